@@ -40,16 +40,48 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+// the shared::cluster address of the same variable in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned mapa_u32(unsigned addr, unsigned rank) {
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// 16 bytes into another CTA's shared memory; on arrival they count on that CTA's mbarrier
+__device__ __forceinline__ void st_async16(unsigned addr, const uint4& v, unsigned bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+               "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+// this CTA's arrival, with the bytes that the phase waits for
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigned parity) {
+  unsigned done;
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+               "selp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done)
+               : "r"(smem_u32(bar)), "r"(parity)
+               : "memory");
+  return done != 0;
+}
+
 // Shared scratch for reductions (static shared memory of the stepper kernel).
 template <class T>
 struct RedBank {
-  T slot[2][kMaxCluster][4];  // [phase][source rank][value]
   T warp[kMaxWarps][4];       // per-warp partials of this CTA
-  T bcast[8];                 // finalised values (double path)
+  T bcast[8];                 // finalised values
 };
 struct RedSmem {
   RedBank<float> f;
   RedBank<double> d;
+  uint4 slot[2][kMaxCluster];    // [phase][source rank]: that rank's partials (up to two values)
+  unsigned long long bar[4];     // the cluster's mbarriers (comm.cuh): two for all-to-all, two for neighbour phases
 };
 template <class T> __device__ __forceinline__ RedBank<T>& bank(RedSmem& rs);
 template <> __device__ __forceinline__ RedBank<float>& bank<float>(RedSmem& rs) { return rs.f; }
@@ -59,75 +91,44 @@ struct NoPost {
   template <class T>
   __device__ __forceinline__ void operator()(T*) const {}
 };
+struct NoPush {
+  __device__ __forceinline__ void operator()() const {}
+};
 
-// Cluster-wide all-reduce of the first NV entries of v (NV <= 4), followed by `post`, which may
-// transform them and fill the NX extra entries v[NV..NV+NX) (for example CG step lengths from
-// the dot products).  Every thread of every CTA of the cluster must call it the same number of
-// times; the result is bitwise identical in every thread of every CTA: the warp butterfly
-// combines the same pairs in every lane, lanes of warp 0 sum the warp partials in warp order,
-// and every CTA writes its partial into every CTA's slot array.  In float every warp sums the
-// slots with a second butterfly (lane r holds rank r) and applies `post` itself.  In double
-// (1/58 of the float rate on this chip) thread 0 sums them in rank order, applies `post` and
-// broadcasts through shared memory.
-// One __syncthreads and one cluster barrier per call (two __syncthreads in double); the
-// cluster barrier also publishes every DSMEM store made before the call.
-template <class T, int NV, int NX = 0, class Post = NoPost>
-__device__ __forceinline__ void cluster_allreduce(T (&v)[NV + NX], RedSmem& rs, int& phase,
-                                                  cg::cluster_group& cluster, int cs, Post post = Post()) {
-  RedBank<T>& rb = bank<T>(rs);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
+// Sum over the warp, the same bits in every lane.
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// In double: an FP64 instruction of a warp holds its FP64 pipe for 64 cycles on this chip
+// (measured, whatever the number of active lanes), so a butterfly costs 320 cycles per warp and
+// value.  Instead the lanes' mantissas are aligned to the largest exponent as 57-bit integers (4
+// guard bits below the 53 of a double, 5 bits of headroom for 32 terms) and summed by three
+// integer reductions; one conversion brings the sum back.  The truncation is at most 32 x 2^-56 of
+// the largest term.  Non-finite, huge and tiny operands take the butterfly.
+__device__ __forceinline__ double warp_sum(double v) {
+  const int hi = __double2hiint(v);
+  const int e = (hi >> 20) & 0x7ff;
+  const int emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (emax < 128 || emax > 0x7f0) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
   }
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) rb.warp[warp][i] = v[i];
-  }
-  __syncthreads();
-  if (warp == 0 && lane < cs) {
-    T s[NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      s[i] = rb.warp[0][i];
-      for (int w = 1; w < nwarps; ++w) s[i] += rb.warp[w][i];
-    }
-    T* dst = cluster.map_shared_rank(&rb.slot[phase][0][0], (unsigned)lane);
-    const int me = (int)cluster.block_rank();
-#pragma unroll
-    for (int i = 0; i < NV; ++i) dst[me * 4 + i] = s[i];
-  }
-  cluster_sync_all();
-  if constexpr (sizeof(T) == 4) {
-    // lane r loads rank r's partial; the same butterfly in every warp of every CTA
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      T t = lane < cs ? rb.slot[phase][lane][i] : T(0);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      v[i] = t;
-    }
-    post(v);
-  } else {
-    if (threadIdx.x == 0) {
-      T t[NV + NX];
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        t[i] = rb.slot[phase][0][i];
-        for (int r = 1; r < cs; ++r) t[i] += rb.slot[phase][r][i];
-      }
-#pragma unroll
-      for (int i = NV; i < NV + NX; ++i) t[i] = T(0);
-      post(t);
-#pragma unroll
-      for (int i = 0; i < NV + NX; ++i) rb.bcast[i] = t[i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < NV + NX; ++i) v[i] = rb.bcast[i];
-  }
-  phase ^= 1;
+  // lanes far below the largest term (denormals among them) shift out to zero
+  const int sh = emax - e;
+  unsigned long long m =
+      (((unsigned long long)((unsigned)(hi & 0xfffff) | 0x100000u) << 32) | (unsigned)__double2loint(v)) << 4;
+  m = sh < 58 ? m >> sh : 0ull;
+  const long long s = hi < 0 ? -(long long)m : (long long)m;
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)s & 0x3fffffu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 22) & 0x3fffffu);
+  const int l2 = __reduce_add_sync(0xffffffffu, (int)(s >> 44));
+  const long long t = (long long)l0 + ((long long)l1 << 22) + ((long long)l2 << 44);
+  if (t == 0) return 0.0;
+  const double d = __ll2double_rn(t);
+  return __hiloint2double(__double2hiint(d) + ((emax - (1023 + 56)) << 20), __double2loint(d));
 }
 
 // ---------------------------------------------------------------------------- slab geometry
@@ -143,29 +144,6 @@ __device__ __forceinline__ void slab_rows(int rows_total, int cs, int rank, int&
   const int base = rows_total / cs, rem = rows_total % cs;
   r0 = rank * base + (rank < rem ? rank : rem);
   R = base + (rank < rem ? 1 : 0);
-}
-
-// Copy this CTA's first and last owned rows of a halo buffer (`buf` points at row -1, row lr at
-// buf + (lr+1)*W) into the halo rows of the CTAs above and below with 16-byte DSMEM stores.
-// Visibility comes from the next cluster barrier.
-template <class T>
-__device__ __forceinline__ void push_halos(T* buf, const Slab& sb, cg::cluster_group& cluster) {
-  constexpr int V = 16 / sizeof(T);           // elements per 16-byte store
-  const int nv = sb.W / V;
-  if (sb.rank > 0) {
-    int r0n, Rn;
-    slab_rows(sb.ny + 1, sb.cs, sb.rank - 1, r0n, Rn);
-    T* dst = cluster.map_shared_rank(buf, (unsigned)(sb.rank - 1));
-    const uint4* s = reinterpret_cast<const uint4*>(buf + 1 * sb.W);                  // own row lr = 0
-    uint4* d = reinterpret_cast<uint4*>(dst + (Rn + 1) * sb.W);                       // its halo row lr = Rn
-    for (int i = threadIdx.x; i < nv; i += blockDim.x) d[i] = s[i];
-  }
-  if (sb.rank < sb.cs - 1) {
-    T* dst = cluster.map_shared_rank(buf, (unsigned)(sb.rank + 1));
-    const uint4* s = reinterpret_cast<const uint4*>(buf + sb.R * sb.W);               // own row lr = R-1
-    uint4* d = reinterpret_cast<uint4*>(dst);                                        // its halo row lr = -1
-    for (int i = threadIdx.x; i < nv; i += blockDim.x) d[i] = s[i];
-  }
 }
 
 // x^(p-1) and x^p for an even integer p >= 2 by repeated squaring (exact operation order is

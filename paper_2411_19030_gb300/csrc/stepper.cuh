@@ -64,6 +64,7 @@ struct Stepper {
   float* tl_gs = nullptr;    // group sums of the vector being restricted, [R * G]
   int* tl_gagg = nullptr;    // local aggregate (row-major in [naj][nax]) of every group, [R * G]
   int* tl_cov = nullptr;     // first / last rank covering each aggregate row, [nay][2]
+  unsigned tl_bytes = 0;     // restricted partials that every rank receives from all ranks together
   // V(1,1) two-grid cycle (P.tl_vc), see vcycle; aj0 / naj then cover the halo rows too
   bool vc = false;
   int ajo0 = 0, najo = 0;    // aggregate rows of the owned rows (the restriction's partials)
@@ -193,6 +194,12 @@ struct Stepper {
             tl_cov[2 * J] = lo;
             tl_cov[2 * J + 1] = hi;
           }
+          for (int q = 0; q < P.cs; ++q) {
+            int r0q, Rq, J0q, R1q;
+            slab_rows(P.ny + 1, P.cs, q, r0q, Rq);
+            l1_rows_of_slab(r0q, Rq, J0q, R1q);
+            tl_bytes += 4u * naxp * (l3_agg(J0q + R1q - 1, P.cm, P.nay) - l3_agg(J0q, P.cm, P.nay) + 1);
+          }
         } else {
         tl_gs = t;    t += groups;
         tl_gagg = reinterpret_cast<int*>(t);  t += P.tl_vc ? groups + 2 * (W / kGroup) : groups;
@@ -218,6 +225,12 @@ struct Stepper {
           }
         }
         naj = ajhi - aj0 + 1;
+        for (int q = 0; q < P.cs; ++q) {
+          int r0q, Rq, a, bq;
+          slab_rows(P.ny + 1, P.cs, q, r0q, Rq);
+          coarse_rows_of_slab(r0q, Rq, P.cm, P.nay, a, bq);
+          tl_bytes += 4u * naxp * (bq - a + 1);
+        }
         for (int J = threadIdx.x; J < P.nay; J += blockDim.x) {
           int lo = -1, hi = -1;
           for (int q = 0; q < P.cs; ++q) {
@@ -264,9 +277,9 @@ struct Stepper {
     return (ix >= 0 && ix <= P.nx) ? (sb.r0 + lr) * (P.nx + 1) + ix : -1;
   }
 
-  template <class T, int NV, int NX = 0, class Post = NoPost>
-  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post()) {
-    comm.template allreduce<T, NV, NX, Post>(v, sb.cs, post);
+  template <class T, int NV, int NX = 0, class Post = NoPost, class Push = NoPush>
+  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post(), Push push = Push()) {
+    comm.template allreduce<T, NV, NX, Post, Push>(v, sb.cs, post, push);
   }
 
   // Select the operator C/dt + K (fine) or C/dtau + K (coarse): per-node FP64 weights for the
@@ -452,8 +465,7 @@ struct Stepper {
   template <class T>
   __device__ void exchange(T* buf) {
     __syncthreads();
-    comm.push_halos(buf, sb);
-    comm.sync();
+    comm.exchange(buf, sb);
   }
   __device__ void exchange_x64() { exchange(x64); }
 
@@ -581,6 +593,7 @@ struct Stepper {
         comm.publish_tl(tl_slot, dst, chunk, lane & 15, sb.cs);
       }
     }
+    comm.expect_tl(tl_bytes);
   }
 
   // After the cluster barrier that follows coarse_restrict_push: qc = sum over the covering
@@ -647,18 +660,18 @@ struct Stepper {
   }
 
   // The owned edge rows (0 and R-1) of a per-thread vector into the neighbours' two-row buffer
-  // `edge` ([0]: the row below the slab, [1]: the row above), straight from registers;
-  // visible after the next barrier.
-  __device__ void put_edges(Real* edge, const Real (&v)[NG][4]) {
+  // `edge` ([0]: the row below the slab, [1]: the row above), straight from registers; visible
+  // after the next all-reduce, or with `own` after comm.finish_edges().
+  __device__ void put_edges(Real* edge, const Real (&v)[NG][4], bool own) {
     comm.begin_edges();
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
       const int lr = l0 / sb.W - 1;
-      if (lr == 0 || lr == sb.R - 1) comm.put_edge(edge, lr, l0 - (lr + 1) * sb.W, v[k], sb);
+      if (lr == 0 || lr == sb.R - 1) comm.put_edge(edge, lr, l0 - (lr + 1) * sb.W, v[k], sb, own);
     }
-    comm.end_edges(edge, sb);
+    comm.end_edges(edge, sb, own);
   }
 
   // offset in a rows -1..R buffer of entry i of the two halo rows ([0, W): row -1, [W, 2W): row R)
@@ -702,7 +715,7 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? rf[k][j] - t[j] : 0.f;
     }
     coarse_restrict_push(w);
-    comm.sync();
+    comm.finish_tl();
     coarse_gather(true, 0.f);
     for (int gi = threadIdx.x; gi < (sb.R + 2) * G; gi += blockDim.x) {
       const int a = tl_gagg[gi];
@@ -797,7 +810,7 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? rf[k][j] - t[j] : 0.f;
     }
     coarse_restrict_push(w);
-    comm.sync();
+    comm.finish_tl();
     coarse_gather(true, 0.f);
     for (int gi = threadIdx.x; gi < (sb.R + 2) * G; gi += blockDim.x) {
       const int a = tl_gagg[gi];
@@ -849,8 +862,7 @@ struct Stepper {
   // refresh the 2h halo rows of every CTA from the neighbours' owned rows
   __device__ void exchange_l1(float* buf) {
     __syncthreads();
-    comm.push_halos_rows(buf, W1, R1, R1b, sb.rank, sb.cs);
-    comm.sync();
+    comm.exchange_rows(buf, W1, R1, R1b, sb.rank, sb.cs);
   }
 
   // P.tl_nu damped-Jacobi steps of A1_s e = s from e = 0 on the owned 2h rows, with the 2h halo
@@ -926,7 +938,8 @@ struct Stepper {
       const int item0 = 4 * c, ajl0 = item0 / naxp, ax0 = item0 - ajl0 * naxp;
       comm.publish_tl(tl_slot, sb.rank * ncp + (ajo0 + ajl0) * naxp + ax0, chunk, t & 15, sb.cs);
     }
-    comm.sync();
+    comm.expect_tl(tl_bytes);
+    comm.finish_tl();
     coarse_gather(true, 0.f);
     // u1 = e1 + P2 ec on the owned and halo 2h rows
     for (int t = threadIdx.x; t < (R1 + 2) * n1; t += blockDim.x) {
@@ -1115,18 +1128,16 @@ struct Stepper {
         v[0] = vcycle_local(r);
       } else if (vc) {
         // r on the halo rows from the neighbours' owned edge rows
-        put_edges(vrh, r);
-        comm.sync();
+        put_edges(vrh, r, true);
+        comm.finish_edges();
         v[0] = vcycle(r);
       } else if (tl) {
         coarse_restrict_push(r);
-        comm.sync();
+        comm.finish_tl();
         coarse_gather(true, 0.f);
         v[0] = prolong_precondition(r);
       }
-      __syncthreads();
-      comm.push_halos(zbuf, sb);
-      allreduce<Real, 1>(v);
+      allreduce<Real, 1>(v, NoPost(), [&] { comm.push_halos(zbuf, sb); });
       rz = v[0];
     }
     int it = 0;
@@ -1153,7 +1164,7 @@ struct Stepper {
       if (vc && !l3 && P.tl_nu < 2) {
         // q's owned edge rows to the neighbours, whose copies of r on their halo rows follow
         // the same recurrence (visible after the all-reduce's barrier)
-        put_edges(vqh, q);
+        put_edges(vqh, q, false);
       } else if (tl && !vc) {
         coarse_restrict_push(q);             // visible after the all-reduce's cluster barrier
       }
@@ -1191,9 +1202,7 @@ struct Stepper {
       } else if (tl) {
         v[0] = prolong_precondition(r);
       }
-      __syncthreads();
-      comm.push_halos(zbuf, sb);
-      allreduce<Real, 2, 1>(v, [rz_c](Real* t) { t[2] = t[0] / rz_c; });
+      allreduce<Real, 2, 1>(v, [rz_c](Real* t) { t[2] = t[0] / rz_c; }, [&] { comm.push_halos(zbuf, sb); });
       ++it;
       if (!(v[1] > target2)) done = true;  // NaN keeps iterating until the limit
       beta = v[2];
@@ -1642,6 +1651,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_kernel(const __gri
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   __shared__ RedSmem rs;
   ClusterComm comm(rs);
+  comm.bind(P);
   Stepper<Real, NG, ClusterComm> st(P, comm, dyn_smem);
   // every CTA of the cluster has initialised its shared memory before any DSMEM traffic
   cluster_sync_all();
@@ -1694,6 +1704,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_batch_kernel(const
     const int t = s_task;                      // identical in every CTA: the loop is uniform
     if (t >= ntasks) break;
     const int2 tk = tasks[t];
+    comm.bind(table[tk.x]);
     Stepper<Real, NG, ClusterComm> st(table[tk.x], comm, dyn_smem);
     cluster_sync_all();
     run_task<Real, NG, KIND>(st, tk.y);
