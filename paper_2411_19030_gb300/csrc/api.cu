@@ -1,5 +1,6 @@
 // api.cu -- the C ABI (include/ptg.h): op lifecycle, argument checks, plan choice, launches.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -62,6 +63,8 @@ struct ptg_op {
   // device workspace
   double *k = nullptr, *c = nullptr, *dk = nullptr, *dc = nullptr;
   double* wE = nullptr;     // [2][3][PEe]: element (D, S, T) weights for dt and dtau (padded)
+  float* ffw = nullptr;     // [2][10][PN]: the weights of C/dt + K and C/dtau + K as float pairs
+  double ff_scale[2] = {1.0, 1.0};
   double* nodew = nullptr;  // [15][PN]: per-node weights of C/dt + K, C/dtau + K and C (padded)
   double* fload = nullptr;
   double *q_elem = nullptr, *q_time = nullptr;
@@ -524,6 +527,8 @@ void base_params(const ptg_op* op, StepParams& P) {
   P.A_fine = nw(0);
   P.A_coarse = nw(5);
   P.mass = nw(10);
+  P.ff_fine = FFWeights{op->ffw + kSlack, (int)PN, op->ff_scale[0]};
+  P.ff_coarse = FFWeights{op->ffw + 10 * PN + kSlack, (int)PN, op->ff_scale[1]};
   if (op->w32) {
     P.w32 = op->w32 + kSlack;
     P.w32_stride = (int)PEe;
@@ -666,7 +671,7 @@ bool window_covers(int j0, int rows, int lo, int hi) { return lo >= j0 && hi < j
 void ptg_op_free(ptg_op* op);
 
 void free_all(ptg_op* op) {
-  void* ptrs[] = {op->k, op->c, op->dk, op->dc, op->wE, op->nodew, op->fload,
+  void* ptrs[] = {op->ffw, op->k, op->c, op->dk, op->dc, op->wE, op->nodew, op->fload,
                   op->q_elem, op->q_time, op->dirichlet, op->sens_partial, op->lam_prev, op->scratch, op->stats,
                   op->g_red, op->g_bar, op->g_halo, op->g_tl,
                   op->tl_Ac, op->tl_band, op->tl_X, op->tl_Ainv,
@@ -928,6 +933,14 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
   A(&op->dc, op->Ne * sizeof(double));
   A(&op->wE, 6 * PEe * sizeof(double));
   A(&op->nodew, 15 * PN * sizeof(double));
+  A(&op->ffw, 20 * PN * sizeof(float));
+  // the power of two that brings the largest possible diagonal of C/step + K to order one
+  for (int i = 0; i < 2; ++i) {
+    const double step = i ? op->dtau : time->dt;
+    const double d = 4.0 * (4.0 / 6.0 * std::max(mat->k0, mat->kmin) +
+                            4.0 * std::max(mat->c0, mat->cmin) * grid->h * grid->h / (36.0 * step));
+    op->ff_scale[i] = std::ldexp(1.0, -std::ilogb(d));
+  }
   A(&op->fload, op->Nn * sizeof(double));
   A(&op->q_elem, op->Ne * sizeof(double));
   A(&op->q_time, (time->Nt + 1) * sizeof(double));
@@ -1048,6 +1061,7 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
   if (e == cudaSuccess) e = cudaMemset(op->fload, 0, op->Nn * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(op->wE, 0, 6 * PEe * sizeof(double));          // slack stays zero
   if (e == cudaSuccess) e = cudaMemset(op->nodew, 0, 15 * PN * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemset(op->ffw, 0, 20 * PN * sizeof(float));
   if (e != cudaSuccess) {
     int rc = cuda_fail(e, "ptg_op_create");
     free_all(op);
@@ -1183,6 +1197,11 @@ int ptg_fe_assemble_operator(ptg_op* op, const double* rho_d, cudaStream_t strea
   out.wEf = op->wE + kSlack;
   out.wEc = op->wE + 3 * PEe + kSlack;
   for (int i = 0; i < 15; ++i) out.node[i] = op->nodew + i * PN + kSlack;
+  for (int i = 0; i < 2; ++i) {
+    out.ff[i] = op->ffw + (size_t)i * 10 * PN + kSlack;
+    out.ff_scale[i] = op->ff_scale[i];
+  }
+  out.ff_stride = (int)PN;
   out.fload = op->fload;
   PTG_CUDA(launch_assemble(op->g.nx, op->g.ny, op->g.h, op->mat, op->tm.dt, op->dtau, rho_d, op->q_elem,
                            op->dirichlet, out, op->stats, stream));

@@ -8,6 +8,9 @@ namespace ptg {
 
 struct NodeOut {
   double* p[15];
+  float* ff[2];
+  int ff_stride;
+  double ff_scale[2];
 };
 
 __device__ __forceinline__ void assemble_error(DevStats* st, int code) {
@@ -103,6 +106,14 @@ __global__ void assemble_nodes(int nx, int ny, int W, int PE, double h, const do
   }
 #pragma unroll
   for (int i = 0; i < 15; ++i) out.p[i][pn] = v[i];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) {
+    const double s = v[i] * out.ff_scale[i / 5];
+    const float h = (float)s;
+    float* f = out.ff[i / 5] + (size_t)(i % 5) * out.ff_stride + pn;
+    f[0] = h;
+    f[5 * (size_t)out.ff_stride] = (float)(s - (double)h);
+  }
 }
 
 // Unit-time load vector f_i = sum_e q_e int N_i = sum over the elements around node i of
@@ -134,6 +145,11 @@ cudaError_t launch_assemble(int nx, int ny, double h, const ptg_material& m, dou
   if (e != cudaSuccess) return e;
   NodeOut no;
   for (int i = 0; i < 15; ++i) no.p[i] = out.node[i];
+  for (int i = 0; i < 2; ++i) {
+    no.ff[i] = out.ff[i];
+    no.ff_scale[i] = out.ff_scale[i];
+  }
+  no.ff_stride = out.ff_stride;
   const int nn_pad = (ny + 3) * W;
   assemble_nodes<<<(nn_pad + 255) / 256, 256, 0, stream>>>(nx, ny, W, PEe, h, out.wEf, out.wEc, out.c, no);
   e = cudaGetLastError();

@@ -110,7 +110,7 @@ struct ClusterComm {
       union { uint4 u; T t[16 / sizeof(T)]; } pk;
       pk.u = make_uint4(0, 0, 0, 0);
 #pragma unroll
-      for (int i = 0; i < NV; ++i) pk.t[i] = warp_sum(lane < nwarps ? rb.warp[lane][i] : T(0));
+      for (int i = 0; i < NV; ++i) pk.t[i] = warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
       if (lane < cs)
         st_async16(mapa_u32(smem_u32(&rs.slot[na & 1][rank()]), (unsigned)lane), pk.u,
                    mapa_u32(smem_u32(bar_a()), (unsigned)lane));
@@ -119,9 +119,9 @@ struct ClusterComm {
       pk.u = rs.slot[na & 1][lane < cs ? lane : 0];
       T t[NV + NX];
 #pragma unroll
-      for (int i = 0; i < NV; ++i) t[i] = warp_sum(lane < cs ? pk.t[i] : T(0));
+      for (int i = 0; i < NV; ++i) t[i] = warp_sum(lane < cs ? pk.t[i] : T{});
 #pragma unroll
-      for (int i = NV; i < NV + NX; ++i) t[i] = T(0);
+      for (int i = NV; i < NV + NX; ++i) t[i] = T{};
       post(t);
       if (lane == 0) {
 #pragma unroll
@@ -234,6 +234,12 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+template <class T>
+__device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
+__device__ __forceinline__ ff ldcg(const ff* p) {
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return make_ff(v.x, v.y);
+}
 __device__ __forceinline__ void st_release_gpu(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -309,62 +315,42 @@ struct GridComm {
     RedBank<T>& rb = bank<T>(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    }
+    for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
     if (lane == 0) {
 #pragma unroll
       for (int i = 0; i < NV; ++i) rb.warp[warp][i] = v[i];
     }
     __syncthreads();
     push();
-    double* slots = P.g_red + (size_t)phase * kMaxGrid * 4;
-    if (threadIdx.x == 0) {
+    T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 4);   // 4 values per block
+    if (warp == 0) {
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        T s = rb.warp[0][i];
-        for (int w = 1; w < nwarps; ++w) s += rb.warp[w][i];
-        slots[(int)blockIdx.x * 4 + i] = (double)s;  // exact for T = float too
+        const T s = warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
+        if (lane == 0) slots[(int)blockIdx.x * 4 + i] = s;
       }
     }
     barrier();
-    if constexpr (sizeof(T) == 4) {
-      // every warp: lane-strided sums over the ranks, then the same butterfly
+    // warp 0: lane-strided sums over the ranks and the warp's sum, then `post`; broadcast
+    if (warp == 0) {
+      T t[NV + NX];
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        T t = T(0);
-        for (int r = lane; r < G; r += 32) t += (T)__ldcg(slots + (base + r) * 4 + i);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        v[i] = t;
+        T a = T{};
+        for (int r = lane; r < G; r += 32) a = a + ldcg(slots + (base + r) * 4 + i);
+        t[i] = warp_sum(a);
       }
-      post(v);
-    } else {
-      // warp 0 sums (lane-strided, then the butterfly), thread 0 applies `post` and
-      // broadcasts: one lane of FP64 work for the divisions instead of every thread
-      if (warp == 0) {
-        T t[NV + NX];
 #pragma unroll
-        for (int i = 0; i < NV; ++i) {
-          T a = T(0);
-          for (int r = lane; r < G; r += 32) a += (T)__ldcg(slots + (base + r) * 4 + i);
+      for (int i = NV; i < NV + NX; ++i) t[i] = T{};
+      post(t);
+      if (lane == 0) {
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-          t[i] = a;
-        }
-        if (lane == 0) {
-#pragma unroll
-          for (int i = NV; i < NV + NX; ++i) t[i] = T(0);
-          post(t);
-#pragma unroll
-          for (int i = 0; i < NV + NX; ++i) rb.bcast[i] = t[i];
-        }
+        for (int i = 0; i < NV + NX; ++i) rb.bcast[i] = t[i];
       }
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < NV + NX; ++i) v[i] = rb.bcast[i];
     }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NV + NX; ++i) v[i] = rb.bcast[i];
     phase ^= 1;
   }
 

@@ -19,6 +19,7 @@
 #pragma once
 #include <cooperative_groups.h>
 #include <cstdint>
+#include "ff.cuh"
 #include "ptg_internal.h"
 
 namespace ptg {
@@ -80,12 +81,14 @@ struct RedBank {
 struct RedSmem {
   RedBank<float> f;
   RedBank<double> d;
+  RedBank<ff> p;
   uint4 slot[2][kMaxCluster];    // [phase][source rank]: that rank's partials (up to two values)
   unsigned long long bar[4];     // the cluster's mbarriers (comm.cuh): two for all-to-all, two for neighbour phases
 };
 template <class T> __device__ __forceinline__ RedBank<T>& bank(RedSmem& rs);
 template <> __device__ __forceinline__ RedBank<float>& bank<float>(RedSmem& rs) { return rs.f; }
 template <> __device__ __forceinline__ RedBank<double>& bank<double>(RedSmem& rs) { return rs.d; }
+template <> __device__ __forceinline__ RedBank<ff>& bank<ff>(RedSmem& rs) { return rs.p; }
 
 struct NoPost {
   template <class T>
@@ -99,6 +102,12 @@ struct NoPush {
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ ff warp_sum(ff v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = v + make_ff(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o));
   return v;
 }
 // In double: an FP64 instruction of a warp holds its FP64 pipe for 64 cycles on this chip
@@ -225,6 +234,64 @@ __device__ __forceinline__ void stencil_node64(const T* __restrict__ x, int loc0
     a = fma(NWo[j], (double)xh[j], a);         // north-west
     a = fma(nwb[j], (double)xl[j + 2], a);     // south-east = NW weight of the SE neighbour
     y[j] = a;
+  }
+}
+
+// y = A z for the 4 nodes of a group: z in float, the per-node weights as float pairs (FFWeights,
+// global memory), summed in pairs.  Row by row, which keeps few weights live.
+__device__ __forceinline__ void stencil_ff(const float* __restrict__ z, int loc0, const FFWeights& nw, int go, int W,
+                                           ff (&y)[4]) {
+  const float *hi = nw.w + go, *lo = hi + 5 * (size_t)nw.stride;
+  const size_t st = (size_t)nw.stride;
+  auto ld = [](const float* p, float (&v)[4]) {
+    const float4 c = *reinterpret_cast<const float4*>(p);
+    v[0] = c.x; v[1] = c.y; v[2] = c.z; v[3] = c.w;
+  };
+  float v[6], ah[4], al[4], bh[4], bl[4], ch[4], cl[4];
+  // the node's row: C, E of the node, E of the west neighbour
+  load_window(z, loc0, v);
+  ld(hi, ah);
+  ld(lo, al);
+  ld(hi + st, bh);
+  ld(lo + st, bl);
+  ch[0] = hi[st - 1];
+  cl[0] = lo[st - 1];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float p, e;
+    ff_prod(make_ff(ah[j], al[j]), v[j + 1], p, e);
+    ff a = make_ff(p, e);
+    a = ff_acc(a, make_ff(bh[j], bl[j]), v[j + 2]);
+    y[j] = ff_acc(a, j == 0 ? make_ff(ch[0], cl[0]) : make_ff(bh[j - 1], bl[j - 1]), v[j]);
+  }
+  // the row above: N, NE, NW of the node
+  load_window(z, loc0 + W, v);
+  ld(hi + 2 * st, ah);
+  ld(lo + 2 * st, al);
+  ld(hi + 3 * st, bh);
+  ld(lo + 3 * st, bl);
+  ld(hi + 4 * st, ch);
+  ld(lo + 4 * st, cl);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    y[j] = ff_acc(y[j], make_ff(ah[j], al[j]), v[j + 1]);
+    y[j] = ff_acc(y[j], make_ff(bh[j], bl[j]), v[j + 2]);
+    y[j] = ff_acc(y[j], make_ff(ch[j], cl[j]), v[j]);
+  }
+  // the row below: N of the south, NE of the south-west, NW of the south-east neighbour
+  load_window(z, loc0 - W, v);
+  ld(hi + 2 * st - W, ah);
+  ld(lo + 2 * st - W, al);
+  ld(hi + 3 * st - W, bh);
+  ld(lo + 3 * st - W, bl);
+  ld(hi + 4 * st - W, ch);
+  ld(lo + 4 * st - W, cl);
+  const ff ne = make_ff(hi[3 * st - W - 1], lo[3 * st - W - 1]), nw4 = make_ff(hi[4 * st - W + 4], lo[4 * st - W + 4]);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    y[j] = ff_acc(y[j], make_ff(ah[j], al[j]), v[j + 1]);
+    y[j] = ff_acc(y[j], j == 0 ? ne : make_ff(bh[j - 1], bl[j - 1]), v[j]);
+    y[j] = ff_acc(y[j], j == 3 ? nw4 : make_ff(ch[j + 1], cl[j + 1]), v[j + 2]);
   }
 }
 

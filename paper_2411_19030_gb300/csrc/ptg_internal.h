@@ -53,6 +53,15 @@ struct NodeWeights {
   const double* NW;
 };
 
+// The same weights as float pairs for the CG of the FP64 kinds (ff.cuh): ten arrays in the padded
+// node layout, stride floats apart, the high parts of (C, E, N, NE, NW) and then their low parts,
+// times a power of two (scale) that makes the largest of order one.
+struct FFWeights {
+  const float* w;            // the first non-slack entry of the first array
+  int stride;
+  double scale;
+};
+
 // Geometric multigrid hierarchy of the coarse-step operator (mg.cu): level l has nx, ny
 // elements (halved per level), the padded width W, arrays of plen floats each (slack included),
 // its six weight arrays (C, E, N, NE, NW, omega/diag) at woff in the op's weight buffer, and its
@@ -89,6 +98,8 @@ struct StepParams {
   NodeWeights A_fine;        // per-node weights of C/dt + K
   NodeWeights A_coarse;      // per-node weights of C/dtau + K
   NodeWeights mass;          // per-node weights of C
+  FFWeights ff_fine;         // A_fine and A_coarse as float pairs
+  FFWeights ff_coarse;
   const double* dk;          // [Ne]
   const double* dc;          // [Ne]
   const double* fload;       // [Nn] unit-time load, zero on Dirichlet nodes
@@ -285,8 +296,8 @@ inline size_t stepper_smem_bytes(int nx, int rmax, int real_bytes, bool keep_ax 
   b += halo * sizeof(double);                  // x64: FP64 state with halos
   b += own * sizeof(double);                   // b64: FP64 right-hand side
   if (keep_ax) b += own * sizeof(double);      // ax64: A x of the last residual evaluation (optional)
-  b += halo * real_bytes;                      // zbuf: CG stencil operand with halos
-  b += own * real_bytes;                       // dinv: Jacobi inverse diagonal (0 off the unknowns)
+  b += halo * 4;                               // zbuf: CG stencil operand with halos (float in both)
+  b += own * 4;                                // dinv: Jacobi inverse diagonal (0 off the unknowns)
   if (real_bytes == 4) b += 3 * elems * 4;     // (D, S, T) element weights for the FP32 CG
   return (b + 15) & ~size_t(15);
 }
@@ -335,6 +346,9 @@ struct AssembleOut {
   double *k, *c, *dk, *dc;            // [Ne]
   double *wEf, *wEc;                  // [3][(ny+2) W] element (D, S, T) weights
   double* node[15];                   // per-node weights: A_fine C,E,N,NE,NW; A_coarse ...; mass ...
+  float* ff[2];                       // float pairs of A_fine and A_coarse (FFWeights), ff_stride apart
+  int ff_stride;
+  double ff_scale[2];                 // their powers of two
   double* fload;                      // [Nn]
 };
 cudaError_t launch_assemble(int nx, int ny, double h, const ptg_material& m, double dt, double dtau, const double* rho,

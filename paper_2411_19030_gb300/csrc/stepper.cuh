@@ -6,9 +6,9 @@
 // nodes of a row.  Each solve of (C/dt + K) x = b (Eq. 2.7 / 4.4) is a Jacobi-preconditioned
 // CG in precision Real inside an FP64 residual loop:
 //     r = b - A x            (FP64, per-node FP64 weights: 9 FMAs per node)
-//     while ||r|| > rtol ||b||:   CG on A d = r / ||r||  (Real),  x += ||r|| d,  r = b - A x
-// With Real = double the first CG already meets the tolerance (plain FP64 PCG on the same
-// per-node weights); with Real = float the CG uses FP32 element weights held in shared memory
+//     while ||r|| > rtol ||b||:   CG on A d = r / 2^k,  x += 2^k d,  r = b - A x
+// With Real = double the CG works in pairs of floats (ff.cuh) on the same per-node weights and the
+// first CG already meets the tolerance; with Real = float the CG uses FP32 element weights held in shared memory
 // and this is iterative refinement with FP64 residuals.  CG carries q = A p by the recurrence
 // q_{k+1} = A z_{k+1} + beta q_k, so each iteration has two cluster reductions and the halo
 // exchange of z, the only stencil operand, rides on the second one.
@@ -28,9 +28,12 @@
 
 namespace ptg {
 
-template <class Real, int NG, class Comm>
+// COARSE: the kinds that solve with C/dtau + K, which alone have the two-level preconditioners.
+template <class Real, int NG, class Comm, bool COARSE>
 struct Stepper {
   static constexpr bool kMixed = std::is_same<Real, float>::value;
+  // the CG's vectors and scalars: floats, or float pairs for the FP64 kinds (ff.cuh)
+  using V = typename std::conditional<kMixed, float, ff>::type;
 
   const StepParams& P;
   Comm& comm;
@@ -38,8 +41,8 @@ struct Stepper {
   // shared memory (each pointer at the first non-slack entry)
   double* x64;      // FP64 state, rows -1..R
   double* b64;      // FP64 right-hand side, rows 0..R-1
-  Real* zbuf;       // CG stencil operand, rows -1..R
-  Real* dinv;       // Jacobi inverse diagonal, rows 0..R-1 (0 on Dirichlet and pad nodes)
+  float* zbuf;      // CG stencil operand, rows -1..R
+  float* dinv;      // Jacobi inverse diagonal, rows 0..R-1 (0 on Dirichlet and pad nodes)
   float* wd = nullptr;  // FP32 element weights (D, S, T), element rows r0-1..r0+R-1 (FP32 CG, V-cycle)
   float* ws = nullptr;
   float* wt = nullptr;
@@ -47,6 +50,7 @@ struct Stepper {
   int loc0[NG];
   unsigned fmask = 0;   // bit 4k+j: node j of group k is an unknown (free, not a pad)
   NodeWeights A;    // per-node FP64 weights of the current operator
+  FFWeights ffw;    // the same as float pairs (FP64 kinds)
   double step_dt = 0.0;
   double inv_dt = 0.0;
   int gshift = 0;   // offset from a halo-buffer node to the same node of the global padded arrays
@@ -68,8 +72,8 @@ struct Stepper {
   // V(1,1) two-grid cycle (P.tl_vc), see vcycle; aj0 / naj then cover the halo rows too
   bool vc = false;
   int ajo0 = 0, najo = 0;    // aggregate rows of the owned rows (the restriction's partials)
-  Real* vqh = nullptr;       // q on the halo rows -1 and R (the neighbours' edge rows), [2][W]
-  Real* vrh = nullptr;       // r on the halo rows -1 and R, [2][W]
+  V* vqh = nullptr;       // q on the halo rows -1 and R (the neighbours' edge rows), [2][W]
+  V* vrh = nullptr;       // r on the halo rows -1 and R, [2][W]
   float* vy = nullptr;       // y = S r, then u = y + P ec, rows -1..R
   float* vsd = nullptr;      // S = omega D^-1, rows -1..R (0 off the unknowns)
   float* ve0 = nullptr;      // slab-local smoothing (P.tl_nu >= 2): ping-pong iterates, rows -1..R,
@@ -106,17 +110,17 @@ struct Stepper {
     double* x64b = reinterpret_cast<double*>(p);  p += sizeof(double) * halo;
     double* b64b = reinterpret_cast<double*>(p);  p += sizeof(double) * own;
     double* axb = reinterpret_cast<double*>(p);   p += P.keep_ax ? sizeof(double) * own : 0;
-    Real* zb = reinterpret_cast<Real*>(p);        p += sizeof(Real) * halo;
-    Real* db = reinterpret_cast<Real*>(p);        p += sizeof(Real) * own;
+    float* zb = reinterpret_cast<float*>(p);      p += sizeof(float) * halo;
+    float* db = reinterpret_cast<float*>(p);      p += sizeof(float) * own;
     float* eb = reinterpret_cast<float*>(p);
     for (int i = threadIdx.x; i < halo; i += blockDim.x) {
       x64b[i] = 0.0;
-      zb[i] = Real(0);
+      zb[i] = 0.f;
     }
     for (int i = threadIdx.x; i < own; i += blockDim.x) {
       b64b[i] = 0.0;
       if (P.keep_ax) axb[i] = 0.0;
-      db[i] = Real(0);
+      db[i] = 0.f;
     }
     if constexpr (kMixed) {
       for (int i = threadIdx.x; i < 3 * elems; i += blockDim.x) eb[i] = 0.f;
@@ -134,10 +138,10 @@ struct Stepper {
         tl_ec = t;    t += P.tl_naj * naxp;
         if (P.tl_vc) {
           // every array a multiple of 4 words, so each starts 16-byte aligned
-          constexpr int rw = (int)(sizeof(Real) / 4);
+          constexpr int rw = (int)(sizeof(V) / 4);
           float* v0 = t;
-          vqh = reinterpret_cast<Real*>(t);  t += 2 * W * rw;
-          vrh = reinterpret_cast<Real*>(t);  t += 2 * W * rw;
+          vqh = reinterpret_cast<V*>(t);  t += 2 * W * rw;
+          vrh = reinterpret_cast<V*>(t);  t += 2 * W * rw;
           vy = t + kSlack;   t += halo;
           vsd = t + kSlack;  t += halo;
           if (P.tl_nu >= 2) {
@@ -285,8 +289,10 @@ struct Stepper {
   // Select the operator C/dt + K (fine) or C/dtau + K (coarse): per-node FP64 weights for the
   // residual (and the FP64 CG), FP32 element weights in shared memory for the FP32 CG, and
   // the Jacobi inverse diagonal (zero on Dirichlet and pad nodes).
-  __device__ void set_operator(bool coarse) {
+  __device__ void set_operator() {
+    constexpr bool coarse = COARSE;
     A = coarse ? P.A_coarse : P.A_fine;
+    ffw = coarse ? P.ff_coarse : P.ff_fine;
     step_dt = coarse ? P.dtau : P.dt;
     inv_dt = 1.0 / step_dt;
     ax_valid = false;
@@ -322,9 +328,12 @@ struct Stepper {
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const int g = gnode(l0, j);
-        Real v = Real(0);
+        float v = 0.f;
         if (g >= 0 && P.dirichlet[g] == 0) {
-          v = Real(1) / (Real)A.C[l0 + gshift + j];
+          // the float pairs are scaled: the CG of the FP64 kinds without a two-level form takes 1/C
+          // in their scale
+          const double c = A.C[l0 + gshift + j];
+          v = 1.f / (float)(kMixed || tl ? c : c * ffw.scale);
           fmask |= 1u << (kGroup * k + j);
         }
         dinv[l0 + j] = v;
@@ -480,7 +489,7 @@ struct Stepper {
       stencil_node64<double>(x64, l0, P.mass, l0 + gshift, sb.W, y);
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
-        const bool free_node = dinv[l0 + j] != Real(0);
+        const bool free_node = dinv[l0 + j] != 0.f;
         b64[l0 + j] = free_node ? fma(y[j], inv_dt, src(gnode(l0, j))) : 0.0;
       }
     }
@@ -529,15 +538,11 @@ struct Stepper {
     return rr;
   }
 
-  __device__ __forceinline__ void apply_A(const Real* z, int l0, Real (&w)[4]) const {
-    if constexpr (kMixed) {
+  __device__ __forceinline__ void apply_A(const float* z, int l0, V (&w)[4]) const {
+    if constexpr (kMixed)
       stencil_elem32(z, wd, ws, wt, l0, sb.W, w);
-    } else {
-      double y[4];
-      stencil_node64<double>(z, l0, A, l0 + gshift, sb.W, y);
-#pragma unroll
-      for (int j = 0; j < kGroup; ++j) w[j] = y[j];
-    }
+    else
+      stencil_ff(z, l0, ffw, l0 + gshift, sb.W, w);
   }
 
   // Two-level preconditioner M^-1 = D^-1 + P Ac^-1 P^T of the coarse-step solves (CG in either
@@ -556,7 +561,7 @@ struct Stepper {
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       if (loc0[k] < 0) continue;
-      tl_gs[threadIdx.x + k * blockDim.x] = (float)((v[k][0] + v[k][1]) + (v[k][2] + v[k][3]));
+      tl_gs[threadIdx.x + k * blockDim.x] = (f32(v[k][0]) + f32(v[k][1])) + (f32(v[k][2]) + f32(v[k][3]));
     }
     __syncthreads();
     // 4 lanes per local aggregate (16 lanes per chunk of 4 aggregates), each summing every
@@ -641,19 +646,18 @@ struct Stepper {
 
   // z = D^-1 r + P ec on the owned nodes (0 off the unknowns), written to zbuf; returns the
   // local part of (r, z).
-  __device__ Real prolong_precondition(const Real (&r)[NG][4]) {
-    Real rz = Real(0);
+  __device__ V prolong_precondition(const V (&r)[NG][4]) {
+    V rz = V{};
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
-      const Real e = (Real)tl_ec[tl_gagg[threadIdx.x + k * blockDim.x]];
+      const float e = tl_ec[tl_gagg[threadIdx.x + k * blockDim.x]];
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
-        const Real di = dinv[l0 + j];
-        const Real z = unknown(k, j) ? fma(di, r[k][j], e) : Real(0);
+        const float z = unknown(k, j) ? fmaf(dinv[l0 + j], f32(r[k][j]), e) : 0.f;
         zbuf[l0 + j] = z;
-        rz = fma(r[k][j], z, rz);
+        rz = vdot(rz, r[k][j], z);
       }
     }
     return rz;
@@ -662,7 +666,7 @@ struct Stepper {
   // The owned edge rows (0 and R-1) of a per-thread vector into the neighbours' two-row buffer
   // `edge` ([0]: the row below the slab, [1]: the row above), straight from registers; visible
   // after the next all-reduce, or with `own` after comm.finish_edges().
-  __device__ void put_edges(Real* edge, const Real (&v)[NG][4], bool own) {
+  __device__ void put_edges(V* edge, const V (&v)[NG][4], bool own) {
     comm.begin_edges();
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
@@ -685,21 +689,21 @@ struct Stepper {
   // aggregate rows its halo rows touch from the same restricted vector, so y and u on a halo
   // row equal the owner's values: M^-1 is one operator across the CTAs.  One cluster barrier
   // (the restricted partials).  z goes to zbuf on the owned rows; returns the local (r, z).
-  __device__ Real vcycle(const Real (&r)[NG][4]) {
+  __device__ V vcycle(const V (&r)[NG][4]) {
     const int W = sb.W, G = sb.G;
     float rf[NG][4];   // r in FP32, converted once (FP64 conversions run on the FP64 pipe)
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) rf[k][j] = (float)r[k][j];
+      for (int j = 0; j < kGroup; ++j) rf[k][j] = f32(r[k][j]);
       if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) vy[l0 + j] = vsd[l0 + j] * rf[k][j];
     }
     for (int i = threadIdx.x; i < 2 * W; i += blockDim.x) {
       const int l = halo_offset(i);
-      vy[l] = vsd[l] * (float)vrh[i];
+      vy[l] = vsd[l] * f32(vrh[i]);
     }
     __syncthreads();
     float w[NG][4];
@@ -725,7 +729,7 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) vy[l + j] = vsd[l + j] != 0.f ? vy[l + j] + e : 0.f;
     }
     __syncthreads();
-    Real rz = Real(0);
+    V rz = V{};
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
@@ -735,8 +739,8 @@ struct Stepper {
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const float z = unknown(k, j) ? fmaf(vsd[l0 + j], rf[k][j] - t[j], vy[l0 + j]) : 0.f;
-        zbuf[l0 + j] = (Real)z;
-        rz = fma(r[k][j], (Real)z, rz);
+        zbuf[l0 + j] = z;
+        rz = vdot(rz, r[k][j], z);
       }
     }
     return rz;
@@ -782,13 +786,13 @@ struct Stepper {
   // exchanged (a cluster barrier) before the residual; u on the halo rows is then the owner's
   // value (e1 from the owner, ec computed from the same restricted vector).  Two cluster
   // barriers.  z goes to zbuf on the owned rows; returns the local (r, z).
-  __device__ Real vcycle_local(const Real (&r)[NG][4]) {
+  __device__ V vcycle_local(const V (&r)[NG][4]) {
     const int W = sb.W, G = sb.G;
     float rf[NG][4], e[NG][4], w[NG][4];
 #pragma unroll
     for (int k = 0; k < NG; ++k)
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) rf[k][j] = (float)r[k][j];
+      for (int j = 0; j < kGroup; ++j) rf[k][j] = f32(r[k][j]);
     smooth_local(rf, e);
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
@@ -827,10 +831,10 @@ struct Stepper {
       float t[4];
       stencil_elem32(vy, wd, ws, wt, l0, W, t);
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? (float)r[k][j] - t[j] : 0.f;
+      for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? f32(r[k][j]) - t[j] : 0.f;
     }
     smooth_local(w, e);
-    Real rz = Real(0);
+    V rz = V{};
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
@@ -838,8 +842,8 @@ struct Stepper {
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const float z = vy[l0 + j] + e[k][j];
-        zbuf[l0 + j] = (Real)z;
-        rz = fma(r[k][j], (Real)z, rz);
+        zbuf[l0 + j] = z;
+        rz = vdot(rz, r[k][j], z);
       }
     }
     return rz;
@@ -973,14 +977,14 @@ struct Stepper {
   // smoother is symmetric, so M^-1 is symmetric.  Values on halo rows equal the owners' (e0 and
   // e1 exchanged, ec from the same restricted vector in every CTA, z1 exchanged), so M^-1 is one
   // operator across the CTAs.  Five cluster barriers.  z goes to zbuf; returns the local (r, z).
-  __device__ Real vcycle3(const Real (&r)[NG][4]) {
+  __device__ V vcycle3(const V (&r)[NG][4]) {
     const int W = sb.W;
     float e[NG][4], w[NG][4];
     // fine pre-smoothing e0 = S0 r, exchanged (r in FP32 in w)
 #pragma unroll
     for (int k = 0; k < NG; ++k)
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) w[k][j] = (float)r[k][j];
+      for (int j = 0; j < kGroup; ++j) w[k][j] = f32(r[k][j]);
     smooth_local(w, e);
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
@@ -1024,10 +1028,10 @@ struct Stepper {
       float t[4];
       stencil_elem32(vy, wd, ws, wt, l0, W, t);
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? (float)r[k][j] - t[j] : 0.f;
+      for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? f32(r[k][j]) - t[j] : 0.f;
     }
     smooth_local(w, e);
-    Real rz = Real(0);
+    V rz = V{};
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
@@ -1035,8 +1039,8 @@ struct Stepper {
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const float z = vy[l0 + j] + e[k][j];
-        zbuf[l0 + j] = (Real)z;
-        rz = fma(r[k][j], (Real)z, rz);
+        zbuf[l0 + j] = z;
+        rz = vdot(rz, r[k][j], z);
       }
     }
     return rz;
@@ -1048,9 +1052,9 @@ struct Stepper {
   // (the FP32 element weights); the first step's iterate goes through zbuf, whose halo rows are
   // not read, so the neighbours may already be writing their new edge rows into them.  No
   // communication; two block barriers.  z goes to zbuf; returns the local (r, z).
-  __device__ Real precond_local2(const Real (&r)[NG][4]) {
+  __device__ V precond_local2(const V (&r)[NG][4]) {
     if constexpr (!kMixed) {
-      return Real(0);   // not used: FP64 CG has no FP32 element weights
+      return V{};       // not used: FP64 CG has no FP32 element weights
     } else {
     const float om = P.tl_omega;
     float e[NG][4];
@@ -1062,8 +1066,8 @@ struct Stepper {
       if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
-        e[k][j] = om * (float)dinv[l0 + j] * (float)r[k][j];
-        zbuf[l0 + j] = (Real)e[k][j];
+        e[k][j] = om * dinv[l0 + j] * f32(r[k][j]);
+        zbuf[l0 + j] = e[k][j];
       }
     }
     __syncthreads();
@@ -1078,142 +1082,141 @@ struct Stepper {
       float t[4];
       stencil_elem32(zbuf, wd, ws, wt, l0, sb.W, t, lr == 0, lr == sb.R - 1);
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) z[k][j] = fmaf(om * (float)dinv[l0 + j], (float)r[k][j] - t[j], e[k][j]);
+      for (int j = 0; j < kGroup; ++j) z[k][j] = fmaf(om * dinv[l0 + j], f32(r[k][j]) - t[j], e[k][j]);
     }
     __syncthreads();
-    Real rz = Real(0);
+    V rz = V{};
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
-        zbuf[l0 + j] = (Real)z[k][j];
-        rz = fma(r[k][j], (Real)z[k][j], rz);
+        zbuf[l0 + j] = z[k][j];
+        rz = vdot(rz, r[k][j], z[k][j]);
       }
     }
     return rz;
     }
   }
 
-  // Jacobi-preconditioned CG in precision Real on A d = r, where r (given per node) is the FP64
-  // residual scaled to unit 2-norm; on return x64 += unscale * d.  Stops when ||r||^2 <= target2
-  // (scaled units) or at the iteration limit; returns the iteration count.  All CG scalars and
-  // dot products are in precision Real.
-  __device__ int cg_correct(Real (&r)[NG][4], Real target2, double unscale) {
-    // FP32 CG without a two-level form: the slab-local two-step preconditioner if asked for
-    const bool local2 = kMixed && !tl && P.local_steps >= 2;
-    Real d[NG][4], p[NG][4], q[NG][4];
-    Real rz;
-    {
-      Real v[1] = {Real(0)};
-#pragma unroll
-      for (int k = 0; k < NG; ++k) {
-        const int l0 = loc0[k];
-#pragma unroll
-        for (int j = 0; j < kGroup; ++j) { d[k][j] = Real(0); p[k][j] = Real(0); q[k][j] = Real(0); }
-        if (l0 < 0 || tl || local2) continue;
-#pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-          const Real z = dinv[l0 + j] * r[k][j];
-          zbuf[l0 + j] = z;
-          v[0] = fma(r[k][j], z, v[0]);
-        }
-      }
-      if (local2) {
-        v[0] = precond_local2(r);
-      } else if (l3) {
-        v[0] = vcycle3(r);
-      } else if (vc && P.tl_nu >= 2) {
-        v[0] = vcycle_local(r);
-      } else if (vc) {
-        // r on the halo rows from the neighbours' owned edge rows
-        put_edges(vrh, r, true);
-        comm.finish_edges();
-        v[0] = vcycle(r);
-      } else if (tl) {
-        coarse_restrict_push(r);
-        comm.finish_tl();
-        coarse_gather(true, 0.f);
-        v[0] = prolong_precondition(r);
-      }
-      allreduce<Real, 1>(v, NoPost(), [&] { comm.push_halos(zbuf, sb); });
-      rz = v[0];
+  // z = M^-1 r to zbuf (owned rows); returns the local (r, z)
+  __device__ V precondition(const V (&r)[NG][4]) {
+    if constexpr (COARSE) {
+      if (l3) return vcycle3(r);
+      if (vc && P.tl_nu >= 2) return vcycle_local(r);
+      if (vc) return vcycle(r);
+      if (tl) return prolong_precondition(r);
     }
-    int it = 0;
-    Real beta = Real(0);
-    bool done = !(Real(1) > target2);
-    while (!done && it < P.itmax) {
-      // q = A z + beta q, p = z + beta p, (p, q); alpha = rz / (p, q)
-      Real pq[1] = {Real(0)};
+    if constexpr (kMixed) {
+      if (P.local_steps >= 2) return precond_local2(r);
+    }
+    V rz = V{};
 #pragma unroll
-      for (int k = 0; k < NG; ++k) {
-        const int l0 = loc0[k];
-        if (l0 < 0) continue;
-        Real w[4];
-        apply_A(zbuf, l0, w);
+    for (int k = 0; k < NG; ++k) {
+      const int l0 = loc0[k];
+      if (l0 < 0) continue;
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-          const Real wj = unknown(k, j) ? w[j] : Real(0);
-          const Real z = zbuf[l0 + j];
-          p[k][j] = fma(beta, p[k][j], z);
-          q[k][j] = fma(beta, q[k][j], wj);
-          pq[0] = fma(p[k][j], q[k][j], pq[0]);
+      for (int j = 0; j < kGroup; ++j) {
+        const float z = dinv[l0 + j] * f32(r[k][j]);
+        zbuf[l0 + j] = z;
+        rz = vdot(rz, r[k][j], z);
+      }
+    }
+    return rz;
+  }
+
+  // Preconditioned CG on A d = r, where r (given per node) is the FP64 residual scaled by a power
+  // of two to a squared 2-norm rr0 in [1, 4); on return x64 += unscale * d.  Stops when
+  // ||r||^2 <= target2 (scaled units) or at the iteration limit; returns the iteration count.
+  // Vectors, scalars and dot products are V; z is float.
+  // The float pairs of the FP64 kinds: on a slab of 9 x 132 nodes (128 x 128 over 16 CTAs) an
+  // iteration's stencil, updates and dot products took 10 100 cycles on the FP64 pipe (17 FP64
+  // instructions per node) and take about 180 FP32 instructions per node in pairs.
+  __device__ int cg_correct(V (&r)[NG][4], float rr0, float target2, double unscale) {
+    V d[NG][4], p[NG][4], q[NG][4];
+#pragma unroll
+    for (int k = 0; k < NG; ++k) {
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) d[k][j] = p[k][j] = q[k][j] = V{};
+    }
+    const bool additive = COARSE && tl && !vc;                   // restricts r once, then q
+    const bool global1 = COARSE && vc && !l3 && P.tl_nu < 2;     // keeps r on the halo rows
+    V rz = V{}, beta = V{};
+    int it = -1;                   // -1: the start, whose z and (r, z) open the iteration
+    bool done = !(rr0 > target2);
+    for (;;) {
+      V v[3] = {V{}, V{}, V{}};
+      if (it < 0) {
+        if (additive) {
+          coarse_restrict_push(r);
+          comm.finish_tl();
+          coarse_gather(true, 0.f);
+        } else if (global1) {
+          put_edges(vrh, r, true);   // r on the halo rows from the neighbours' owned edge rows
+          comm.finish_edges();
         }
-      }
-      if (vc && !l3 && P.tl_nu < 2) {
-        // q's owned edge rows to the neighbours, whose copies of r on their halo rows follow
-        // the same recurrence (visible after the all-reduce's barrier)
-        put_edges(vqh, q, false);
-      } else if (tl && !vc) {
-        coarse_restrict_push(q);             // visible after the all-reduce's cluster barrier
-      }
-      const Real rz_c = rz;
-      allreduce<Real, 1>(pq, [rz_c](Real* t) { t[0] = rz_c / t[0]; });
-      const Real alpha = pq[0];
-      if (tl && !vc) coarse_gather(false, (float)alpha);
-      // d += alpha p, r -= alpha q, z = D^-1 r; (r, z), (r, r) and beta = (r, z)_new / (r, z)
-      Real v[3] = {Real(0), Real(0), Real(0)};
+      } else {
+        // q = A z + beta q, p = z + beta p, (p, q); alpha = rz / (p, q)
+        V pq[1] = {V{}};
 #pragma unroll
-      for (int k = 0; k < NG; ++k) {
-        const int l0 = loc0[k];
-        if (l0 < 0) continue;
+        for (int k = 0; k < NG; ++k) {
+          const int l0 = loc0[k];
+          if (l0 < 0) continue;
+          V w[4];
+          apply_A(zbuf, l0, w);
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-          d[k][j] = fma(alpha, p[k][j], d[k][j]);
-          r[k][j] = fma(-alpha, q[k][j], r[k][j]);
-          v[1] = fma(r[k][j], r[k][j], v[1]);
-          if (!tl && !local2) {
-            const Real z = dinv[l0 + j] * r[k][j];
-            zbuf[l0 + j] = z;
-            v[0] = fma(r[k][j], z, v[0]);
+          for (int j = 0; j < kGroup; ++j) {
+            const V wj = unknown(k, j) ? w[j] : V{};
+            p[k][j] = vfma(beta, p[k][j], zbuf[l0 + j]);
+            q[k][j] = vfma(beta, q[k][j], wj);
+            pq[0] = vdot(pq[0], p[k][j], q[k][j]);
           }
         }
+        if (global1)
+          put_edges(vqh, q, false);  // the neighbours' copies of r on their halo rows follow q
+        else if (additive)
+          coarse_restrict_push(q);   // (both visible after the all-reduce)
+        const V rz_c = rz;
+        allreduce<V, 1>(pq, [rz_c](V* t) { t[0] = vdiv(rz_c, t[0]); });
+        const V alpha = pq[0], nalpha = vneg(alpha);
+        if (additive) coarse_gather(false, f32(alpha));
+        // d += alpha p, r -= alpha q; (r, r)
+#pragma unroll
+        for (int k = 0; k < NG; ++k) {
+          if (loc0[k] < 0) continue;
+#pragma unroll
+          for (int j = 0; j < kGroup; ++j) {
+            d[k][j] = vfma(alpha, p[k][j], d[k][j]);
+            r[k][j] = vfma(nalpha, q[k][j], r[k][j]);
+            v[1] = vdot(v[1], r[k][j], r[k][j]);
+          }
+        }
+        if (global1)
+          for (int i = threadIdx.x; i < 2 * sb.W; i += blockDim.x) vrh[i] = vfma(nalpha, vqh[i], vrh[i]);
       }
-      if (local2) {
-        v[0] = precond_local2(r);
-      } else if (l3) {
-        v[0] = vcycle3(r);
-      } else if (vc && P.tl_nu >= 2) {
-        v[0] = vcycle_local(r);
-      } else if (vc) {
-        for (int i = threadIdx.x; i < 2 * sb.W; i += blockDim.x) vrh[i] = fma(-alpha, vqh[i], vrh[i]);
-        v[0] = vcycle(r);
-      } else if (tl) {
-        v[0] = prolong_precondition(r);
-      }
-      allreduce<Real, 2, 1>(v, [rz_c](Real* t) { t[2] = t[0] / rz_c; }, [&] { comm.push_halos(zbuf, sb); });
+      // z = M^-1 r, (r, z) and beta = (r, z)_new / (r, z)
+      v[0] = precondition(r);
+      const V rz_c = rz;
+      const bool start = it < 0;
+      allreduce<V, 2, 1>(v, [rz_c, start](V* t) { if (!start) t[2] = vdiv(t[0], rz_c); },
+                         [&] { comm.push_halos(zbuf, sb); });
       ++it;
-      if (!(v[1] > target2)) done = true;  // NaN keeps iterating until the limit
+      if (!start && !(f32(v[1]) > target2)) done = true;
       beta = v[2];
       rz = v[0];
+      if (done || it >= P.itmax) break;
     }
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) x64[l0 + j] = fma((double)d[k][j], unscale, x64[l0 + j]);
+      for (int j = 0; j < kGroup; ++j) {
+        double x = x64[l0 + j];
+        if constexpr (!kMixed) x = fma(widen(d[k][j].l), unscale, x);
+        x64[l0 + j] = fma((double)f32(d[k][j]), unscale, x);
+      }
     }
     return it;
   }
@@ -1239,15 +1242,25 @@ struct Stepper {
     const double tol2 = P.rtol * P.rtol * bb;
     int sweeps = 0, its = 0;
     while (rr > tol2 && sweeps < P.refmax) {
-      // scale the residual to unit norm so the Real-precision CG works on O(1) values
-      const double nrm = sqrt(rr), scale = 1.0 / nrm;
-      Real r[NG][4];
+      // scale the residual by 2^-k to a squared norm in [1, 4), so that the CG works on O(1) values
+      const int k2 = (((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1;
+      const double rr0 = rr * exp2_int(-k2) * exp2_int(-k2);
+      V r[NG][4];
 #pragma unroll
-      for (int k = 0; k < NG; ++k)
+      for (int k = 0; k < NG; ++k) {
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) r[k][j] = (Real)(r64[k][j] * scale);
-      const Real target2 = (Real)fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr);
-      its += cg_correct(r, target2, nrm);
+        for (int j = 0; j < kGroup; ++j) {
+          const ff s = split_scaled(r64[k][j], -k2);
+          if constexpr (kMixed)
+            r[k][j] = s.h + s.l;
+          else
+            r[k][j] = s;
+        }
+      }
+      // (the pairs carry a residual to about 1e-15 of its start)
+      const float target2 = fmaxf((float)(fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr) * rr0), 1e-30f);
+      // A d = r in the scale of the float pairs gives d / scale
+      its += cg_correct(r, (float)rr0, target2, exp2_int(k2) * (kMixed ? 1.0 : ffw.scale));
       ++sweeps;
       exchange_x64();
       double v[1] = {residual(r64)};
@@ -1280,7 +1293,7 @@ struct Stepper {
       if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j)
-        if (dinv[l0 + j] != Real(0)) v[0] += ipow(x64[l0 + j], P.p_int);
+        if (dinv[l0 + j] != 0.f) v[0] += ipow(x64[l0 + j], P.p_int);
     }
     allreduce<double, 1>(v);
     return v[0];
@@ -1346,7 +1359,7 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) {
         const int g = gnode(l0, j);
         if (g < 0) continue;
-        const double t = dinv[l0 + j] != Real(0) ? (x64[l0 + j] + Fs[g]) - Gs[g] : 0.0;
+        const double t = dinv[l0 + j] != 0.f ? (x64[l0 + j] + Fs[g]) - Gs[g] : 0.0;
         x64[l0 + j] = t;
         X[g] = t;
         if (Y) Y[g] = t;
@@ -1387,7 +1400,7 @@ struct Stepper {
     const int sb_end = P.chained ? P.s0 + P.ns : sa + 1;
     const int M = P.M;
     const double inv_norm = 1.0 / ((double)P.Nt * (double)P.Ne);
-    set_operator(false);
+    set_operator();
     load_x64(P.in_field + (size_t)sa * P.Nn);
     double theta = P.in_aux[sa];
     if (P.chained) {                              // a sequential run also records its start
@@ -1412,10 +1425,8 @@ struct Stepper {
           for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.Nn;
           extrapolate_x64(n, X, ring + (size_t)((j - 1) % nring) * P.Nn);
           ++saved;
-          solve(j, false);
-        } else {
-          solve(j, true);
         }
+        solve(j, ring == nullptr);
         const double sp = pnorm_p();
         if (threadIdx.x == 0) theta = accumulate_theta(theta, sp * inv_norm);  // used by thread 0 only
         if (double* row = hist_row(j)) store_x64(row);
@@ -1427,7 +1438,7 @@ struct Stepper {
 
   __device__ void coarse_primal(int task) {
     const int s = P.s0 + task;
-    set_operator(true);
+    set_operator();
     load_x64(P.in_field + (size_t)s * P.Nn);
     const double theta0 = P.in_aux[s];
     const int j = P.M * (s + 1);
@@ -1446,7 +1457,7 @@ struct Stepper {
   }
 
   __device__ void correct_primal() {
-    if (!P.plt) set_operator(true);
+    if (!P.plt) set_operator();
     double theta;
     if (P.in_field) {                           // u_0 taken from the guess states, copied to X[0]
       load_x64(P.in_field);
@@ -1506,7 +1517,7 @@ struct Stepper {
     const int M = P.M;
     const double Theta = *P.Theta;
     const double scale = adjoint_scale(Theta);
-    set_operator(false);
+    set_operator();
     load_x64(P.in_field + (size_t)(s_hi + 1) * P.Nn);
     const double* gsrc = P.in_aux + (size_t)(s_hi + 1) * P.Ne;
     // initial guess: the extrapolation through lambda_{j+1} (in x64) .. lambda_{j+n}, kept in a
@@ -1533,10 +1544,8 @@ struct Stepper {
           for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.Nn;
           extrapolate_x64(n, X, ring + (size_t)((j + 1) % nring) * P.Nn);
           ++saved;
-          solve(j, false);
-        } else {
-          solve(j, true);
         }
+        solve(j, ring == nullptr);
         accumulate_g(Tj, Tjm, P.dt, (double)P.Nt, gsrc, gdst, nullptr, nullptr);
         gsrc = gdst;
         __syncthreads();
@@ -1556,7 +1565,7 @@ struct Stepper {
     const double scale = P.src_mode == 0 ? adjoint_scale(*P.Theta) : (P.src_mode == 1 ? 0.0 : 1.0);
     const double* Tk = P.hist + (size_t)kidx * P.Nn;
     const double* Tkm = P.hist + (size_t)kprev * P.Nn;
-    set_operator(true);
+    set_operator();
     if (P.src_mode == 2)
       zero_x64();
     else
@@ -1572,7 +1581,7 @@ struct Stepper {
   __device__ void correct_adjoint() {
     const double Theta = *P.Theta;
     const double scale = adjoint_scale(Theta);
-    if (!P.plt) set_operator(true);
+    if (!P.plt) set_operator();
     // v_Ntau = 0
     {
       double* Xl = P.out_field + (size_t)P.Ntau * P.Nn;
@@ -1636,8 +1645,11 @@ struct Stepper {
 // plan picks the block size), at most 128 registers per thread.
 constexpr int kStepMaxThreads = 512;
 
+template <int KIND>
+constexpr bool kCoarseStep = KIND != KIND_FINE_PRI && KIND != KIND_FINE_ADJ;
+
 template <class Real, int NG, int KIND, class Comm>
-__device__ __forceinline__ void run_task(Stepper<Real, NG, Comm>& st, int task) {
+__device__ __forceinline__ void run_task(Stepper<Real, NG, Comm, kCoarseStep<KIND>>& st, int task) {
   if constexpr (KIND == KIND_FINE_PRI) st.fine_primal(task);
   if constexpr (KIND == KIND_COARSE_PRI) st.coarse_primal(task);
   if constexpr (KIND == KIND_CORRECT_PRI) st.correct_primal();
@@ -1652,7 +1664,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_kernel(const __gri
   __shared__ RedSmem rs;
   ClusterComm comm(rs);
   comm.bind(P);
-  Stepper<Real, NG, ClusterComm> st(P, comm, dyn_smem);
+  Stepper<Real, NG, ClusterComm, kCoarseStep<KIND>> st(P, comm, dyn_smem);
   // every CTA of the cluster has initialised its shared memory before any DSMEM traffic
   cluster_sync_all();
   run_task<Real, NG, KIND>(st, (int)(blockIdx.x / (unsigned)P.cs));
@@ -1672,7 +1684,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_wide_kernel(const 
   GridComm comm(P, rs);
   const int ngroups = (int)gridDim.x / P.cs;
   for (int task = comm.gid; task < P.wide_tasks; task += ngroups) {
-    Stepper<Real, NG, GridComm> st(P, comm, dyn_smem);
+    Stepper<Real, NG, GridComm, kCoarseStep<KIND>> st(P, comm, dyn_smem);
     run_task<Real, NG, KIND>(st, task);
     comm.sync();                               // the group's halo slots are free again
   }
@@ -1705,7 +1717,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_batch_kernel(const
     if (t >= ntasks) break;
     const int2 tk = tasks[t];
     comm.bind(table[tk.x]);
-    Stepper<Real, NG, ClusterComm> st(table[tk.x], comm, dyn_smem);
+    Stepper<Real, NG, ClusterComm, kCoarseStep<KIND>> st(table[tk.x], comm, dyn_smem);
     cluster_sync_all();
     run_task<Real, NG, KIND>(st, tk.y);
     cluster_sync_all();
