@@ -322,12 +322,15 @@ struct GridComm {
     }
     __syncthreads();
     push();
-    T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 4);   // 4 values per block
+    // 32 bytes per block whatever T: the groups of a launch are not in step, and one may reduce floats
+    // while another reduces doubles
+    constexpr int kPer = 32 / (int)sizeof(T);
+    T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 4);
     if (warp == 0) {
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
         const T s = warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
-        if (lane == 0) slots[(int)blockIdx.x * 4 + i] = s;
+        if (lane == 0) slots[(int)blockIdx.x * kPer + i] = s;
       }
     }
     barrier();
@@ -337,7 +340,7 @@ struct GridComm {
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
         T a = T{};
-        for (int r = lane; r < G; r += 32) a = a + ldcg(slots + (base + r) * 4 + i);
+        for (int r = lane; r < G; r += 32) a = a + ldcg(slots + (base + r) * kPer + i);
         t[i] = warp_sum(a);
       }
 #pragma unroll
