@@ -921,8 +921,8 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
   op->W = padded_width(grid->nx);
   const size_t PEe = (size_t)(grid->ny + 2) * op->W + 2 * kSlack;
   const size_t PN = (size_t)(grid->ny + 3) * op->W + 2 * kSlack;
-  const int blocks_e = (op->Ne + 255) / 256;
-  op->sens_chunks = std::max(1, std::min(64, (4 * 152 + blocks_e - 1) / blocks_e));
+  const int blocks_s = sens_blocks(grid->nx, grid->ny);
+  op->sens_chunks = std::max(1, std::min(64, (8 * 152 + blocks_s - 1) / blocks_s));
   cudaError_t e = cudaSuccess;
   auto A = [&](auto** p, size_t bytes) {
     if (e == cudaSuccess) e = cudaMalloc((void**)p, bytes);

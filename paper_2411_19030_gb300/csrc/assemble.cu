@@ -160,24 +160,35 @@ cudaError_t launch_assemble(int nx, int ny, double h, const ptg_material& m, dou
 }
 
 // a6, Eq. 4.7: per element e and time chunk, sum over j of
-//   lambda_j,e^T ( dk_e Ke T_j,e + dc_e/dt Me (T_j - T_{j-1})_e )   (sens_element_sum).
-// One thread per element; blockIdx.y selects a contiguous chunk of time steps.
-__global__ void sens_kernel(int nx, int ny, double h, double dt, int has_dc, const double* __restrict__ dk,
-                            const double* __restrict__ dc, const double* __restrict__ lam, int j0, int j1,
-                            const double* __restrict__ T, int hist_j0, int steps_per_chunk,
-                            double* __restrict__ partial) {
+//   lambda_j,e^T ( dk_e Ke T_j,e + dc_e/dt Me (T_j - T_{j-1})_e )   (sens_strip_sum).
+// One thread per strip of kSensRows elements above one another (see sens_strip_sum for what that
+// shares); blockIdx.y selects a contiguous chunk of time steps, as many chunks as give every SM
+// about eight blocks, since the FP64 pipes bound it: 256 x 256 over 512 steps with the capacity
+// term 3.89 ms with one element per thread and the 4 x 4 forms.
+__global__ void __launch_bounds__(kSensThreads)
+sens_kernel(int nx, int ny, double h, double dt, int has_dc, const double* __restrict__ dk,
+            const double* __restrict__ dc, const double* __restrict__ lam, int j0, int j1,
+            const double* __restrict__ T, int hist_j0, int steps_per_chunk, double* __restrict__ partial) {
   const int Ne = nx * ny, nn = nx + 1, Nn = nn * (ny + 1);
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= Ne) return;
+  const int strips = (ny + kSensRows - 1) / kSensRows;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nx * strips) return;
   const int chunk = blockIdx.y;
   const int ja = j0 + chunk * steps_per_chunk;
   const int jb = min(j1, ja + steps_per_chunk - 1);
-  const int ey = e / nx, ex = e % nx;
-  const double dke = dk[e], dce = has_dc ? dc[e] / dt : 0.0;
-  const double acc = ja <= jb ? sens_element_sum(ey * nn + ex, nn, Nn, h * h / 36.0, dke, dce, has_dc != 0, lam, j0,
-                                                 T, hist_j0, ja, jb)
-                              : 0.0;
-  partial[(size_t)chunk * Ne + e] = acc;
+  const int st = t / nx, ex = t - st * nx, ey = st * kSensRows, rows = min(kSensRows, ny - ey);
+  double dke[kSensRows], dce[kSensRows], out[kSensRows];
+#pragma unroll
+  for (int i = 0; i < kSensRows; ++i) {
+    dke[i] = i < rows ? dk[(ey + i) * nx + ex] : 0.0;
+    dce[i] = i < rows && has_dc ? dc[(ey + i) * nx + ex] / dt : 0.0;
+    out[i] = 0.0;
+  }
+  if (ja <= jb)
+    sens_strip_sum<kSensRows>(ey * nn + ex, nn, Nn, h * h, dke, dce, has_dc != 0, rows, lam, j0, T, hist_j0, ja, jb, out);
+#pragma unroll
+  for (int i = 0; i < kSensRows; ++i)
+    if (i < rows) partial[(size_t)chunk * Ne + (ey + i) * nx + ex] = out[i];
 }
 
 // grad_e += -(1/Nt) sum over chunks (fixed order) of the partial sums.
@@ -223,8 +234,8 @@ cudaError_t launch_sensitivities(int nx, int ny, int Nt, double h, double dt, in
   const int nsteps = j1 - j0 + 1;
   const int spc = (nsteps + nchunks - 1) / nchunks;
   const int used = (nsteps + spc - 1) / spc;
-  dim3 grid((Ne + 255) / 256, used);
-  sens_kernel<<<grid, 256, 0, stream>>>(nx, ny, h, dt, has_dc, dk, dc, lam, j0, j1, T, hist_j0, spc, partial);
+  dim3 grid(sens_blocks(nx, ny), used);
+  sens_kernel<<<grid, kSensThreads, 0, stream>>>(nx, ny, h, dt, has_dc, dk, dc, lam, j0, j1, T, hist_j0, spc, partial);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   sens_reduce_kernel<<<(Ne + 255) / 256, 256, 0, stream>>>(Ne, used, 1.0 / Nt, partial, grad);

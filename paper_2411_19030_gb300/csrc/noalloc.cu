@@ -7,7 +7,7 @@
 // in host code it is only a stand-in for the device symbol, so its device address is looked
 // up once per device with cudaGetSymbolAddress and passed to the kernel.
 //
-// The per-element accumulation (sens_element_sum) and the chunk reduction are the ones of
+// The per-element accumulation (sens_strip_sum) and the chunk reduction are the ones of
 // ptg_sensitivities; only the source of dk/drho and dc/drho differs (evaluated from rho here,
 // read from the op's workspace there).
 #include <algorithm>
@@ -29,7 +29,7 @@ std::mutex g_mu;
 double* g_scratch_ptr[kMaxDevices] = {};
 
 // Partial sums over a contiguous chunk of time steps of
-//   lambda_j,e^T ( dk_e Ke T_j,e + dc_e/dt Me (T_j - T_{j-1})_e )   (sens_element_sum),
+//   lambda_j,e^T ( dk_e Ke T_j,e + dc_e/dt Me (T_j - T_{j-1})_e )   (sens_strip_sum),
 // with dk_e and dc_e evaluated from rho (Eq. 2.5-2.6 differentiated) inside the kernel, so
 // the call needs no coefficient workspace.  A value of rho outside [0, 1] (or NaN) is taken
 // as 0, as the assembly does (which also records the error in its op's status word).
@@ -48,10 +48,11 @@ __global__ void sens_noalloc_kernel(int nx, int ny, double h, double dt, ptg_mat
   const bool has_dc = m.c0 != m.cmin;
   const double dke = (m.k0 == m.kmin) ? 0.0 : m.pk * (m.k0 - m.kmin) * pow(r, m.pk - 1.0);
   const double dce = has_dc ? m.pc * (m.c0 - m.cmin) * pow(r, m.pc - 1.0) / dt : 0.0;
-  const double acc = ja <= jb ? ptg::sens_element_sum(ey * nn + ex, nn, Nn, h * h / 36.0, dke, dce, has_dc, lam, j0,
-                                                      T, hist_j0, ja, jb)
-                              : 0.0;
-  partial[(size_t)chunk * Ne + e] = acc;
+  const double dk1[1] = {dke}, dc1[1] = {dce};
+  double acc[1] = {0.0};
+  if (ja <= jb)
+    ptg::sens_strip_sum<1>(ey * nn + ex, nn, Nn, h * h, dk1, dc1, has_dc, 1, lam, j0, T, hist_j0, ja, jb, acc);
+  partial[(size_t)chunk * Ne + e] = acc[0];
 }
 
 // Device address of the scratch array for the current device, looked up once per device and

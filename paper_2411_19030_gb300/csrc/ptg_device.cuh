@@ -155,14 +155,17 @@ __device__ __forceinline__ void slab_rows(int rows_total, int cs, int rank, int&
   R = base + (rank < rem ? 1 : 0);
 }
 
-// x^(p-1) and x^p for an even integer p >= 2 by repeated squaring (exact operation order is
-// fixed so every CTA and every run computes the same value).
+// x^e for an integer exponent e >= 1 by squaring, without the multiplications by one (exact
+// operation order is fixed so every CTA and every run computes the same value).
 __device__ __forceinline__ double ipow(double x, int e) {
-  double r = 1.0, b = x;
-  while (e > 0) {
-    if (e & 1) r *= b;
-    b *= b;
+  while (!(e & 1)) {
+    x *= x;
     e >>= 1;
+  }
+  double r = x;
+  while ((e >>= 1) > 0) {
+    x *= x;
+    if (e & 1) r *= x;
   }
   return r;
 }
@@ -342,41 +345,89 @@ __device__ __forceinline__ void stencil_elem32(const float* __restrict__ z, cons
   }
 }
 
-// Eq. 4.7, one element over the contiguous steps ja..jb (ja <= jb): the sum over j of
-//   lambda_j,e^T ( dke Ke T_j,e + dce Me (T_j - T_{j-1})_e ),
-// with dce already divided by the step size and Me = (h^2/36)[4 2 1 2; 2 4 2 1; 1 2 4 2; 2 1 2 4],
-// Ke = (1/6)[4 -1 -2 -1; -1 4 -1 -2; -2 -1 4 -1; -1 -2 -1 4] in the local order SW, SE, NE, NW.
-// g0 is the element's SW node, nn = nx + 1, Nn the node count; lambda_j is row j - j0 of lam and
-// T_j row j - hist_j0 of T.  T_{j-1} is carried in registers, so each step reads lambda_j and T_j
-// once.  The capacity term is evaluated only when has_dc is set.
-__device__ __forceinline__ double sens_element_sum(int g0, int nn, int Nn, double h2, double dke, double dce,
-                                                   bool has_dc, const double* __restrict__ lam, int j0,
-                                                   const double* __restrict__ T, int hist_j0, int ja, int jb) {
-  double acc = 0.0;
-  const double* Tp = T + (size_t)(ja - 1 - hist_j0) * Nn;
-  double psw = Tp[g0], pse = Tp[g0 + 1], pne = Tp[g0 + nn + 1], pnw = Tp[g0 + nn];
-  for (int j = ja; j <= jb; ++j) {
-    const double* Tj = T + (size_t)(j - hist_j0) * Nn;
-    const double* Lj = lam + (size_t)(j - j0) * Nn;
-    const double tsw = Tj[g0], tse = Tj[g0 + 1], tne = Tj[g0 + nn + 1], tnw = Tj[g0 + nn];
-    const double lsw = Lj[g0], lse = Lj[g0 + 1], lne = Lj[g0 + nn + 1], lnw = Lj[g0 + nn];
-    const double ksw = 4.0 * tsw - tse - 2.0 * tne - tnw;
-    const double kse = -tsw + 4.0 * tse - tne - 2.0 * tnw;
-    const double kne = -2.0 * tsw - tse + 4.0 * tne - tnw;
-    const double knw = -tsw - 2.0 * tse - tne + 4.0 * tnw;
-    double term = dke * (lsw * ksw + lse * kse + lne * kne + lnw * knw) / 6.0;
-    if (has_dc) {
-      const double dsw = tsw - psw, dse = tse - pse, dne = tne - pne, dnw = tnw - pnw;
-      const double msw = 4.0 * dsw + 2.0 * dse + dne + 2.0 * dnw;
-      const double mse = 2.0 * dsw + 4.0 * dse + 2.0 * dne + dnw;
-      const double mne = dsw + 2.0 * dse + 4.0 * dne + 2.0 * dnw;
-      const double mnw = 2.0 * dsw + dse + 2.0 * dne + 4.0 * dnw;
-      term += dce * (lsw * msw + lse * mse + lne * mne + lnw * mnw) * h2;
-    }
-    acc += term;
-    psw = tsw; pse = tse; pne = tne; pnw = tnw;
+// Element bilinear forms of Eq. 4.7 in the modes that Ke and Me share as eigenvectors: with the
+// corner values in the order SW, SE, NE, NW the sums a = (1, 1, 1, 1), b = (-1, 1, 1, -1),
+// c = (-1, -1, 1, 1) and d = (1, -1, 1, -1) have the eigenvalues 0, 1, 1, 2/3 of Ke and
+// (h^2/36) (9, 3, 3, 1) of Me, so
+//   lambda^T Ke T = (b b' + c c' + (2/3) d d') / 4,
+//   lambda^T Me T = (h^2/36) (9 a a' + 3 (b b' + c c') + d d') / 4.
+// The sums are bound by the FP64 pipe (an FP64 instruction of a warp takes 64 cycles on this
+// chip): 8 additions per field and 3 or 4 products replace the 20 multiply-adds of each 4 x 4 form.
+struct Modes {
+  double a, b, c, d;
+};
+__device__ __forceinline__ Modes elem_modes(double sw, double se, double ne, double nw) {
+  const double p = se - sw, q = ne - nw, bot = sw + se, top = nw + ne;
+  return Modes{top + bot, p + q, top - bot, q - p};
+}
+__device__ __forceinline__ double elem_stiffness(const Modes& l, const Modes& t) {
+  return fma(l.d * t.d, 1.0 / 6.0, 0.25 * fma(l.b, t.b, l.c * t.c));
+}
+// (times h^2)
+__device__ __forceinline__ double elem_mass(const Modes& l, const Modes& t) {
+  return fma(l.a * t.a, 1.0 / 16.0, fma(l.d * t.d, 1.0 / 144.0, fma(l.b, t.b, l.c * t.c) * (1.0 / 48.0)));
+}
+
+// Eq. 4.7 for H elements above one another over the contiguous steps ja..jb (ja <= jb): the sums
+// over j of lambda_j,e^T ( dke Ke T_j,e + dce Me (T_j - T_{j-1})_e ), dce already divided by the
+// step size.  g0 is the lowest element's SW node, nn = nx + 1, Nn the node count; lambda_j is row
+// j - j0 of lam and T_j row j - hist_j0 of T; rows from `rows` on (1 <= rows <= H) are left out.
+// The row differences and sums of two neighbouring elements are shared, and each step's modes of
+// T serve the next one as T_{j-1}, so a step costs 13 FP64 instructions per element, 23 with the
+// capacity term (has_dc).
+template <int H>
+__device__ __forceinline__ void sens_strip_sum(int g0, int nn, int Nn, double h2, const double (&dke)[H],
+                                               const double (&dce)[H], bool has_dc, int rows,
+                                               const double* __restrict__ lam, int j0, const double* __restrict__ T,
+                                               int hist_j0, int ja, int jb, double (&out)[H]) {
+  double k1[H], k2[H], m9[H], m3[H], m1[H];
+  Modes prev[H];
+#pragma unroll
+  for (int i = 0; i < H; ++i) k1[i] = k2[i] = m9[i] = m3[i] = m1[i] = 0.0;
+  const double* Tp = T + (size_t)(ja - 1 - hist_j0) * Nn + g0;
+  const double* Lj = lam + (size_t)(ja - j0) * Nn + g0;
+  if (has_dc) {
+#pragma unroll
+    for (int i = 0; i < H; ++i)
+      if (i < rows) prev[i] = elem_modes(Tp[i * nn], Tp[i * nn + 1], Tp[(i + 1) * nn + 1], Tp[(i + 1) * nn]);
   }
-  return acc;
+  for (int j = ja; j <= jb; ++j) {
+    Tp += Nn;                                  // T_j
+    double tp, ts, lp, ls;                     // difference and sum along the row below
+    {
+      const double t0 = Tp[0], t1 = Tp[1], l0 = Lj[0], l1 = Lj[1];
+      tp = t1 - t0;
+      ts = t0 + t1;
+      lp = l1 - l0;
+      ls = l0 + l1;
+    }
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      if (i >= rows) break;
+      const double t0 = Tp[(i + 1) * nn], t1 = Tp[(i + 1) * nn + 1], l0 = Lj[(i + 1) * nn], l1 = Lj[(i + 1) * nn + 1];
+      const double tq = t1 - t0, tt = t0 + t1, lq = l1 - l0, lt = l0 + l1;
+      const Modes t{has_dc ? tt + ts : 0.0, tp + tq, tt - ts, tq - tp};
+      const Modes l{has_dc ? lt + ls : 0.0, lp + lq, lt - ls, lq - lp};
+      k1[i] = fma(l.b, t.b, fma(l.c, t.c, k1[i]));
+      k2[i] = fma(l.d, t.d, k2[i]);
+      if (has_dc) {
+        m9[i] = fma(l.a, t.a - prev[i].a, m9[i]);
+        m3[i] = fma(l.b, t.b - prev[i].b, fma(l.c, t.c - prev[i].c, m3[i]));
+        m1[i] = fma(l.d, t.d - prev[i].d, m1[i]);
+        prev[i] = t;
+      }
+      tp = tq;
+      ts = tt;
+      lp = lq;
+      ls = lt;
+    }
+    Lj += Nn;
+  }
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    out[i] = dke[i] * 0.25 * fma(2.0 / 3.0, k2[i], k1[i]);
+    if (has_dc) out[i] += dce[i] * h2 * (1.0 / 144.0) * fma(9.0, m9[i], fma(3.0, m3[i], m1[i]));
+  }
 }
 
 }  // namespace ptg

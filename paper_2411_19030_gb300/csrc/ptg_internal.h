@@ -355,6 +355,11 @@ cudaError_t launch_assemble(int nx, int ny, double h, const ptg_material& m, dou
                             const double* q_elem, const uint8_t* dirichlet, const AssembleOut& out, DevStats* st,
                             cudaStream_t stream);
 
+// The sensitivity reduction: strips of kSensRows elements per thread, blocks of a time chunk.
+constexpr int kSensRows = 4, kSensThreads = 128;
+inline int sens_blocks(int nx, int ny) {
+  return (nx * ((ny + kSensRows - 1) / kSensRows) + kSensThreads - 1) / kSensThreads;
+}
 cudaError_t launch_objective_from_modified(int Ne, double p, const double* Theta_mod, const double* grad_mod,
                                           double* Theta, double* grad, double* scratch, cudaStream_t stream);
 cudaError_t launch_sensitivities(int nx, int ny, int Nt, double h, double dt, int has_dc, const double* dk,

@@ -1309,33 +1309,21 @@ struct Stepper {
     const int nx = P.nx, nn = P.nx + 1;
     const int er = min(sb.R, P.ny - sb.r0);  // owned element rows ey in [r0, r0+er)
     const int nel = er > 0 ? er * nx : 0;
-    const double h2 = P.h * P.h / 36.0;
+    const double mass_scale = P.h * P.h / dt_step, inv_norm = 1.0 / nnorm;
     for (int t = threadIdx.x; t < nel; t += blockDim.x) {
       const int ler = t / nx, ex = t - ler * nx;
       const int ey = sb.r0 + ler;
       const int e = ey * nx + ex;
       const int l0 = (ler + 1) * sb.W + ex + 1;   // SW node in x64
-      const double lsw = x64[l0], lse = x64[l0 + 1], lne = x64[l0 + sb.W + 1], lnw = x64[l0 + sb.W];
+      const Modes l = elem_modes(x64[l0], x64[l0 + 1], x64[l0 + sb.W + 1], x64[l0 + sb.W]);
       const int g0 = ey * nn + ex;
       const double tsw = Tj[g0], tse = Tj[g0 + 1], tne = Tj[g0 + nn + 1], tnw = Tj[g0 + nn];
-      // lambda^T Ke T, Ke = (1/6)[[4,-1,-2,-1],[-1,4,-1,-2],[-2,-1,4,-1],[-1,-2,-1,4]] (order SW,SE,NE,NW)
-      const double ksw = 4.0 * tsw - tse - 2.0 * tne - tnw;
-      const double kse = -tsw + 4.0 * tse - tne - 2.0 * tnw;
-      const double kne = -2.0 * tsw - tse + 4.0 * tne - tnw;
-      const double knw = -tsw - 2.0 * tse - tne + 4.0 * tnw;
-      const double kterm = (lsw * ksw + lse * kse + lne * kne + lnw * knw) / 6.0;
-      double term = P.dk[e] * kterm;
-      if (P.has_dc) {
-        const double dsw = tsw - Tjm[g0], dse = tse - Tjm[g0 + 1], dne = tne - Tjm[g0 + nn + 1], dnw = tnw - Tjm[g0 + nn];
-        // lambda^T Me dT, Me = h^2/36 [[4,2,1,2],[2,4,2,1],[1,2,4,2],[2,1,2,4]]
-        const double msw = 4.0 * dsw + 2.0 * dse + dne + 2.0 * dnw;
-        const double mse = 2.0 * dsw + 4.0 * dse + 2.0 * dne + dnw;
-        const double mne = dsw + 2.0 * dse + 4.0 * dne + 2.0 * dnw;
-        const double mnw = 2.0 * dsw + dse + 2.0 * dne + 4.0 * dnw;
-        const double cterm = (lsw * msw + lse * mse + lne * mne + lnw * mnw) * h2;
-        term += P.dc[e] * cterm / dt_step;
-      }
-      double g = (gsrc ? gsrc[e] : 0.0) - term / nnorm;
+      double term = P.dk[e] * elem_stiffness(l, elem_modes(tsw, tse, tne, tnw));
+      if (P.has_dc)
+        term = fma(P.dc[e] * mass_scale,
+                   elem_mass(l, elem_modes(tsw - Tjm[g0], tse - Tjm[g0 + 1], tne - Tjm[g0 + nn + 1], tnw - Tjm[g0 + nn])),
+                   term);
+      double g = fma(-inv_norm, term, gsrc ? gsrc[e] : 0.0);
       if (addF) g += addF[e] - subG[e];
       gdst[e] = g;
     }
