@@ -88,14 +88,14 @@ struct ClusterComm {
     pend_n = 0;
   }
 
-  // All-reduce of the first NV (1 or 2) entries of v, then `post` as in GridComm.  `push` (sends of
-  // the same all-to-all phase) runs after the block barrier that makes this CTA's shared-memory
-  // writes visible.  Warp sums, then warp 0 adds the warps' partials and sends the CTA's sums to
-  // every rank; warp 0 waits, adds the ranks' sums, applies `post` and hands the result to the
-  // CTA.  Every rank adds the same values in the same order: the same bits everywhere.
-  template <class T, int NV, int NX, class Post, class Push = NoPush>
-  __device__ void allreduce(T (&v)[NV + NX], int cs, Post post, Push push = Push()) {
-    static_assert(NV <= 2 && NV * sizeof(T) <= 16, "one 16-byte slot per rank");
+  // All-reduce of the first NV entries of v, then `post` as in GridComm.  Warp sums, then warp 0
+  // adds the warps' partials and sends the CTA's sums to every rank; warp 0 waits, adds the ranks'
+  // sums, applies `post` and hands the result to the CTA.  Every rank adds the same values in the
+  // same order: the same bits everywhere.
+  template <class T, int NV, int NX, class Post>
+  __device__ void allreduce(T (&v)[NV + NX], int cs, Post post) {
+    constexpr int kWords = NV * (int)sizeof(T) > 16 ? 2 : 1;
+    static_assert(NV <= 4 && NV * sizeof(T) <= 32, "two 16-byte words per rank");
     RedBank<T>& rb = bank<T>(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -105,21 +105,25 @@ struct ClusterComm {
       for (int i = 0; i < NV; ++i) rb.warp[warp][i] = v[i];
     }
     __syncthreads();
-    push();
     if (warp == 0) {
-      union { uint4 u; T t[16 / sizeof(T)]; } pk;
-      pk.u = make_uint4(0, 0, 0, 0);
+      union { uint4 u[kWords]; T t[16 * kWords / sizeof(T)]; } pk;
 #pragma unroll
-      for (int i = 0; i < NV; ++i) pk.t[i] = warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
-      if (lane < cs)
-        st_async16(mapa_u32(smem_u32(&rs.slot[na & 1][rank()]), (unsigned)lane), pk.u,
-                   mapa_u32(smem_u32(bar_a()), (unsigned)lane));
-      if (lane == 0) mbar_expect(bar_a(), pend_a + 16u * (unsigned)cs);
+      for (int w = 0; w < kWords; ++w) pk.u[w] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) pk.t[i] = half_warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
+      if (lane < cs) {
+        const unsigned b = mapa_u32(smem_u32(bar_a()), (unsigned)lane);
+#pragma unroll
+        for (int w = 0; w < kWords; ++w)
+          st_async16(mapa_u32(smem_u32(&rs.slot[na & 1][w][rank()]), (unsigned)lane), pk.u[w], b);
+      }
+      if (lane == 0) mbar_expect(bar_a(), pend_a + 16u * kWords * (unsigned)cs);
       wait(bar_a(), (na >> 1) & 1);
-      pk.u = rs.slot[na & 1][lane < cs ? lane : 0];
+#pragma unroll
+      for (int w = 0; w < kWords; ++w) pk.u[w] = rs.slot[na & 1][w][lane < cs ? lane : 0];
       T t[NV + NX];
 #pragma unroll
-      for (int i = 0; i < NV; ++i) t[i] = warp_sum(lane < cs ? pk.t[i] : T{});
+      for (int i = 0; i < NV; ++i) t[i] = half_warp_sum(lane < cs ? pk.t[i] : T{});
 #pragma unroll
       for (int i = NV; i < NV + NX; ++i) t[i] = T{};
       post(t);
@@ -154,17 +158,8 @@ struct ClusterComm {
     return 16u * (unsigned)words16 * ((rank_ > 0 ? 1u : 0u) + (rank_ < cs - 1 ? 1u : 0u));
   }
   // Own first / last rows of a halo buffer (`buf` at row -1, row lr at buf + (lr+1) W) into the
-  // neighbours' halo rows, as part of the next all-to-all phase.
-  template <class T>
-  __device__ void push_halos(T* buf, const Slab& sb) {
-    const int n16 = sb.W * (int)sizeof(T) / 16;
-    int r0n = 0, Rn = 0;
-    if (sb.rank > 0) slab_rows(sb.ny + 1, sb.cs, sb.rank - 1, r0n, Rn);
-    send_rows(buf + sb.W, buf + sb.R * sb.W, buf + (Rn + 1) * sb.W, buf, n16, sb.rank, sb.cs, bar_a());
-    pend_a += row_bytes(n16, sb.rank, sb.cs);
-  }
-  // The same as a neighbour phase of its own: on return the halo rows are the neighbours' rows.
-  // The caller's block barrier has made this CTA's rows visible.
+  // neighbours' halo rows; on return the own halo rows are the neighbours' rows.  The caller's
+  // block barrier has made this CTA's rows visible.
   template <class T>
   __device__ void exchange(T* buf, const Slab& sb) {
     const int n16 = sb.W * (int)sizeof(T) / 16;
@@ -184,12 +179,11 @@ struct ClusterComm {
   }
   // Edge rows sent straight from registers: the thread holding columns [col, col+4) of the
   // owned row lr (0 or R-1) stores them into the neighbour's two-row buffer `edge` ([0]: the
-  // row below that CTA's slab, [1]: the row above).  They belong to the next all-to-all phase, or
-  // with `own` to a neighbour phase that finish_edges ends.
+  // row below that CTA's slab, [1]: the row above); a neighbour phase that finish_edges ends.
   __device__ void begin_edges() {}
   template <class T>
-  __device__ void put_edge(T* edge, int lr, int col, const T (&v)[4], const Slab& sb, bool own) {
-    unsigned long long* bar = own ? bar_n() : bar_a();
+  __device__ void put_edge(T* edge, int lr, int col, const T (&v)[4], const Slab& sb) {
+    unsigned long long* bar = bar_n();
     union { uint4 u[sizeof(T) / 4]; T t[4]; } pk;
 #pragma unroll
     for (int j = 0; j < 4; ++j) pk.t[j] = v[j];
@@ -207,8 +201,8 @@ struct ClusterComm {
     }
   }
   template <class T>
-  __device__ void end_edges(T*, const Slab& sb, bool own) {
-    (own ? pend_n : pend_a) += row_bytes(sb.W * (int)sizeof(T) / 16, sb.rank, sb.cs);
+  __device__ void end_edges(T*, const Slab& sb) {
+    pend_n += row_bytes(sb.W * (int)sizeof(T) / 16, sb.rank, sb.cs);
   }
   __device__ void finish_edges() { finish_n(); }
   // a 16-byte chunk of restricted partials, written at offset dst of every rank's slot array;
@@ -310,8 +304,8 @@ struct GridComm {
   }
   __device__ void sync() { barrier(); }
 
-  template <class T, int NV, int NX, class Post, class Push = NoPush>
-  __device__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post, Push push = Push()) {
+  template <class T, int NV, int NX, class Post>
+  __device__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post) {
     RedBank<T>& rb = bank<T>(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -321,7 +315,6 @@ struct GridComm {
       for (int i = 0; i < NV; ++i) rb.warp[warp][i] = v[i];
     }
     __syncthreads();
-    push();
     // 32 bytes per block whatever T: the groups of a launch are not in step, and one may reduce floats
     // while another reduces doubles
     constexpr int kPer = 32 / (int)sizeof(T);
@@ -411,7 +404,7 @@ struct GridComm {
   // Edge rows from registers (see ClusterComm::put_edge): into this CTA's slots of the next set.
   __device__ void begin_edges() { hset ^= 1; }
   template <class T>
-  __device__ void put_edge(T*, int lr, int col, const T (&v)[4], const Slab& sb, bool /*own*/) {
+  __device__ void put_edge(T*, int lr, int col, const T (&v)[4], const Slab& sb) {
     unsigned char* out = reinterpret_cast<unsigned char*>(P.g_halo) + halo_slot(hset, (int)blockIdx.x);
     if (lr == 0) {
       T* d = reinterpret_cast<T*>(out) + col;
@@ -426,7 +419,7 @@ struct GridComm {
     __threadfence();                                // each writer orders its own stores
   }
   template <class T>
-  __device__ void end_edges(T* edge, const Slab& sb, bool /*own*/) {
+  __device__ void end_edges(T* edge, const Slab& sb) {
     pending_lo = reinterpret_cast<unsigned char*>(edge);
     pending_hi = reinterpret_cast<unsigned char*>(edge + sb.W);
     pending_bytes = sb.W * (int)sizeof(T);

@@ -84,6 +84,12 @@ __device__ __forceinline__ ff vfma(const ff& a, const ff& x, float y) { return v
 __device__ __forceinline__ float vdot(float acc, float x, float y) { return fmaf(x, y, acc); }
 __device__ __forceinline__ ff vdot(const ff& acc, const ff& x, const ff& y) { return ff_acc(acc, x, y); }
 __device__ __forceinline__ ff vdot(const ff& acc, const ff& x, float y) { return ff_acc(acc, x, y); }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ ff vmul(const ff& a, const ff& b) {
+  float p, e;
+  ff_prod(a, b, p, e);
+  return fast_two_sum(p, e);
+}
 __device__ __forceinline__ float vdiv(float a, float b) { return a / b; }
 __device__ __forceinline__ ff vdiv(const ff& a, const ff& b) { return ff_div(a, b); }
 __device__ __forceinline__ float vneg(float a) { return -a; }

@@ -82,7 +82,7 @@ struct RedSmem {
   RedBank<float> f;
   RedBank<double> d;
   RedBank<ff> p;
-  uint4 slot[2][kMaxCluster];    // [phase][source rank]: that rank's partials (up to two values)
+  uint4 slot[2][2][kMaxCluster]; // [phase][16-byte word][source rank]: that rank's partials
   unsigned long long bar[4];     // the cluster's mbarriers (comm.cuh): two for all-to-all, two for neighbour phases
 };
 template <class T> __device__ __forceinline__ RedBank<T>& bank(RedSmem& rs);
@@ -94,11 +94,9 @@ struct NoPost {
   template <class T>
   __device__ __forceinline__ void operator()(T*) const {}
 };
-struct NoPush {
-  __device__ __forceinline__ void operator()() const {}
-};
 
-// Sum over the warp, the same bits in every lane.
+// Sum over the warp, the same bits in every lane; half_warp_sum: over lanes 0..15, in lane 0 .. 15
+// (the others' values are not used there).
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -107,6 +105,17 @@ __device__ __forceinline__ float warp_sum(float v) {
 __device__ __forceinline__ ff warp_sum(ff v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
+    v = v + make_ff(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o));
+  return v;
+}
+__device__ __forceinline__ float half_warp_sum(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ ff half_warp_sum(ff v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
     v = v + make_ff(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o));
   return v;
 }
@@ -139,6 +148,9 @@ __device__ __forceinline__ double warp_sum(double v) {
   const double d = __ll2double_rn(t);
   return __hiloint2double(__double2hiint(d) + ((emax - (1023 + 56)) << 20), __double2loint(d));
 }
+
+// (the lanes from 16 on hold zeros where this is called)
+__device__ __forceinline__ double half_warp_sum(double v) { return warp_sum(v); }
 
 // ---------------------------------------------------------------------------- slab geometry
 struct Slab {

@@ -220,7 +220,7 @@ inline __host__ __device__ int coarse_row_stride(int nax) { return (nax + 3) / 4
 // Shared-memory bytes of the two-level preconditioner for one CTA (naj aggregate rows); the
 // partials of every rank sit in shared memory for a cluster (slots = true), in global memory
 // for a grid-wide launch.  The V-cycle (vc) adds its smoother buffers over the slab and its
-// halo rows, the halo rows of q and r in the CG precision (real_bytes), and FP32 element
+// halo rows, the halo rows of r in the CG precision (real_bytes), and FP32 element
 // weights where the CG runs in FP64 (the FP32 CG has them already).
 inline size_t twolevel_smem_bytes(int W, int rmax, int cs, int nax, int nay, int naj, bool slots = true,
                                   bool vc = false, int real_bytes = 4, int nu = 1) {
@@ -235,7 +235,7 @@ inline size_t twolevel_smem_bytes(int W, int rmax, int cs, int nax, int nay, int
   b += ncp * 4;                             // their sum over the covering ranks
   b += (size_t)naj * naxp * 4;              // coarse correction of the CTA's aggregates
   if (vc) {
-    b += 4 * (size_t)W * real_bytes;        // q and r on the two halo rows
+    b += 2 * (size_t)W * real_bytes;        // r on the two halo rows
     b += 2 * halo * 4;                      // the smoother iterate (y, then u) and omega D^-1
     if (real_bytes == 8) b += 3 * elems * 4;  // FP32 (D, S, T) element weights
     if (nu >= 2) b += 2 * halo * 4;         // the slab-local smoother's two iterates
@@ -274,7 +274,7 @@ inline size_t threelevel_smem_bytes(int W, int rmax, int cs, int W1, int r1max, 
   if (slots) b += (size_t)cs * ncp * 4;     // restricted partials of every rank
   b += ncp * 4;                             // their sum over the covering ranks
   b += (size_t)naj * naxp * 4;              // coarse correction of the CTA's aggregates
-  b += 4 * (size_t)W * real_bytes;          // (the V-cycle's halo rows of q and r, unused here)
+  b += 2 * (size_t)W * real_bytes;          // (the V-cycle's halo rows of r, unused here)
   b += 2 * halo * 4;                        // fine smoother iterate and omega D^-1
   if (real_bytes == 8) b += 3 * elems * 4;  // FP32 (D, S, T) element weights
   if (nu >= 2) b += 2 * halo * 4;           // the slab-local smoother's two iterates

@@ -10,8 +10,8 @@
 // With Real = double the CG works in pairs of floats (ff.cuh) on the same per-node weights and the
 // first CG already meets the tolerance; with Real = float the CG uses FP32 element weights held in shared memory
 // and this is iterative refinement with FP64 residuals.  CG carries q = A p by the recurrence
-// q_{k+1} = A z_{k+1} + beta q_k, so each iteration has two cluster reductions and the halo
-// exchange of z, the only stencil operand, rides on the second one.
+// q_{k+1} = A z_{k+1} + beta q_k, so z is the only stencil operand and an iteration has one
+// exchange of its halo rows and one reduction.
 //
 // Task kinds (StepParams::kind), one task per cluster:
 //   FINE_PRI    Alg. 1 repeated M times from u_s (or chained over slices), history written.
@@ -72,7 +72,6 @@ struct Stepper {
   // V(1,1) two-grid cycle (P.tl_vc), see vcycle; aj0 / naj then cover the halo rows too
   bool vc = false;
   int ajo0 = 0, najo = 0;    // aggregate rows of the owned rows (the restriction's partials)
-  V* vqh = nullptr;       // q on the halo rows -1 and R (the neighbours' edge rows), [2][W]
   V* vrh = nullptr;       // r on the halo rows -1 and R, [2][W]
   float* vy = nullptr;       // y = S r, then u = y + P ec, rows -1..R
   float* vsd = nullptr;      // S = omega D^-1, rows -1..R (0 off the unknowns)
@@ -140,7 +139,6 @@ struct Stepper {
           // every array a multiple of 4 words, so each starts 16-byte aligned
           constexpr int rw = (int)(sizeof(V) / 4);
           float* v0 = t;
-          vqh = reinterpret_cast<V*>(t);  t += 2 * W * rw;
           vrh = reinterpret_cast<V*>(t);  t += 2 * W * rw;
           vy = t + kSlack;   t += halo;
           vsd = t + kSlack;  t += halo;
@@ -281,9 +279,9 @@ struct Stepper {
     return (ix >= 0 && ix <= P.nx) ? (sb.r0 + lr) * (P.nx + 1) + ix : -1;
   }
 
-  template <class T, int NV, int NX = 0, class Post = NoPost, class Push = NoPush>
-  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post(), Push push = Push()) {
-    comm.template allreduce<T, NV, NX, Post, Push>(v, sb.cs, post, push);
+  template <class T, int NV, int NX = 0, class Post = NoPost>
+  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post()) {
+    comm.template allreduce<T, NV, NX, Post>(v, sb.cs, post);
   }
 
   // Select the operator C/dt + K (fine) or C/dtau + K (coarse): per-node FP64 weights for the
@@ -553,8 +551,6 @@ struct Stepper {
   // cluster (16-byte stores of 4 aggregates); the next cluster barrier (the one of the
   // following all-reduce) makes them visible.  coarse_gather then adds, chunk by chunk, the
   // partials of the covering ranks in rank order and multiplies by the CTA's rows of Ac^-1.
-  // In the CG loop the coarse correction follows r by the same recurrence as r,
-  // ec -= alpha Ac^-1 P^T q, so restricting q needs no cluster barrier of its own.
   template <class T>
   __device__ void coarse_restrict_push(const T (&v)[NG][4]) {
     const int G = sb.G, m4 = P.cm / 4, nax = P.nax, naxp = coarse_row_stride(nax), ncp = naxp * P.nay;
@@ -601,10 +597,10 @@ struct Stepper {
     comm.expect_tl(tl_bytes);
   }
 
-  // After the cluster barrier that follows coarse_restrict_push: qc = sum over the covering
-  // ranks of the partials (in rank order), then ec = Ac^-1 qc (first == true) or
-  // ec -= alpha Ac^-1 qc on the CTA's aggregate rows (8 lanes per row of Ac^-1, 16-byte loads).
-  __device__ void coarse_gather(bool first, float alpha) {
+  // After the phase that follows coarse_restrict_push: qc = sum over the covering ranks of the
+  // partials (in rank order), then ec = Ac^-1 qc on the CTA's aggregate rows (8 lanes per row of
+  // Ac^-1, 16-byte loads).
+  __device__ void coarse_gather() {
     const int naxp = coarse_row_stride(P.nax), ncp = naxp * P.nay;
     const float* slots = comm.tl_slots(tl_slot);
     for (int L4 = threadIdx.x; L4 < ncp / 4; L4 += blockDim.x) {
@@ -639,7 +635,7 @@ struct Stepper {
       acc += __shfl_xor_sync(0xffffffffu, acc, 1);
       acc += __shfl_xor_sync(0xffffffffu, acc, 2);
       acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-      if (part == 0 && row < nrows) tl_ec[row] = first ? acc : fmaf(-alpha, acc, tl_ec[row]);
+      if (part == 0 && row < nrows) tl_ec[row] = acc;
     }
     __syncthreads();
   }
@@ -665,17 +661,17 @@ struct Stepper {
 
   // The owned edge rows (0 and R-1) of a per-thread vector into the neighbours' two-row buffer
   // `edge` ([0]: the row below the slab, [1]: the row above), straight from registers; visible
-  // after the next all-reduce, or with `own` after comm.finish_edges().
-  __device__ void put_edges(V* edge, const V (&v)[NG][4], bool own) {
+  // after comm.finish_edges().
+  __device__ void put_edges(V* edge, const V (&v)[NG][4]) {
     comm.begin_edges();
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
       const int lr = l0 / sb.W - 1;
-      if (lr == 0 || lr == sb.R - 1) comm.put_edge(edge, lr, l0 - (lr + 1) * sb.W, v[k], sb, own);
+      if (lr == 0 || lr == sb.R - 1) comm.put_edge(edge, lr, l0 - (lr + 1) * sb.W, v[k], sb);
     }
-    comm.end_edges(edge, sb, own);
+    comm.end_edges(edge, sb);
   }
 
   // offset in a rows -1..R buffer of entry i of the two halo rows ([0, W): row -1, [W, 2W): row R)
@@ -685,7 +681,7 @@ struct Stepper {
   //   y = S r,  ec = Ac^-1 P^T (r - A y),  u = y + P ec (in place of y),  z = u + S (r - A u),
   // with the damped-Jacobi smoother S = omega D^-1 and A applied with the FP32 element weights,
   // so that I - M^-1 A = (I - S A)(I - P Ac^-1 P^T A)(I - S A) (symmetric).  The halo rows of r
-  // (vrh) follow the owners' CG recurrence bit for bit, and every CTA computes ec for the
+  // (vrh) are the owners' rows, and every CTA computes ec for the
   // aggregate rows its halo rows touch from the same restricted vector, so y and u on a halo
   // row equal the owner's values: M^-1 is one operator across the CTAs.  One cluster barrier
   // (the restricted partials).  z goes to zbuf on the owned rows; returns the local (r, z).
@@ -720,7 +716,7 @@ struct Stepper {
     }
     coarse_restrict_push(w);
     comm.finish_tl();
-    coarse_gather(true, 0.f);
+    coarse_gather();
     for (int gi = threadIdx.x; gi < (sb.R + 2) * G; gi += blockDim.x) {
       const int a = tl_gagg[gi];
       const float e = a >= 0 ? tl_ec[a] : 0.f;
@@ -815,7 +811,7 @@ struct Stepper {
     }
     coarse_restrict_push(w);
     comm.finish_tl();
-    coarse_gather(true, 0.f);
+    coarse_gather();
     for (int gi = threadIdx.x; gi < (sb.R + 2) * G; gi += blockDim.x) {
       const int a = tl_gagg[gi];
       const float ea = a >= 0 ? tl_ec[a] : 0.f;
@@ -944,7 +940,7 @@ struct Stepper {
     }
     comm.expect_tl(tl_bytes);
     comm.finish_tl();
-    coarse_gather(true, 0.f);
+    coarse_gather();
     // u1 = e1 + P2 ec on the owned and halo 2h rows
     for (int t = threadIdx.x; t < (R1 + 2) * n1; t += blockDim.x) {
       const int lr1 = t / n1 - 1, I = t - (lr1 + 1) * n1, J = J0 + lr1;
@@ -1130,6 +1126,9 @@ struct Stepper {
   // of two to a squared 2-norm rr0 in [1, 4); on return x64 += unscale * d.  Stops when
   // ||r||^2 <= target2 (scaled units) or at the iteration limit; returns the iteration count.
   // Vectors, scalars and dot products are V; z is float.
+  // One reduction per iteration (Chronopoulos and Gear's arrangement): A z instead of A p, with
+  // q = A p and (p, q) by recurrence, so the iteration waits for the neighbours' rows of z and for
+  // one all-reduce instead of two.
   // The float pairs of the FP64 kinds: on a slab of 9 x 132 nodes (128 x 128 over 16 CTAs) an
   // iteration's stencil, updates and dot products took 10 100 cycles on the FP64 pipe (17 FP64
   // instructions per node) and take about 180 FP32 instructions per node in pairs.
@@ -1140,72 +1139,65 @@ struct Stepper {
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) d[k][j] = p[k][j] = q[k][j] = V{};
     }
-    const bool additive = COARSE && tl && !vc;                   // restricts r once, then q
-    const bool global1 = COARSE && vc && !l3 && P.tl_nu < 2;     // keeps r on the halo rows
-    V rz = V{}, beta = V{};
-    int it = -1;                   // -1: the start, whose z and (r, z) open the iteration
-    bool done = !(rr0 > target2);
+    const bool additive = COARSE && tl && !vc;                   // needs r restricted
+    const bool global1 = COARSE && vc && !l3 && P.tl_nu < 2;     // needs r on the halo rows
+    V rz_old = V{}, pq_old = V{};
+    int it = 0;
     for (;;) {
-      V v[3] = {V{}, V{}, V{}};
-      if (it < 0) {
-        if (additive) {
-          coarse_restrict_push(r);
-          comm.finish_tl();
-          coarse_gather(true, 0.f);
-        } else if (global1) {
-          put_edges(vrh, r, true);   // r on the halo rows from the neighbours' owned edge rows
-          comm.finish_edges();
-        }
-      } else {
-        // q = A z + beta q, p = z + beta p, (p, q); alpha = rz / (p, q)
-        V pq[1] = {V{}};
-#pragma unroll
-        for (int k = 0; k < NG; ++k) {
-          const int l0 = loc0[k];
-          if (l0 < 0) continue;
-          V w[4];
-          apply_A(zbuf, l0, w);
-#pragma unroll
-          for (int j = 0; j < kGroup; ++j) {
-            const V wj = unknown(k, j) ? w[j] : V{};
-            p[k][j] = vfma(beta, p[k][j], zbuf[l0 + j]);
-            q[k][j] = vfma(beta, q[k][j], wj);
-            pq[0] = vdot(pq[0], p[k][j], q[k][j]);
-          }
-        }
-        if (global1)
-          put_edges(vqh, q, false);  // the neighbours' copies of r on their halo rows follow q
-        else if (additive)
-          coarse_restrict_push(q);   // (both visible after the all-reduce)
-        const V rz_c = rz;
-        allreduce<V, 1>(pq, [rz_c](V* t) { t[0] = vdiv(rz_c, t[0]); });
-        const V alpha = pq[0], nalpha = vneg(alpha);
-        if (additive) coarse_gather(false, f32(alpha));
-        // d += alpha p, r -= alpha q; (r, r)
-#pragma unroll
-        for (int k = 0; k < NG; ++k) {
-          if (loc0[k] < 0) continue;
-#pragma unroll
-          for (int j = 0; j < kGroup; ++j) {
-            d[k][j] = vfma(alpha, p[k][j], d[k][j]);
-            r[k][j] = vfma(nalpha, q[k][j], r[k][j]);
-            v[1] = vdot(v[1], r[k][j], r[k][j]);
-          }
-        }
-        if (global1)
-          for (int i = threadIdx.x; i < 2 * sb.W; i += blockDim.x) vrh[i] = vfma(nalpha, vqh[i], vrh[i]);
+      if (additive) {
+        coarse_restrict_push(r);
+        comm.finish_tl();
+        coarse_gather();
+      } else if (global1) {
+        put_edges(vrh, r);
+        comm.finish_edges();
       }
-      // z = M^-1 r, (r, z) and beta = (r, z)_new / (r, z)
+      // z = M^-1 r and w = A z; (r, z), (z, w) and (r, r) in one reduction; then
+      //   beta = (r, z) / (r, z)_old,  (p, q) = (z, w) - beta^2 (p, q)_old,  alpha = (r, z) / (p, q)
+      V v[6] = {V{}, V{}, V{}, V{}, V{}, V{}};
       v[0] = precondition(r);
-      const V rz_c = rz;
-      const bool start = it < 0;
-      allreduce<V, 2, 1>(v, [rz_c, start](V* t) { if (!start) t[2] = vdiv(t[0], rz_c); },
-                         [&] { comm.push_halos(zbuf, sb); });
-      ++it;
-      if (!start && !(f32(v[1]) > target2)) done = true;
-      beta = v[2];
-      rz = v[0];
-      if (done || it >= P.itmax) break;
+      exchange(zbuf);
+      V w[NG][4];
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const int l0 = loc0[k];
+        if (l0 < 0) continue;
+        apply_A(zbuf, l0, w[k]);
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) {
+          if (!unknown(k, j)) w[k][j] = V{};
+          v[1] = vdot(v[1], w[k][j], zbuf[l0 + j]);
+          v[2] = vdot(v[2], r[k][j], r[k][j]);
+        }
+      }
+      const bool start = it == 0;
+      allreduce<V, 3, 3>(v, [start, rz_old, pq_old](V* t) {
+        if (start) {
+          t[5] = t[1];
+        } else {
+          t[4] = vdiv(t[0], rz_old);
+          t[5] = vfma(vneg(vmul(t[4], t[4])), pq_old, t[1]);
+        }
+        t[3] = vdiv(t[0], t[5]);
+      });
+      if (!((start ? rr0 : f32(v[2])) > target2)) break;
+      const V alpha = v[3], nalpha = vneg(alpha), beta = v[4];
+      rz_old = v[0];
+      pq_old = v[5];
+      // p = z + beta p, q = w + beta q, d += alpha p, r -= alpha q
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const int l0 = loc0[k];
+        if (l0 < 0) continue;
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) {
+          p[k][j] = vfma(beta, p[k][j], zbuf[l0 + j]);
+          q[k][j] = vfma(beta, q[k][j], w[k][j]);
+          d[k][j] = vfma(alpha, p[k][j], d[k][j]);
+          r[k][j] = vfma(nalpha, q[k][j], r[k][j]);
+        }
+      }
+      if (++it >= P.itmax) break;
     }
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
