@@ -70,7 +70,7 @@ struct ptg_op {
   double *q_elem = nullptr, *q_time = nullptr;
   uint8_t* dirichlet = nullptr;
   double* sens_partial = nullptr;
-  double* lam_prev = nullptr;  // [n Ntau][Nn] ring of the last n states of each fine task (primal or adjoint)
+  double* lam_prev = nullptr;  // [n Ntau][(ny + 1) W] ring of the last n states of each fine task (primal or adjoint)
   double* scratch = nullptr;   // [2] small device scalars
   // grid-wide launches (one system over every SM): reduction partials, barrier, halo rows,
   // two-level partials
@@ -263,18 +263,6 @@ size_t wide_twolevel_bytes(const void* ctx, int G) {
   return twolevel_bytes(c->op, c->precision, c->kind, G, c->tl_mode, false);
 }
 
-// Inner tolerance of an FP64 CG with the additive two-level preconditioner.  Its coarse
-// correction is applied in FP32 and carried by the CG recurrence, so its rounding is relative
-// to the residual the CG started from.  Once the CG has reduced its residual by much more than
-// 1e-4 that rounding dominates the coarse correction and the CG stalls (measured: 2000 instead
-// of 61 iterations per solve at 1e-5 on a near-binary design).  So each CG stops at a 1e-4
-// reduction (or the op's looser inner_rtol) and the FP64 residual loop restarts it from the
-// exact residual.  The two-grid cycle is recomputed from r at every iteration and carries no
-// such error, so its FP64 CG runs to the final tolerance in one go (measured on the 128 x 128
-// pass: one refinement sweep per solve instead of two, 53.8 instead of 55.9 ms, and no stall
-// on near-binary designs).
-constexpr double kTwoLevelInnerFp64 = 1e-4;
-
 void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode) {
   P.tl_naj = twolevel_rows(op, precision, P.kind, P.cs, tl_mode);
   P.tl_vc = P.tl_naj > 0 && uses_vcycle(op, tl_mode);
@@ -283,10 +271,8 @@ void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode
   // local_steps 3 (multigrid) applies to streamed fine propagators only: the default elsewhere
   const int ls = op->sv.local_steps == 3 ? 0 : op->sv.local_steps;
   P.local_steps = ls > 0 ? ls : kLocalSteps;
-  // FP32 CG: the op's inner tolerance; FP64 CG: to the final tolerance in one go, or in
-  // kTwoLevelInnerFp64 steps with the additive two-level preconditioner
-  if (precision == PTG_FP64)
-    P.inner_rtol = P.tl_naj > 0 && !P.tl_vc ? std::max(kTwoLevelInnerFp64, op->sv.inner_rtol) : 0.0;
+  // FP32 CG: the op's inner tolerance; FP64 CG: to the final tolerance in one go
+  if (precision == PTG_FP64) P.inner_rtol = 0.0;
   if (P.tl_naj == 0) return;
   if (tl_mode >= TL_VCYCLE3) {
     // the V-cycle's fine buffers plus the 2h level; the aggregate level is on the 2h grid
@@ -302,7 +288,6 @@ void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode
     P.cm = op->tl3_m;
     P.nax = op->tl3_nax;
     P.nay = op->tl3_nay;
-    P.inner_rtol = precision == PTG_FP64 ? 0.0 : P.inner_rtol;
     return;
   }
   P.Ainv = op->tl_Ainv;
@@ -311,12 +296,19 @@ void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode
   P.nay = op->tl_nay;
 }
 
+// Whether a kind reads the saved A x of its last residual: fine steps that start from the last
+// state alone (ptg_solve.initial_guess = 1).
+bool uses_saved_ax(const ptg_op* op, int kind) {
+  return !coarse_kind(kind) && op->sv.initial_guess == 1;
+}
+
 // Best plan for `ntasks` concurrent clusters with or without the two-level preconditioner:
 // fewest waves, then the shortest per-thread work (ng), then the largest cluster.  Returns
 // the number of waves, or -1 if nothing fits.
 long best_plan(ptg_op* op, int precision, int kind, int ntasks, int tl_mode, Plan* out, bool keep_ax = true) {
   const int nx = op->g.nx, ny = op->g.ny;
   const int G = op->W / kGroup;
+  keep_ax = keep_ax && uses_saved_ax(op, kind);
   long best_waves = -1;
   for (int cs : {16, 8, 4, 2, 1}) {
     const int rmax = (ny + 1 + cs - 1) / cs;
@@ -464,7 +456,7 @@ int choose_plan(ptg_op* op, int precision, int kind, int ntasks, Plan* out) {
         Plan w;
         WideCtx ctx{op, precision, kind, mode};
         if (query_wide_plan(op->g.nx, op->g.ny, precision, kind, ntasks, spread, wide_twolevel_bytes, &ctx, &w,
-                            keep_ax) == cudaSuccess) {
+                            keep_ax && uses_saved_ax(op, kind)) == cudaSuccess) {
           w.twolevel = twolevel_rows(op, precision, kind, w.cs, mode) > 0;
           w.vc = w.twolevel && uses_vcycle(op, mode);
           op->plans[key] = w;
@@ -548,6 +540,8 @@ void base_params(const ptg_op* op, StepParams& P) {
   P.extrap = guess_states(op->sv);
   P.guess_next = P.extrap > 1;
   P.prev_field = op->lam_prev;
+  P.ring_stride = (long long)(op->g.ny + 1) * op->W;
+  P.mass_uniform = op->has_dc ? 0.0 : op->mat.c0 * op->g.h * op->g.h / 36.0;
 }
 
 #ifdef PTG_DEBUG
@@ -947,7 +941,7 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
   A(&op->dirichlet, op->Nn);
   A(&op->sens_partial, (size_t)op->sens_chunks * op->Ne * sizeof(double));
   if (guess_states(*solve) > 1)
-    A(&op->lam_prev, (size_t)guess_states(*solve) * time->Ntau * op->Nn * sizeof(double));
+    A(&op->lam_prev, (size_t)guess_states(*solve) * time->Ntau * (grid->ny + 1) * op->W * sizeof(double));
   // two-level preconditioner: aggregates of m x m nodes, m the smallest multiple of 4 giving
   // at most kCoarseMaxAgg aggregates per direction
   if (solve->twolevel) {
@@ -1145,7 +1139,8 @@ int ptg_op_set_plan(ptg_op* op, int kind, int cs, int ng) {
     for (bool keep_ax : {true, false}) {
       Plan p;
       cudaError_t e = query_stepper_plan(op->g.nx, op->g.ny, prec, kind, cs, ng, nthreads,
-                                         twolevel_bytes(op, prec, kind, cs, mode), &p, keep_ax);
+                                         twolevel_bytes(op, prec, kind, cs, mode), &p,
+                                         keep_ax && uses_saved_ax(op, kind));
       if (e != cudaSuccess) {
         cudaGetLastError();
         continue;
@@ -1509,7 +1504,7 @@ constexpr int kPhases = 10;
 struct BatchBuf {
   double *T_hist, *U_T, *U_th, *V_l, *V_g, *U_T_new, *U_th_new, *V_l_new, *V_g_new;
   double *F_T, *F_th, *G_T, *G_th, *F_l, *F_g, *G_l, *G_g, *rho;
-  double* lam_prev;   // [n Ntau][Nn] fine-step initial guesses (null when the op starts plainly)
+  double* lam_prev;   // [n Ntau][(ny + 1) W] fine-step initial guesses (null when the op starts plainly)
 };
 
 struct PhasePlan {
@@ -1648,12 +1643,19 @@ std::vector<int2> phase_tasks(const ptg_batch* b, int ph) {
   return t;
 }
 
+bool batch_saves_ax(const ptg_batch* b, int kind) {
+  for (const ptg_op* op : b->ops)
+    if (uses_saved_ax(op, kind)) return true;
+  return false;
+}
+
 // Install a plan for a phase: validate it for every design, upload the parameter table and
 // the task list, and size the persistent grid.  tl_mode: the strongest two-level form the
 // designs may use where it applies.
 int batch_install(ptg_batch* b, int ph, int cs, int ng, int nthreads, int tl_mode, bool keep_ax = true) {
   const int kind = phase_kind(ph);
   const int prec = kind_precision(b->precision, kind);
+  keep_ax = keep_ax && batch_saves_ax(b, kind);
   size_t smem = 0;
   for (int d = 0; d < (int)b->ops.size(); ++d) {
     if (!in_launch(b, d, ph)) continue;
@@ -1699,6 +1701,7 @@ long batch_best(ptg_batch* b, int ph, int tl_mode, int ntasks, int* best_cs, int
                 bool keep_ax = true) {
   long best_waves = -1;
   const int prec = kind_precision(b->precision, phase_kind(ph));
+  keep_ax = keep_ax && batch_saves_ax(b, phase_kind(ph));
   for (int cs : {16, 8, 4, 2}) {
     for (int ng : kStepNG) {
       int nt = 32;
@@ -1960,7 +1963,7 @@ int ptg_batch_create(ptg_op* const* ops, int nops, ptg_batch** out) {
     A(&B.F_l, T * Nn); A(&B.F_g, T * Ne); A(&B.G_l, T * Nn); A(&B.G_g, T * Ne);
     A(&B.rho, Ne);
     B.lam_prev = nullptr;
-    if (guess_states(op->sv) > 1) A(&B.lam_prev, guess_states(op->sv) * T * Nn);
+    if (guess_states(op->sv) > 1) A(&B.lam_prev, (size_t)guess_states(op->sv) * T * (op->g.ny + 1) * op->W);
     b->bufs.push_back(B);
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->queue, kPhases * sizeof(int));

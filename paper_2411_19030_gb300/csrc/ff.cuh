@@ -112,11 +112,12 @@ __device__ __forceinline__ ff split_scaled(double v, int k) {
   r.l = ef > 52 ? __uint2float_rn(lo & 0x1fffffffu) * __uint_as_float(sign | ((unsigned)(ef - 52) << 23)) : 0.f;
   return r;
 }
-// a float as a double by integer operations; 0 below the normal range, not for infinities
+// a float as a double by integer operations; 0 below the normal range
 __device__ __forceinline__ double widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  if ((u & 0x7f800000u) == 0u) return 0.0;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+  const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m < 0x00800000u) return 0.0;
+  const unsigned hi = m >= 0x7f800000u ? (m >> 3) | 0x7ff00000u : (m >> 3) + (896u << 20);
+  return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
 }
 
 }  // namespace ptg

@@ -135,8 +135,10 @@ struct StepParams {
   int extrap;                // fine kinds: start each CG from the extrapolation through the slice's
                              // last `extrap` states (1: the last state alone; up to kMaxExtrap)
   int guess_next;            // coarse kinds: start each CG from the guess state at the slice's other end
-  double* prev_field;        // fine kinds with extrap > 1: [extrap tasks][Nn] ring of each task's last
-                             // states (or null: every step starts from the last state)
+  double* prev_field;        // fine kinds with extrap > 1: [extrap tasks][ring_stride] ring of each task's
+                             // last states (or null: every step starts from the last state)
+  long long ring_stride;     // entries of one state: padded node rows 0 .. ny
+  double mass_uniform;       // c h^2 / 36 where the capacity does not depend on rho (has_dc == 0)
   int tl_nu;                 // V-cycle smoothing: <= 1 one global Jacobi step before and after; k >= 2 k
                              // slab-local steps before and after
   // three-level cycle (P.tl_l3): the V-cycle's coarse correction becomes a two-grid cycle of its

@@ -40,7 +40,7 @@ struct Stepper {
   Slab sb;
   // shared memory (each pointer at the first non-slack entry)
   double* x64;      // FP64 state, rows -1..R
-  double* b64;      // FP64 right-hand side, rows 0..R-1
+  double* b64;      // FP64 right-hand side, rows 0..R-1 (in an FP32 kind's solve: the residual)
   float* zbuf;      // CG stencil operand, rows -1..R
   float* dinv;      // Jacobi inverse diagonal, rows 0..R-1 (0 on Dirichlet and pad nodes)
   float* wd = nullptr;  // FP32 element weights (D, S, T), element rows r0-1..r0+R-1 (FP32 CG, V-cycle)
@@ -426,30 +426,38 @@ struct Stepper {
   // CTA evaluates the same expression on the same operands and the halos stay exact: no
   // exchange is needed.  If wr is given, x_1 is first saved there on the owned rows (the
   // slice's ring of states; wr is none of the X).  Ends with __syncthreads.
+  // The ring's rows are padded node rows (P.W entries a row, rows 0 .. ny), so a thread moves groups
+  // of 4 with 16-byte loads; pads and Dirichlet nodes are zero in every state.
   __device__ void extrapolate_x64(int n, const double* const* X, double* __restrict__ wr) {
     ax_valid = false;
     __syncthreads();
-    const int nn = P.nx + 1;
-    const int rows = sb.R + 2;
-    for (int t = threadIdx.x; t < rows * nn; t += blockDim.x) {
-      const int row = t / nn, ix = t - row * nn;
-      const int g = sb.r0 - 1 + row;
-      if (g >= 0 && g <= P.ny) {
-        const int gi = g * nn + ix;
-        double& x = x64[row * sb.W + ix + 1];
-        const double x1 = x;
-        if (wr && row >= 1 && row <= sb.R) wr[gi] = x1;
-        if (n < 2) continue;
-        double v;
-        if (n == 2) {
-          v = fma(2.0, x1, -X[0][gi]);
-        } else if (n == 3) {
-          v = fma(3.0, x1 - X[0][gi], X[1][gi]);
-        } else {
-          v = fma(4.0, x1 + X[1][gi], -fma(6.0, X[0][gi], X[2][gi]));
-        }
-        x = P.dirichlet[gi] ? 0.0 : v;
+    const int G = sb.G, total = (sb.R + 2) * G;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+      const int row = t / G, y = sb.r0 - 1 + row;
+      if (y < 0 || y > P.ny) continue;
+      double* x = x64 + kGroup * t;
+      const size_t o = (size_t)(sb.r0 - 1) * P.W + kGroup * t;
+      double x1[4], v[4], a[4], b[4], c[4];
+      load4(x, x1);
+      if (n >= 2) load4(X[0] + o, a);
+      if (n >= 3) load4(X[1] + o, b);
+      if (n >= 4) load4(X[2] + o, c);
+      if (wr && row >= 1 && row <= sb.R) {
+        *reinterpret_cast<double2*>(wr + o) = make_double2(x1[0], x1[1]);
+        *reinterpret_cast<double2*>(wr + o + 2) = make_double2(x1[2], x1[3]);
       }
+      if (n < 2) continue;
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) {
+        if (n == 2)
+          v[j] = fma(2.0, x1[j], -a[j]);
+        else if (n == 3)
+          v[j] = fma(3.0, x1[j] - a[j], b[j]);
+        else
+          v[j] = fma(4.0, x1[j] + b[j], -fma(6.0, a[j], c[j]));
+      }
+      *reinterpret_cast<double2*>(x) = make_double2(v[0], v[1]);
+      *reinterpret_cast<double2*>(x + 2) = make_double2(v[2], v[3]);
     }
     __syncthreads();
   }
@@ -476,6 +484,30 @@ struct Stepper {
   }
   __device__ void exchange_x64() { exchange(x64); }
 
+  // (C/dt) x64 on a group.  With a uniform capacity the mass stencil is (c h^2/36) (1 4 1) x (1 4 1)
+  // (2 instead of 4 on the boundary): 4 FP64 instructions per node and no weights, instead of 9.
+  __device__ __forceinline__ void mass_dt(int l0, double (&y)[4]) const {
+    if (P.has_dc) {
+      stencil_node64<double>(x64, l0, P.mass, l0 + gshift, sb.W, y);
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) y[j] *= inv_dt;
+      return;
+    }
+    const int lr = l0 / sb.W - 1, iy = sb.r0 + lr, ix0 = l0 - (lr + 1) * sb.W - 1;
+    const double dy = iy == 0 || iy == P.ny ? 2.0 : 4.0, s = P.mass_uniform * inv_dt;
+    double xl[6], xm[6], xh[6];
+    load_window(x64, l0 - sb.W, xl);
+    load_window(x64, l0, xm);
+    load_window(x64, l0 + sb.W, xh);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) xm[i] = fma(dy, xm[i], xl[i] + xh[i]);
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) {
+      const double dx = ix0 + j == 0 || ix0 + j == P.nx ? 2.0 : 4.0;
+      y[j] = s * fma(dx, xm[j + 1], xm[j] + xm[j + 2]);
+    }
+  }
+
   // b64 = (C/dt) x64 + src, with src(global node) supplied per owned free node.
   template <class Src>
   __device__ void build_rhs(Src src) {
@@ -484,11 +516,11 @@ struct Stepper {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
       double y[4];
-      stencil_node64<double>(x64, l0, P.mass, l0 + gshift, sb.W, y);
+      mass_dt(l0, y);
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const bool free_node = dinv[l0 + j] != 0.f;
-        b64[l0 + j] = free_node ? fma(y[j], inv_dt, src(gnode(l0, j))) : 0.0;
+        b64[l0 + j] = free_node ? y[j] + src(gnode(l0, j)) : 0.0;
       }
     }
   }
@@ -1199,6 +1231,17 @@ struct Stepper {
       }
       if (++it >= P.itmax) break;
     }
+    if constexpr (kMixed) {
+      // d with its halo rows in zbuf
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const int l0 = loc0[k];
+        if (l0 < 0) continue;
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) zbuf[l0 + j] = d[k][j];
+      }
+      exchange(zbuf);
+    }
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
@@ -1207,10 +1250,44 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) {
         double x = x64[l0 + j];
         if constexpr (!kMixed) x = fma(widen(d[k][j].l), unscale, x);
-        x64[l0 + j] = fma((double)f32(d[k][j]), unscale, x);
+        x64[l0 + j] = fma(widen(f32(d[k][j])), unscale, x);
       }
     }
     return it;
+  }
+
+  // After an FP32 CG (d with its halo rows in zbuf): x64's halo rows follow their owners' update bit
+  // for bit, and the residual in b64 follows x64 += unscale d by
+  //   r -= unscale A d,
+  // A d summed in float pairs: d is a small correction of x64, so the 48 bits of its product are
+  // finer than the rounding of an FP64 b - A x64, and a refinement costs 3 FP64 instructions per
+  // node here instead of 11.  Returns the local sum of r^2.
+  __device__ double update_residual(double unscale, double (&r64)[NG][4]) {
+    for (int i = threadIdx.x; i < 2 * sb.W; i += blockDim.x) {
+      const int l = halo_offset(i);
+      x64[l] = fma(widen(zbuf[l]), unscale, x64[l]);
+    }
+    const double us = -unscale / ffw.scale;   // powers of two
+    double rr = 0.0;
+#pragma unroll
+    for (int k = 0; k < NG; ++k) {
+      const int l0 = loc0[k];
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) r64[k][j] = 0.0;
+      if (l0 < 0) continue;
+      ff y[4];
+      stencil_ff(zbuf, l0, ffw, l0 + gshift, sb.W, y);
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) {
+        if (!unknown(k, j)) continue;
+        const double t = fma(widen(y[j].l), us, fma(widen(y[j].h), us, b64[l0 + j]));
+        if (ax64) ax64[l0 + j] -= t - b64[l0 + j];
+        b64[l0 + j] = t;
+        r64[k][j] = t;
+        rr = fma(t, t, rr);
+      }
+    }
+    return rr;
   }
 
   // Solve (C/dt + K) x = b64 with x64 (owned + halos) as initial guess; on return x64 holds
@@ -1226,7 +1303,10 @@ struct Stepper {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) bb_rr[0] = fma(b64[l0 + j], b64[l0 + j], bb_rr[0]);
+      for (int j = 0; j < kGroup; ++j) {
+        bb_rr[0] = fma(b64[l0 + j], b64[l0 + j], bb_rr[0]);
+        if constexpr (kMixed) b64[l0 + j] = r64[k][j];   // the residual from here on (update_residual)
+      }
     }
     allreduce<double, 2>(bb_rr);
     const double bb = bb_rr[0];
@@ -1252,10 +1332,16 @@ struct Stepper {
       // (the pairs carry a residual to about 1e-15 of its start)
       const float target2 = fmaxf((float)(fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr) * rr0), 1e-30f);
       // A d = r in the scale of the float pairs gives d / scale
-      its += cg_correct(r, (float)rr0, target2, exp2_int(k2) * (kMixed ? 1.0 : ffw.scale));
+      const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
+      its += cg_correct(r, (float)rr0, target2, unscale);
       ++sweeps;
-      exchange_x64();
-      double v[1] = {residual(r64)};
+      double v[1];
+      if constexpr (kMixed) {
+        v[0] = update_residual(unscale, r64);
+      } else {
+        exchange_x64();
+        v[0] = residual(r64);
+      }
       allreduce<double, 1>(v);
       rr = v[0];
     }
@@ -1382,12 +1468,15 @@ struct Stepper {
     const double inv_norm = 1.0 / ((double)P.Nt * (double)P.Ne);
     set_operator();
     load_x64(P.in_field + (size_t)sa * P.Nn);
-    double theta = P.in_aux[sa];
+    // theta^p (or theta of the modified objective), a plain sum over the steps: the root is taken at
+    // the end of a slice only (an FP64 pow takes 6 000 cycles of the one thread that needs it)
+    const bool power = P.objective != PTG_OBJ_MODIFIED;
+    double theta = power ? ipow(P.in_aux[sa], P.p_int) : P.in_aux[sa];
     if (P.chained) {                              // a sequential run also records its start
       if (double* row = hist_row(M * sa)) store_x64(row);
     }
     const int nring = P.extrap;
-    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.Nn : nullptr;
+    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.ring_stride : nullptr;
     int saved = 0;                                // states of this slice in the ring
     for (int s = sa; s < sb_end; ++s) {
       for (int j = M * s + 1; j <= M * (s + 1); ++j) {
@@ -1402,17 +1491,17 @@ struct Stepper {
           if (j == M * s + 1) saved = 0;
           const int n = min(saved + 1, nring);
           const double* X[kMaxExtrap - 1];
-          for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.Nn;
-          extrapolate_x64(n, X, ring + (size_t)((j - 1) % nring) * P.Nn);
+          for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.ring_stride;
+          extrapolate_x64(n, X, ring + (size_t)((j - 1) % nring) * P.ring_stride);
           ++saved;
         }
         solve(j, ring == nullptr);
         const double sp = pnorm_p();
-        if (threadIdx.x == 0) theta = accumulate_theta(theta, sp * inv_norm);  // used by thread 0 only
+        theta = fma(sp, inv_norm, theta);
         if (double* row = hist_row(j)) store_x64(row);
       }
       store_x64(P.out_field + (size_t)s * P.Nn);
-      if (threadIdx.x == 0 && sb.rank == 0) P.out_aux[s] = theta;
+      if (threadIdx.x == 0 && sb.rank == 0) P.out_aux[s] = power ? pow(theta, 1.0 / P.p) : theta;
     }
   }
 
@@ -1505,7 +1594,7 @@ struct Stepper {
     // (j+1) mod P.extrap and reads the n-1 <= P.extrap-1 others, so no CTA writes a row that a
     // neighbour reads in the same step
     const int nring = P.extrap;
-    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.Nn : nullptr;
+    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.ring_stride : nullptr;
     int saved = 0;   // states of this slice in the ring
     for (int s = s_hi; s >= s_lo; --s) {
       double* gdst = P.out_aux + (size_t)s * P.Ne;
@@ -1521,8 +1610,8 @@ struct Stepper {
         if (ring) {
           const int n = min(saved + 1, nring);
           const double* X[kMaxExtrap - 1];
-          for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.Nn;
-          extrapolate_x64(n, X, ring + (size_t)((j + 1) % nring) * P.Nn);
+          for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.ring_stride;
+          extrapolate_x64(n, X, ring + (size_t)((j + 1) % nring) * P.ring_stride);
           ++saved;
         }
         solve(j, ring == nullptr);

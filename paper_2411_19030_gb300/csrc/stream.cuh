@@ -713,31 +713,31 @@ struct Streamer {
 
   // b = (C/dt) xp + src(node) on the own rows; xn = the start of the step: the extrapolation
   // through xp and the ring rows X[0..n-2] (n = 1: xp itself); the ring row wr receives xp.
-  // The ring rows are node vectors ([Nn], unpadded).
+  // The ring rows are padded node rows 0 .. ny; pads and Dirichlet nodes are zero in every state.
   template <class Src>
   __device__ void begin_step(const double* __restrict__ xp, double* __restrict__ xn, int n, const double* const* X,
                              double* __restrict__ wr, Src src) {
     for_groups([&](int loc, int iy, int g) {
-      double y[4], x1[4], bv[4], xv[4];
-      stencil_node64<double>(xp, loc, P.mass, loc, P.W, y);
+      double y[4], x1[4], bv[4], xv[4], a[4], b_[4], c[4];
+      const int o = loc - P.W;
       load4(xp + loc, x1);
+      if (n >= 2) load4(X[0] + o, a);
+      if (n >= 3) load4(X[1] + o, b_);
+      if (n >= 4) load4(X[2] + o, c);
+      stencil_node64<double>(xp, loc, P.mass, loc, P.W, y);
+      if (wr) st4d(wr, o, x1);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int gi = gnode(iy, g, j);
-        bv[j] = 0.0;
-        xv[j] = 0.0;
-        if (gi < 0) continue;
-        if (wr) wr[gi] = x1[j];
-        if (P.dirichlet[gi]) continue;
-        bv[j] = fma(y[j], inv_dt, src(gi));
+        bv[j] = gi < 0 || P.dirichlet[gi] ? 0.0 : fma(y[j], inv_dt, src(gi));
         if (n <= 1)
           xv[j] = x1[j];
         else if (n == 2)
-          xv[j] = fma(2.0, x1[j], -X[0][gi]);
+          xv[j] = fma(2.0, x1[j], -a[j]);
         else if (n == 3)
-          xv[j] = fma(3.0, x1[j] - X[0][gi], X[1][gi]);
+          xv[j] = fma(3.0, x1[j] - a[j], b_[j]);
         else
-          xv[j] = fma(4.0, x1[j] + X[1][gi], -fma(6.0, X[0][gi], X[2][gi]));
+          xv[j] = fma(4.0, x1[j] + b_[j], -fma(6.0, a[j], c[j]));
       }
       st4d(b, loc, bv);
       st4d(xn, loc, xv);
@@ -889,7 +889,7 @@ struct Streamer {
     comm.sync();
     double theta = P.in_aux[s];
     const int nring = P.extrap;
-    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.Nn : nullptr;
+    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.ring_stride : nullptr;
     int saved = 0;
     for (int j = M * s + 1; j <= M * (s + 1); ++j) {
       const double qj = P.q_time[j];
@@ -898,8 +898,8 @@ struct Streamer {
       double* wr = nullptr;
       if (ring) {
         n = min(saved + 1, nring);
-        for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.Nn;
-        wr = ring + (size_t)((j - 1) % nring) * P.Nn;
+        for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.ring_stride;
+        wr = ring + (size_t)((j - 1) % nring) * P.ring_stride;
         ++saved;
       }
       begin_step(x_prev, x_cur, n, X, wr, [&](int g) { return qj * P.fload[g]; });
@@ -926,7 +926,7 @@ struct Streamer {
     const double* gsrc = P.in_aux + (size_t)(s + 1) * P.Ne;
     double* gdst = P.out_aux + (size_t)s * P.Ne;
     const int nring = P.extrap;
-    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.Nn : nullptr;
+    double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.ring_stride : nullptr;
     int saved = 0;
     for (int j = M * (s + 1); j >= M * s + 1; --j) {
       const double* Tj = hist_row(j);
@@ -940,8 +940,8 @@ struct Streamer {
       double* wr = nullptr;
       if (ring) {
         n = min(saved + 1, nring);
-        for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.Nn;
-        wr = ring + (size_t)((j + 1) % nring) * P.Nn;
+        for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.ring_stride;
+        wr = ring + (size_t)((j + 1) % nring) * P.ring_stride;
         ++saved;
       }
       begin_step(x_prev, x_cur, n, X, wr, [&](int g) { return scale * ipow(Tj[g], P.p_int - 1); });
