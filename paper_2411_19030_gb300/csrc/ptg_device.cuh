@@ -357,6 +357,74 @@ __device__ __forceinline__ void stencil_elem32(const float* __restrict__ z, cons
   }
 }
 
+// The same from the elements' conductivity and capacity parts k = k_e/6 and m = c_e h^2/(36 step),
+// D = 4 (k + m), S = 2 m - k, T = m - 2 k, and with the window entries beyond a lane's own 16 bytes
+// taken from the neighbouring lanes: the groups of a warp are consecutive in the row-padded
+// buffers (from one row's last group to the next row's first, whose pads are zero), so only the
+// warp's first and last lane load them.  A 4-byte load at a 16-byte stride takes 4 shared-memory
+// wavefronts, like the 16-byte load beside it; this form takes about 45 wavefronts per warp where
+// stencil_elem32 takes 84, and the smoothers and the FP32 CG are bound by them (17 x 132 nodes in
+// two CTAs: 2 860 cycles per application).  Every lane of the warp calls it.
+__device__ __forceinline__ void warp_window(const float* __restrict__ x, int b, int lane, float (&w)[6]) {
+  const float4 c = *reinterpret_cast<const float4*>(x + b);
+  float e = 0.f;
+  if (lane == 0 || lane == 31) e = x[lane == 0 ? b - 1 : b + 4];
+  const float l = __shfl_up_sync(0xffffffffu, c.w, 1), r = __shfl_down_sync(0xffffffffu, c.x, 1);
+  w[0] = lane == 0 ? e : l;
+  w[1] = c.x; w[2] = c.y; w[3] = c.z; w[4] = c.w;
+  w[5] = lane == 31 ? e : r;
+}
+__device__ __forceinline__ void warp_ewindow(const float* __restrict__ x, int b, int lane, float (&w)[5]) {
+  const float4 c = *reinterpret_cast<const float4*>(x + b);
+  float e = 0.f;
+  if (lane == 0) e = x[b - 1];
+  const float l = __shfl_up_sync(0xffffffffu, c.w, 1);
+  w[0] = lane == 0 ? e : l;
+  w[1] = c.x; w[2] = c.y; w[3] = c.z; w[4] = c.w;
+}
+__device__ __forceinline__ void stencil_km32(const float* __restrict__ z, const float* __restrict__ wk,
+                                             const float* __restrict__ wm, int loc0, int W, int lane, float (&y)[4],
+                                             bool no_lo = false, bool no_hi = false) {
+  float zl[6], zm[6], zh[6], kl[5], ml[5], ku[5], mu[5];
+  warp_window(z, loc0 - W, lane, zl);
+  warp_window(z, loc0, lane, zm);
+  warp_window(z, loc0 + W, lane, zh);
+  warp_ewindow(wk, loc0 - W, lane, kl);
+  warp_ewindow(wm, loc0 - W, lane, ml);
+  warp_ewindow(wk, loc0, lane, ku);
+  warp_ewindow(wm, loc0, lane, mu);
+  if (no_lo) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) zl[i] = 0.f;
+  }
+  if (no_hi) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) zh[i] = 0.f;
+  }
+  float d[5], sl[5], su[5], tl[5], tu[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    d[i] = (kl[i] + ml[i]) + (ku[i] + mu[i]);
+    sl[i] = fmaf(2.f, ml[i], -kl[i]);
+    su[i] = fmaf(2.f, mu[i], -ku[i]);
+    tl[i] = fmaf(-2.f, kl[i], ml[i]);
+    tu[i] = fmaf(-2.f, ku[i], mu[i]);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float a = 4.f * (d[j] + d[j + 1]) * zm[j + 1];
+    a = fmaf(sl[j] + su[j], zm[j], a);             // west
+    a = fmaf(sl[j + 1] + su[j + 1], zm[j + 2], a); // east
+    a = fmaf(sl[j] + sl[j + 1], zl[j + 1], a);     // south
+    a = fmaf(su[j] + su[j + 1], zh[j + 1], a);     // north
+    a = fmaf(tl[j], zl[j], a);
+    a = fmaf(tl[j + 1], zl[j + 2], a);
+    a = fmaf(tu[j], zh[j], a);
+    a = fmaf(tu[j + 1], zh[j + 2], a);
+    y[j] = a;
+  }
+}
+
 // Element bilinear forms of Eq. 4.7 in the modes that Ke and Me share as eigenvectors: with the
 // corner values in the order SW, SE, NE, NW the sums a = (1, 1, 1, 1), b = (-1, 1, 1, -1),
 // c = (-1, -1, 1, 1) and d = (1, -1, 1, -1) have the eigenvalues 0, 1, 1, 2/3 of Ke and

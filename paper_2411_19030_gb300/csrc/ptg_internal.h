@@ -239,7 +239,7 @@ inline size_t twolevel_smem_bytes(int W, int rmax, int cs, int nax, int nay, int
   if (vc) {
     b += 2 * (size_t)W * real_bytes;        // r on the two halo rows
     b += 2 * halo * 4;                      // the smoother iterate (y, then u) and omega D^-1
-    if (real_bytes == 8) b += 3 * elems * 4;  // FP32 (D, S, T) element weights
+    if (real_bytes == 8) b += 2 * elems * 4;  // FP32 element weights (k, m)
     if (nu >= 2) b += 2 * halo * 4;         // the slab-local smoother's two iterates
   }
   b += groups * 4;                          // group sums of the restricted vector
@@ -278,7 +278,7 @@ inline size_t threelevel_smem_bytes(int W, int rmax, int cs, int W1, int r1max, 
   b += (size_t)naj * naxp * 4;              // coarse correction of the CTA's aggregates
   b += 2 * (size_t)W * real_bytes;          // (the V-cycle's halo rows of r, unused here)
   b += 2 * halo * 4;                        // fine smoother iterate and omega D^-1
-  if (real_bytes == 8) b += 3 * elems * 4;  // FP32 (D, S, T) element weights
+  if (real_bytes == 8) b += 2 * elems * 4;  // FP32 element weights (k, m)
   if (nu >= 2) b += 2 * halo * 4;           // the slab-local smoother's two iterates
   b += halo * 4;                            // fine residual with halo rows
   b += 5 * halo1 * 4;                       // 2h: e1, u1, z1, two smoother iterates
@@ -300,7 +300,7 @@ inline size_t stepper_smem_bytes(int nx, int rmax, int real_bytes, bool keep_ax 
   if (keep_ax) b += own * sizeof(double);      // ax64: A x of the last residual evaluation (optional)
   b += halo * 4;                               // zbuf: CG stencil operand with halos (float in both)
   b += own * 4;                                // dinv: Jacobi inverse diagonal (0 off the unknowns)
-  if (real_bytes == 4) b += 3 * elems * 4;     // (D, S, T) element weights for the FP32 CG
+  if (real_bytes == 4) b += 2 * elems * 4;     // (k, m) element weights for the FP32 CG
   return (b + 15) & ~size_t(15);
 }
 

@@ -43,9 +43,8 @@ struct Stepper {
   double* b64;      // FP64 right-hand side, rows 0..R-1 (in an FP32 kind's solve: the residual)
   float* zbuf;      // CG stencil operand, rows -1..R
   float* dinv;      // Jacobi inverse diagonal, rows 0..R-1 (0 on Dirichlet and pad nodes)
-  float* wd = nullptr;  // FP32 element weights (D, S, T), element rows r0-1..r0+R-1 (FP32 CG, V-cycle)
-  float* ws = nullptr;
-  float* wt = nullptr;
+  float* wk = nullptr;  // FP32 element weights, element rows r0-1..r0+R-1 (FP32 CG, V-cycle): the conductivity
+  float* wm = nullptr;  // and the capacity part, k_e / 6 and c_e h^2 / (36 step) (stencil_km32)
   // per-thread groups: loc0[k] = offset of the group's first node in the halo buffers, -1 if none
   int loc0[NG];
   unsigned fmask = 0;   // bit 4k+j: node j of group k is an unknown (free, not a pad)
@@ -122,7 +121,7 @@ struct Stepper {
       db[i] = 0.f;
     }
     if constexpr (kMixed) {
-      for (int i = threadIdx.x; i < 3 * elems; i += blockDim.x) eb[i] = 0.f;
+      for (int i = threadIdx.x; i < 2 * elems; i += blockDim.x) eb[i] = 0.f;
     }
     {
       if (P.tl_naj > 0) {
@@ -130,7 +129,7 @@ struct Stepper {
         const int groups = P.rmax * (W / kGroup);
         // after the element weights (FP32 CG only); 16-byte aligned: every earlier array is a
         // multiple of 4 words
-        float* t = eb + (kMixed ? 3 * elems : 0);
+        float* t = eb + (kMixed ? 2 * elems : 0);
         tl_ainv = t;  t += P.tl_naj * naxp * ncp;
         tl_slot = t;  t += P.wide ? 0 : P.cs * ncp;   // grid-wide: the partials are in global memory
         tl_qc = t;    t += ncp;
@@ -147,10 +146,9 @@ struct Stepper {
             ve1 = t + kSlack;  t += halo;
           }
           if constexpr (!kMixed) {
-            wd = t + kSlack;
-            ws = t + elems + kSlack;
-            wt = t + 2 * elems + kSlack;
-            t += 3 * elems;
+            wk = t + kSlack;
+            wm = t + elems + kSlack;
+            t += 2 * elems;
           }
           for (float* z = v0 + threadIdx.x; z < t; z += blockDim.x) *z = 0.f;
         }
@@ -256,9 +254,8 @@ struct Stepper {
     zbuf = zb + kSlack;
     dinv = db + kSlack - W;    // dinv[loc] likewise
     if constexpr (kMixed) {
-      wd = eb + kSlack;
-      ws = eb + elems + kSlack;
-      wt = eb + 2 * elems + kSlack;
+      wk = eb + kSlack;
+      wm = eb + elems + kSlack;
     }
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
@@ -313,9 +310,9 @@ struct Stepper {
       const int n = (sb.R + 1) * W;
       const double* src = wE + sb.r0 * W;               // padded element row r0 = element row r0 - 1
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        wd[i] = (float)src[i];
-        ws[i] = (float)src[PE + i];
-        wt[i] = (float)src[2 * PE + i];
+        const double Dw = src[i], Sw = src[PE + i];   // 4 (k + m) and 2 m - k
+        wk[i] = (float)(fma(-2.0, Sw, Dw) * (1.0 / 6.0));
+        wm[i] = (float)(fma(4.0, Sw, Dw) * (1.0 / 12.0));
       }
     }
     fmask = 0;
@@ -568,11 +565,11 @@ struct Stepper {
     return rr;
   }
 
-  __device__ __forceinline__ void apply_A(const float* z, int l0, V (&w)[4]) const {
-    if constexpr (kMixed)
-      stencil_elem32(z, wd, ws, wt, l0, sb.W, w);
-    else
-      stencil_ff(z, l0, ffw, l0 + gshift, sb.W, w);
+  // A z on group k with the FP32 element weights; every lane calls it (a lane without the group
+  // computes on the first one)
+  __device__ __forceinline__ void apply32(const float* z, int k, float (&y)[4], bool no_lo = false,
+                                          bool no_hi = false) const {
+    stencil_km32(z, wk, wm, loc0[k] < 0 ? sb.W : loc0[k], sb.W, threadIdx.x & 31, y, no_lo, no_hi);
   }
 
   // Two-level preconditioner M^-1 = D^-1 + P Ac^-1 P^T of the coarse-step solves (CG in either
@@ -740,9 +737,9 @@ struct Stepper {
       const int l0 = loc0[k];
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = 0.f;
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? rf[k][j] - t[j] : 0.f;
     }
@@ -761,9 +758,9 @@ struct Stepper {
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const float z = unknown(k, j) ? fmaf(vsd[l0 + j], rf[k][j] - t[j], vy[l0 + j]) : 0.f;
@@ -799,9 +796,9 @@ struct Stepper {
 #pragma unroll
       for (int k = 0; k < NG; ++k) {
         const int l0 = loc0[k];
-        if (l0 < 0) continue;
         float t[4];
-        stencil_elem32(buf, wd, ws, wt, l0, sb.W, t);
+        apply32(buf, k, t);
+        if (l0 < 0) continue;
 #pragma unroll
         for (int j = 0; j < kGroup; ++j) e[k][j] = fmaf(vsd[l0 + j], s[k][j] - t[j], e[k][j]);
       }
@@ -835,9 +832,9 @@ struct Stepper {
       const int l0 = loc0[k];
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = 0.f;
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? rf[k][j] - t[j] : 0.f;
     }
@@ -855,9 +852,9 @@ struct Stepper {
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? f32(r[k][j]) - t[j] : 0.f;
     }
@@ -1026,9 +1023,9 @@ struct Stepper {
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
       const int l0 = loc0[k];
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) vw[l0 + j] = unknown(k, j) ? w[k][j] - t[j] : 0.f;
     }
@@ -1052,9 +1049,9 @@ struct Stepper {
       const int l0 = loc0[k];
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = 0.f;
-      if (l0 < 0) continue;
       float t[4];
-      stencil_elem32(vy, wd, ws, wt, l0, W, t);
+      apply32(vy, k, t);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) w[k][j] = unknown(k, j) ? f32(r[k][j]) - t[j] : 0.f;
     }
@@ -1105,10 +1102,10 @@ struct Stepper {
       const int l0 = loc0[k];
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) z[k][j] = 0.f;
-      if (l0 < 0) continue;
       const int lr = l0 / sb.W - 1;
       float t[4];
-      stencil_elem32(zbuf, wd, ws, wt, l0, sb.W, t, lr == 0, lr == sb.R - 1);
+      apply32(zbuf, k, t, lr == 0, lr == sb.R - 1);
+      if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) z[k][j] = fmaf(om * dinv[l0 + j], f32(r[k][j]) - t[j], e[k][j]);
     }
@@ -1193,8 +1190,9 @@ struct Stepper {
 #pragma unroll
       for (int k = 0; k < NG; ++k) {
         const int l0 = loc0[k];
+        if constexpr (kMixed) apply32(zbuf, k, w[k]);
         if (l0 < 0) continue;
-        apply_A(zbuf, l0, w[k]);
+        if constexpr (!kMixed) stencil_ff(zbuf, l0, ffw, l0 + gshift, sb.W, w[k]);
 #pragma unroll
         for (int j = 0; j < kGroup; ++j) {
           if (!unknown(k, j)) w[k][j] = V{};
