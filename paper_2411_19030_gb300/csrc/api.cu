@@ -296,6 +296,21 @@ void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode
   P.nay = op->tl_nay;
 }
 
+// Threads per CTA for ng groups per thread.  The three-level cycle holds its 2h nodes ng + 1 to a
+// thread; with one group per thread the block gets a thread per 2h node, so that every pass over
+// them is one trip (128 x 128 over 16 CTAs: 325 nodes, 297 groups).  Too many for a block where the
+// 2h nodes do not fit.
+int step_threads(const ptg_op* op, int kind, int cs, int ng, int groups, int tl_mode) {
+  int nthreads = ((groups + ng - 1) / ng + 31) / 32 * 32;
+  int r1max = 0;
+  if (tl_mode >= TL_VCYCLE3 && threelevel_rows(op, kind, cs, tl_mode, &r1max) > 0) {
+    const int nodes = r1max * (op->g.nx / 2 + 1);
+    if (ng == 1) nthreads = std::max(nthreads, std::min((nodes + 31) / 32 * 32, kStepMaxThreadsHost));
+    if (nodes > (ng + 1) * nthreads) return kStepMaxThreadsHost + 32;
+  }
+  return nthreads;
+}
+
 // Whether a kind reads the saved A x of its last residual: fine steps that start from the last
 // state alone (ptg_solve.initial_guess = 1).
 bool uses_saved_ax(const ptg_op* op, int kind) {
@@ -315,7 +330,7 @@ long best_plan(ptg_op* op, int precision, int kind, int ntasks, int tl_mode, Pla
     if (rmax < 2) continue;
     const int groups = rmax * G;
     for (int ng : kStepNG) {
-      const int nthreads = ((groups + ng - 1) / ng + 31) / 32 * 32;
+      const int nthreads = step_threads(op, kind, cs, ng, groups, tl_mode);
       if (nthreads > kStepMaxThreadsHost) continue;
       Plan p;
       cudaError_t e = query_stepper_plan(nx, ny, precision, kind, cs, ng, nthreads,
@@ -1130,12 +1145,13 @@ int ptg_op_set_plan(ptg_op* op, int kind, int cs, int ng) {
   if (rmax < 2) return PTG_EINVAL;
   const int groups = rmax * (op->W / kGroup);
   if (ng < 1 || ng > kStepNG[kNumStepNG - 1]) return PTG_EINVAL;
-  const int nthreads = ((groups + ng - 1) / ng + 31) / 32 * 32;
-  if (nthreads > kStepMaxThreadsHost) return PTG_EINVAL;
+  if (((groups + ng - 1) / ng + 31) / 32 * 32 > kStepMaxThreadsHost) return PTG_EINVAL;
   // with the strongest two-level form where it applies and fits, else with Jacobi
   for (int mode = strongest_mode(op); mode >= TL_NONE; --mode) {
     const int prec = kind_precision(op->sv.precision, kind);
     if (mode > TL_NONE && twolevel_rows(op, prec, kind, cs, mode) == 0) continue;
+    const int nthreads = step_threads(op, kind, cs, ng, groups, mode);
+    if (nthreads > kStepMaxThreadsHost) continue;
     for (bool keep_ax : {true, false}) {
       Plan p;
       cudaError_t e = query_stepper_plan(op->g.nx, op->g.ny, prec, kind, cs, ng, nthreads,

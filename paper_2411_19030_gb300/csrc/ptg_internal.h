@@ -282,8 +282,7 @@ inline size_t threelevel_smem_bytes(int W, int rmax, int cs, int W1, int r1max, 
   if (nu >= 2) b += 2 * halo * 4;           // the slab-local smoother's two iterates
   b += halo * 4;                            // fine residual with halo rows
   b += 5 * halo1 * 4;                       // 2h: e1, u1, z1, two smoother iterates
-  b += 11 * own1 * 4;                       // 2h: restricted residual, 9 weights, omega / diag
-  b += (size_t)naj * naxp * 4;              // per-aggregate partial sums
+  b += 10 * own1 * 4;                       // 2h: 9 weights, omega / diag
   b += (size_t)nay * 2 * 4;                 // covering rank range per aggregate row
   return (b + 15) & ~size_t(15);
 }

@@ -80,16 +80,17 @@ struct Stepper {
   // of the CTA below), padded 2h row width W1, stride own1s of the owned-row 2h arrays
   bool l3 = false;
   int J0 = 0, R1 = 0, R1b = 0, W1 = 0, own1s = 0;
+  // this thread's owned 2h nodes: offset in the halo buffers (-1 if none) and local aggregate
+  static constexpr int K1 = NG + 1;
+  int n1o[K1], n1a[K1];
   float* vw = nullptr;       // fine residual w0 = r - A e0, rows -1..R
   float* b1x = nullptr;      // 2h rows -1..R1: e1 = S1 r1 (halo rows from the neighbours)
   float* b1u = nullptr;      //                 u1 = e1 + P2 ec (owned and halo rows, computed here)
   float* b1z = nullptr;      //                 z1 = u1 + S1 (r1 - A1 u1) (halo rows from the neighbours)
   float* s1a = nullptr;      //                 slab-local smoothing iterates (halo rows kept at zero)
   float* s1b = nullptr;
-  float* r1 = nullptr;       // owned 2h rows: restricted residual r1 = P1^T w0 (then r1 - A1 u1)
   float* a1w = nullptr;      // [9][own1s] A1 weights of the owned 2h nodes, k = (dJ + 1) * 3 + (dI + 1)
   float* s1d = nullptr;      // omega / diag(A1) of the owned 2h nodes
-  float* l3_items = nullptr; // partial sums of the 2h residual per aggregate of the owned rows
 
   __device__ Stepper(const StepParams& P_, Comm& comm_, unsigned char* dyn) : P(P_), comm(comm_) {
     sb.nx = P.nx;
@@ -163,10 +164,8 @@ struct Stepper {
           b1z = t + kSlack;  t += halo1;
           s1a = t + kSlack;  t += halo1;
           s1b = t + kSlack;  t += halo1;
-          r1 = t + kSlack - W1;  t += own1s;     // r1[lr1 * W1 + I + 1]: owned rows from lr1 = 0
-          a1w = t + kSlack - W1; t += 9 * own1s;
+          a1w = t + kSlack - W1; t += 9 * own1s;     // indexed like the halo buffers from lr1 = 0
           s1d = t + kSlack - W1; t += own1s;
-          l3_items = t;      t += P.tl_naj * naxp;
           for (float* z = l0 + threadIdx.x; z < t; z += blockDim.x) *z = 0.f;
           tl_cov = reinterpret_cast<int*>(t);
           l1_rows_of_slab(sb.r0, sb.R, J0, R1);
@@ -180,6 +179,17 @@ struct Stepper {
           naj = l3_agg(J0 + R1 <= ny1 ? J0 + R1 : ny1, P.cm, P.nay) - aj0 + 1;
           ajo0 = l3_agg(J0, P.cm, P.nay);
           najo = l3_agg(J0 + R1 - 1, P.cm, P.nay) - ajo0 + 1;
+#pragma unroll
+          for (int u = 0; u < K1; ++u) {
+            const int n1 = P.l3_nx1 + 1, i = threadIdx.x + u * blockDim.x;
+            n1o[u] = -1;
+            n1a[u] = 0;
+            if (i < R1 * n1) {
+              const int lr1 = i / n1, I = i - lr1 * n1;
+              n1o[u] = (lr1 + 1) * W1 + I + 1;
+              n1a[u] = (l3_agg(J0 + lr1, P.cm, P.nay) - aj0) * naxp + l3_agg(I, P.cm, P.nax);
+            }
+          }
           for (int J = threadIdx.x; J < P.nay; J += blockDim.x) {
             int lo = -1, hi = -1;
             for (int q = 0; q < P.cs; ++q) {
@@ -338,7 +348,7 @@ struct Stepper {
       // the 2h stencil and omega / diag of the owned 2h nodes (FP32)
       const int n1 = P.l3_nx1 + 1, nn1 = n1 * (P.l3_ny1 + 1);
       for (int t = threadIdx.x; t < R1 * n1; t += blockDim.x) {
-        const int lr1 = t / n1, I = t - lr1 * n1, o = lr1 * W1 + I + 1;
+        const int lr1 = t / n1, I = t - lr1 * n1, o = (lr1 + 1) * W1 + I + 1;
         const int g = (J0 + lr1) * n1 + I;
 #pragma unroll
         for (int k = 0; k < 9; ++k) a1w[k * own1s + o] = (float)P.A1[(size_t)k * nn1 + g];
@@ -875,17 +885,20 @@ struct Stepper {
   }
 
   // ---------------------------------------------------------------- three-level cycle
-  // 2h buffers: halo buffers (rows -1..R1) at (lr1 + 1) W1 + I + 1, owned-row arrays at lr1 W1 + I + 1
-  __device__ __forceinline__ int h1(int lr1, int I) const { return (lr1 + 1) * W1 + I + 1; }
-  __device__ __forceinline__ int o1(int lr1, int I) const { return lr1 * W1 + I + 1; }
+  // 2h buffers: halo buffers (rows -1..R1) at (lr1 + 1) W1 + I + 1; the owned-row arrays a1w and s1d
+  // are addressed by the same offset
 
-  // (A1 x) at the owned 2h node (lr1, I) from a halo buffer x (zero outside the 2h grid)
-  __device__ __forceinline__ float a1_apply(const float* __restrict__ x, int lr1, int I) const {
-    const int c = h1(lr1, I), o = o1(lr1, I);
-    float y = 0.f;
+  // (A1 x) at the owned 2h node with offset c from a halo buffer x (zero outside the 2h grid)
+  __device__ __forceinline__ float a1_apply(const float* __restrict__ x, int c) const {
+    const float* w = a1w + c;
+    float lo = 0.f, mid = 0.f, hi = 0.f;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) y = fmaf(a1w[k * own1s + o], x[c + (k / 3 - 1) * W1 + (k % 3 - 1)], y);
-    return y;
+    for (int k = 0; k < 3; ++k) {
+      lo = fmaf(w[k * own1s], x[c - W1 + k - 1], lo);
+      mid = fmaf(w[(3 + k) * own1s], x[c + k - 1], mid);
+      hi = fmaf(w[(6 + k) * own1s], x[c + W1 + k - 1], hi);
+    }
+    return (lo + hi) + mid;
   }
 
   // refresh the 2h halo rows of every CTA from the neighbours' owned rows
@@ -896,100 +909,126 @@ struct Stepper {
 
   // P.tl_nu damped-Jacobi steps of A1_s e = s from e = 0 on the owned 2h rows, with the 2h halo
   // rows held at zero (the diagonal block of A1 of this CTA's rows: a fixed polynomial in
-  // S1 A1_s times S1, symmetric, no communication); e goes to the owned rows of `out`.
-  __device__ void smooth_l1(const float* __restrict__ s, float* __restrict__ out) {
-    const int n1 = P.l3_nx1 + 1, n = R1 * n1;
+  // S1 A1_s times S1, symmetric, no communication).  Every thread keeps its nodes in registers; the
+  // iterates ping-pong through s1a and s1b.
+  __device__ __forceinline__ void smooth_l1(const float (&sv)[K1], float (&e)[K1]) {
+#pragma unroll
+    for (int u = 0; u < K1; ++u) e[u] = n1o[u] >= 0 ? s1d[n1o[u]] * sv[u] : 0.f;
     float* cur = s1a;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      cur[h1(lr1, I)] = s1d[o1(lr1, I)] * s[o1(lr1, I)];
-    }
-    __syncthreads();
     for (int it = 1; it < P.tl_nu; ++it) {
-      float* nxt = cur == s1a ? s1b : s1a;
-      for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int lr1 = t / n1, I = t - lr1 * n1;
-        nxt[h1(lr1, I)] = fmaf(s1d[o1(lr1, I)], s[o1(lr1, I)] - a1_apply(cur, lr1, I), cur[h1(lr1, I)]);
-      }
+#pragma unroll
+      for (int u = 0; u < K1; ++u)
+        if (n1o[u] >= 0) cur[n1o[u]] = e[u];
       __syncthreads();
-      cur = nxt;
+#pragma unroll
+      for (int u = 0; u < K1; ++u)
+        if (n1o[u] >= 0) e[u] = fmaf(s1d[n1o[u]], sv[u] - a1_apply(cur, n1o[u]), e[u]);
+      cur = cur == s1a ? s1b : s1a;
     }
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      out[h1(lr1, I)] = cur[h1(lr1, I)];
-    }
-    __syncthreads();
   }
 
   // The 2h part of the three-level cycle, from the fine residual w0 in vw (halo rows exchanged):
   //   r1 = P1^T w0;  e1 = S1 r1;  ec = A2^-1 P2^T (r1 - A1 e1);  u1 = e1 + P2 ec;
   //   z1 = u1 + S1 (r1 - A1 u1) into b1z with its halo rows exchanged.
+  // The plan gives the block a thread per owned 2h node, so a pass over them is one trip with
+  // precomputed offsets: the passes are bound by latency (barriers, shared-memory round trips).
   __device__ __forceinline__ void l1_correct() {
     const int W = sb.W, n1 = P.l3_nx1 + 1, ny1 = P.l3_ny1;
     const int naxp = coarse_row_stride(P.nax), ncp = naxp * P.nay;
-    // r1 = P1^T w0 on the owned 2h rows: fine rows 2J-1 .. 2J+1 lie in -1 .. R
-    for (int t = threadIdx.x; t < R1 * n1; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      const int lr = 2 * (J0 + lr1) - sb.r0;
-      const float* c = vw + (lr + 1) * W + 2 * I + 1;
+    // r1 = P1^T w0 on the owned 2h rows: fine rows 2J-1 .. 2J+1 lie in -1 .. R.  The 2h node at
+    // offset o = (lr1 + 1) W1 + I + 1 sits on the fine offset of row 2 (J0 + lr1) - r0, column 2I.
+    float r1[K1], e1[K1];
+    const int fshift = (2 * J0 - sb.r0 + 1) * W - 1;
+#pragma unroll
+    for (int u = 0; u < K1; ++u) {
+      r1[u] = 0.f;
+      if (n1o[u] < 0) continue;
+      const int lr1 = n1o[u] / W1 - 1, I1 = n1o[u] - (lr1 + 1) * W1;   // I1 = I + 1
+      const float* c = vw + fshift + 2 * (lr1 * W + I1);
       const float mid = fmaf(0.5f, c[-1] + c[1], c[0]);
       const float lo = fmaf(0.5f, c[-W - 1] + c[-W + 1], c[-W]);
       const float hi = fmaf(0.5f, c[W - 1] + c[W + 1], c[W]);
-      r1[o1(lr1, I)] = fmaf(0.5f, lo + hi, mid);
+      r1[u] = fmaf(0.5f, lo + hi, mid);
     }
-    __syncthreads();
     // 2h pre-smoothing e1 = S1 r1, exchanged
-    smooth_l1(r1, b1x);
+    smooth_l1(r1, e1);
+#pragma unroll
+    for (int u = 0; u < K1; ++u)
+      if (n1o[u] >= 0) b1x[n1o[u]] = e1[u];
     exchange_l1(b1x);
-    // 2h residual r1 - A1 e1 (in s1a's owned rows), summed per aggregate of the owned rows and
-    // published to every CTA (16-byte chunks of 4 aggregates)
-    for (int t = threadIdx.x; t < R1 * n1; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      s1a[h1(lr1, I)] = r1[o1(lr1, I)] - a1_apply(b1x, lr1, I);
-    }
+    // 2h residual r1 - A1 e1 (in b1u's owned rows), summed per aggregate of the owned rows by 4
+    // lanes each and published to every CTA (16 lanes per 16-byte chunk of 4 aggregates)
+#pragma unroll
+    for (int u = 0; u < K1; ++u)
+      if (n1o[u] >= 0) b1u[n1o[u]] = r1[u] - a1_apply(b1x, n1o[u]);
     __syncthreads();
-    const int items = najo * naxp;
-    for (int it = threadIdx.x; it < items; it += blockDim.x) {
-      const int ay = ajo0 + it / naxp, ax = it % naxp;
+    const int items = najo * naxp, padded = ((4 * items + 31) / 32) * 32, lane = threadIdx.x & 31;
+    for (int t = threadIdx.x; t < padded; t += blockDim.x) {
+      const int item = t >> 2, ajl = item / naxp, ax = item - ajl * naxp, ay = ajo0 + ajl;
       float acc = 0.f;
-      if (ax < P.nax) {
+      if (item < items && ax < P.nax) {
         const int ya = max(ay * P.cm, J0), yb = min(ay == P.nay - 1 ? ny1 : ay * P.cm + P.cm - 1, J0 + R1 - 1);
         const int xa = ax * P.cm, xb = ax == P.nax - 1 ? n1 - 1 : ax * P.cm + P.cm - 1;
-        for (int J = ya; J <= yb; ++J)
-          for (int I = xa; I <= xb; ++I) acc += s1a[h1(J - J0, I)];
+        for (int J = ya + (t & 3); J <= yb; J += 4) {
+          const float* row = b1u + (J - J0 + 1) * W1 + 1;
+          for (int I = xa; I <= xb; ++I) acc += row[I];
+        }
       }
-      l3_items[it] = acc;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < (items / 4) * 16; t += blockDim.x) {
-      const int c = t >> 4;
-      const float4 chunk = reinterpret_cast<const float4*>(l3_items)[c];
-      const int item0 = 4 * c, ajl0 = item0 / naxp, ax0 = item0 - ajl0 * naxp;
-      comm.publish_tl(tl_slot, sb.rank * ncp + (ajo0 + ajl0) * naxp + ax0, chunk, t & 15, sb.cs);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      const int base = lane & 16;
+      float4 chunk;
+      chunk.x = __shfl_sync(0xffffffffu, acc, base + 0);
+      chunk.y = __shfl_sync(0xffffffffu, acc, base + 4);
+      chunk.z = __shfl_sync(0xffffffffu, acc, base + 8);
+      chunk.w = __shfl_sync(0xffffffffu, acc, base + 12);
+      const int item0 = (t & ~15) >> 2;                // first aggregate of the chunk
+      if (item0 < items) {
+        const int ajl0 = item0 / naxp, ax0 = item0 - ajl0 * naxp;
+        comm.publish_tl(tl_slot, sb.rank * ncp + (ajo0 + ajl0) * naxp + ax0, chunk, lane & 15, sb.cs);
+      }
     }
     comm.expect_tl(tl_bytes);
     comm.finish_tl();
     coarse_gather();
-    // u1 = e1 + P2 ec on the owned and halo 2h rows
-    for (int t = threadIdx.x; t < (R1 + 2) * n1; t += blockDim.x) {
-      const int lr1 = t / n1 - 1, I = t - (lr1 + 1) * n1, J = J0 + lr1;
+    // u1 = e1 + P2 ec on the owned and halo 2h rows (b1u's owned rows have been read: coarse_gather
+    // ends with a block barrier)
+#pragma unroll
+    for (int u = 0; u < K1; ++u) {
+      if (n1o[u] < 0) continue;
+      e1[u] += tl_ec[n1a[u]];
+      b1u[n1o[u]] = e1[u];
+    }
+    for (int t = threadIdx.x; t < 2 * n1; t += blockDim.x) {
+      const int lr1 = t < n1 ? -1 : R1, I = t < n1 ? t : t - n1, J = J0 + lr1;
       if (J < 0 || J > ny1) continue;
-      const float ec = tl_ec[(l3_agg(J, P.cm, P.nay) - aj0) * naxp + l3_agg(I, P.cm, P.nax)];
-      b1u[h1(lr1, I)] = b1x[h1(lr1, I)] + ec;
+      const int o = (lr1 + 1) * W1 + I + 1;
+      b1u[o] = b1x[o] + tl_ec[(l3_agg(J, P.cm, P.nay) - aj0) * naxp + l3_agg(I, P.cm, P.nax)];
     }
     __syncthreads();
     // 2h post-smoothing z1 = u1 + S1 (r1 - A1 u1), exchanged
-    for (int t = threadIdx.x; t < R1 * n1; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      r1[o1(lr1, I)] -= a1_apply(b1u, lr1, I);
-    }
-    __syncthreads();
-    smooth_l1(r1, b1z);
-    for (int t = threadIdx.x; t < R1 * n1; t += blockDim.x) {
-      const int lr1 = t / n1, I = t - lr1 * n1;
-      b1z[h1(lr1, I)] += b1u[h1(lr1, I)];
-    }
+    float z1[K1];
+#pragma unroll
+    for (int u = 0; u < K1; ++u)
+      if (n1o[u] >= 0) r1[u] -= a1_apply(b1u, n1o[u]);
+    smooth_l1(r1, z1);
+#pragma unroll
+    for (int u = 0; u < K1; ++u)
+      if (n1o[u] >= 0) b1z[n1o[u]] = e1[u] + z1[u];
     exchange_l1(b1z);
+  }
+
+  // P1 z1 on the fine group g of local row lr: columns 4g-1 .. 4g+2 take the 2h columns 2g-1, 2g and
+  // 2g+1, an odd row the mean of the 2h rows below and above
+  __device__ __forceinline__ void prolong_l1(int lr, int g, float (&v)[4]) const {
+    const int y = sb.r0 + lr;
+    const float* ra = b1z + ((y >> 1) - J0 + 1) * W1 + 2 * g;
+    const float* rb = b1z + (((y + 1) >> 1) - J0 + 1) * W1 + 2 * g;
+    const float z0 = 0.5f * (ra[0] + rb[0]), z1 = 0.5f * (ra[1] + rb[1]), z2 = 0.5f * (ra[2] + rb[2]);
+    v[0] = 0.5f * (z0 + z1);
+    v[1] = z1;
+    v[2] = 0.5f * (z1 + z2);
+    v[3] = z2;
   }
 
   // Three-level cycle z = M^-1 r in FP32 over the fine, 2h and aggregate levels:
@@ -1032,15 +1071,26 @@ struct Stepper {
     exchange(vw);
     l1_correct();
     // u0 = e0 + P1 z1 on the owned and halo fine rows (in vy); 0 off the unknowns
-    for (int i = threadIdx.x; i < (sb.R + 2) * W; i += blockDim.x) {
-      if (vsd[i] == 0.f) {
-        vy[i] = 0.f;
-        continue;
-      }
-      const int lr = i / W - 1, ix = i - (lr + 1) * W - 1, y = sb.r0 + lr;
-      const int ja = y / 2 - J0, jb = (y + 1) / 2 - J0, ia = ix / 2, ib = (ix + 1) / 2;
-      const float z = 0.25f * ((b1z[h1(ja, ia)] + b1z[h1(ja, ib)]) + (b1z[h1(jb, ia)] + b1z[h1(jb, ib)]));
-      vy[i] += z;
+#pragma unroll
+    for (int k = 0; k < NG; ++k) {
+      const int l0 = loc0[k];
+      if (l0 < 0) continue;
+      const int lr = l0 / W - 1;
+      float v[4];
+      prolong_l1(lr, (l0 - (lr + 1) * W) / kGroup, v);
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j)
+        if (unknown(k, j)) vy[l0 + j] += v[j];
+    }
+    for (int t = threadIdx.x; t < 2 * sb.G; t += blockDim.x) {
+      const int lr = t < sb.G ? -1 : sb.R, g = t < sb.G ? t : t - sb.G, y = sb.r0 + lr;
+      if (y < 0 || y > P.ny) continue;
+      const int l0 = (lr + 1) * W + kGroup * g;
+      float v[4];
+      prolong_l1(lr, g, v);
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j)
+        if (vsd[l0 + j] != 0.f) vy[l0 + j] += v[j];
     }
     __syncthreads();
     // fine post-smoothing z = u0 + S0 (r - A u0)
