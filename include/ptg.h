@@ -255,8 +255,9 @@ int ptg_op_sizes(const ptg_op* op, int* Nn, int* Ne, int* Nt, int* Ntau, int* M)
 /* Tuning of the multigrid cycle of the streamed solves (ptg_solve.coarse_stream, local_steps = 3)
  * for the launches that follow: solo_rows, levels with at most this many node rows run on the
  * first CTA of a group alone (block barriers instead of the group's); coarse_steps, damped-Jacobi
- * steps on the coarsest level (1..64); fused, 1 prolongation and post-smoothing in one pass, 0 in
- * two.  0 (solo_rows, coarse_steps) and -1 (fused) restore the library's defaults (33, 10, 1).
+ * steps on the coarsest level (1..64); fused, -1, 0 or 1, has no effect any more: prolongation and
+ * post-smoothing are always one pass.  0 (solo_rows, coarse_steps) restores the library's
+ * defaults (33, 10).
  * Results change only within the solver tolerance.  PTG_EINVAL on other values. */
 int ptg_op_set_multigrid(ptg_op* op, int solo_rows, int coarse_steps, int fused);
 

@@ -41,7 +41,6 @@ struct ptg_op {
   // 1/C ([6][PN]), the FP64 1/C ([PN]), and the workspace of st_groups concurrent slices
   float* w32 = nullptr;         // [3][PEe] FP32 element weights (D, S, T) of C/dt + K
   float* w32_inv = nullptr;     // [PN] FP32 1/C
-  double* w64_inv = nullptr;    // [PN] FP64 1/C
   double* st_w64 = nullptr;     // [st_groups][3][PN] (x, x, b), padded node layout
   void* st_wr = nullptr;        // [st_groups][5][PN] (r, z, p, q, d) of the FP64 CG kinds
   void* st_wr32 = nullptr;      // the same for the FP32 CG kinds: the two layouts never share
@@ -53,11 +52,12 @@ struct ptg_op {
   int mg_L = 0;
   MgLevel mg_lv[kMgMaxLevels] = {};
   float* mg_w = nullptr;
+  float *mg_elem = nullptr, *mg_elemf = nullptr;   // their finest levels in element form
   float* mg_wf = nullptr;       // the same hierarchy of C/dt + K for the streamed fine propagators
   int mg_Lf = 0;                // its levels (0: the fine kinds stream with Jacobi)
   float* mg_ws = nullptr;
   long long mg_ws_stride = 0;
-  int mg_solo = 0, mg_csteps = 0, mg_fuse = -1;   // ptg_op_set_multigrid (0 / -1: the defaults)
+  int mg_solo = 0, mg_csteps = 0;   // ptg_op_set_multigrid (0: the defaults)
   double* sw_red = nullptr;     // the correction sweeps' reduction partials and barrier, so that the
   unsigned* sw_bar = nullptr;   // adjoint coarse parts may run beside the forward sweep
   // device workspace
@@ -244,14 +244,12 @@ constexpr int kWideMinNodes = 40000;
 // took longer than a 256 x 256 one with the same slices (214 against 187 ms at 64 slices).
 constexpr int kCoarseStreamMinNodes = 30000;
 // Streamed coarse-step solves (stream.cuh, mg.cu): node rows per CTA of a correction sweep's
-// group, the multigrid's smoothing steps, the damped-Jacobi steps on its coarsest level (at most
+// group, the damped-Jacobi steps on the multigrid's coarsest level (at most
 // 9 x 9 nodes) where no dense inverse applies, and the levels with at most kMgSoloRows node rows, which the group's first CTA
 // runs alone (block barriers instead of the group's).
 constexpr int kSweepRowsPerCta = 2;
-constexpr int kMgNu = 1;
 constexpr int kMgCoarseSteps = 10;
 constexpr int kMgSoloRows = 33;
-constexpr int kMgFuse = 1;
 
 // two-level bytes of a grid-wide launch of G CTAs (the partials live in global memory)
 struct WideCtx {
@@ -540,7 +538,6 @@ void base_params(const ptg_op* op, StepParams& P) {
     P.w32 = op->w32 + kSlack;
     P.w32_stride = (int)PEe;
     P.w32_inv = op->w32_inv + kSlack;
-    P.w64_inv = op->w64_inv + kSlack;
     P.st_pv = (long long)PN;
   }
   P.dk = op->dk;
@@ -626,12 +623,11 @@ int run(ptg_op* op, StepParams& P, int ntasks, cudaStream_t stream, int stats_ki
     const int L = coarse_kind(P.kind) ? op->mg_L : op->mg_Lf;
     if (L > 0) {
       P.mg_levels = L;
-      P.mg_nu = kMgNu;
       P.mg_coarse_steps = op->mg_csteps > 0 ? op->mg_csteps : kMgCoarseSteps;
       P.mg_solo_rows = op->mg_solo > 0 ? op->mg_solo : kMgSoloRows;
-      P.mg_fuse = op->mg_fuse >= 0 ? op->mg_fuse : kMgFuse;
       for (int l = 0; l < L; ++l) P.mg[l] = op->mg_lv[l];
       P.mg_w = coarse_kind(P.kind) ? op->mg_w : op->mg_wf;
+      P.mg_elem = coarse_kind(P.kind) ? op->mg_elem : op->mg_elemf;
       P.mg_ws = op->mg_ws;
       P.mg_ws_stride = op->mg_ws_stride;
       if (P.kind == KIND_CORRECT_PRI || P.kind == KIND_CORRECT_ADJ) {
@@ -648,7 +644,7 @@ int run(ptg_op* op, StepParams& P, int ntasks, cudaStream_t stream, int stats_ki
     if (const int rc = debug_check(op, P, plan, ntasks)) return rc;
 #endif
     op->last_stream = stream;
-    PTG_CUDA(launch_stream(P, prec, plan.max_active_clusters, plan.nthreads, stream));
+    PTG_CUDA(launch_stream(P, prec, plan.max_active_clusters, stream));
     return PTG_OK;
   }
   if (plan.wide) {
@@ -685,7 +681,7 @@ void free_all(ptg_op* op) {
                   op->g_red, op->g_bar, op->g_halo, op->g_tl,
                   op->tl_Ac, op->tl_band, op->tl_X, op->tl_Ainv,
                   op->tl3_A1, op->tl3_Ac, op->tl3_band, op->tl3_X, op->tl3_Ainv,
-                  op->w32, op->w32_inv, op->w64_inv, op->st_w64, op->st_wr, op->st_wr32, op->mg_w, op->mg_wf, op->mg_ws, op->sw_red,
+                  op->w32, op->w32_inv, op->st_w64, op->st_wr, op->st_wr32, op->mg_w, op->mg_wf, op->mg_elem, op->mg_elemf, op->mg_ws, op->sw_red,
                   op->sw_bar,
                   op->mesh_rho, op->mesh_XH, op->mesh_FH, op->mesh_GH, op->mesh_SH, op->mesh_YH,
                   op->mesh_zero, op->mesh_aux, op->mesh_pn, op->mesh_lam, op->mesh_dg};
@@ -1019,7 +1015,6 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
     const bool f32 = (fine_st && pf != PTG_FP64) || (op->mg_L > 0 && pc != PTG_FP64);
     A(&op->w32, 3 * PEs * sizeof(float));
     A(&op->w32_inv, PNs * sizeof(float));
-    A(&op->w64_inv, PNs * sizeof(double));
     A(&op->st_w64, ng * 3 * PNs * sizeof(double));
     if (f64) A(&op->st_wr, ng * 5 * PNs * sizeof(double));
     if (f32) A(&op->st_wr32, ng * 5 * PNs * sizeof(float));
@@ -1040,6 +1035,10 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
         if (!w) continue;
         A(w, (size_t)wf * sizeof(float));
         if (e == cudaSuccess) e = cudaMemset(*w, 0, (size_t)wf * sizeof(float));
+        const size_t ef = ((size_t)(grid->ny + 3) * 3 * op->W + 2 * kSlack) * sizeof(float);
+        float** el = w == &op->mg_w ? &op->mg_elem : &op->mg_elemf;
+        A(el, ef);
+        if (e == cudaSuccess) e = cudaMemset(*el, 0, ef);
       }
     }
   }
@@ -1176,7 +1175,6 @@ int ptg_op_set_multigrid(ptg_op* op, int solo_rows, int coarse_steps, int fused)
   if (!op || solo_rows < 0 || coarse_steps < 0 || coarse_steps > 64 || fused < -1 || fused > 1) return PTG_EINVAL;
   op->mg_solo = solo_rows;
   op->mg_csteps = coarse_steps;
-  op->mg_fuse = fused;
   return PTG_OK;
 }
 
@@ -1218,14 +1216,14 @@ int ptg_fe_assemble_operator(ptg_op* op, const double* rho_d, cudaStream_t strea
                            op->dirichlet, out, op->stats, stream));
   if (op->w32)
     PTG_CUDA(launch_stream_weights((int)PEe, (int)PN, op->wE, op->nodew, op->dirichlet, op->g.nx, op->g.ny, op->W,
-                                   op->w32, op->w32_inv, op->w64_inv, stream));
+                                   op->w32, op->w32_inv, stream));
   if (op->mg_L > 0) {
     NodeWeights Ac{out.node[5], out.node[6], out.node[7], out.node[8], out.node[9]};
-    PTG_CUDA(launch_mg_setup(Ac, op->dirichlet, op->mg_lv, op->mg_L, op->mg_w, stream));
+    PTG_CUDA(launch_mg_setup(Ac, out.wEc, (int)PEe, op->dirichlet, op->mg_lv, op->mg_L, op->mg_w, op->mg_elem, stream));
   }
   if (op->mg_Lf > 0) {
     NodeWeights Af{out.node[0], out.node[1], out.node[2], out.node[3], out.node[4]};
-    PTG_CUDA(launch_mg_setup(Af, op->dirichlet, op->mg_lv, op->mg_Lf, op->mg_wf, stream));
+    PTG_CUDA(launch_mg_setup(Af, out.wEf, (int)PEe, op->dirichlet, op->mg_lv, op->mg_Lf, op->mg_wf, op->mg_elemf, stream));
   }
   if (op->tl_m) {
     NodeWeights Ac;

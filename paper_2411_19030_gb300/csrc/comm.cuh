@@ -274,38 +274,40 @@ struct GridComm {
   // records PTG_ETIMEOUT and returns; once any CTA has recorded it (the group's broken flag,
   // P.g_bar[4 gid + 2]), every later wait returns at once, so a broken launch ends quickly with
   // the error instead of waiting out every barrier.
-  __device__ void barrier() {
+  __device__ __forceinline__ void barrier() {
     __syncthreads();
     if (G == 1) {                // a group of one CTA: the block barrier orders its global accesses
       pull_halos();
       return;
     }
-    if (threadIdx.x == 0) {
-      unsigned* count = P.g_bar + 4 * gid;
-      unsigned* broken = count + 2;
-      ++epoch;
-      const unsigned target = epoch * (unsigned)G;
-      __threadfence();
-      red_release_add_gpu(count, 1u);
-      const long long limit = P.wait_limit > 0 ? P.wait_limit : (long long)kGridSpinLimit;
-      long long spins = 0;
-      while ((int)(ld_acquire_gpu(count) - target) < 0) {
-        if ((++spins & 255) == 0 && ld_acquire_gpu(broken) != 0u) break;
-        if (spins >= limit) {
-          record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
-          atomicExch(broken, 1u);
-          break;
-        }
-      }
-      __threadfence();
-    }
+    if (threadIdx.x == 0) arrive_and_wait();
     __syncthreads();
     pull_halos();
+  }
+  // One thread's part, after a block barrier (or its own stores).  The release of the arrival and
+  // the acquire of the poll order every store of the CTA that the block barrier put before it, and
+  // every load after the next block barrier; a fence on top of each would cost a round trip.
+  __device__ __forceinline__ void arrive_and_wait() {
+    unsigned* count = P.g_bar + 4 * gid;
+    unsigned* broken = count + 2;
+    ++epoch;
+    const unsigned target = epoch * (unsigned)G;
+    red_release_add_gpu(count, 1u);
+    const long long limit = P.wait_limit > 0 ? P.wait_limit : (long long)kGridSpinLimit;
+    long long spins = 0;
+    while ((int)(ld_acquire_gpu(count) - target) < 0) {
+      if ((++spins & 255) == 0 && ld_acquire_gpu(broken) != 0u) break;
+      if (spins >= limit) {
+        record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
+        atomicExch(broken, 1u);
+        break;
+      }
+    }
   }
   __device__ void sync() { barrier(); }
 
   template <class T, int NV, int NX, class Post>
-  __device__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post) {
+  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post) {
     RedBank<T>& rb = bank<T>(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -319,16 +321,16 @@ struct GridComm {
     // while another reduces doubles
     constexpr int kPer = 32 / (int)sizeof(T);
     T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 4);
+    // warp 0 alone: the CTA's sums into its slots, the barrier, lane-strided sums over the ranks and
+    // the warp's sum, then `post`; broadcast
     if (warp == 0) {
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        const T s = warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
+        const T s = half_warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
         if (lane == 0) slots[(int)blockIdx.x * kPer + i] = s;
       }
-    }
-    barrier();
-    // warp 0: lane-strided sums over the ranks and the warp's sum, then `post`; broadcast
-    if (warp == 0) {
+      if (lane == 0 && G > 1) arrive_and_wait();
+      __syncwarp();
       T t[NV + NX];
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
@@ -345,6 +347,7 @@ struct GridComm {
       }
     }
     __syncthreads();
+    pull_halos();
 #pragma unroll
     for (int i = 0; i < NV + NX; ++i) v[i] = rb.bcast[i];
     phase ^= 1;

@@ -10,7 +10,8 @@
 // bounds on the eigenvalues of D^-1 A, and with them the Jacobi damping, carry over to every
 // level.  Every level is stored as FP32 per-node weights in the padded node layout of the fine
 // arrays (centre, east, north, north-east, north-west; the other four couplings are those of the
-// neighbour on the other side) plus omega/diag (0 off the unknowns).
+// neighbour on the other side) plus omega/diag (0 off the unknowns), the six interleaved row by row
+// so that one bulk copy brings some rows of all of them.
 #include <algorithm>
 #include "ptg_internal.h"
 
@@ -19,25 +20,30 @@ namespace ptg {
 namespace {
 
 // coupling of node i = (x, y) of a level to its neighbour (x + c, y + d), |c|, |d| <= 1, from the
-// five stored weights
-__device__ __forceinline__ double coupling(const float* __restrict__ w, long long plen, int W, int loc, int c, int d) {
+// five stored weights; wl is the node's index in the interleaved rows (6 W floats a row)
+__device__ __forceinline__ double coupling(const float* __restrict__ w, int W, int wl, int c, int d) {
   const float* C = w;
-  const float* E = w + plen;
-  const float* N = w + 2 * plen;
-  const float* NE = w + 3 * plen;
-  const float* NW = w + 4 * plen;
-  if (d == 0) return c == 0 ? C[loc] : (c == 1 ? E[loc] : E[loc - 1]);
-  if (c == 0) return d == 1 ? N[loc] : N[loc - W];
-  if (c == d) return d == 1 ? NE[loc] : NE[loc - W - 1];
-  return d == 1 ? NW[loc] : NW[loc - W + 1];   // (-1, 1): own NW; (1, -1): NW of the SE neighbour
+  const float* E = w + W;
+  const float* N = w + 2 * W;
+  const float* NE = w + 3 * W;
+  const float* NW = w + 4 * W;
+  const int row = 6 * W;
+  if (d == 0) return c == 0 ? C[wl] : (c == 1 ? E[wl] : E[wl - 1]);
+  if (c == 0) return d == 1 ? N[wl] : N[wl - row];
+  if (c == d) return d == 1 ? NE[wl] : NE[wl - row - 1];
+  return d == 1 ? NW[wl] : NW[wl - row + 1];   // (-1, 1): own NW; (1, -1): NW of the SE neighbour
 }
 
 __device__ __forceinline__ double hat(int a) { return a == 0 ? 1.0 : 0.5; }   // |a| <= 1
 
 // Level 0: FP32 copy of the FP64 node weights; omega/diag on the unknowns.  One thread per
 // padded entry (rows -1 .. ny + 1); entries outside the grid are zero.
+// Beside them the element form (omega/diag of the nodes of row y, then k = k_e/6 and m = c_e h^2/(36
+// step) of the elements above it) interleaved row by row, from the element weights wE (D = 4 (k + m)
+// and S = 2 m - k, PE apart, rows ey = -1 .. ny).
 __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ dirichlet, int nx, int ny, int W,
-                                 float* __restrict__ w, long long plen, float omega) {
+                                 float* __restrict__ w, float omega, const double* __restrict__ wE, int PE,
+                                 float* __restrict__ elem) {
   const int n = (ny + 3) * W;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int iy = t / W - 1, ix = t % W - 1;
@@ -52,12 +58,20 @@ __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ diri
       nw = (float)A.NW[loc];
       if (!dirichlet[iy * (nx + 1) + ix] && A.C[loc] > 0.0) wd = (float)(omega / A.C[loc]);
     }
-    w[loc] = c;
-    w[plen + loc] = e;
-    w[2 * plen + loc] = no;
-    w[3 * plen + loc] = ne;
-    w[4 * plen + loc] = nw;
-    w[5 * plen + loc] = wd;
+    const int o = 6 * (t / W) * W + t % W;
+    w[o] = c;
+    w[o + W] = e;
+    w[o + 2 * W] = no;
+    w[o + 3 * W] = ne;
+    w[o + 4 * W] = nw;
+    w[o + 5 * W] = wd;
+    // the node rows are -1 .. ny + 1, the element rows -1 .. ny
+    const bool row = t < (ny + 2) * W;
+    const double Dw = row ? wE[t] : 0.0, Sw = row ? wE[PE + t] : 0.0;
+    const int oe = 3 * (t / W) * W + t % W;
+    elem[oe] = wd;
+    elem[oe + W] = (float)(fma(-2.0, Sw, Dw) * (1.0 / 6.0));
+    elem[oe + 2 * W] = (float)(fma(4.0, Sw, Dw) * (1.0 / 12.0));
   }
 }
 
@@ -65,9 +79,9 @@ __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ diri
 // (P^T A P)[(I,J), (I,J) + o] for o = (0,0), (1,0), (0,1), (1,1), (-1,1): the sum over the fine
 // nodes i around (2I, 2J) and their neighbours k around (2I, 2J) + 2o of P[i,(I,J)] A[i,k]
 // P[k,(I,J)+o], over unknowns only (omega/diag of the fine level nonzero).  FP64 sums.
-__global__ void mg_galerkin_kernel(const float* __restrict__ wf, long long plf, int nxf, int nyf, int Wf,
-                                   float* __restrict__ wc, long long plc, int nxc, int nyc, int Wc, float omega) {
-  const float* wdf = wf + 5 * plf;
+__global__ void mg_galerkin_kernel(const float* __restrict__ wf, int nxf, int nyf, int Wf, float* __restrict__ wc,
+                                   int nxc, int nyc, int Wc, float omega) {
+  const float* wdf = wf + 5 * Wf;
   const int n = (nyc + 3) * Wc;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int J = t / Wc - 1, I = t % Wc - 1;
@@ -84,7 +98,7 @@ __global__ void mg_galerkin_kernel(const float* __restrict__ wf, long long plf, 
           for (int a = -1; a <= 1; ++a) {
             const int x = 2 * I + a;
             if (x < 0 || x > nxf) continue;
-            const int li = (y + 1) * Wf + x + 1;
+            const int li = 6 * (y + 1) * Wf + x + 1;
             if (wdf[li] == 0.f) continue;
             const double pi = hat(a) * hat(b);
             for (int d = -1; d <= 1; ++d) {
@@ -93,8 +107,8 @@ __global__ void mg_galerkin_kernel(const float* __restrict__ wf, long long plf, 
               for (int c = -1; c <= 1; ++c) {
                 const int kx = x + c, ka = kx - 2 * K;
                 if (kx < 0 || kx > nxf || ka < -1 || ka > 1) continue;
-                if (wdf[(ky + 1) * Wf + kx + 1] == 0.f) continue;
-                s += pi * coupling(wf, plf, Wf, li, c, d) * (hat(ka) * hat(kb));
+                if (wdf[6 * (ky + 1) * Wf + kx + 1] == 0.f) continue;
+                s += pi * coupling(wf, Wf, li, c, d) * (hat(ka) * hat(kb));
               }
             }
           }
@@ -102,8 +116,9 @@ __global__ void mg_galerkin_kernel(const float* __restrict__ wf, long long plf, 
         out[o] = s;
       }
     }
-    for (int o = 0; o < 5; ++o) wc[o * plc + t] = (float)out[o];
-    wc[5 * plc + t] = out[0] > 0.0 ? (float)(omega / out[0]) : 0.f;
+    const int o0 = 6 * (t / Wc) * Wc + t % Wc;
+    for (int o = 0; o < 5; ++o) wc[o0 + o * Wc] = (float)out[o];
+    wc[o0 + 5 * Wc] = out[0] > 0.0 ? (float)(omega / out[0]) : 0.f;
   }
 }
 
@@ -138,18 +153,18 @@ long long mg_layout(int nx, int ny, MgLevel* lv, int L, long long* ws_floats) {
   return woff;
 }
 
-cudaError_t launch_mg_setup(NodeWeights A, const uint8_t* dirichlet, const MgLevel* lv, int L, float* w,
-                            cudaStream_t stream) {
+cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, const uint8_t* dirichlet, const MgLevel* lv, int L,
+                            float* w, float* elem, cudaStream_t stream) {
   const MgLevel& l0 = lv[0];
   const int threads = 256;
   auto blocks = [&](long long n) { return (int)std::min<long long>((n + threads - 1) / threads, 4096); };
   mg_level0_kernel<<<blocks((long long)(l0.ny + 3) * l0.W), threads, 0, stream>>>(
-      A, dirichlet, l0.nx, l0.ny, l0.W, w + l0.woff + kSlack, l0.plen, kMgOmega);
+      A, dirichlet, l0.nx, l0.ny, l0.W, w + l0.woff + kSlack, kMgOmega, wE, PE, elem + kSlack);
   for (int l = 0; l + 1 < L; ++l) {
     const MgLevel& f = lv[l];
     const MgLevel& c = lv[l + 1];
     mg_galerkin_kernel<<<blocks((long long)(c.ny + 3) * c.W), threads, 0, stream>>>(
-        w + f.woff + kSlack, f.plen, f.nx, f.ny, f.W, w + c.woff + kSlack, c.plen, c.nx, c.ny, c.W, kMgOmega);
+        w + f.woff + kSlack, f.nx, f.ny, f.W, w + c.woff + kSlack, c.nx, c.ny, c.W, kMgOmega);
   }
   return cudaGetLastError();
 }

@@ -382,25 +382,11 @@ __device__ __forceinline__ void warp_ewindow(const float* __restrict__ x, int b,
   w[0] = lane == 0 ? e : l;
   w[1] = c.x; w[2] = c.y; w[3] = c.z; w[4] = c.w;
 }
-__device__ __forceinline__ void stencil_km32(const float* __restrict__ z, const float* __restrict__ wk,
-                                             const float* __restrict__ wm, int loc0, int W, int lane, float (&y)[4],
-                                             bool no_lo = false, bool no_hi = false) {
-  float zl[6], zm[6], zh[6], kl[5], ml[5], ku[5], mu[5];
-  warp_window(z, loc0 - W, lane, zl);
-  warp_window(z, loc0, lane, zm);
-  warp_window(z, loc0 + W, lane, zh);
-  warp_ewindow(wk, loc0 - W, lane, kl);
-  warp_ewindow(wm, loc0 - W, lane, ml);
-  warp_ewindow(wk, loc0, lane, ku);
-  warp_ewindow(wm, loc0, lane, mu);
-  if (no_lo) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) zl[i] = 0.f;
-  }
-  if (no_hi) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) zh[i] = 0.f;
-  }
+// A z on a group from z's windows and the element windows (columns b-1 .. b+3) below and above
+template <int N>
+__device__ __forceinline__ void km_combine(const float (&zl)[6], const float (&zm)[6], const float (&zh)[6],
+                                           const float (&kl)[N], const float (&ml)[N], const float (&ku)[N],
+                                           const float (&mu)[N], float (&y)[4]) {
   float d[5], sl[5], su[5], tl[5], tu[5];
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
@@ -423,6 +409,27 @@ __device__ __forceinline__ void stencil_km32(const float* __restrict__ z, const 
     a = fmaf(tu[j + 1], zh[j + 2], a);
     y[j] = a;
   }
+}
+__device__ __forceinline__ void stencil_km32(const float* __restrict__ z, const float* __restrict__ wk,
+                                             const float* __restrict__ wm, int loc0, int W, int lane, float (&y)[4],
+                                             bool no_lo = false, bool no_hi = false) {
+  float zl[6], zm[6], zh[6], kl[5], ml[5], ku[5], mu[5];
+  warp_window(z, loc0 - W, lane, zl);
+  warp_window(z, loc0, lane, zm);
+  warp_window(z, loc0 + W, lane, zh);
+  warp_ewindow(wk, loc0 - W, lane, kl);
+  warp_ewindow(wm, loc0 - W, lane, ml);
+  warp_ewindow(wk, loc0, lane, ku);
+  warp_ewindow(wm, loc0, lane, mu);
+  if (no_lo) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) zl[i] = 0.f;
+  }
+  if (no_hi) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) zh[i] = 0.f;
+  }
+  km_combine(zl, zm, zh, kl, ml, ku, mu, y);
 }
 
 // Element bilinear forms of Eq. 4.7 in the modes that Ke and Me share as eigenvectors: with the

@@ -64,7 +64,8 @@ struct FFWeights {
 
 // Geometric multigrid hierarchy of the coarse-step operator (mg.cu): level l has nx, ny
 // elements (halved per level), the padded width W, arrays of plen floats each (slack included),
-// its six weight arrays (C, E, N, NE, NW, omega/diag) at woff in the op's weight buffer, and its
+// its six weight arrays (C, E, N, NE, NW, omega/diag; interleaved row by row) at woff in the op's
+// weight buffer, and its
 // vectors at voff in a group's workspace (level 0: u, res; coarser: f, u, res, e).
 constexpr int kMgMaxLevels = 10;
 constexpr int kMgMinCells = 8;       // a level with min(nx, ny) <= 8 is the coarsest
@@ -150,17 +151,17 @@ struct StepParams {
   int l3_W1;                 // padded row width of the 2h buffers
   int l3_r1max;              // most 2h rows owned by a CTA of the launch
   const double* A1;          // [9][(ny1 + 1) (nx1 + 1)] 2h stencil, k = (dJ + 1) * 3 + (dI + 1)
-  // streamed fine propagators (stream.cuh): per group of P.cs CTAs, three FP64 vectors (x, x, b)
-  // and five CG vectors (r, z, p, q, d) in the kernel's precision, each st_pv entries in the padded
-  // node layout with its slack; the FP32 element weights (D, S, T) of C/dt + K, w32_stride floats
-  // apart in the padded element layout; 1/C (0 off the unknowns) in FP32 and FP64, padded node layout
+  // streamed propagators (stream.cuh): per group of P.cs CTAs, three FP64 vectors (x, x, b) and the
+  // CG vectors (r, z, p, q, d) of one float array each, two in the FP64 kinds (float pairs), st_pv
+  // entries an array in the padded node layout with its slack; the FP32 element weights (D, S, T)
+  // of C/dt + K, w32_stride floats apart in the padded element layout; 1/C of C/dt + K (0 off the
+  // unknowns) in the padded node layout
   double* st_w64;
   void* st_wr;
   long long st_pv;
   const float* w32;
   int w32_stride;
   const float* w32_inv;
-  const double* w64_inv;
   // one system over a whole cooperative grid (GridComm): global scratch of the op
   int wide;                  // 1: launched as stepper_wide_kernel, groups of cs CTAs
   int wide_tasks;            // tasks of a grid-wide launch (group g runs g, g + groups, ...)
@@ -174,13 +175,11 @@ struct StepParams {
   // multigrid hierarchy (mg_levels = 0: Jacobi); mg_ws + group * mg_ws_stride is a group's
   // workspace; levels with at most mg_solo_rows node rows run on the group's first CTA alone
   int mg_levels;
-  int mg_nu;                 // damped-Jacobi steps before and after the coarse correction
   int mg_coarse_steps;       // damped-Jacobi steps on the coarsest level (from zero)
   int mg_solo_rows;
-  int mg_fuse;               // nu = 1: prolongation and post-smoothing in one pass (one barrier less
-                             // per level)
   MgLevel mg[kMgMaxLevels];
   const float* mg_w;
+  const float* mg_elem;      // level 0 in element form: [ny + 3][3][W] omega/diag, k, m (mg.cu), after the slack
   float* mg_ws;
   long long mg_ws_stride;
 };
@@ -368,20 +367,19 @@ cudaError_t launch_sensitivities(int nx, int ny, int Nt, double h, double dt, in
                                  double* partial, int nchunks, double* grad, cudaStream_t stream);
 
 // For the streamed fine propagators: FP32 copies of the 3 x PE FP64 element weights (D, S, T) of
-// C/dt + K (slack included), and 1/C in FP32 and FP64 (0 off the unknowns) on the PN entries of
+// C/dt + K (slack included), and 1/C in FP32 (0 off the unknowns) on the PN entries of
 // the padded node layout (slack included; C the node weight array with its slack).
 cudaError_t launch_stream_weights(int PE, int PN, const double* wE, const double* C_node, const uint8_t* dirichlet,
-                                  int nx, int ny, int W, float* w32, float* w32_inv, double* w64_inv,
-                                  cudaStream_t stream);
-cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, int nthreads, cudaStream_t stream);
+                                  int nx, int ny, int W, float* w32, float* w32_inv, cudaStream_t stream);
+cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, cudaStream_t stream);
 // Multigrid hierarchy: the number of levels of an nx x ny grid (1: no coarsening), the layout of
 // L levels (returns the floats of the weight buffer; *ws_floats the floats of one group's
-// workspace), and the set-up of every level's weights from the FP64 node weights A (buffer
-// zeroed beforehand: the slack and the rows outside the grid stay zero).
+// workspace), and the set-up of every level's weights from the FP64 node weights A and element
+// weights wE (buffers zeroed beforehand: the slack and the rows outside the grid stay zero).
 int mg_level_count(int nx, int ny);
 long long mg_layout(int nx, int ny, MgLevel* lv, int L, long long* ws_floats);
-cudaError_t launch_mg_setup(NodeWeights A, const uint8_t* dirichlet, const MgLevel* lv, int L, float* w,
-                            cudaStream_t stream);
+cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, const uint8_t* dirichlet, const MgLevel* lv, int L,
+                            float* w, float* elem, cudaStream_t stream);
 // G_l = H_l + c S_l ([n_l]) and G_g = H_g + c S_g ([n_g]), c the adjoint source scale of Theta
 cudaError_t launch_adjoint_combine(long long n_l, long long n_g, const double* Theta, double p, int Ne, int modified,
                                    const double* H_l, const double* H_g, const double* S_l, const double* S_g,

@@ -4,7 +4,7 @@
 
 namespace ptg {
 
-cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, int nthreads, cudaStream_t stream) {
+cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, cudaStream_t stream) {
   StreamKernels ks{nullptr, nullptr};
   switch (P.kind) {
     case KIND_FINE_PRI: ks = stream_select_0(); break;
@@ -17,13 +17,22 @@ cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, int n
   }
   const StreamKernel k = precision == PTG_FP32_REFINE ? ks.f32 : ks.f64;
   if (!k || ngroups < 1 || ngroups * P.cs > kMaxGrid) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaMemsetAsync(P.g_bar, 0, 4 * sizeof(unsigned) * ngroups, stream);
+  // shared memory of the largest level's rings
+  size_t smem = 0;
+  for (int l = 0; l + 1 < P.mg_levels; ++l) {
+    const int G4 = P.mg[l].W / kGroup;
+    const int weights = l == 0 ? kElemWeights : kNodeWeights;
+    if (pipe_rows(G4, weights) > 0 && pipe_bytes(G4, weights) > smem) smem = pipe_bytes(G4, weights);
+  }
+  cudaError_t e = configure_kernel((const void*)k, smem, false);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(P.g_bar, 0, 4 * sizeof(unsigned) * ngroups, stream);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   cfg.gridDim = dim3((unsigned)(ngroups * P.cs), 1, 1);
-  cfg.blockDim = dim3((unsigned)(nthreads < kStreamThreads ? nthreads : kStreamThreads), 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3((unsigned)kStreamThreads, 1, 1);   // the row rings count on it
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;

@@ -12,19 +12,61 @@
 //
 // Each step is the same as the stepper's (stepper.cuh): b = (C/dt) x_{j-1} + source, the start
 // extrapolated through the slice's last states (the same ring of states per task), the FP64
-// residual loop around a Jacobi-preconditioned CG in Real on A d = r / ||r||, then theta (primal)
-// or the Eq. 4.7 element sums (adjoint).  Per CG iteration the group sums two sets of dot
-// products (fixed order, identical in every CTA of the group: GridComm) and each CTA streams its
-// rows: q = A z + beta q, p = z + beta p with z = D^-1 r formed on the fly from r, then
-// d += alpha p, r -= alpha q; 44 bytes per node and iteration in FP32.  The FP32 operator
-// (per-node weights C, E, N, NE, NW and 1/C, shared by every slice) stays in L2.
+// residual loop around a preconditioned CG on A d = r / 2^k, then theta (primal) or the Eq. 4.7
+// element sums (adjoint).  The CG's vectors are floats, or float pairs (ff.cuh) in the FP64 kinds,
+// its preconditioned vector z a float.  Per CG iteration the group sums two sets of dot products
+// (fixed order, identical in every CTA of the group: GridComm) and each CTA streams its rows.
+//
+// What bounds the passes: at one CTA of 512 threads per SM a pass that loads its stencil operands
+// straight from global memory waits for them (256 x 256 and 512 x 512: 5 100 cycles per 512 groups
+// of 4 nodes, 12% of the HBM bandwidth).  The passes of the multigrid cycle's large levels and the
+// FP32 CG's operator therefore march down the rows through a ring in shared memory that bulk copies
+// (cp.async.bulk) fill several rows ahead (march below).
 #pragma once
 #include "comm.cuh"
 
 namespace ptg {
 
+constexpr int kStreamThreads = 512;   // one CTA per SM, 128 registers per thread
+constexpr int kPipeRows = 32;         // most rows of a ring (one mbarrier each)
+
+// Weights of a ring row per node: level 0 has the element form (omega/diag, k, m: stencil_km32's k_e/6
+// and c_e h^2/(36 step)), which halves the bytes of a pass (the passes of 128 slices were bound by
+// the weights' way from L2: 12 bytes per cycle and SM); a Galerkin level its six node weights.
+constexpr int kElemWeights = 3, kNodeWeights = 6;
+constexpr int kPipeBytes = 200 * 1024;
+// rows of the ring that holds a level's residual until it is restricted (G4 groups per row): those
+// of two trips of 512 groups and the ones that wait for their last row
+inline __host__ __device__ int res_rows(int G4) { return 2 * ((kStreamThreads - 1) / G4 + 2) + 4; }
+// rows that 512 consecutive groups touch, with a row on each side
+inline __host__ __device__ int trip_rows(int G4) { return (kStreamThreads - 1) / G4 + 4; }
+// Rows of a level's ring: a trip's rows and up to 16 ahead if the shared memory allows; 0 where
+// fewer than 2 ahead remain (short rows, whose 512 groups span too many of them, and rows of more
+// than 3 KB): such levels load straight from global memory.
+inline __host__ __device__ int pipe_rows(int G4, int weights) {
+  const int need = trip_rows(G4);
+  const int cap = (kPipeBytes / (16 * G4) - res_rows(G4)) / (1 + weights);
+  const int rows = cap < need + 16 ? cap : need + 16;
+  return need <= 32 && rows >= need + 2 ? rows : 0;
+}
+// Rows of a bulk copy: the largest chunk of which the ring holds a trip's rows, wherever they
+// start, and one more chunk.  A bulk copy costs about 175 cycles of the copy engine whatever its
+// size (1 KB and 2 KB rows alike), so the weights of a level are interleaved row by row and a
+// chunk is two copies.
+inline __host__ __device__ int chunk_rows(int S, int need) {
+  int c = (S - need + 1) / 2;
+  while (c > 1 && (S / c) * c < need + 2 * c - 1) --c;
+  return c < 1 ? 1 : c;
+}
+// shared memory of a level's rings
+inline size_t pipe_bytes(int G4, int weights) {
+  return 16 * (size_t)G4 * (size_t)((1 + weights) * pipe_rows(G4, weights) + res_rows(G4));
+}
+
 template <class Real, int KIND>
 struct Streamer {
+  static constexpr bool kMixed = std::is_same<Real, float>::value;
+  using V = typename std::conditional<kMixed, float, ff>::type;
   const StepParams& P;
   GridComm& comm;
   int rank = 0, r0 = 0, R = 0;   // this CTA's node rows [r0, r0 + R) of the group's system
@@ -33,14 +75,21 @@ struct Streamer {
   // group workspace, padded node layout (node (iy, ix) at (iy + 1) W + ix + 1, the layout of the
   // per-node weights), zero off the unknowns
   double *xa = nullptr, *xb = nullptr, *b = nullptr;
-  Real *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *d = nullptr;
+  float *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *d = nullptr;   // high parts; low parts
+  size_t lo = 0;                                                                // `lo` floats after (FP64 kinds)
   double step_dt = 0.0, inv_dt = 0.0;
   static constexpr bool kCoarse = KIND == KIND_COARSE_PRI || KIND == KIND_COARSE_ADJ || KIND == KIND_CORRECT_PRI ||
                                   KIND == KIND_CORRECT_ADJ;
   NodeWeights A64;               // the operator of the kind's step: C/dt + K or C/dtau + K
+  FFWeights ffw;                 // the same as float pairs
   float* mgws = nullptr;         // the group's multigrid workspace
+  // the row ring: shared memory, one mbarrier per row slot and the parity each waits for next
+  float* ring_sm;
+  unsigned long long* ring_bar;
+  unsigned& ring_phase;
 
-  __device__ Streamer(const StepParams& P_, GridComm& comm_) : P(P_), comm(comm_) {
+  __device__ Streamer(const StepParams& P_, GridComm& comm_, float* sm, unsigned long long* bar, unsigned& phase)
+      : P(P_), comm(comm_), ring_sm(sm), ring_bar(bar), ring_phase(phase) {
     rank = comm.rank();
     slab_rows(P.ny + 1, P.cs, rank, r0, R);
     nn = P.nx + 1;
@@ -51,15 +100,18 @@ struct Streamer {
     xa = w64;
     xb = w64 + pv;
     b = w64 + 2 * pv;
-    Real* wr = reinterpret_cast<Real*>(P.st_wr) + (size_t)grp * 5 * pv + kSlack;
+    constexpr int kParts = kMixed ? 1 : 2;
+    float* wr = reinterpret_cast<float*>(P.st_wr) + (size_t)grp * 5 * kParts * pv + kSlack;
+    lo = pv;
     r = wr;
-    z = wr + pv;
-    p = wr + 2 * pv;
-    q = wr + 3 * pv;
-    d = wr + 4 * pv;
+    z = wr + kParts * pv;
+    p = wr + 2 * kParts * pv;
+    q = wr + 3 * kParts * pv;
+    d = wr + 4 * kParts * pv;
     step_dt = kCoarse ? P.dtau : P.dt;
     inv_dt = 1.0 / step_dt;
     A64 = kCoarse ? P.A_coarse : P.A_fine;
+    ffw = kCoarse ? P.ff_coarse : P.ff_fine;
     if (P.mg_levels > 0) mgws = P.mg_ws + (size_t)grp * P.mg_ws_stride;
   }
 
@@ -98,100 +150,8 @@ struct Streamer {
     return (ix >= 0 && ix <= P.nx) ? iy * nn + ix : -1;
   }
 
-  // 1/C of the 4 nodes (0 off the unknowns) in the CG precision
-  __device__ __forceinline__ void dinv4(int loc, Real (&v)[4]) const {
-    if constexpr (sizeof(Real) == 8) {
-      load4(P.w64_inv + loc, v);
-    } else {
-      const float4 c = *reinterpret_cast<const float4*>(P.w32_inv + loc);
-      v[0] = c.x; v[1] = c.y; v[2] = c.z; v[3] = c.w;
-    }
-  }
-  __device__ __forceinline__ void ld4(const Real* __restrict__ a, int loc, Real (&v)[4]) const {
-    if constexpr (sizeof(Real) == 8) {
-      load4(a + loc, v);
-    } else {
-      const float4 c = *reinterpret_cast<const float4*>(a + loc);
-      v[0] = c.x; v[1] = c.y; v[2] = c.z; v[3] = c.w;
-    }
-  }
-  __device__ __forceinline__ void st4(Real* __restrict__ a, int loc, const Real (&v)[4]) const {
-    if constexpr (sizeof(Real) == 8) {
-      *reinterpret_cast<double2*>(a + loc) = make_double2(v[0], v[1]);
-      *reinterpret_cast<double2*>(a + loc + 2) = make_double2(v[2], v[3]);
-    } else {
-      *reinterpret_cast<float4*>(a + loc) = make_float4(v[0], v[1], v[2], v[3]);
-    }
-  }
-  __device__ __forceinline__ void st4d(double* __restrict__ a, int loc, const double (&v)[4]) const {
-    *reinterpret_cast<double2*>(a + loc) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2*>(a + loc + 2) = make_double2(v[2], v[3]);
-  }
-
-  // (A z) on a group in the CG precision (FP32 coarse-step operator: the multigrid's level 0)
-  __device__ __forceinline__ void apply_z(int loc, Real (&w)[4]) const {
-    if constexpr (sizeof(Real) == 8) {
-      double y[4];
-      stencil_node64<double>(z, loc, A64, loc, P.W, y);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = y[j];
-    } else if constexpr (kCoarse) {
-      float zl[6], zm[6], zh[6];
-      load_window(z, loc - P.W, zl);
-      load_window(z, loc, zm);
-      load_window(z, loc + P.W, zh);
-      lstencil(0, loc, zl, zm, zh, w);
-    } else {
-      float y[4];
-      stencil_elem32(z, P.w32, P.w32 + P.w32_stride, P.w32 + 2 * P.w32_stride, loc, P.W, y);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = y[j];
-    }
-  }
-
-  template <class T, int NV, int NX = 0, class Post = NoPost>
-  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post()) {
-    comm.template allreduce<T, NV, NX, Post>(v, P.cs, post);
-  }
-
-  // ------------------------------------------------------------------ multigrid
-  // z = M^-1 r by one V(nu, nu)-cycle over the levels of mg.cu, all in FP32:
-  //   level l < L-1: u = S^nu f (damped Jacobi from zero), res = f - A u, f_{l+1} = P^T res,
-  //                  e_{l+1} from the level below, u += P e_{l+1}, e = S^nu applied from u;
-  //   level L-1:     e = mg_coarse_steps damped-Jacobi steps from zero,
-  // with f = r on level 0 and e = z there.  Pre- and post-smoothing are the same symmetric
-  // steps and restriction is the transpose of prolongation, so M^-1 is symmetric (and positive
-  // definite: omega lambda_max(D^-1 A) < 2), as CG needs.  Levels with few rows run on the
-  // group's first CTA alone with block barriers; a barrier between passes on two such levels is
-  // a block barrier, every other one the group's barrier.
-  __device__ __forceinline__ const float* lw(int l, int a) const {
-    return P.mg_w + P.mg[l].woff + (size_t)a * P.mg[l].plen + kSlack;
-  }
-  __device__ __forceinline__ float* lv(int l, int a) const {
-    return mgws + P.mg[l].voff + (size_t)a * P.mg[l].plen + kSlack;
-  }
-  __device__ __forceinline__ bool solo(int l) const { return P.cs == 1 || P.mg[l].ny + 1 <= P.mg_solo_rows; }
-  __device__ __forceinline__ void xsync(int a, int b) {
-    if (solo(a) && solo(b))
-      __syncthreads();
-    else
-      comm.sync();
-  }
-  // f(loc) for this CTA's groups of 4 nodes of level l
-  template <class F>
-  __device__ __forceinline__ void for_lgroups(int l, F f) const {
-    int r0l = 0, Rl = 0;
-    if (solo(l)) {
-      Rl = rank == 0 ? P.mg[l].ny + 1 : 0;
-    } else {
-      slab_rows(P.mg[l].ny + 1, P.cs, rank, r0l, Rl);
-    }
-    const int Wl = P.mg[l].W, G4l = Wl / kGroup;
-    for (int t = threadIdx.x; t < Rl * G4l; t += blockDim.x) {
-      const int lr = t / G4l, g = t - lr * G4l;
-      f((r0l + lr + 1) * Wl + kGroup * g);
-    }
-  }
+  // 1/C of the 4 nodes (0 off the unknowns)
+  __device__ __forceinline__ void dinv4(int loc, float (&v)[4]) const { ld4f(P.w32_inv, loc, v); }
   __device__ __forceinline__ void ld4f(const float* __restrict__ a, int loc, float (&v)[4]) const {
     const float4 c = *reinterpret_cast<const float4*>(a + loc);
     v[0] = c.x; v[1] = c.y; v[2] = c.z; v[3] = c.w;
@@ -199,21 +159,233 @@ struct Streamer {
   __device__ __forceinline__ void st4f(float* __restrict__ a, int loc, const float (&v)[4]) const {
     *reinterpret_cast<float4*>(a + loc) = make_float4(v[0], v[1], v[2], v[3]);
   }
+  // a CG vector's entries on a group
+  __device__ __forceinline__ void ldv(const float* __restrict__ a, int loc, V (&v)[4]) const {
+    if constexpr (kMixed) {
+      ld4f(a, loc, v);
+    } else {
+      float h[4], l[4];
+      ld4f(a, loc, h);
+      ld4f(a + lo, loc, l);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = make_ff(h[j], l[j]);
+    }
+  }
+  __device__ __forceinline__ void stv(float* __restrict__ a, int loc, const V (&v)[4]) const {
+    if constexpr (kMixed) {
+      st4f(a, loc, v);
+    } else {
+      float h[4], l[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h[j] = v[j].h;
+        l[j] = v[j].l;
+      }
+      st4f(a, loc, h);
+      st4f(a + lo, loc, l);
+    }
+  }
+  __device__ __forceinline__ void st4d(double* __restrict__ a, int loc, const double (&v)[4]) const {
+    *reinterpret_cast<double2*>(a + loc) = make_double2(v[0], v[1]);
+    *reinterpret_cast<double2*>(a + loc + 2) = make_double2(v[2], v[3]);
+  }
+
+  // Group barriers.  A pass's stores may be read by bulk copies of the next: every thread orders
+  // its stores before the barrier for the async proxy.
+  __device__ __forceinline__ void sync() {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    comm.sync();
+  }
+  template <class T, int NV, int NX = 0, class Post = NoPost>
+  __device__ __forceinline__ void allreduce(T (&v)[NV + NX], Post post = Post()) {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    comm.template allreduce<T, NV, NX, Post>(v, P.cs, post);
+  }
+
+  // ------------------------------------------------------------------ row rings
+  static __device__ __forceinline__ void bulk_load(unsigned dst, const float* src, unsigned bytes, unsigned bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+  }
+  __device__ __forceinline__ void ring_wait(int slot) {
+    bool in = false;
+    for (int i = 0; i < (1 << 20) && !in; ++i) in = mbar_try(ring_bar + slot, (ring_phase >> slot) & 1u);
+    if (!in) record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
+    ring_phase ^= 1u << slot;
+  }
+  // The rows below, at and above a group's row in the ring: the vector (v) and the weights (w, array
+  // a of C, E, N, NE, NW, omega/diag, or of omega/diag, k, m)
+  template <int NW>
+  struct RowRef {
+    const float *vec, *wts;   // the ring's vector rows and weight rows
+    int W, so, sm, su;        // row indexes in the ring
+    __device__ __forceinline__ const float* v(int s) const { return vec + s * W; }
+    __device__ __forceinline__ const float* w(int s, int a) const { return wts + (NW * s + a) * W; }
+    __device__ __forceinline__ const float* wd(int s) const { return w(s, NW == kNodeWeights ? 5 : 0); }
+  };
+  // Visit the groups of rows ya .. yb of level l, 512 consecutive groups at a time: body(rows, y, g,
+  // ok) finds the rows y-1, y, y+1 of the vector `vec` (padded layout of the level) and of the
+  // level's weights in shared memory (every lane calls it; one without a group has ok = false and
+  // the last group's operands), then after(y_done) runs behind a block barrier, rows below y_done
+  // visited.  The rows ya-1 .. yb+1 (all inside the padded layout) come in chunks of CR rows, one
+  // mbarrier and two bulk copies each; a chunk's slot is filled again once its rows are done.
+  template <int NW, class Body, class After>
+  __device__ __forceinline__ void march(int l, const float* vec, int ya, int yb, Body body, After after) {
+    const int Wl = P.mg[l].W, G4l = Wl / kGroup, first = ya - 1, nr = yb - ya + 3, n = (yb - ya + 1) * G4l;
+    const int Smax = pipe_rows(G4l, NW), CR = nr <= Smax ? nr : chunk_rows(Smax, trip_rows(G4l));
+    const int NS = Smax / CR, S = NS * CR, nchunks = (nr + CR - 1) / CR;
+    float* svec = ring_sm;
+    float* swts = ring_sm + Smax * Wl;
+    const float* gvec = vec + (size_t)(first + 1) * Wl;
+    const float* gwts = (NW == kNodeWeights ? lwb(l) : P.mg_elem + kSlack) + (size_t)(first + 1) * NW * Wl;
+    int issued = 0, ready = 0;
+    auto issue = [&](int upto) {           // chunks
+      if (threadIdx.x != 0) return;
+      for (; issued < upto; ++issued) {
+        const int slot = issued % NS, row = issued * CR, rows = min(CR, nr - row);
+        const unsigned bytes = 4u * (unsigned)(rows * Wl), bar = smem_u32(ring_bar + slot);
+        mbar_expect(ring_bar + slot, (1u + NW) * bytes);
+        bulk_load(smem_u32(svec + slot * CR * Wl), gvec + (size_t)row * Wl, bytes, bar);
+        bulk_load(smem_u32(swts + slot * CR * NW * Wl), gwts + (size_t)row * NW * Wl, NW * bytes, bar);
+      }
+    };
+    asm volatile("fence.proxy.async;" ::: "memory");
+    issue(min(NS, nchunks));
+    for (int t0 = 0; t0 < n; t0 += kStreamThreads) {
+      const int t = t0 + (int)threadIdx.x, tc = min(t, n - 1);
+      const int need = ((min(n, t0 + kStreamThreads) - 1) / G4l + 2) / CR;   // last chunk of the trip
+      for (; ready <= need; ++ready) ring_wait(ready % NS);
+      const int ry = tc / G4l, g = tc - ry * G4l;
+      RowRef<NW> rr;
+      rr.vec = svec;
+      rr.wts = swts;
+      rr.W = Wl;
+      rr.so = ry % S;
+      rr.sm = rr.so + 1 == S ? 0 : rr.so + 1;
+      rr.su = rr.sm + 1 == S ? 0 : rr.sm + 1;
+      body(rr, ya + ry, g, t < n);
+      __syncthreads();
+      const int done = min(n, t0 + kStreamThreads) / G4l;   // whole rows visited: chunks below are free
+      issue(min(nchunks, done / CR + NS));
+      after(ya + done);
+    }
+    __syncthreads();   // the ring is free for the next pass
+  }
+  // 6-entry window of a group in a ring row; entries beyond the lane's own 16 bytes come from the
+  // neighbouring lanes (their groups follow one another, a row's last entry is a zero pad)
+  __device__ __forceinline__ void rwin(const float* row, int g, int G4l, float (&w)[6]) const {
+    const int lane = threadIdx.x & 31;
+    const float* x = row + kGroup * g;
+    const float4 c = *reinterpret_cast<const float4*>(x);
+    float e = 0.f;
+    if (lane == 0 && g > 0) e = x[-1];
+    if (lane == 31 && g < G4l - 1) e = x[4];
+    const float l = __shfl_up_sync(0xffffffffu, c.w, 1), u = __shfl_down_sync(0xffffffffu, c.x, 1);
+    w[0] = lane == 0 ? e : l;
+    w[1] = c.x; w[2] = c.y; w[3] = c.z; w[4] = c.w;
+    w[5] = lane == 31 ? e : u;
+  }
+  // A v on a group from v's windows and the weights' rows in the ring
+  __device__ __forceinline__ void rstencil(const RowRef<kElemWeights>& rr, int g, int G4l, const float (&vl)[6],
+                                           const float (&vm)[6], const float (&vh)[6], float (&y)[4]) const {
+    float kl[6], ml[6], ku[6], mu[6];
+    rwin(rr.w(rr.so, 1), g, G4l, kl);
+    rwin(rr.w(rr.so, 2), g, G4l, ml);
+    rwin(rr.w(rr.sm, 1), g, G4l, ku);
+    rwin(rr.w(rr.sm, 2), g, G4l, mu);
+    km_combine(vl, vm, vh, kl, ml, ku, mu, y);
+  }
+  __device__ __forceinline__ void rstencil(const RowRef<kNodeWeights>& rr, int g, int G4l, const float (&vl)[6],
+                                           const float (&vm)[6], const float (&vh)[6], float (&y)[4]) const {
+    float c4[4], n4[4], ne4[4], nw4[4], nb[4], e6[6], s6[6], t6[6];
+    ld4f(rr.w(rr.sm, 0), kGroup * g, c4);
+    rwin(rr.w(rr.sm, 1), g, G4l, e6);
+    ld4f(rr.w(rr.sm, 2), kGroup * g, n4);
+    ld4f(rr.w(rr.sm, 3), kGroup * g, ne4);
+    ld4f(rr.w(rr.sm, 4), kGroup * g, nw4);
+    ld4f(rr.w(rr.so, 2), kGroup * g, nb);
+    rwin(rr.w(rr.so, 3), g, G4l, s6);     // NE of the row below: the south-west neighbours' weights
+    rwin(rr.w(rr.so, 4), g, G4l, t6);     // NW of the row below: the south-east neighbours' weights
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float a = c4[j] * vm[j + 1];
+      a = fmaf(e6[j + 1], vm[j + 2], a);
+      a = fmaf(e6[j], vm[j], a);
+      a = fmaf(n4[j], vh[j + 1], a);
+      a = fmaf(nb[j], vl[j + 1], a);
+      a = fmaf(ne4[j], vh[j + 2], a);
+      a = fmaf(s6[j], vl[j], a);
+      a = fmaf(nw4[j], vh[j], a);
+      a = fmaf(t6[j + 2], vl[j + 2], a);
+      y[j] = a;
+    }
+  }
+
+  // ------------------------------------------------------------------ multigrid
+  // z = M^-1 r by one V(1, 1)-cycle over the levels of mg.cu, all in FP32:
+  //   level l < L-1: u = S f (one damped-Jacobi step from zero), f_{l+1} = P^T (f - A u),
+  //                  e_{l+1} from the level below, u' = u + P e_{l+1}, e = u' + S (f - A u');
+  //   level L-1:     e = mg_coarse_steps damped-Jacobi steps from zero,
+  // with f = r (its high parts) on level 0 and e = z there.  Pre- and post-smoothing are the same
+  // symmetric step and restriction is the transpose of prolongation, so M^-1 is symmetric (and
+  // positive definite: omega lambda_max(D^-1 A) < 2), as CG needs.  Levels with few rows run on the
+  // group's first CTA alone with block barriers; a barrier between passes on two such levels is
+  // a block barrier, every other one the group's barrier.  A large level is one march down (the
+  // residual is restricted from shared memory) and one up (u is formed again from f).
+  // level l's weights: six arrays (C, E, N, NE, NW, omega/diag) interleaved row by row, so array a of
+  // node (iy, ix) is at (6 (iy + 1) + a) W + ix + 1
+  __device__ __forceinline__ const float* lwb(int l) const { return P.mg_w + P.mg[l].woff + kSlack; }
+  __device__ __forceinline__ const float* lw(int l, int a) const { return lwb(l) + a * P.mg[l].W; }
+  __device__ __forceinline__ float* lv(int l, int a) const {
+    return mgws + P.mg[l].voff + (size_t)a * P.mg[l].plen + kSlack;
+  }
+  __device__ __forceinline__ bool solo(int l) const { return P.cs == 1 || P.mg[l].ny + 1 <= P.mg_solo_rows; }
+  __device__ __forceinline__ bool piped(int l) const { return pipe_rows(P.mg[l].W / kGroup, l == 0 ? kElemWeights : kNodeWeights) > 0; }
+  __device__ __forceinline__ void xsync(int a, int b) {
+    if (solo(a) && solo(b)) {
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      __syncthreads();
+    } else {
+      sync();
+    }
+  }
+  // this CTA's node rows [y0, y0 + n) of level l
+  __device__ __forceinline__ void lrows(int l, int& y0, int& n) const {
+    y0 = 0;
+    n = 0;
+    if (solo(l))
+      n = rank == 0 ? P.mg[l].ny + 1 : 0;
+    else
+      slab_rows(P.mg[l].ny + 1, P.cs, rank, y0, n);
+  }
+  // f(loc, wloc) for this CTA's groups of 4 nodes of level l: their padded index, and the index of
+  // their weights
+  template <class F>
+  __device__ __forceinline__ void for_lgroups(int l, F f) const {
+    int r0l, Rl;
+    lrows(l, r0l, Rl);
+    const int Wl = P.mg[l].W, G4l = Wl / kGroup;
+    for (int t = threadIdx.x; t < Rl * G4l; t += blockDim.x) {
+      const int lr = t / G4l, g = t - lr * G4l;
+      const int row = r0l + lr + 1;
+      f(row * Wl + kGroup * g, 6 * row * Wl + kGroup * g);
+    }
+  }
   // y = A_l v on a group from v's windows on the rows below, at and above it (FP32 node weights)
-  template <class T>
-  __device__ __forceinline__ void lstencil(int l, int loc, const float (&vl)[6], const float (&vm)[6],
-                                           const float (&vh)[6], T (&y)[4]) const {
-    const int Wl = P.mg[l].W;
+  __device__ __forceinline__ void lstencil(int l, int wloc, const float (&vl)[6], const float (&vm)[6],
+                                           const float (&vh)[6], float (&y)[4]) const {
+    const int Wl = P.mg[l].W, wb = wloc - 6 * Wl;       // the row below
     const float *C = lw(l, 0), *E = lw(l, 1), *N = lw(l, 2), *NE = lw(l, 3), *NW = lw(l, 4);
     float c4[4], n4[4], nb[4], ne4[4], nw4[4], e5[5];
-    ld4f(C, loc, c4);
-    ld4f(N, loc, n4);
-    ld4f(N, loc - Wl, nb);
-    ld4f(NE, loc, ne4);
-    ld4f(NW, loc, nw4);
-    load_ewindow(E, loc, e5);
-    const float* neb = NE + loc - Wl - 1;   // NE weights of the row below, shifted left
-    const float* nwb = NW + loc - Wl + 1;   // NW weights of the row below, shifted right
+    ld4f(C, wloc, c4);
+    ld4f(N, wloc, n4);
+    ld4f(N, wb, nb);
+    ld4f(NE, wloc, ne4);
+    ld4f(NW, wloc, nw4);
+    load_ewindow(E, wloc, e5);
+    const float* neb = NE + wb - 1;         // NE weights of the row below, shifted left
+    const float* nwb = NW + wb + 1;         // NW weights of the row below, shifted right
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float a = c4[j] * vm[j + 1];
@@ -225,89 +397,202 @@ struct Streamer {
       a = fmaf(neb[j], vl[j], a);
       a = fmaf(nw4[j], vh[j], a);
       a = fmaf(nwb[j], vl[j + 2], a);
-      y[j] = (T)a;
+      y[j] = a;
     }
   }
-  template <class T>
-  __device__ __forceinline__ void lwindows(const T* __restrict__ v, int loc, int Wl, float (&a)[6], float (&b)[6],
-                                           float (&c)[6]) const {
-    T t[6];
-    load_window(v, loc - Wl, t);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) a[i] = (float)t[i];
-    load_window(v, loc, t);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) b[i] = (float)t[i];
-    load_window(v, loc + Wl, t);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) c[i] = (float)t[i];
+  // windows on the rows below, at and above (rows `stride` floats apart)
+  __device__ __forceinline__ void lwindows(const float* __restrict__ v, int loc, int stride, float (&a)[6],
+                                           float (&b)[6], float (&c)[6]) const {
+    load_window(v, loc - stride, a);
+    load_window(v, loc, b);
+    load_window(v, loc + stride, c);
   }
-  // Pre-smoothing of level l from zero on f: nu = 1: u = S f = omega D^-1 f and res = f - A u in
-  // one pass (u of the neighbours formed from their f); nu = 2: u = S f + S (f - A S f) in one
-  // pass, then res = f - A u after a barrier.  res is 0 off the unknowns.
-  template <class T>
-  __device__ void mg_pre(int l, const T* __restrict__ f) {
+  // a large level on the way down: u = S f and res = f - A u row by row, f_{l+1} = P^T res.  The CTA
+  // writes the coarse rows J with 2J among its rows, for which it also forms the residual on the
+  // row on each side of them; the residual waits in a ring of its own behind the arrays'.
+  template <int NW>
+  __device__ __forceinline__ void mg_down_march(int l, const float* __restrict__ f) {
+    int y0, n;
+    lrows(l, y0, n);
+    const int ny = P.mg[l].ny, Wl = P.mg[l].W, G4l = Wl / kGroup, Wc = P.mg[l + 1].W, G4c = Wc / kGroup;
+    const int nxc = P.mg[l + 1].nx;
+    if (n > 0) {
+      const int ya = max(y0 - 1, 0), yb = min(y0 + n, ny), SR = res_rows(G4l);
+      float* res = ring_sm + (1 + NW) * pipe_rows(G4l, NW) * Wl;
+      const float* wdc = lw(l + 1, 5);
+      float* fc = lv(l + 1, 0);
+      int J = (y0 + 1) / 2;
+      const int Jend = (y0 + n + 1) / 2;           // coarse rows J .. Jend - 1
+      march<NW>(l, f, ya, yb,
+               [&](const RowRef<NW>& rr, int y, int g, bool ok) {
+                 float vl[6], vm[6], vh[6], dw[6], t[4], fc4[4], o[4];
+                 rwin(rr.v(rr.so), g, G4l, vl);
+                 rwin(rr.wd(rr.so), g, G4l, dw);
+#pragma unroll
+                 for (int i = 0; i < 6; ++i) vl[i] *= dw[i];
+                 rwin(rr.v(rr.su), g, G4l, vh);
+                 rwin(rr.wd(rr.su), g, G4l, dw);
+#pragma unroll
+                 for (int i = 0; i < 6; ++i) vh[i] *= dw[i];
+                 rwin(rr.v(rr.sm), g, G4l, vm);
+                 rwin(rr.wd(rr.sm), g, G4l, dw);
+#pragma unroll
+                 for (int j = 0; j < 4; ++j) fc4[j] = vm[j + 1];
+#pragma unroll
+                 for (int i = 0; i < 6; ++i) vm[i] *= dw[i];
+                 rstencil(rr, g, G4l, vl, vm, vh, t);
+#pragma unroll
+                 for (int j = 0; j < 4; ++j) o[j] = dw[j + 1] != 0.f ? fc4[j] - t[j] : 0.f;
+                 if (ok) st4f(res, ((y - ya) % SR) * Wl + kGroup * g, o);
+               },
+               [&](int ydone) {
+                 // coarse rows whose fine rows 2J-1 .. 2J+1 are all there
+                 const int Jn = ydone > yb ? Jend : max(J, min(Jend, ydone / 2));
+                 for (int t = threadIdx.x; t < (Jn - J) * G4c; t += kStreamThreads) {
+                   const int jr = t / G4c, gc = t - jr * G4c, Jc = J + jr, I0 = kGroup * gc - 1;
+                   float dv[4], o[4] = {0.f, 0.f, 0.f, 0.f};
+                   const int loc = (Jc + 1) * Wc + kGroup * gc;
+                   ld4f(wdc, 6 * (Jc + 1) * Wc + kGroup * gc, dv);
+#pragma unroll
+                   for (int b = -1; b <= 1; ++b) {
+                     const int y = 2 * Jc + b;
+                     if (y < 0 || y > ny) continue;
+                     // entries 8 gc - 4 .. 8 gc + 7 of the row: column 2 I of node j is entry 3 + 2 j
+                     const float* row = res + ((y - ya) % SR) * Wl + 2 * kGroup * gc - 4;
+                     // (those outside the row belong to pads of the coarse row)
+                     const int at = 2 * kGroup * gc;
+                     float4 ca = make_float4(0.f, 0.f, 0.f, 0.f), cb = ca, cc = ca;
+                     if (gc > 0) ca = *reinterpret_cast<const float4*>(row);
+                     if (at < Wl) cb = *reinterpret_cast<const float4*>(row + 4);
+                     if (at + 4 < Wl) cc = *reinterpret_cast<const float4*>(row + 8);
+                     const float hb = b == 0 ? 1.f : 0.5f;
+                     o[0] = fmaf(hb, fmaf(0.5f, ca.z + cb.x, ca.w), o[0]);
+                     o[1] = fmaf(hb, fmaf(0.5f, cb.x + cb.z, cb.y), o[1]);
+                     o[2] = fmaf(hb, fmaf(0.5f, cb.z + cc.x, cb.w), o[2]);
+                     o[3] = fmaf(hb, fmaf(0.5f, cc.x + cc.z, cc.y), o[3]);
+                   }
+#pragma unroll
+                   for (int j = 0; j < 4; ++j)
+                     if (dv[j] == 0.f || I0 + j < 0 || I0 + j > nxc) o[j] = 0.f;
+                   st4f(fc, loc, o);
+                 }
+                 J = Jn;
+               });
+    }
+  }
+  // a large level on the way up: u' = S f + P e_{l+1}, out = u' + S (f - A u'); level 0 writes z and
+  // returns the local (r, z)
+  template <int NW>
+  __device__ __forceinline__ V mg_up_march(int l, const float* __restrict__ f) {
+    int y0, n;
+    lrows(l, y0, n);
+    V rz = V{};
+    if (n == 0) return rz;
+    const int Wl = P.mg[l].W, G4l = Wl / kGroup, Wc = P.mg[l + 1].W;
+    const float* ec = lv(l + 1, 3);
+    float* out = l == 0 ? z : lv(l, 3);
+    march<NW>(l, f, y0, y0 + n - 1,
+             [&](const RowRef<NW>& rr, int y, int g, bool ok) {
+               // coarse rows A, B, C: row y-1 takes A and B (y even) or A, row y B or A and B, row
+               // y+1 B and C or B; columns 2g-1 .. 2g+2
+               const bool even = (y & 1) == 0;
+               const int c0 = 2 * g;
+               const float* eA = ec + (((y - 1) >> 1) + 1) * Wc + c0;
+               const float* eB = ec + (((y + 1) >> 1) + 1) * Wc + c0;
+               const float* eC = ec + (((y + 2) >> 1) + 1) * Wc + c0;
+               float pa[4], pb[4], pc[4];
+               auto ld = [](const float* q_, float (&v)[4]) {
+                 const float2 a = *reinterpret_cast<const float2*>(q_), b = *reinterpret_cast<const float2*>(q_ + 2);
+                 v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+               };
+               ld(eA, pa);
+               ld(eB, pb);
+               ld(eC, pc);
+               const int loc = (y + 1) * Wl + kGroup * g;
+               V rv[4];
+               if (l == 0) ldv(r, loc, rv);
+               float vl[6], vm[6], vh[6], dw[6], t[4], fc4[4], o[4];
+               // the row's window of P e: even window columns on coarse columns, odd ones between
+               auto add = [&](float (&v)[6], const float (&c)[4]) {
+#pragma unroll
+                 for (int i = 0; i < 6; ++i) {
+                   const float pe = i & 1 ? 0.5f * (c[i >> 1] + c[(i >> 1) + 1]) : c[i >> 1];
+                   v[i] = dw[i] != 0.f ? fmaf(v[i], dw[i], pe) : 0.f;
+                 }
+               };
+               float m[4];
+#pragma unroll
+               for (int i = 0; i < 4; ++i) m[i] = 0.5f * (pa[i] + pb[i]);
+               rwin(rr.v(rr.so), g, G4l, vl);
+               rwin(rr.wd(rr.so), g, G4l, dw);
+               float c_[4];
+#pragma unroll
+               for (int i = 0; i < 4; ++i) c_[i] = even ? m[i] : pa[i];
+               add(vl, c_);
+               rwin(rr.v(rr.su), g, G4l, vh);
+               rwin(rr.wd(rr.su), g, G4l, dw);
+#pragma unroll
+               for (int i = 0; i < 4; ++i) c_[i] = even ? 0.5f * (pb[i] + pc[i]) : pb[i];
+               add(vh, c_);
+               rwin(rr.v(rr.sm), g, G4l, vm);
+               rwin(rr.wd(rr.sm), g, G4l, dw);
+#pragma unroll
+               for (int j = 0; j < 4; ++j) fc4[j] = vm[j + 1];
+#pragma unroll
+               for (int i = 0; i < 4; ++i) c_[i] = even ? pb[i] : m[i];
+               add(vm, c_);
+               rstencil(rr, g, G4l, vl, vm, vh, t);
+#pragma unroll
+               for (int j = 0; j < 4; ++j) o[j] = fmaf(dw[j + 1], fc4[j] - t[j], vm[j + 1]);
+               if (!ok) return;
+               if (l == 0) {
+#pragma unroll
+                 for (int j = 0; j < 4; ++j) rz = vdot(rz, rv[j], o[j]);
+               }
+               st4f(out, loc, o);
+             },
+             [](int) {});
+    return rz;
+  }
+  // a small level on the way down: u = S f and res = f - A u (u of the neighbours from their f)
+  __device__ __forceinline__ void mg_pre(int l, const float* __restrict__ f) {
     const int Wl = P.mg[l].W;
     const float* wd = lw(l, 5);
     float* u = lv(l, l == 0 ? 0 : 1);
     float* res = lv(l, l == 0 ? 1 : 2);
-    for_lgroups(l, [&](int loc) {
+    for_lgroups(l, [&](int loc, int wloc) {
       float fl[6], fm[6], fh[6], dl[6], dm[6], dh[6], y[4], uo[4], ro[4], fc[4];
       lwindows(f, loc, Wl, fl, fm, fh);
-      lwindows(wd, loc, Wl, dl, dm, dh);
+      lwindows(wd, wloc, 6 * Wl, dl, dm, dh);
 #pragma unroll
       for (int j = 0; j < 4; ++j) fc[j] = fm[j + 1];
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
-        fl[i] *= dl[i];   // u = S f on the window (fl.. now hold u)
+        fl[i] *= dl[i];
         fm[i] *= dm[i];
         fh[i] *= dh[i];
       }
-      lstencil(l, loc, fl, fm, fh, y);
+      lstencil(l, wloc, fl, fm, fh, y);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float rj = dm[j + 1] != 0.f ? fc[j] - y[j] : 0.f;
+        ro[j] = dm[j + 1] != 0.f ? fc[j] - y[j] : 0.f;
         uo[j] = fm[j + 1];
-        if (P.mg_nu >= 2) uo[j] = fmaf(dm[j + 1], rj, uo[j]);
-        ro[j] = rj;
       }
       st4f(u, loc, uo);
-      if (P.mg_nu < 2) st4f(res, loc, ro);
+      st4f(res, loc, ro);
     });
-    if (P.mg_nu >= 2) {
-      xsync(l, l);
-      for_lgroups(l, [&](int loc) {
-        float ul[6], um[6], uh[6], y[4], ro[4], dv[4];
-        T fv[4];
-        lwindows(u, loc, Wl, ul, um, uh);
-        lstencil(l, loc, ul, um, uh, y);
-        ld4f(wd, loc, dv);
-        ldv(f, loc, fv);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) ro[j] = dv[j] != 0.f ? (float)fv[j] - y[j] : 0.f;
-        st4f(res, loc, ro);
-      });
-    }
-  }
-  template <class T>
-  __device__ __forceinline__ void ldv(const T* __restrict__ a, int loc, T (&v)[4]) const {
-    if constexpr (sizeof(T) == 8) {
-      load4(a + loc, v);
-    } else {
-      ld4f(a, loc, v);
-    }
   }
   // f_{l+1} = P^T res_l on the nodes of level l+1 (0 off its unknowns)
-  __device__ void mg_restrict(int l) {
+  __device__ __forceinline__ void mg_restrict(int l) {
     const int c = l + 1, Wf = P.mg[l].W, nxc = P.mg[c].nx;
     const float* res = lv(l, l == 0 ? 1 : 2);
     const float* wdc = lw(c, 5);
     float* fc = lv(c, 0);
     const int Wc = P.mg[c].W;
-    for_lgroups(c, [&](int loc) {
+    for_lgroups(c, [&](int loc, int wloc) {
       const int J = loc / Wc - 1, I0 = loc - (J + 1) * Wc - 1;
       float dv[4], o[4];
-      ld4f(wdc, loc, dv);
+      ld4f(wdc, wloc, dv);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int I = I0 + j;
@@ -327,7 +612,7 @@ struct Streamer {
     });
   }
   // coarsest level: e = mg_coarse_steps damped-Jacobi steps from zero, the last into e
-  __device__ void mg_coarsest(int l) {
+  __device__ __forceinline__ void mg_coarsest(int l) {
     const int Wl = P.mg[l].W, n = P.mg_coarse_steps;
     const float* f = lv(l, 0);
     const float* wd = lw(l, 5);
@@ -335,17 +620,17 @@ struct Streamer {
     for (int k = 1; k <= n; ++k) {
       float* dst = bufs[(n - k) & 1];
       const float* src = bufs[(n - k + 1) & 1];
-      for_lgroups(l, [&](int loc) {
+      for_lgroups(l, [&](int loc, int wloc) {
         float fv[4], dv[4], o[4];
         ld4f(f, loc, fv);
-        ld4f(wd, loc, dv);
+        ld4f(wd, wloc, dv);
         if (k == 1) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) o[j] = dv[j] * fv[j];
         } else {
           float vl[6], vm[6], vh[6], y[4];
           lwindows(src, loc, Wl, vl, vm, vh);
-          lstencil(l, loc, vl, vm, vh, y);
+          lstencil(l, wloc, vl, vm, vh, y);
 #pragma unroll
           for (int j = 0; j < 4; ++j) o[j] = fmaf(dv[j], fv[j] - y[j], vm[j + 1]);
         }
@@ -354,150 +639,50 @@ struct Streamer {
       xsync(l, l);
     }
   }
-  // u_l += P e_{l+1} on the unknowns of level l
-  __device__ void mg_prolong(int l) {
-    const int c = l + 1, Wl = P.mg[l].W, Wc = P.mg[c].W;
-    const float* ec = lv(c, 3);
-    const float* wd = lw(l, 5);
-    float* u = lv(l, l == 0 ? 0 : 1);
-    for_lgroups(l, [&](int loc) {
-      const int y = loc / Wl - 1, x0 = loc - (y + 1) * Wl - 1;
-      float dv[4], uv[4];
-      ld4f(wd, loc, dv);
-      ld4f(u, loc, uv);
-      const int Ja = y >> 1, Jb = (y + 1) >> 1;   // y even: Ja = Jb = y / 2
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int x = x0 + j;
-        if (dv[j] == 0.f) continue;               // also every pad column
-        const int Ia = x >> 1, Ib = (x + 1) >> 1;
-        const float* ra = ec + (Ja + 1) * Wc + 1;
-        const float* rb = ec + (Jb + 1) * Wc + 1;
-        const float v = 0.25f * ((ra[Ia] + ra[Ib]) + (rb[Ia] + rb[Ib]));
-        uv[j] += v;
-      }
-      st4f(u, loc, uv);
-    });
-  }
-  // Post-smoothing of level l from u: nu steps out = v + S (f - A v); level 0 writes z in the CG
-  // precision and returns the local (r, z); nu = 2 goes through res.
-  template <class T>
-  __device__ Real mg_post(int l, const T* __restrict__ f) {
-    const int Wl = P.mg[l].W;
-    const float* wd = lw(l, 5);
-    float* u = lv(l, l == 0 ? 0 : 1);
-    float* tmp = lv(l, l == 0 ? 1 : 2);
-    Real rz = Real(0);
-    for (int step = 0; step < P.mg_nu; ++step) {
-      const bool last = step == P.mg_nu - 1;
-      const float* src = step == 0 ? u : tmp;
-      if (step > 0) xsync(l, l);
-      for_lgroups(l, [&](int loc) {
-        float vl[6], vm[6], vh[6], y[4], dv[4], o[4];
-        T fv[4];
-        lwindows(src, loc, Wl, vl, vm, vh);
-        lstencil(l, loc, vl, vm, vh, y);
-        ld4f(wd, loc, dv);
-        ldv(f, loc, fv);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) o[j] = fmaf(dv[j], (float)fv[j] - y[j], vm[j + 1]);
-        if (!last) {
-          st4f(tmp, loc, o);
-        } else if (l == 0) {
-          Real zv[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            zv[j] = (Real)o[j];
-            rz = fma((Real)fv[j], zv[j], rz);
-          }
-          st4(z, loc, zv);
-        } else {
-          st4f(lv(l, 3), loc, o);
-        }
-      });
-    }
-    return rz;
-  }
-  // nu = 1: the prolongation and the post-smoothing step in one pass, out = u' + S (f - A u') with
-  // u' = u + P e_{l+1} formed on the window from u and the coarse e (no barrier between them);
-  // level 0 writes z in the CG precision and returns the local (r, z)
-  template <class T>
-  __device__ Real mg_prolong_post(int l, const T* __restrict__ f) {
+  // a small level on the way up: the prolongation and the post-smoothing step in one pass, with
+  // u' = u + P e_{l+1} formed on the window from u and the coarse e
+  __device__ __forceinline__ V mg_up(int l, const float* __restrict__ f) {
     const int c = l + 1, Wl = P.mg[l].W, Wc = P.mg[c].W;
     const float* ec = lv(c, 3);
     const float* wd = lw(l, 5);
     const float* u = lv(l, l == 0 ? 0 : 1);
-    const float *C = lw(l, 0), *E = lw(l, 1), *N = lw(l, 2), *NE = lw(l, 3), *NW = lw(l, 4);
-    Real rz = Real(0);
-    for_lgroups(l, [&](int loc) {
+    V rz = V{};
+    for_lgroups(l, [&](int loc, int wloc) {
       const int y = loc / Wl - 1, x0 = loc - (y + 1) * Wl - 1;   // first node of the group
-      // A u' accumulated row by row (rows y-1, y, y+1) from the window of u' = u + P e_{l+1};
       // x0 = 4g - 1 is odd, so window column i (node x0 - 1 + i) lies between coarse columns
       // cx0 + i/2 and cx0 + (i+1)/2 (equal for even i)
       const int cx0 = (x0 - 1) >> 1;
-      float acc[4] = {0.f, 0.f, 0.f, 0.f}, uc[4];
+      float win[3][6];
 #pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const int row = loc + (r - 1) * Wl;
-        float v[6], d[6];
+      for (int r_ = 0; r_ < 3; ++r_) {
+        const int row = loc + (r_ - 1) * Wl;
+        float v[6], d_[6];
         load_window(u, row, v);
-        load_window(wd, row, d);
-        const int yy = y - 1 + r, Ja = yy >> 1, Jb = (yy + 1) >> 1;
+        load_window(wd, wloc + (r_ - 1) * 6 * Wl, d_);
+        const int yy = y - 1 + r_, Ja = yy >> 1, Jb = (yy + 1) >> 1;
         const float* ra = ec + (Ja + 1) * Wc + 1 + cx0;
         const float* rb = ec + (Jb + 1) * Wc + 1 + cx0;
-        float ca[4], cb[4];
+        float cc[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          ca[q] = ra[q];
-          cb[q] = rb[q];
-        }
+        for (int q_ = 0; q_ < 4; ++q_) cc[q_] = 0.5f * (ra[q_] + rb[q_]);
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
-          const int Ia = i >> 1, Ib = (i + 1) >> 1;
-          const float pv = 0.25f * ((ca[Ia] + ca[Ib]) + (cb[Ia] + cb[Ib]));
-          if (d[i] != 0.f) v[i] += pv;
-        }
-        if (r == 0) {          // the row below: N of the node below, NE of the SW, NW of the SE node
-          float nb[4];
-          ld4f(N, loc - Wl, nb);
-          const float* neb = NE + loc - Wl - 1;
-          const float* nwb = NW + loc - Wl + 1;
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            acc[j] = fmaf(nb[j], v[j + 1], fmaf(neb[j], v[j], fmaf(nwb[j], v[j + 2], acc[j])));
-        } else if (r == 1) {   // the node's row: C, E of the node, E of the west neighbour
-          float c4[4], e5[5];
-          ld4f(C, loc, c4);
-          load_ewindow(E, loc, e5);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            acc[j] = fmaf(c4[j], v[j + 1], fmaf(e5[j + 1], v[j + 2], fmaf(e5[j], v[j], acc[j])));
-            uc[j] = v[j + 1];
-          }
-        } else {               // the row above: the node's N, NE, NW
-          float n4[4], ne4[4], nw4[4];
-          ld4f(N, loc, n4);
-          ld4f(NE, loc, ne4);
-          ld4f(NW, loc, nw4);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            acc[j] = fmaf(n4[j], v[j + 1], fmaf(ne4[j], v[j + 2], fmaf(nw4[j], v[j], acc[j])));
+          const float pv = i & 1 ? 0.5f * (cc[i >> 1] + cc[(i >> 1) + 1]) : cc[i >> 1];
+          win[r_][i] = d_[i] != 0.f ? v[i] + pv : v[i];
         }
       }
-      float dv[4], o[4];
-      T fv[4];
-      ld4f(wd, loc, dv);
-      ldv(f, loc, fv);
+      float t[4], dv[4], fv[4], o[4];
+      lstencil(l, wloc, win[0], win[1], win[2], t);
+      ld4f(wd, wloc, dv);
+      ld4f(f, loc, fv);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) o[j] = fmaf(dv[j], (float)fv[j] - acc[j], uc[j]);
+      for (int j = 0; j < 4; ++j) o[j] = fmaf(dv[j], fv[j] - t[j], win[1][j + 1]);
       if (l == 0) {
-        Real zv[4];
+        V rv[4];
+        ldv(r, loc, rv);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          zv[j] = (Real)o[j];
-          rz = fma((Real)fv[j], zv[j], rz);
-        }
-        st4(z, loc, zv);
+        for (int j = 0; j < 4; ++j) rz = vdot(rz, rv[j], o[j]);
+        st4f(z, loc, o);
       } else {
         st4f(lv(l, 3), loc, o);
       }
@@ -507,178 +692,254 @@ struct Streamer {
 
   // z = M^-1 r from r (every row of r visible); returns the local (r, z).  z is visible to the
   // group after the next group barrier.
-  __device__ Real vcycle() {
+  __device__ __forceinline__ V vcycle() {
     const int L = P.mg_levels;
     for (int l = 0; l < L - 1; ++l) {
-      if (l == 0)
-        mg_pre(0, r);
-      else
-        mg_pre(l, (const float*)lv(l, 0));
-      xsync(l, l + 1);
-      mg_restrict(l);
-      xsync(l + 1, l + 1);
+      const float* f = l == 0 ? r : lv(l, 0);
+      if (piped(l)) {
+        if (l == 0)
+          mg_down_march<kElemWeights>(0, f);
+        else
+          mg_down_march<kNodeWeights>(l, f);
+        xsync(l, l + 1);
+      } else {
+        mg_pre(l, f);
+        xsync(l, l + 1);
+        mg_restrict(l);
+        xsync(l + 1, l + 1);
+      }
     }
     mg_coarsest(L - 1);                 // ends with a barrier
-    Real rz = Real(0);
+    V rz = V{};
     for (int l = L - 2; l >= 0; --l) {
       if (l < L - 2) xsync(l + 1, l);   // e_{l+1} of the level above is visible
-      else if (!(solo(l + 1) && solo(l))) comm.sync();
-      if (P.mg_nu == 1 && P.mg_fuse) {
-        if (l == 0)
-          rz = mg_prolong_post(0, r);
-        else
-          mg_prolong_post(l, (const float*)lv(l, 0));
-        continue;
-      }
-      mg_prolong(l);
-      xsync(l, l);
+      else if (!(solo(l + 1) && solo(l))) sync();
+      const float* f = l == 0 ? r : lv(l, 0);
       if (l == 0)
-        rz = mg_post(0, r);
+        rz = piped(0) ? mg_up_march<kElemWeights>(0, f) : mg_up(0, f);
+      else if (piped(l))
+        mg_up_march<kNodeWeights>(l, f);
       else
-        mg_post(l, (const float*)lv(l, 0));
+        mg_up(l, f);
     }
     return rz;
   }
 
-  // r = b - A x (FP64, stored in the CG precision unscaled, 0 off the unknowns); the local
-  // (b, b) and (r, r)
-  __device__ void residual(const double* __restrict__ x, double& bb, double& rr) const {
+  // b <- b - A x (FP64, 0 off the unknowns); the local (b, b) of the old b and (r, r)
+  __device__ __forceinline__ void residual(const double* __restrict__ x, double& bb, double& rr) const {
     bb = 0.0;
     rr = 0.0;
     for_groups([&](int loc, int, int) {
       double y[4], bv[4];
-      Real di[4], rv[4];
+      float di[4];
       stencil_node64<double>(x, loc, A64, loc, P.W, y);
       load4(b + loc, bv);
       dinv4(loc, di);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const double t = di[j] != Real(0) ? bv[j] - y[j] : 0.0;
         bb = fma(bv[j], bv[j], bb);
-        rr = fma(t, t, rr);
-        rv[j] = (Real)t;
+        bv[j] = di[j] != 0.f ? bv[j] - y[j] : 0.0;
+        rr = fma(bv[j], bv[j], rr);
       }
-      st4(r, loc, rv);
+      st4d(b, loc, bv);
     });
   }
+  // After a CG: x += unscale d, and b <- b - unscale A d with A d summed in float pairs (see
+  // Stepper::update_residual: d is a small correction of x, so the 48 bits of its product are finer
+  // than the rounding of an FP64 b - A x); returns the local (r, r)
+  __device__ __forceinline__ double update_residual(double* __restrict__ x, double unscale) const {
+    const double us = -unscale / ffw.scale;
+    double rr = 0.0;
+    for_groups([&](int loc, int, int) {
+      ff y[4];
+      stencil_ff(d, loc, ffw, loc, P.W, y);
+      if constexpr (!kMixed) {
+        ff yl[4];
+        stencil_ff(d + lo, loc, ffw, loc, P.W, yl);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = y[j] + yl[j];
+      }
+      V dv[4];
+      double xv[4], bv[4];
+      float di[4];
+      ldv(d, loc, dv);
+      load4(x + loc, xv);
+      load4(b + loc, bv);
+      dinv4(loc, di);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if constexpr (!kMixed) xv[j] = fma(widen(dv[j].l), unscale, xv[j]);
+        xv[j] = fma(widen(f32(dv[j])), unscale, xv[j]);
+        bv[j] = di[j] != 0.f ? fma(widen(y[j].l), us, fma(widen(y[j].h), us, bv[j])) : 0.0;
+        rr = fma(bv[j], bv[j], rr);
+      }
+      st4d(x, loc, xv);
+      st4d(b, loc, bv);
+    });
+    return rr;
+  }
 
-  // Solve (C/dt + K) x = b from the start in x (every row of x readable).
-  __device__ void solve(double* __restrict__ x, int step) {
+  // q = A z + beta q, p = z + beta p on the own rows (q = A z, p = z at the start); the local (p, q)
+  __device__ __forceinline__ V direction(bool start, const V& beta) {
+    V pq = V{};
+    auto update = [&](int loc, const V (&w)[4], const float (&zv)[4], const float (&di)[4]) {
+      V qv[4] = {V{}, V{}, V{}, V{}}, pv[4] = {V{}, V{}, V{}, V{}};
+      if (!start) {
+        ldv(q, loc, qv);
+        ldv(p, loc, pv);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        qv[j] = di[j] != 0.f ? vfma(beta, qv[j], w[j]) : V{};
+        pv[j] = vfma(beta, pv[j], zv[j]);
+        pq = vdot(pq, pv[j], qv[j]);
+      }
+      stv(q, loc, qv);
+      stv(p, loc, pv);
+    };
+    if constexpr (kMixed) {
+      if (P.mg_levels > 0 && piped(0)) {
+        const int W = P.W;
+        constexpr int NW = kElemWeights;
+        march<NW>(0, z, r0, r0 + R - 1,
+                 [&](const RowRef<NW>& rr, int y, int g, bool ok) {
+                   float vl[6], vm[6], vh[6], w[4], zv[4], di[4];
+                   rwin(rr.v(rr.so), g, G4, vl);
+                   rwin(rr.v(rr.sm), g, G4, vm);
+                   rwin(rr.v(rr.su), g, G4, vh);
+                   rstencil(rr, g, G4, vl, vm, vh, w);
+                   ld4f(rr.wd(rr.sm), kGroup * g, di);
+#pragma unroll
+                   for (int j = 0; j < 4; ++j) zv[j] = vm[j + 1];
+                   if (ok) update((y + 1) * W + kGroup * g, w, zv, di);
+                 },
+                 [](int) {});
+        return pq;
+      }
+    }
+    for_groups([&](int loc, int iy, int g) {
+      V w[4];
+      float zv[4], di[4];
+      if constexpr (!kMixed) {
+        stencil_ff(z, loc, ffw, loc, P.W, w);
+      } else if (P.mg_levels > 0) {
+        float zl[6], zm[6], zh[6];
+        lwindows(z, loc, P.W, zl, zm, zh);
+        lstencil(0, 6 * (iy + 1) * P.W + kGroup * g, zl, zm, zh, w);
+      } else {
+        stencil_elem32(z, P.w32, P.w32 + P.w32_stride, P.w32 + 2 * P.w32_stride, loc, P.W, w);
+      }
+      ld4f(z, loc, zv);
+      dinv4(loc, di);
+      update(loc, w, zv, di);
+    });
+    return pq;
+  }
+
+  // z = D^-1 r on a group; acc + (r, z)
+  __device__ __forceinline__ V jacobi(int loc, const V (&rv)[4], V acc) const {
+    float di[4], zv[4];
+    dinv4(loc, di);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      zv[j] = di[j] * f32(rv[j]);
+      acc = vdot(acc, rv[j], zv[j]);
+    }
+    st4f(z, loc, zv);
+    return acc;
+  }
+
+  // Solve (C/dt + K) x = b from the start in x (every row of x readable); b becomes the residual.
+  __device__ __forceinline__ void solve(double* __restrict__ x, int step) {
     double v2[2];
     residual(x, v2[0], v2[1]);
     allreduce<double, 2>(v2);
     const double bb = v2[0];
     double rr = v2[1];
     const double tol2 = P.rtol * P.rtol * bb;
+    const bool mg = P.mg_levels > 0;
     int sweeps = 0, its = 0;
     while (rr > tol2 && sweeps < P.refmax) {
-      const double nrm = sqrt(rr);
-      const Real scale = (Real)(1.0 / nrm);
-      const Real target2 = (Real)fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr);
-      // r /= ||r||, z = M^-1 r, d = p = q = 0; (r, z)
-      const bool mg = P.mg_levels > 0;
-      Real a[1] = {Real(0)};
-      for_groups([&](int loc, int, int) {
-        Real rv[4], di[4], zv[4], zero[4] = {Real(0), Real(0), Real(0), Real(0)};
-        ld4(r, loc, rv);
-        dinv4(loc, di);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          rv[j] *= scale;
-          zv[j] = di[j] * rv[j];
-          a[0] = fma(rv[j], zv[j], a[0]);
-        }
-        st4(r, loc, rv);
-        if (!mg) st4(z, loc, zv);
-        st4(d, loc, zero);
-        st4(p, loc, zero);
-        st4(q, loc, zero);
-      });
-      if (mg) {
-        comm.sync();
-        a[0] = vcycle();
-      }
-      allreduce<Real, 1>(a);
-      Real rz = a[0], beta = Real(0);
-      int it = 0;
-      bool done = !(Real(1) > target2);
-      while (!done && it < P.itmax) {
-        // q = A z + beta q, p = z + beta p, (p, q); alpha = rz / (p, q)
-        Real pq[1] = {Real(0)};
-        for_groups([&](int loc, int, int) {
-          Real w[4], qv[4], pv[4], zv[4], di[4];
-          apply_z(loc, w);
-          ld4(q, loc, qv);
-          ld4(p, loc, pv);
-          ld4(z, loc, zv);
-          dinv4(loc, di);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            qv[j] = di[j] != Real(0) ? fma(beta, qv[j], w[j]) : Real(0);
-            pv[j] = fma(beta, pv[j], zv[j]);
-            pq[0] = fma(pv[j], qv[j], pq[0]);
-          }
-          st4(q, loc, qv);
-          st4(p, loc, pv);
-        });
-        const Real rz_c = rz;
-        allreduce<Real, 1>(pq, [rz_c](Real* t) { t[0] = rz_c / t[0]; });
-        const Real alpha = pq[0];
-        // d += alpha p, r -= alpha q, z = D^-1 r; (r, z), (r, r), beta = (r, z)_new / (r, z)
-        Real v[3] = {Real(0), Real(0), Real(0)};
-        for_group_pairs([&](const int (&loc)[2], const bool (&ok)[2]) {
-          Real dv[2][4], pv[2][4], rv[2][4], qv[2][4], di[2][4];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            if (!ok[u]) continue;
-            ld4(d, loc[u], dv[u]);
-            ld4(p, loc[u], pv[u]);
-            ld4(r, loc[u], rv[u]);
-            ld4(q, loc[u], qv[u]);
-            dinv4(loc[u], di[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            if (!ok[u]) continue;
-            Real zv[4];
+      // r / 2^k of squared norm in [1, 4)
+      const int k2 = (((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1;
+      const double rr0 = rr * exp2_int(-k2) * exp2_int(-k2);
+      const float target2 = fmaxf((float)(fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr) * rr0), 1e-30f);
+      V rz = V{}, beta = V{};
+      int it = -1;                     // -1: the start, whose z and (r, z) open the iteration
+      bool done = !((float)rr0 > target2);
+      const bool none = done;
+      for (;;) {
+        V v[3] = {V{}, V{}, V{}};
+        const bool start = it < 0;
+        if (start) {
+          for_groups([&](int loc, int, int) {
+            double bv[4];
+            V rv[4];
+            load4(b + loc, bv);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              dv[u][j] = fma(alpha, pv[u][j], dv[u][j]);
-              rv[u][j] = fma(-alpha, qv[u][j], rv[u][j]);
-              zv[j] = di[u][j] * rv[u][j];
-              if (!mg) v[0] = fma(rv[u][j], zv[j], v[0]);
-              v[1] = fma(rv[u][j], rv[u][j], v[1]);
+              const ff s = split_scaled(bv[j], -k2);
+              if constexpr (kMixed)
+                rv[j] = s.h + s.l;
+              else
+                rv[j] = s;
             }
-            st4(d, loc[u], dv[u]);
-            st4(r, loc[u], rv[u]);
-            if (!mg) st4(z, loc[u], zv);
-          }
-        });
+            stv(r, loc, rv);
+            if (!mg) v[0] = jacobi(loc, rv, v[0]);
+          });
+        } else {
+          // alpha = rz / (p, q)
+          V pq[1] = {direction(it == 0, beta)};
+          const V rz_c = rz;
+          allreduce<V, 1>(pq, [rz_c](V* t) { t[0] = vdiv(rz_c, t[0]); });
+          const V alpha = pq[0], nalpha = vneg(alpha);
+          // d += alpha p (d = alpha p at first), r -= alpha q; (r, r)
+          const bool first = it == 0;
+          for_group_pairs([&](const int (&loc)[2], const bool (&ok)[2]) {
+            V dv[2][4], pv[2][4], rv[2][4], qv[2][4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              if (!ok[u]) continue;
+#pragma unroll
+              for (int j = 0; j < 4; ++j) dv[u][j] = V{};
+              if (!first) ldv(d, loc[u], dv[u]);
+              ldv(p, loc[u], pv[u]);
+              ldv(r, loc[u], rv[u]);
+              ldv(q, loc[u], qv[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              if (!ok[u]) continue;
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                dv[u][j] = vfma(alpha, pv[u][j], dv[u][j]);
+                rv[u][j] = vfma(nalpha, qv[u][j], rv[u][j]);
+                v[1] = vdot(v[1], rv[u][j], rv[u][j]);
+              }
+              stv(d, loc[u], dv[u]);
+              stv(r, loc[u], rv[u]);
+              if (!mg) v[0] = jacobi(loc[u], rv[u], v[0]);
+            }
+          });
+        }
+        // z = M^-1 r; (r, z), (r, r), beta = (r, z)_new / (r, z)
         if (mg) {
-          comm.sync();
+          sync();
           v[0] = vcycle();
         }
-        allreduce<Real, 2, 1>(v, [rz_c](Real* t) { t[2] = t[0] / rz_c; });
+        const V rz_c = rz;
+        allreduce<V, 2, 1>(v, [rz_c, start](V* t) { if (!start) t[2] = vdiv(t[0], rz_c); });
         ++it;
-        if (!(v[1] > target2)) done = true;   // NaN keeps iterating until the limit
+        if (!start && !(f32(v[1]) > target2)) done = true;   // NaN keeps iterating until the limit
         beta = v[2];
         rz = v[0];
+        if (done || it >= P.itmax) break;
       }
       its += it;
       ++sweeps;
-      // x += ||r|| d on the own rows, then the FP64 residual of the whole system
-      for_groups([&](int loc, int, int) {
-        double xv[4];
-        Real dv[4];
-        load4(x + loc, xv);
-        ld4(d, loc, dv);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xv[j] = fma((double)dv[j], nrm, xv[j]);
-        st4d(x, loc, xv);
-      });
-      comm.sync();
-      residual(x, v2[0], v2[1]);
-      double w1[1] = {v2[1]};
+      if (none) break;                             // no iteration: there is no d
+      const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
+      double w1[1] = {update_residual(x, unscale)};
       allreduce<double, 1>(w1);
       rr = w1[0];
     }
@@ -711,11 +972,34 @@ struct Streamer {
     return (P.objective == PTG_OBJ_MODIFIED ? P.p : pow(Theta, 1.0 - P.p)) / (double)P.Ne;
   }
 
+  // (C/dt) x on a group: without weights where the capacity is uniform (see Stepper::mass_dt)
+  __device__ __forceinline__ void mass_dt(const double* __restrict__ x, int loc, int iy, int g, double (&y)[4]) const {
+    if (P.has_dc) {
+      stencil_node64<double>(x, loc, P.mass, loc, P.W, y);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) y[j] *= inv_dt;
+      return;
+    }
+    const double dy = iy == 0 || iy == P.ny ? 2.0 : 4.0, s = P.mass_uniform * inv_dt;
+    double xl[6], xm[6], xh[6];
+    load_window(x, loc - P.W, xl);
+    load_window(x, loc, xm);
+    load_window(x, loc + P.W, xh);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) xm[i] = fma(dy, xm[i], xl[i] + xh[i]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int ix = kGroup * g - 1 + j;
+      const double dx = ix == 0 || ix == P.nx ? 2.0 : 4.0;
+      y[j] = s * fma(dx, xm[j + 1], xm[j] + xm[j + 2]);
+    }
+  }
+
   // b = (C/dt) xp + src(node) on the own rows; xn = the start of the step: the extrapolation
   // through xp and the ring rows X[0..n-2] (n = 1: xp itself); the ring row wr receives xp.
   // The ring rows are padded node rows 0 .. ny; pads and Dirichlet nodes are zero in every state.
   template <class Src>
-  __device__ void begin_step(const double* __restrict__ xp, double* __restrict__ xn, int n, const double* const* X,
+  __device__ __forceinline__ void begin_step(const double* __restrict__ xp, double* __restrict__ xn, int n, const double* const* X,
                              double* __restrict__ wr, Src src) {
     for_groups([&](int loc, int iy, int g) {
       double y[4], x1[4], bv[4], xv[4], a[4], b_[4], c[4];
@@ -724,12 +1008,12 @@ struct Streamer {
       if (n >= 2) load4(X[0] + o, a);
       if (n >= 3) load4(X[1] + o, b_);
       if (n >= 4) load4(X[2] + o, c);
-      stencil_node64<double>(xp, loc, P.mass, loc, P.W, y);
+      mass_dt(xp, loc, iy, g, y);
       if (wr) st4d(wr, o, x1);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int gi = gnode(iy, g, j);
-        bv[j] = gi < 0 || P.dirichlet[gi] ? 0.0 : fma(y[j], inv_dt, src(gi));
+        bv[j] = gi < 0 || P.dirichlet[gi] ? 0.0 : y[j] + src(gi);
         if (n <= 1)
           xv[j] = x1[j];
         else if (n == 2)
@@ -768,14 +1052,19 @@ struct Streamer {
     });
   }
 
-  __device__ double pnorm_p(const double* __restrict__ x) {
+  // sum of x^p over the nodes; x is stored to the node vector dst (if given) in the same pass
+  __device__ __forceinline__ double pnorm_store(const double* __restrict__ x, double* __restrict__ dst) {
     double v[1] = {0.0};
     for_groups([&](int loc, int iy, int g) {
       double xv[4];
       load4(x + loc, xv);
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (gnode(iy, g, j) >= 0) v[0] += ipow(xv[j], P.p_int);   // 0 on Dirichlet nodes
+      for (int j = 0; j < 4; ++j) {
+        const int gi = gnode(iy, g, j);
+        if (gi < 0) continue;
+        v[0] += ipow(xv[j], P.p_int);   // 0 on Dirichlet nodes
+        if (dst) dst[gi] = xv[j];
+      }
     });
     allreduce<double, 1>(v);
     return v[0];
@@ -784,7 +1073,7 @@ struct Streamer {
   // Eq. 4.7 element sums of the own element rows (rows r0 .. r0 + R - 1 below ny); lam padded,
   // Tj and Tjm node vectors
   // (the gsrc row is 0 if null; addF - subG is added if given)
-  __device__ void accumulate_g(const double* __restrict__ lam, const double* __restrict__ Tj,
+  __device__ __forceinline__ void accumulate_g(const double* __restrict__ lam, const double* __restrict__ Tj,
                                const double* __restrict__ Tjm, const double* __restrict__ gsrc,
                                double* __restrict__ gdst, double nnorm, const double* __restrict__ addF = nullptr,
                                const double* __restrict__ subG = nullptr) const {
@@ -813,14 +1102,14 @@ struct Streamer {
 
   // b = (C/dt) xp + src(node) on the own rows (xp padded, every row visible), 0 off the unknowns
   template <class Src>
-  __device__ void build_rhs(const double* __restrict__ xp, Src src) {
+  __device__ __forceinline__ void build_rhs(const double* __restrict__ xp, Src src) {
     for_groups([&](int loc, int iy, int g) {
       double y[4], bv[4];
-      stencil_node64<double>(xp, loc, P.mass, loc, P.W, y);
+      mass_dt(xp, loc, iy, g, y);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int gi = gnode(iy, g, j);
-        bv[j] = (gi < 0 || P.dirichlet[gi]) ? 0.0 : fma(y[j], inv_dt, src(gi));
+        bv[j] = (gi < 0 || P.dirichlet[gi]) ? 0.0 : y[j] + src(gi);
       }
       st4d(b, loc, bv);
     });
@@ -829,7 +1118,7 @@ struct Streamer {
   // extrapolation of the last m (1..3) increments of the correction sweep (as the stepper's
   // load_x64_increment): d_i = X_i - Fm[i], X_0 = xc (padded, the state the step propagates),
   // X_1, X_2 node vectors of earlier corrected states; inc = d0, 2 d0 - d1 or 3 (d0 - d1) + d2
-  __device__ void load_increment(const double* __restrict__ Gs, int m, const double* const* Fm,
+  __device__ __forceinline__ void load_increment(const double* __restrict__ Gs, int m, const double* const* Fm,
                                  const double* const* X, const double* __restrict__ xc,
                                  double* __restrict__ x) const {
     for_groups([&](int loc, int iy, int g) {
@@ -853,7 +1142,7 @@ struct Streamer {
   }
   // Parareal correction (Eq. 4.9 / 4.14): x = xs + Fs - Gs on the own rows into the padded x and
   // the node vectors X (and Y if given); 0 off the unknowns
-  __device__ void correction(const double* __restrict__ xs, const double* __restrict__ Fs,
+  __device__ __forceinline__ void correction(const double* __restrict__ xs, const double* __restrict__ Fs,
                              const double* __restrict__ Gs, double* __restrict__ x, double* __restrict__ X,
                              double* __restrict__ Y) const {
     for_groups([&](int loc, int iy, int g) {
@@ -879,7 +1168,7 @@ struct Streamer {
   }
 
   // ------------------------------------------------------------------ task bodies
-  __device__ void fine_primal(int task) {
+  __device__ __forceinline__ void fine_primal(int task) {
     const int s = P.s0 + task;
     const int M = P.M;
     const double inv_norm = 1.0 / ((double)P.Nt * (double)P.Ne);
@@ -887,7 +1176,8 @@ struct Streamer {
     double* x_cur = xb;
     load(P.in_field + (size_t)s * P.Nn, x_prev);
     comm.sync();
-    double theta = P.in_aux[s];
+    const bool power = P.objective != PTG_OBJ_MODIFIED;   // (see the stepper: one root per slice)
+    double theta = power ? ipow(P.in_aux[s], P.p_int) : P.in_aux[s];
     const int nring = P.extrap;
     double* ring = nring > 1 && P.prev_field ? P.prev_field + (size_t)task * nring * P.ring_stride : nullptr;
     int saved = 0;
@@ -904,18 +1194,16 @@ struct Streamer {
       }
       begin_step(x_prev, x_cur, n, X, wr, [&](int g) { return qj * P.fload[g]; });
       solve(x_cur, j);
-      const double sp = pnorm_p(x_cur);
-      if (threadIdx.x == 0) theta = accumulate_theta(theta, sp * inv_norm);
-      store(x_cur, hist_row(j));
+      theta = fma(pnorm_store(x_cur, hist_row(j)), inv_norm, theta);
       double* t = x_prev;
       x_prev = x_cur;
       x_cur = t;
     }
     store(x_prev, P.out_field + (size_t)s * P.Nn);
-    if (threadIdx.x == 0 && rank == 0) P.out_aux[s] = theta;
+    if (threadIdx.x == 0 && rank == 0) P.out_aux[s] = power ? pow(theta, 1.0 / P.p) : theta;
   }
 
-  __device__ void fine_adjoint(int task) {
+  __device__ __forceinline__ void fine_adjoint(int task) {
     const int s = P.s0 + task;
     const int M = P.M;
     const double scale = adjoint_scale(*P.Theta);
@@ -957,7 +1245,7 @@ struct Streamer {
   }
 
   // G_pri of slice s (one step of size dtau from u_s, started from the guess u_{s+1})
-  __device__ void coarse_primal(int task) {
+  __device__ __forceinline__ void coarse_primal(int task) {
     const int s = P.s0 + task;
     const int j = P.M * (s + 1);
     load(P.in_field + (size_t)s * P.Nn, xa);
@@ -972,14 +1260,13 @@ struct Streamer {
     load(P.in_field + (size_t)(P.guess_next ? s + 1 : s) * P.Nn, xb);
     comm.sync();
     solve(xb, j);
-    const double sp = pnorm_p(xb);
-    store(xb, P.out_field + (size_t)s * P.Nn);
+    const double sp = pnorm_store(xb, P.out_field + (size_t)s * P.Nn);
     if (threadIdx.x == 0 && rank == 0)
       P.out_aux[s] = accumulate_theta(P.in_aux[s], sp / ((double)P.Ntau * (double)P.Ne));
   }
 
   // G_adj of slice s; src_mode 1 / 2 one of its two Theta-free parts (as the stepper)
-  __device__ void coarse_adjoint(int task) {
+  __device__ __forceinline__ void coarse_adjoint(int task) {
     const int s = P.s0 + task;
     const int kidx = P.M * s + 1;
     const int kprev = max(kidx - P.M, 0);
@@ -1006,7 +1293,7 @@ struct Streamer {
   }
 
   // Eq. 4.9 forward correction sweep (one task): u_{s+1} = G(u_s) + F[s] - G_old[s]
-  __device__ void correct_primal() {
+  __device__ __forceinline__ void correct_primal() {
     double theta;
     if (P.in_field) {                           // u_0 taken from the guess states, copied to X[0]
       load(P.in_field, xa);
@@ -1051,7 +1338,7 @@ struct Streamer {
       }
       comm.sync();
       solve(xb, j);
-      const double sp = pnorm_p(xb);
+      const double sp = pnorm_store(xb, nullptr);
       correction(xb, P.F_field + (size_t)s * P.Nn, P.G_field + (size_t)s * P.Nn, xa,
                  P.out_field + (size_t)(s + 1) * P.Nn, hist_row(j));
       if (threadIdx.x == 0) {
@@ -1064,7 +1351,7 @@ struct Streamer {
   }
 
   // Eq. 4.14 reverse correction sweep (one task): v_s = G(v_{s+1}) + F[s] - G_old[s], v_Ntau = 0
-  __device__ void correct_adjoint() {
+  __device__ __forceinline__ void correct_adjoint() {
     const double scale = adjoint_scale(*P.Theta);
     const int er = min(R, P.ny - r0);
     const int ne_own = er > 0 ? er * P.nx : 0;
@@ -1120,15 +1407,21 @@ struct Streamer {
   }
 };
 
-constexpr int kStreamThreads = 512;   // one CTA per SM, 128 registers per thread
-
 // ngroups groups of P.cs CTAs; group g runs tasks g, g + ngroups, ... < P.wide_tasks (the
 // correction sweeps are one task).
 template <class Real, int KIND>
 __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_constant__ StepParams P) {
+  extern __shared__ __align__(128) float stream_smem[];
   __shared__ RedSmem rs;
+  __shared__ unsigned long long ring_bar[kPipeRows];
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kPipeRows; ++i) mbar_init(&ring_bar[i]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  unsigned ring_phase = 0;
   GridComm comm(P, rs);
-  Streamer<Real, KIND> st(P, comm);
+  Streamer<Real, KIND> st(P, comm, stream_smem, ring_bar, ring_phase);
   const int ngroups = (int)gridDim.x / P.cs;
   for (int task = comm.gid; task < P.wide_tasks; task += ngroups) {
     if constexpr (KIND == KIND_FINE_PRI) st.fine_primal(task);
