@@ -1,7 +1,7 @@
 """Build the CUDA library ``libptg.so`` (sm_103a) in-tree.
 
-The stepper is compiled once per (precision, task kind) pair so the translation units
-build in parallel; the objects are linked with the assembly kernels and the C ABI layer
+The stepper is compiled once per (precision, task kind, range of groups per thread) so the
+translation units build in parallel; the objects are linked with the assembly kernels and the C ABI layer
 into ``paper_2411_19030_gb300/libptg.so``.  Objects go to ``paper_2411_19030_gb300/_build``.
 A rebuild happens only when a source or header is newer than the library.
 
@@ -45,9 +45,11 @@ def _units() -> list[tuple[str, list[str], str]]:
     units = []
     for tag, real in (("f32", "float"), ("f64", "double")):
         for kind in range(6):
-            units.append((os.path.join(CSRC, "stepper_inst.cu"),
-                          [f"-DPTG_REAL={real}", f"-DPTG_TAG={tag}", f"-DPTG_KIND={kind}"],
-                          f"stepper_{tag}_k{kind}.o"))
+            for part, first in (("lo", 1), ("hi", 4)):
+                units.append((os.path.join(CSRC, "stepper_inst.cu"),
+                              [f"-DPTG_REAL={real}", f"-DPTG_TAG={tag}", f"-DPTG_KIND={kind}", f"-DPTG_SET={part}",
+                               f"-DPTG_FIRST_NG={first}"],
+                              f"stepper_{tag}_k{kind}_{part}.o"))
     for kind in range(6):
         units.append((os.path.join(CSRC, "stream_inst.cu"), [f"-DPTG_KIND={kind}"], f"stream_k{kind}.o"))
     for name in ("plan.cu", "assemble.cu", "coarse.cu", "api.cu", "noalloc.cu", "design.cu", "mesh.cu", "stream.cu",

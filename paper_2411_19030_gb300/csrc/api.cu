@@ -330,21 +330,25 @@ long best_plan(ptg_op* op, int precision, int kind, int ntasks, int tl_mode, Pla
     for (int ng : kStepNG) {
       const int nthreads = step_threads(op, kind, cs, ng, groups, tl_mode);
       if (nthreads > kStepMaxThreadsHost) continue;
-      Plan p;
-      cudaError_t e = query_stepper_plan(nx, ny, precision, kind, cs, ng, nthreads,
-                                         twolevel_bytes(op, precision, kind, cs, tl_mode), &p, keep_ax);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        continue;
-      }
-      if (p.max_active_clusters <= 0) continue;
-      const long waves = (ntasks + p.max_active_clusters - 1) / p.max_active_clusters;
-      if (best_waves < 0 || waves < best_waves || (waves == best_waves && ng < out->ng)) {
-        p.twolevel = twolevel_rows(op, precision, kind, cs, tl_mode) > 0;
-        p.vc = p.twolevel && uses_vcycle(op, tl_mode);
-        p.l3 = p.twolevel && uses_three(op, tl_mode);
-        *out = p;
-        best_waves = waves;
+      // the kernel with more registers unless they cost a wave (200 x 150, 24 slices: 14 clusters
+      // of 16 CTAs at a time without it and 7 with it, 10.6 against 16 ms)
+      for (bool narrow : {true, false}) {
+        Plan p;
+        cudaError_t e = query_stepper_plan(nx, ny, precision, kind, cs, ng, nthreads,
+                                           twolevel_bytes(op, precision, kind, cs, tl_mode), &p, keep_ax, narrow);
+        if (e != cudaSuccess) {
+          cudaGetLastError();
+          continue;
+        }
+        if (p.max_active_clusters <= 0) continue;
+        const long waves = (ntasks + p.max_active_clusters - 1) / p.max_active_clusters;
+        if (best_waves < 0 || waves < best_waves || (waves == best_waves && ng < out->ng)) {
+          p.twolevel = twolevel_rows(op, precision, kind, cs, tl_mode) > 0;
+          p.vc = p.twolevel && uses_vcycle(op, tl_mode);
+          p.l3 = p.twolevel && uses_three(op, tl_mode);
+          *out = p;
+          best_waves = waves;
+        }
       }
     }
   }
@@ -484,7 +488,8 @@ int choose_plan(ptg_op* op, int precision, int kind, int ntasks, Plan* out) {
     std::snprintf(g_last_error, sizeof(g_last_error), "no launch plan fits a %dx%d grid", op->g.nx, op->g.ny);
     return PTG_EINVAL;
   }
-  const Plan best = wt >= 0 ? two : jac;
+  Plan best = wt >= 0 ? two : jac;
+  if (spread_plan(precision, kind, ntasks, &best) != cudaSuccess) cudaGetLastError();
   op->plans[key] = best;
   *out = best;
   return PTG_OK;
@@ -1153,13 +1158,14 @@ int ptg_op_set_plan(ptg_op* op, int kind, int cs, int ng) {
     if (nthreads > kStepMaxThreadsHost) continue;
     for (bool keep_ax : {true, false}) {
       Plan p;
-      cudaError_t e = query_stepper_plan(op->g.nx, op->g.ny, prec, kind, cs, ng, nthreads,
-                                         twolevel_bytes(op, prec, kind, cs, mode), &p,
-                                         keep_ax && uses_saved_ax(op, kind));
-      if (e != cudaSuccess) {
+      cudaError_t e = cudaErrorInvalidConfiguration;
+      for (bool narrow : {true, false}) {
+        e = query_stepper_plan(op->g.nx, op->g.ny, prec, kind, cs, ng, nthreads,
+                               twolevel_bytes(op, prec, kind, cs, mode), &p, keep_ax && uses_saved_ax(op, kind), narrow);
+        if (e == cudaSuccess) break;
         cudaGetLastError();
-        continue;
       }
+      if (e != cudaSuccess) continue;
       if (p.max_active_clusters <= 0) continue;
       p.twolevel = mode > TL_NONE;
       p.vc = uses_vcycle(op, mode);

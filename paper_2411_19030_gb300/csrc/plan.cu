@@ -72,7 +72,7 @@ cudaError_t launch_stepper(const StepParams& P, const Plan& plan, int precision,
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, P);
   }
-  StepKernel k = stepper_kernel_for(precision, P.kind, plan.ng);
+  StepKernel k = stepper_kernel_for(precision, P.kind, plan.ng, plan.narrow);
   if (!k) return cudaErrorInvalidConfiguration;
   cudaError_t e = configure((const void*)k, plan.cs, plan.smem);
   if (e != cudaSuccess) return e;
@@ -106,8 +106,9 @@ static cudaError_t occupancy(const void* k, int cs, int nthreads, size_t smem, i
 }
 
 cudaError_t query_stepper_plan(int nx, int ny, int precision, int kind, int cs, int ng, int nthreads, size_t extra_smem,
-                               Plan* plan, bool keep_ax) {
-  StepKernel k = stepper_kernel_for(precision, kind, ng);
+                               Plan* plan, bool keep_ax, bool narrow) {
+  StepKernel k = stepper_kernel_for(precision, kind, ng, narrow);
+  if (narrow && nthreads > kStepNarrowThreads) return cudaErrorInvalidConfiguration;
   if (!k || nthreads < 32 || nthreads > kStepMaxThreadsHost || nthreads % 32) return cudaErrorInvalidConfiguration;
   plan->cs = cs;
   plan->nthreads = nthreads;
@@ -115,12 +116,35 @@ cudaError_t query_stepper_plan(int nx, int ny, int precision, int kind, int cs, 
   plan->rmax = (ny + 1 + cs - 1) / cs;
   plan->smem = stepper_smem_bytes(nx, plan->rmax, precision == PTG_FP32_REFINE ? 4 : 8, keep_ax) + extra_smem;
   plan->keep_ax = keep_ax;
+  plan->narrow = narrow;
   plan->max_active_clusters = 0;
   if (plan->smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   int n = 0;
   cudaError_t e = occupancy((const void*)k, cs, nthreads, plan->smem, &n);
   plan->max_active_clusters = n;
   return e;
+}
+
+// One CTA of shared memory size s takes s + its static and reserved part of the SM's 228 KB; this size
+// leaves room for k CTAs and not for k + 1.
+static size_t smem_for_residents(int k) { return 233472 / (size_t)(k + 1) - 3072; }
+
+cudaError_t spread_plan(int precision, int kind, int ntasks, Plan* plan) {
+  StepKernel k = stepper_kernel_for(precision, kind, plan->ng, plan->narrow);
+  if (!k) return cudaErrorInvalidConfiguration;
+  for (int per_sm = 1; per_sm <= 4; ++per_sm) {
+    const size_t smem = smem_for_residents(per_sm);
+    if (smem <= plan->smem) return cudaSuccess;        // its own size bounds it already
+    int n = 0;
+    cudaError_t e = occupancy((const void*)k, plan->cs, plan->nthreads, smem, &n);
+    if (e != cudaSuccess) return e;
+    if (n >= ntasks) {
+      plan->smem = smem;
+      plan->max_active_clusters = n;
+      return cudaSuccess;
+    }
+  }
+  return cudaSuccess;
 }
 
 cudaError_t query_wide_plan(int nx, int ny, int precision, int kind, int ntasks, bool spread,

@@ -311,6 +311,7 @@ struct Plan {
   bool vc = false;           // ... in the V(1,1) cycle form (else additive)
   bool l3 = false;           // ... as the three-level cycle
   bool keep_ax = true;       // the saved A x of the last residual is in smem
+  bool narrow = false;       // the kernel for blocks of at most kStepNarrowThreads threads
   bool wide = false;         // one task over a cooperative grid of cs CTAs (GridComm), no clusters
   bool stream = false;       // fine kinds: the streamed propagator (stream.cuh), cs CTAs per slice
 };
@@ -333,7 +334,11 @@ cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A,
 // device; later calls with no larger footprint make no attribute call.
 cudaError_t configure_kernel(const void* k, size_t smem, bool cluster);
 cudaError_t query_stepper_plan(int nx, int ny, int precision, int kind, int cs, int ng, int nthreads, size_t extra_smem,
-                               Plan* plan, bool keep_ax = true);
+                               Plan* plan, bool keep_ax, bool narrow);
+// Raises a cluster plan's shared memory to the size that lets the fewest CTAs share an SM with which
+// all ntasks clusters still run at once: the hardware packs the CTAs of a cluster onto SMs as long
+// as they fit, and leaves other SMs idle.
+cudaError_t spread_plan(int precision, int kind, int ntasks, Plan* plan);
 // Plan of the grid-wide variant.  spread: one system over as many CTAs as there are SMs (rmax
 // >= 2 rows each); otherwise the fewest CTAs per group whose slabs fit, and as many groups as
 // fit the chip (plan.max_active_clusters = groups, at most ntasks).  extra_smem(G) gives the

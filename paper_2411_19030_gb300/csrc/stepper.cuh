@@ -1761,6 +1761,9 @@ struct Stepper {
 // body, which keeps register pressure and compile time down.  Up to 512 threads per CTA (the
 // plan picks the block size), at most 128 registers per thread.
 constexpr int kStepMaxThreads = 512;
+// Blocks of at most kStepNarrowThreads threads run a second instantiation of the same kernel that
+// may use 168 registers: at 128 the CG of the FP32 kinds with two or three groups per thread and the
+// three-level cycle spill (up to 750 bytes a thread).
 
 template <int KIND>
 constexpr bool kCoarseStep = KIND != KIND_FINE_PRI && KIND != KIND_FINE_ADJ;
@@ -1775,8 +1778,8 @@ __device__ __forceinline__ void run_task(Stepper<Real, NG, Comm, kCoarseStep<KIN
   if constexpr (KIND == KIND_CORRECT_ADJ) st.correct_adjoint();
 }
 
-template <class Real, int NG, int KIND>
-__global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_kernel(const __grid_constant__ StepParams P) {
+template <class Real, int NG, int KIND, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) stepper_kernel(const __grid_constant__ StepParams P) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   __shared__ RedSmem rs;
   ClusterComm comm(rs);

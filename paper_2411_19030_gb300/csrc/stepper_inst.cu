@@ -1,5 +1,5 @@
 // stepper_inst.cu -- instantiates the cluster stepper for one precision and one task kind.
-// Compiled once per (PTG_REAL, PTG_KIND) pair so the kernels build in parallel:
+// Compiled once per (PTG_REAL, PTG_KIND, PTG_SET) so the kernels build in parallel:
 //   PTG_REAL = float (FP32 CG + FP64 refinement) or double (FP64 CG); PTG_KIND = 0..5.
 #include "stepper.cuh"
 #include "stepper_launch.cuh"
@@ -14,10 +14,16 @@
 #error "define PTG_TAG (f32 or f64)"
 #endif
 
-#define PTG_CAT3(a, b, c) a##_##b##_##c
-#define PTG_SELECT_NAME(tag, kind) PTG_CAT3(stepper_select, tag, kind)
+#if !defined(PTG_SET) || !defined(PTG_FIRST_NG)
+#error "define PTG_SET and PTG_FIRST_NG (lo and 1: NG 1..3; hi and 4: NG 4..6)"
+#endif
+
+#define PTG_CAT4(a, b, c, d) a##_##b##_##c##_##d
+#define PTG_SELECT_NAME(tag, kind, set) PTG_CAT4(stepper_select, tag, kind, set)
 
 namespace ptg {
+
+namespace {   // every unit has its own
 
 // The grid-wide (grouped) variant exists for every kind and precision, for up to 3 groups
 // per thread.
@@ -27,20 +33,26 @@ StepKernel wide_kernel() {
   else return nullptr;
 }
 
-StepKernels PTG_SELECT_NAME(PTG_TAG, PTG_KIND)(int ng) {
-#define PTG_PAIR(NG_)                                                                                   \
-  StepKernels{&stepper_kernel<PTG_REAL, NG_, PTG_KIND>, &stepper_batch_kernel<PTG_REAL, NG_, PTG_KIND>, \
-              wide_kernel<NG_>()}
-  switch (ng) {
-    case 1: return PTG_PAIR(1);
-    case 2: return PTG_PAIR(2);
-    case 3: return PTG_PAIR(3);
-    case 4: return PTG_PAIR(4);
-    case 5: return PTG_PAIR(5);
-    case 6: return PTG_PAIR(6);
-    default: return StepKernels{nullptr, nullptr, nullptr};
+template <int NG>
+StepKernels kernels() {
+  if constexpr (NG <= 3)
+    return StepKernels{&stepper_kernel<PTG_REAL, NG, PTG_KIND, kStepMaxThreads>,
+                       &stepper_kernel<PTG_REAL, NG, PTG_KIND, kStepNarrowThreads>,
+                       &stepper_batch_kernel<PTG_REAL, NG, PTG_KIND>, wide_kernel<NG>()};
+  else
+    return StepKernels{&stepper_kernel<PTG_REAL, NG, PTG_KIND, kStepMaxThreads>, nullptr,
+                       &stepper_batch_kernel<PTG_REAL, NG, PTG_KIND>, nullptr};
+}
+
+}  // namespace
+
+StepKernels PTG_SELECT_NAME(PTG_TAG, PTG_KIND, PTG_SET)(int ng) {
+  switch (ng - PTG_FIRST_NG) {
+    case 0: return kernels<PTG_FIRST_NG>();
+    case 1: return kernels<PTG_FIRST_NG + 1>();
+    case 2: return kernels<PTG_FIRST_NG + 2>();
+    default: return StepKernels{nullptr, nullptr, nullptr, nullptr};
   }
-#undef PTG_PAIR
 }
 
 }  // namespace ptg

@@ -8,6 +8,7 @@ using StepKernel = void (*)(const StepParams);
 using BatchKernel = void (*)(const StepParams*, const int2*, int, int*);
 struct StepKernels {
   StepKernel single;
+  StepKernel narrow;    // the same for blocks of at most kStepNarrowThreads threads, with more registers each
   BatchKernel batch;
   StepKernel wide;      // grid-wide variant (FP64, single-task kinds, NG <= 3), else null
 };
@@ -17,9 +18,12 @@ struct StepKernels {
 constexpr int kStepNG[] = {1, 2, 3, 4, 5, 6};
 constexpr int kNumStepNG = sizeof(kStepNG) / sizeof(kStepNG[0]);
 constexpr int kStepMaxThreadsHost = 512;
+constexpr int kStepNarrowThreads = 384;
 
 // Defined by the per-(precision, kind) translation units.
-#define PTG_DECLARE_SELECT(P, K) StepKernels stepper_select_##P##_##K(int ng);
+#define PTG_DECLARE_SELECT(P, K) \
+  StepKernels stepper_select_##P##_##K##_lo(int ng); /* ng 1..3 */ \
+  StepKernels stepper_select_##P##_##K##_hi(int ng); /* ng 4..6 */
 PTG_DECLARE_SELECT(f32, 0) PTG_DECLARE_SELECT(f32, 1) PTG_DECLARE_SELECT(f32, 2)
 PTG_DECLARE_SELECT(f32, 3) PTG_DECLARE_SELECT(f32, 4) PTG_DECLARE_SELECT(f32, 5)
 PTG_DECLARE_SELECT(f64, 0) PTG_DECLARE_SELECT(f64, 1) PTG_DECLARE_SELECT(f64, 2)
@@ -28,16 +32,19 @@ PTG_DECLARE_SELECT(f64, 3) PTG_DECLARE_SELECT(f64, 4) PTG_DECLARE_SELECT(f64, 5)
 
 inline StepKernels stepper_kernels_for(int precision, int kind, int ng) {
   const bool f32 = precision == PTG_FP32_REFINE;
+#define PTG_PICK(K)                                                                       \
+  case K:                                                                                 \
+    return f32 ? (ng <= 3 ? stepper_select_f32_##K##_lo(ng) : stepper_select_f32_##K##_hi(ng)) \
+               : (ng <= 3 ? stepper_select_f64_##K##_lo(ng) : stepper_select_f64_##K##_hi(ng))
   switch (kind) {
-    case 0: return f32 ? stepper_select_f32_0(ng) : stepper_select_f64_0(ng);
-    case 1: return f32 ? stepper_select_f32_1(ng) : stepper_select_f64_1(ng);
-    case 2: return f32 ? stepper_select_f32_2(ng) : stepper_select_f64_2(ng);
-    case 3: return f32 ? stepper_select_f32_3(ng) : stepper_select_f64_3(ng);
-    case 4: return f32 ? stepper_select_f32_4(ng) : stepper_select_f64_4(ng);
-    case 5: return f32 ? stepper_select_f32_5(ng) : stepper_select_f64_5(ng);
-    default: return StepKernels{nullptr, nullptr, nullptr};
+    PTG_PICK(0); PTG_PICK(1); PTG_PICK(2); PTG_PICK(3); PTG_PICK(4); PTG_PICK(5);
+    default: return StepKernels{nullptr, nullptr, nullptr, nullptr};
   }
+#undef PTG_PICK
 }
-inline StepKernel stepper_kernel_for(int precision, int kind, int ng) { return stepper_kernels_for(precision, kind, ng).single; }
+inline StepKernel stepper_kernel_for(int precision, int kind, int ng, bool narrow) {
+  const StepKernels k = stepper_kernels_for(precision, kind, ng);
+  return narrow ? k.narrow : k.single;
+}
 
 }  // namespace ptg
