@@ -84,6 +84,12 @@ __global__ void galerkin_kernel(int nx, int ny, int W, int m, int nax, int nay, 
 // same positions and 1/D[i] in the diagonal slot.  A pivot D[k] <= 0 (an aggregate made only
 // of Dirichlet nodes has an empty row) is replaced by 1 so that the preconditioner stays
 // defined.
+//
+// The nc steps are a serial chain, so a step's latency is the cost: the row of a lane is read
+// whole before any of it is written (kBandMax independent loads in flight; a read-modify-write
+// per entry put that many shared-memory round trips in a row: assembly with both coarse set-ups at
+// 64 x 64 and 128 x 128 takes 0.45 instead of 0.56 ms).
+constexpr int kBandMax = kCoarseMaxAgg + 1;
 __global__ void band_ldlt_kernel(int nc, int b, const double* __restrict__ Ac, float* __restrict__ band) {
   extern __shared__ float w[];
   const int bw = b + 1;
@@ -103,10 +109,15 @@ __global__ void band_ldlt_kernel(int nc, int b, const double* __restrict__ Ac, f
     if (lane == 0) band[k * bw] = r;
     if (mine) band[i * bw + (i - k)] = aik * r;
     const float sik = aik * r;
-    for (int jj = 0; jj < b; ++jj) {      // j = k+1+jj
-      const float ajk = __shfl_sync(0xffffffffu, aik, jj);
-      if (mine && jj <= lane) w[i * bw + (lane - jj)] -= sik * ajk;
-    }
+    float* row = w + i * bw + lane;       // entry j = k+1+jj at row[-jj]
+    float v[kBandMax];
+#pragma unroll
+    for (int jj = 0; jj < kBandMax; ++jj) v[jj] = mine && jj <= lane ? row[-jj] : 0.f;
+#pragma unroll
+    for (int jj = 0; jj < kBandMax; ++jj) v[jj] -= sik * __shfl_sync(0xffffffffu, aik, jj);
+#pragma unroll
+    for (int jj = 0; jj < kBandMax; ++jj)
+      if (mine && jj <= lane) row[-jj] = v[jj];
     __syncwarp();
   }
 }
@@ -114,21 +125,20 @@ __global__ void band_ldlt_kernel(int nc, int b, const double* __restrict__ Ac, f
 // Columns of Ac^-1 from the LDL^T factor: one lane per column, 32 columns per CTA, the
 // substitutions L y = e_c, z = D^-1 y, L^T x = z in FP32 (the inverse is only a
 // preconditioner and is stored in FP32).  X[i * nc + c] is the compact result.  The band
-// loops run over a fixed kBandMax terms with out-of-band terms reading a zero, so that the
-// loads of a row are issued together.
-constexpr int kBandMax = kCoarseMaxAgg + 1;
+// loops run over a fixed kBandMax terms with out-of-band terms reading a zero (kBandMax zero
+// rows stand before and after y, and after L), so that the loads of a row are issued together.
 __global__ void band_inverse_kernel(int nc, int b, const float* __restrict__ band, float* __restrict__ X) {
   extern __shared__ float fsm[];
   constexpr int bw = kBandMax + 1;
-  float* L = fsm;                       // [nc][bw], zero beyond the band
-  float* y = fsm + nc * bw;             // [nc + kBandMax][32], rows -kBandMax..-1 and beyond stay 0
-  for (int t = threadIdx.x; t < nc * bw; t += blockDim.x) {
+  float* L = fsm;                       // [nc + kBandMax][bw], zero beyond the band and the rows
+  float* y = fsm + (nc + kBandMax) * bw;   // [nc + 2 kBandMax][32], only rows 0..nc-1 leave 0
+  for (int t = threadIdx.x; t < (nc + kBandMax) * bw; t += blockDim.x) {
     const int i = t / bw, d = t - i * bw;
-    L[t] = (d <= b && i - d >= 0) ? band[i * (b + 1) + d] : 0.f;
+    L[t] = (i < nc && d <= b && i - d >= 0) ? band[i * (b + 1) + d] : 0.f;
   }
-  for (int t = threadIdx.x; t < (nc + kBandMax) * 32; t += blockDim.x) y[t] = 0.f;
+  for (int t = threadIdx.x; t < (nc + 2 * kBandMax) * 32; t += blockDim.x) y[t] = 0.f;
   __syncthreads();
-  float* yv = y + kBandMax * 32;        // yv[i * 32 + lane], i = -kBandMax .. nc-1
+  float* yv = y + kBandMax * 32;        // yv[i * 32 + lane], i = -kBandMax .. nc+kBandMax-1
   const int lane = threadIdx.x;
   const int c = blockIdx.x * 32 + lane;
   const bool live = c < nc;
@@ -144,13 +154,13 @@ __global__ void band_inverse_kernel(int nc, int b, const float* __restrict__ ban
   }
   for (int i = 0; i < nc; ++i) yv[i * 32 + lane] *= L[i * bw];   // z = D^-1 y
   __syncwarp();
-  for (int i = nc - 1; i >= 0; --i) {   // L^T x = z; rows j > nc-1 read L = 0 via the guard
+  for (int i = nc - 1; i >= 0; --i) {   // L^T x = z
     float s0 = yv[i * 32 + lane], s1 = 0.f;
 #pragma unroll
     for (int d = 1; d <= kBandMax; d += 2) {
       const int j = i + d;
-      if (j < nc) s0 = fmaf(-L[j * bw + d], yv[j * 32 + lane], s0);
-      if (d + 1 <= kBandMax && j + 1 < nc) s1 = fmaf(-L[(j + 1) * bw + d + 1], yv[(j + 1) * 32 + lane], s1);
+      s0 = fmaf(-L[j * bw + d], yv[j * 32 + lane], s0);
+      if (d + 1 <= kBandMax) s1 = fmaf(-L[(j + 1) * bw + d + 1], yv[(j + 1) * 32 + lane], s1);
     }
     yv[i * 32 + lane] = s0 + s1;
     __syncwarp();
@@ -282,7 +292,7 @@ cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A,
   galerkin_l2_kernel<<<nc, 128, 0, stream>>>(nx1, ny1, m, nax, nay, A1, Ac);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t ldlt_smem = sizeof(float) * nc * (b + 1);
-  const size_t inv_smem = sizeof(float) * (nc * (kBandMax + 1) + (nc + kBandMax) * 32);
+  const size_t inv_smem = sizeof(float) * ((nc + kBandMax) * (kBandMax + 1) + (nc + 2 * kBandMax) * 32);
   if ((e = configure_kernel((const void*)band_ldlt_kernel, ldlt_smem, false)) != cudaSuccess) return e;
   if ((e = configure_kernel((const void*)band_inverse_kernel, inv_smem, false)) != cudaSuccess) return e;
   band_ldlt_kernel<<<1, 32, ldlt_smem, stream>>>(nc, b, Ac, band);
@@ -303,7 +313,7 @@ cudaError_t launch_coarse_setup(int nx, int ny, int W, int m, const NodeWeights&
   galerkin_kernel<<<nc, 256, 0, stream>>>(nx, ny, W, m, nax, nay, A, dirichlet, Ac);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t ldlt_smem = sizeof(float) * nc * (b + 1);
-  const size_t inv_smem = sizeof(float) * (nc * (kBandMax + 1) + (nc + kBandMax) * 32);
+  const size_t inv_smem = sizeof(float) * ((nc + kBandMax) * (kBandMax + 1) + (nc + 2 * kBandMax) * 32);
   if ((e = configure_kernel((const void*)band_ldlt_kernel, ldlt_smem, false)) != cudaSuccess) return e;
   if ((e = configure_kernel((const void*)band_inverse_kernel, inv_smem, false)) != cudaSuccess) return e;
   band_ldlt_kernel<<<1, 32, ldlt_smem, stream>>>(nc, b, Ac, band);
