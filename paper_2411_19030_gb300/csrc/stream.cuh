@@ -190,8 +190,8 @@ struct Streamer {
     *reinterpret_cast<double2*>(a + loc + 2) = make_double2(v[2], v[3]);
   }
 
-  // Group barriers.  A pass's stores may be read by bulk copies of the next: every thread orders
-  // its stores before the barrier for the async proxy.
+  // Group barriers after a pass whose stores bulk copies of the next may read (r, z, the right-hand
+  // side of a large level): every thread orders its stores before the barrier for the async proxy.
   __device__ __forceinline__ void sync() {
     asm volatile("fence.proxy.async.global;" ::: "memory");
     comm.sync();
@@ -250,7 +250,7 @@ struct Streamer {
         bulk_load(smem_u32(swts + slot * CR * NW * Wl), gwts + (size_t)row * NW * Wl, NW * bytes, bar);
       }
     };
-    asm volatile("fence.proxy.async;" ::: "memory");
+    if (threadIdx.x == 0) asm volatile("fence.proxy.async;" ::: "memory");
     issue(min(NS, nchunks));
     for (int t0 = 0; t0 < n; t0 += kStreamThreads) {
       const int t = t0 + (int)threadIdx.x, tc = min(t, n - 1);
@@ -270,7 +270,9 @@ struct Streamer {
       issue(min(nchunks, done / CR + NS));
       after(ya + done);
     }
-    __syncthreads();   // the ring is free for the next pass
+    // the ring is free for the next pass, whose copies may overwrite what `after` left in it
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
   }
   // 6-entry window of a group in a ring row; entries beyond the lane's own 16 bytes come from the
   // neighbouring lanes (their groups follow one another, a row's last entry is a zero pad)
@@ -342,13 +344,14 @@ struct Streamer {
   }
   __device__ __forceinline__ bool solo(int l) const { return P.cs == 1 || P.mg[l].ny + 1 <= P.mg_solo_rows; }
   __device__ __forceinline__ bool piped(int l) const { return pipe_rows(P.mg[l].W / kGroup, l == 0 ? kElemWeights : kNodeWeights) > 0; }
-  __device__ __forceinline__ void xsync(int a, int b) {
-    if (solo(a) && solo(b)) {
-      asm volatile("fence.proxy.async.global;" ::: "memory");
+  // Barrier between passes on levels a and b.  `bulk`: the pass before it wrote a vector that bulk
+  // copies read (the fence costs 400 cycles of 512 threads, as much as a pass of a small level).
+  __device__ __forceinline__ void xsync(int a, int b, bool bulk = false) {
+    if (bulk) asm volatile("fence.proxy.async.global;" ::: "memory");
+    if (solo(a) && solo(b))
       __syncthreads();
-    } else {
-      sync();
-    }
+    else
+      comm.sync();
   }
   // this CTA's node rows [y0, y0 + n) of level l
   __device__ __forceinline__ void lrows(int l, int& y0, int& n) const {
@@ -372,33 +375,47 @@ struct Streamer {
       f(row * Wl + kGroup * g, 6 * row * Wl + kGroup * g);
     }
   }
-  // y = A_l v on a group from v's windows on the rows below, at and above it (FP32 node weights)
-  __device__ __forceinline__ void lstencil(int l, int wloc, const float (&vl)[6], const float (&vm)[6],
-                                           const float (&vh)[6], float (&y)[4]) const {
+  // The node weights of a group's stencil on level l: its own and those of the row below and to the left
+  struct GroupWeights {
+    float c[4], e[5], n[4], nb[4], ne[4], neb[4], nw[4], nwb[4];
+  };
+  __device__ __forceinline__ void lweights(int l, int wloc, GroupWeights& w) const {
     const int Wl = P.mg[l].W, wb = wloc - 6 * Wl;       // the row below
     const float *C = lw(l, 0), *E = lw(l, 1), *N = lw(l, 2), *NE = lw(l, 3), *NW = lw(l, 4);
-    float c4[4], n4[4], nb[4], ne4[4], nw4[4], e5[5];
-    ld4f(C, wloc, c4);
-    ld4f(N, wloc, n4);
-    ld4f(N, wb, nb);
-    ld4f(NE, wloc, ne4);
-    ld4f(NW, wloc, nw4);
-    load_ewindow(E, wloc, e5);
-    const float* neb = NE + wb - 1;         // NE weights of the row below, shifted left
-    const float* nwb = NW + wb + 1;         // NW weights of the row below, shifted right
+    ld4f(C, wloc, w.c);
+    ld4f(N, wloc, w.n);
+    ld4f(N, wb, w.nb);
+    ld4f(NE, wloc, w.ne);
+    ld4f(NW, wloc, w.nw);
+    load_ewindow(E, wloc, w.e);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float a = c4[j] * vm[j + 1];
-      a = fmaf(e5[j + 1], vm[j + 2], a);
-      a = fmaf(e5[j], vm[j], a);
-      a = fmaf(n4[j], vh[j + 1], a);
-      a = fmaf(nb[j], vl[j + 1], a);
-      a = fmaf(ne4[j], vh[j + 2], a);
-      a = fmaf(neb[j], vl[j], a);
-      a = fmaf(nw4[j], vh[j], a);
-      a = fmaf(nwb[j], vl[j + 2], a);
+      w.neb[j] = NE[wb - 1 + j];            // NE weights of the row below, shifted left
+      w.nwb[j] = NW[wb + 1 + j];            // NW weights of the row below, shifted right
+    }
+  }
+  // y = A_l v on a group from v's windows on the rows below, at and above it (FP32 node weights)
+  static __device__ __forceinline__ void lapply(const GroupWeights& w, const float (&vl)[6], const float (&vm)[6],
+                                                const float (&vh)[6], float (&y)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float a = w.c[j] * vm[j + 1];
+      a = fmaf(w.e[j + 1], vm[j + 2], a);
+      a = fmaf(w.e[j], vm[j], a);
+      a = fmaf(w.n[j], vh[j + 1], a);
+      a = fmaf(w.nb[j], vl[j + 1], a);
+      a = fmaf(w.ne[j], vh[j + 2], a);
+      a = fmaf(w.neb[j], vl[j], a);
+      a = fmaf(w.nw[j], vh[j], a);
+      a = fmaf(w.nwb[j], vl[j + 2], a);
       y[j] = a;
     }
+  }
+  __device__ __forceinline__ void lstencil(int l, int wloc, const float (&vl)[6], const float (&vm)[6],
+                                           const float (&vh)[6], float (&y)[4]) const {
+    GroupWeights w;
+    lweights(l, wloc, w);
+    lapply(w, vl, vm, vh, y);
   }
   // windows on the rows below, at and above (rows `stride` floats apart)
   __device__ __forceinline__ void lwindows(const float* __restrict__ v, int loc, int stride, float (&a)[6],
@@ -611,11 +628,60 @@ struct Streamer {
       st4f(fc, loc, o);
     });
   }
-  // coarsest level: e = mg_coarse_steps damped-Jacobi steps from zero, the last into e
+  // coarsest level: e = mg_coarse_steps damped-Jacobi steps from zero, the last into e.  A level of at
+  // most 32 groups on one CTA (9 x 9 nodes: 27) is one warp's: the iterate and the weights stay in
+  // registers, the neighbours' values come by shuffles, and a step has no barrier.
   __device__ __forceinline__ void mg_coarsest(int l) {
     const int Wl = P.mg[l].W, n = P.mg_coarse_steps;
     const float* f = lv(l, 0);
     const float* wd = lw(l, 5);
+    const int G4l = Wl / kGroup, cnt = (P.mg[l].ny + 1) * G4l;
+    if (solo(l) && cnt <= 32) {
+      if (rank == 0 && threadIdx.x < 32) {
+        const int lane = threadIdx.x, t = min(lane, cnt - 1), lr = t / G4l, g = t - lr * G4l;
+        const int loc = (lr + 1) * Wl + kGroup * g, wloc = 6 * (lr + 1) * Wl + kGroup * g;
+        GroupWeights w;
+        lweights(l, wloc, w);
+        float fv[4], dv[4], v[4];
+        ld4f(f, loc, fv);
+        ld4f(wd, wloc, dv);
+        // lanes beyond the level and rows beyond it hold 0; a row's first and last entries are zero
+        // pads, so the window's ends may come from the lane of another row
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (lane >= cnt) dv[j] = fv[j] = 0.f;
+          v[j] = dv[j] * fv[j];
+        }
+        const bool below = lane >= G4l, above = lane + G4l < cnt;
+        auto from = [&](float x, int src) { return __shfl_sync(0xffffffffu, x, src & 31); };
+        for (int k = 2; k <= n; ++k) {
+          float vl[6], vm[6], vh[6], y[4];
+          vm[0] = from(v[3], lane - 1);
+          vm[5] = from(v[0], lane + 1);
+          vl[0] = from(v[3], lane - G4l - 1);
+          vl[5] = from(v[0], lane - G4l + 1);
+          vh[0] = from(v[3], lane + G4l - 1);
+          vh[5] = from(v[0], lane + G4l + 1);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            vm[j + 1] = v[j];
+            vl[j + 1] = from(v[j], lane - G4l);
+            vh[j + 1] = from(v[j], lane + G4l);
+          }
+#pragma unroll
+          for (int i = 0; i < 6; ++i) {
+            vl[i] = below ? vl[i] : 0.f;
+            vh[i] = above ? vh[i] : 0.f;
+          }
+          lapply(w, vl, vm, vh, y);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = fmaf(dv[j], fv[j] - y[j], v[j]);
+        }
+        if (lane < cnt) st4f(lv(l, 3), loc, v);
+      }
+      xsync(l, l);
+      return;
+    }
     float* bufs[2] = {lv(l, 3), lv(l, 1)};   // step k writes bufs[(n - k) % 2]: the last lands in e
     for (int k = 1; k <= n; ++k) {
       float* dst = bufs[(n - k) & 1];
@@ -701,19 +767,19 @@ struct Streamer {
           mg_down_march<kElemWeights>(0, f);
         else
           mg_down_march<kNodeWeights>(l, f);
-        xsync(l, l + 1);
+        xsync(l, l + 1, piped(l + 1));
       } else {
         mg_pre(l, f);
         xsync(l, l + 1);
         mg_restrict(l);
-        xsync(l + 1, l + 1);
+        xsync(l + 1, l + 1, piped(l + 1));
       }
     }
     mg_coarsest(L - 1);                 // ends with a barrier
     V rz = V{};
     for (int l = L - 2; l >= 0; --l) {
       if (l < L - 2) xsync(l + 1, l);   // e_{l+1} of the level above is visible
-      else if (!(solo(l + 1) && solo(l))) sync();
+      else if (!(solo(l + 1) && solo(l))) comm.sync();
       const float* f = l == 0 ? r : lv(l, 0);
       if (l == 0)
         rz = piped(0) ? mg_up_march<kElemWeights>(0, f) : mg_up(0, f);
@@ -891,7 +957,7 @@ struct Streamer {
           // alpha = rz / (p, q)
           V pq[1] = {direction(it == 0, beta)};
           const V rz_c = rz;
-          allreduce<V, 1>(pq, [rz_c](V* t) { t[0] = vdiv(rz_c, t[0]); });
+          comm.template allreduce<V, 1, 0>(pq, P.cs, [rz_c](V* t) { t[0] = vdiv(rz_c, t[0]); });   // p, q: no bulk copies
           const V alpha = pq[0], nalpha = vneg(alpha);
           // d += alpha p (d = alpha p at first), r -= alpha q; (r, r)
           const bool first = it == 0;
