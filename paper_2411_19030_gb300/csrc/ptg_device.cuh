@@ -310,28 +310,16 @@ __device__ __forceinline__ void stencil_ff(const float* __restrict__ z, int loc0
   }
 }
 
-// y = A z for the 4 nodes of a group, FP32 element weights (D, S, T) in shared memory.
+// y = A z for the 4 nodes of a group, FP32 element weights (D, S, T).
 // For the node at window position c = j+1: elements a, b below-left / below-right and c, d
 // above-left / above-right, i.e. element windows lower[j], lower[j+1], upper[j], upper[j+1].
-// no_lo / no_hi: the node row below / above is left out (taken as zero), which applies the
-// slab's diagonal block of the operator on its first / last row.
 __device__ __forceinline__ void stencil_elem32(const float* __restrict__ z, const float* __restrict__ wd,
                                                const float* __restrict__ ws, const float* __restrict__ wt, int loc0,
-                                               int W, float (&y)[4], bool no_lo = false, bool no_hi = false) {
+                                               int W, float (&y)[4]) {
   float zl[6], zm[6], zh[6];
-  if (no_lo) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) zl[i] = 0.f;
-  } else {
-    load_window(z, loc0 - W, zl);
-  }
+  load_window(z, loc0 - W, zl);
   load_window(z, loc0, zm);
-  if (no_hi) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) zh[i] = 0.f;
-  } else {
-    load_window(z, loc0 + W, zh);
-  }
+  load_window(z, loc0 + W, zh);
   float dl[5], sl[5], tl[5], du[5], su[5], tu[5];
   const int el = loc0 - W, eu = loc0;   // element windows share the node buffers' row offsets
   load_ewindow(wd, el, dl);

@@ -83,6 +83,30 @@ def test_streamed_marches(nx, ny, precision):
     assert op.stats()["status"] == 0
 
 
+@pytest.mark.parametrize("nx,ny,Ntau,solo", [(64, 64, 2, 0), (64, 64, 2, 257), (64, 64, 160, 0), (66, 66, 2, 0),
+                                             (20, 132, 4, 0), (100, 36, 2, 9), (40, 24, 160, 2)])
+def test_small_levels(nx, ny, Ntau, solo):
+    """The levels that one block works on: the last three, all, a coarsest level of one warp and one of
+    more than 32 groups of nodes, none (solo = 2: then the coarsest level is the group's)."""
+    prob = make_problem(nx, ny, Nt=Ntau, Ntau=Ntau, dt=1 / 64, material="simp_k", sink="left_wide")
+    rho = W.rho_uniform(nx, ny, 12, 0.2, 0.8)
+    U_old, V_old, _ = coarse_states_from_sequential(OracleOp(prob, W.rho_warm_perturb(rho, seed=3, amp=0.05)))
+    ref = o_oneshot(OracleOp(prob, rho), U_old, V_old)
+    op = gpu_operator(prob, "fp32_refine", rtol=1e-12, coarse_stream=2, fine_stream=2)
+    if solo:
+        op.set_multigrid(solo_rows=solo)
+    buf = PassBuffers(op)
+    for t, a in ((buf.U_T, U_old[0]), (buf.U_th, U_old[1]), (buf.V_l, V_old[0]), (buf.V_g, V_old[1])):
+        t.copy_(dev(a))
+    op.assemble(dev(rho))
+    Theta, grad = oneshot_pass(op, buf)
+    # every step's solve leaves rtol 1e-12, in the state and again in the adjoint and the gradient
+    tol = max(FP64_TOL, 5 * Ntau * 1e-12)
+    assert_close("T_hist", host(buf.T_hist), ref["T_hist"], tol)
+    assert_close("grad", host(grad), ref["grad"], tol)
+    assert op.stats()["status"] == 0
+
+
 @pytest.mark.parametrize("scale", [1e-30, 1e30])
 def test_float_pair_cg_is_independent_of_the_units(scale):
     """Conductivity, capacity and source times a factor far from one: the same temperatures."""
