@@ -335,8 +335,8 @@ def run_gpu(args):
                     f64_ms.append(a.elapsed_time(b))
             f64_mean = slowest_rank_ms(float(np.mean(f64_ms)), device)
             f64_st = f64_op.stats()
-            fp64_arm = {"what": "the same one-shot pass with every CG and sum in FP64 (rtol 1e-13), timed like the "
-                                "main steps", "ms_per_step": f64_mean, "value": job_throughput(dof_steps, world, f64_mean),
+            fp64_arm = {"what": "the same one-shot pass in the FP64 kinds (CG in float pairs, every residual and sum "
+                                "in FP64; rtol 1e-13), timed like the main steps", "ms_per_step": f64_mean, "value": job_throughput(dof_steps, world, f64_mean),
                         "unit": UNIT, "sequential_fp64_rtol_1e-13_ms": tight_ms,
                         "speedup_vs_sequential_fp64_same_rtol": tight_ms / f64_mean,
                         "mixed_over_fp64_speedup": f64_mean / ms,
@@ -553,7 +553,8 @@ def ncu_traffic(kind: str, workload: str = WORKLOAD, precision: str = "fp32_refi
 
 
 # FP64 peak of the chip (nominal, 1.25 TFLOP/s; MEASURED_PEAKS.json holds no FP64 figure) and the
-# FLOPs of one FP64 CG iteration per unknown: the 9-point stencil (9 FMA), the p, q, d, r
+# FLOPs of one CG iteration per unknown, whatever its arithmetic (the FP64 kinds' is in float
+# pairs): the 9-point stencil (9 FMA), the p, q, d, r
 # updates (4 FMA), three dot products (3 FMA) and the preconditioned residual (1 FMA) = 17 FMA;
 # one FP64 residual evaluation per refinement sweep and per solve: stencil + subtraction + dot.
 FP64_PEAK_TFLOPS = 1.25
@@ -627,7 +628,7 @@ def roofline(kind_ms: dict, stats: dict, N_free: int, launches: int, precision: 
                            "peak_source": "nominal FP64 peak of the chip (no measured FP64 peak)"}
     out["note"] = ("the CG vectors of a system stay on chip, so the bytes are what a streaming CG would move; the "
                    "correction sweeps are sequential (one system on one 16-CTA cluster at a time) and bound by the "
-                   "latency of their cluster barriers and by the FP64 pipes of 16 SMs, not by HBM")
+                   "latency of their exchanges and block barriers, not by HBM")
     return out
 
 
