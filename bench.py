@@ -519,17 +519,18 @@ def run_gpu(args):
 # kernel source they were taken from: the hash of the stepper sources at capture time is stored
 # beside them.  Any other workload, precision or source hash reports traffic as null.
 NCU_TRAFFIC = {
-    "captured": "2026-12-03",
-    "sources_sha16": "a6f7f5ec6bb57ab9",
+    "captured": "2026-12-05",
+    "sources_sha16": "3568ff7231bf5f38",
     "workload": WORKLOAD,
     "precision": "fp32_refine",
     # the adjoint coarse propagator runs as its two Theta-free parts (two launches per pass)
-    "bytes": {"fine_primal": 8.002304e6 + 108.280064e6, "coarse_primal": 7.368448e6 + 256.0,
-              "correct_primal": 11.627264e6 + 768.0, "fine_adjoint": 149.358848e6 + 2.136320e6,
-              "coarse_adjoint": (15.459840e6 + 0.0) + (7.042304e6 + 512.0),
-              "correct_adjoint": 24.212224e6 + 0.0},
+    "bytes": {"fine_primal": 10.605824e6 + 129.631488e6, "coarse_primal": 7.128576e6 + 0.269056e6,
+              "correct_primal": 11.402496e6 + 0.0, "fine_adjoint": 151.732992e6 + 8.669440e6,
+              "coarse_adjoint": (15.538944e6 + 0.282112e6) + (6.909952e6 + 0.419584e6),
+              "correct_adjoint": 23.983104e6 + 256.0},
 }
-STEPPER_SOURCES = ("stepper.cuh", "comm.cuh", "ptg_device.cuh", "stepper_inst.cu", "stepper_launch.cuh", "plan.cu")
+STEPPER_SOURCES = ("stepper.cuh", "comm.cuh", "ff.cuh", "ptg_device.cuh", "stepper_inst.cu", "stepper_launch.cuh",
+                   "plan.cu")
 
 
 def stepper_sources_sha16() -> str:
