@@ -61,6 +61,12 @@ struct ClusterComm {
   __device__ void bind(const StepParams& P_) { P = &P_; }
   __device__ int rank() const { return (int)cl.block_rank(); }
   __device__ void sync() { cluster_sync_all(); }
+  // Orders the cluster's global stores before its global loads: between a CTA's stores to a global row
+  // and a neighbour's loads of it.  The phases above order shared memory alone: the completion of
+  // an st.async releases that store, not the earlier global stores of the CTA's other threads, and
+  // a row that is written again may still sit in the reader's L1.  The hardware barrier's release and
+  // acquire cover both (16 CTAs: 430 cycles, once per time step).
+  __device__ void order_global() { cluster_sync_all(); }
 
   __device__ __forceinline__ unsigned long long* bar_a() { return &rs.bar[na & 1]; }
   __device__ __forceinline__ unsigned long long* bar_n() { return &rs.bar[2 + (nn & 1)]; }
@@ -305,6 +311,8 @@ struct GridComm {
     }
   }
   __device__ void sync() { barrier(); }
+  // every phase of a group is its barrier, a release and an acquire at gpu scope: nothing left to order
+  __device__ void order_global() {}
 
   template <class T, int NV, int NX, class Post>
   __device__ __forceinline__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post) {

@@ -1540,6 +1540,7 @@ struct Stepper {
           const int n = min(saved + 1, nring);
           const double* X[kMaxExtrap - 1];
           for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j - i) % nring) * P.ring_stride;
+          if (n >= 2) comm.order_global();   // the neighbours' ring rows
           extrapolate_x64(n, X, ring + (size_t)((j - 1) % nring) * P.ring_stride);
           ++saved;
         }
@@ -1611,6 +1612,7 @@ struct Stepper {
         const double* X[3] = {nullptr, nullptr, nullptr};
         for (int i = 0; i < m; ++i) Fm[i] = P.F_field + (size_t)(s - 1 - i) * P.Nn;
         for (int i = 1; i < m; ++i) X[i] = P.out_field + (size_t)(s - i) * P.Nn;
+        if (m >= 2) comm.order_global();      // the neighbours' rows of the corrected states
         load_x64_increment(P.G_field + (size_t)s * P.Nn, m, Fm, X);
       } else {
         load_x64(P.G_field + (size_t)s * P.Nn);
@@ -1659,6 +1661,7 @@ struct Stepper {
           const int n = min(saved + 1, nring);
           const double* X[kMaxExtrap - 1];
           for (int i = 2; i <= n; ++i) X[i - 2] = ring + (size_t)((j + i) % nring) * P.ring_stride;
+          if (n >= 2) comm.order_global();   // the neighbours' ring rows
           extrapolate_x64(n, X, ring + (size_t)((j + 1) % nring) * P.ring_stride);
           ++saved;
         }
@@ -1749,7 +1752,8 @@ struct Stepper {
       // g_s = g_{s+1} - (1/Ntau) term(lambda_G) + F_g[s] - G_g[s]
       accumulate_g(Tk, Tkm, P.dtau, (double)P.Ntau, P.out_aux + (size_t)(s + 1) * P.Ne, P.out_aux + (size_t)s * P.Ne,
                    P.F_aux + (size_t)s * P.Ne, P.G_aux + (size_t)s * P.Ne);
-      comm.sync();                              // every CTA is done reading lambda_G halos
+      comm.sync();                              // every CTA is done reading lambda_G halos; also orders the
+                                                // corrected states of the steps before for the next start
       apply_correction(P.F_field + (size_t)s * P.Nn, P.G_field + (size_t)s * P.Nn, P.out_field + (size_t)s * P.Nn,
                        nullptr);
       exchange_x64();
