@@ -569,13 +569,15 @@ int ptg_mma_set_state(ptg_mma* m, long long k, const double* x1, const double* x
 int ptg_get_stats(ptg_op* op, ptg_stats* out);
 
 /*
- * Bound of the device-side waits of this op's cooperative-grid launches (ptg_solve.grid_wide):
- * a CTA that has polled a grid barrier `polls` times without the release records PTG_ETIMEOUT
- * in the status word and stops waiting, and so does every later wait of that launch, so the
- * launch ends with the error and meaningless results instead of hanging.  0 restores the
- * default (2^20 polls, never reached by a correct co-resident launch); a small value makes the
- * waits give up early (failure-detection tests).  Negative: PTG_EINVAL.  Applies to launches
- * made after the call.
+ * Bound of the device-side waits of this op's launches: the grid barriers of cooperative-grid
+ * launches, the exchanges of cluster launches and the row copies of the streamed solves.  A thread
+ * that has polled `polls` times in vain records PTG_ETIMEOUT in the status word; its CTA, and with it
+ * its group or cluster, stops waiting and sending, and its reductions return NaN, so the launch ends
+ * with the error and meaningless results instead of hanging.  In a batch, a cluster that gave up in one
+ * design's task records PTG_ETIMEOUT for every design whose tasks it takes afterwards, and runs none of
+ * them.  0 restores the default (2^20 polls, never reached by a correct launch); a small value makes
+ * the waits give up early (failure-detection tests).  Negative: PTG_EINVAL.  Applies to launches made
+ * after the call; a batch takes the limit when its plans are made (created or tuned).
  */
 int ptg_op_set_wait_limit(ptg_op* op, long long polls);
 

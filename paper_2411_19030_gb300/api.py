@@ -283,7 +283,7 @@ class Operator:
         return out
 
     def set_wait_limit(self, polls: int):
-        """Bound of the grid-barrier waits of cooperative-grid launches (0: the default)."""
+        """Bound of the device waits of this operator's launches, in polls (0: the default)."""
         _check(_lib().ptg_op_set_wait_limit(self._h, int(polls)), "ptg_op_set_wait_limit")
 
     def reset_stats(self, stream=None):

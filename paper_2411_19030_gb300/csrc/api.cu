@@ -76,7 +76,7 @@ struct ptg_op {
   // two-level partials
   double* g_red = nullptr;
   unsigned* g_bar = nullptr;
-  long long wait_limit = 0;  // polls of a grid barrier before PTG_ETIMEOUT (0: the kernel's default)
+  long long wait_limit = 0;  // polls of a device wait before PTG_ETIMEOUT (0: the kernels' default)
   void* g_halo = nullptr;
   float* g_tl = nullptr;
   int sens_chunks = 0;
@@ -559,6 +559,7 @@ void base_params(const ptg_op* op, StepParams& P) {
   P.guess_next = P.extrap > 1;
   P.prev_field = op->lam_prev;
   P.ring_stride = (long long)(op->g.ny + 1) * op->W;
+  P.wait_limit = op->wait_limit;
   P.mass_uniform = op->has_dc ? 0.0 : op->mat.c0 * op->g.h * op->g.h / 36.0;
 }
 
@@ -620,7 +621,6 @@ int run(ptg_op* op, StepParams& P, int ntasks, cudaStream_t stream, int stats_ki
     P.wide_tasks = ntasks;
     P.g_red = op->g_red;
     P.g_bar = op->g_bar;
-    P.wait_limit = op->wait_limit;
     P.st_w64 = op->st_w64;
     P.st_wr = prec == PTG_FP64 ? op->st_wr : op->st_wr32;
     const size_t rbytes = prec == PTG_FP64 ? sizeof(double) : sizeof(float);
@@ -658,7 +658,6 @@ int run(ptg_op* op, StepParams& P, int ntasks, cudaStream_t stream, int stats_ki
     P.wide_tasks = ntasks;
     P.g_red = op->g_red;
     P.g_bar = op->g_bar;
-    P.wait_limit = op->wait_limit;
     P.g_halo = op->g_halo;
     P.g_halo_row_bytes = op->W * (int)sizeof(double);
     P.g_tl = op->g_tl;

@@ -37,10 +37,16 @@ constexpr long kGridSpinLimit = 1L << 20; // polls of a grid barrier before it r
 // of a buffer and the next send into it; the stepper has one between any two sends into the same
 // buffer.
 //
-// Every wait is bounded: after kClusterPolls polls a thread records PTG_ETIMEOUT and stops waiting
-// for the rest of the launch.  Loop decisions come from values that warp 0 publishes to the whole
-// CTA, so the CTA's threads stay together even then.
-constexpr int kClusterPolls = 1 << 20;
+// Every wait is bounded (P.wait_limit polls, kMbarPolls if not positive).  A thread whose wait runs out
+// records PTG_ETIMEOUT, and its CTA gives up: from the next reduction on no thread of it sends, expects
+// bytes or waits, and every reduction returns NaN, which ends each CG and each residual loop at once.
+// The other CTAs, whose waits for it run out in turn, follow.  So
+//   - an mbarrier is never armed for a phase while its phase before is open (only thread 0 arms them, and
+//     only after its own wait for the phase before);
+//   - loop decisions come from values that warp 0 publishes to the whole CTA, and the hardware barriers
+//     (sync, order_global) stand outside those loops: every CTA passes the same number of them;
+//   - a CTA that has given up may still be sent the bytes of a phase or two (a few KB, within an
+//     mbarrier's range).  drain() keeps it until they have landed.
 
 struct ClusterComm {
   cg::cluster_group cl;
@@ -48,11 +54,12 @@ struct ClusterComm {
   const StepParams* P = nullptr;   // for error reports
   unsigned na = 0, nn = 0;         // all-to-all and neighbour phases completed
   unsigned pend_a = 0, pend_n = 0; // bytes this CTA expects in the next phase of each kind
-  bool broken = false;
+  bool broken = false;             // a wait of this thread ran out, or it has seen that the CTA gave up
 
   // Before the first use: the CTA's mbarriers; the caller follows with cluster_sync_all().
   __device__ ClusterComm(RedSmem& rs_) : cl(cg::this_cluster()), rs(rs_) {
     if (threadIdx.x == 0) {
+      rs.dead = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) mbar_init(&rs.bar[i]);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -71,11 +78,21 @@ struct ClusterComm {
   __device__ __forceinline__ unsigned long long* bar_a() { return &rs.bar[na & 1]; }
   __device__ __forceinline__ unsigned long long* bar_n() { return &rs.bar[2 + (nn & 1)]; }
   __device__ __forceinline__ void wait(unsigned long long* bar, unsigned parity) {
-    if (broken) return;
-    for (int i = 0; i < kClusterPolls; ++i)
-      if (mbar_try(bar, parity)) return;
+    if (broken || mbar_test(bar, parity)) return;
+    if (mbar_wait(bar, parity, P->wait_limit)) return;
     broken = true;
-    if (P) record_error(P->stats, PTG_ETIMEOUT, P->stats_kind, -1);
+    rs.dead = 1;
+    record_error(P->stats, PTG_ETIMEOUT, P->stats_kind, -1);
+  }
+  // After a block barrier behind the last wait: whether this CTA gave up.
+  __device__ bool dead() const { return rs.dead != 0; }
+  // The end of a launch, after the cluster barrier behind which no CTA sends: where this CTA gave up,
+  // nobody has counted the bytes that are still on their way to its shared memory (they take about a
+  // microsecond); it stays for 200 000 cycles.
+  __device__ void drain() const {
+    if (threadIdx.x != 0 || !dead()) return;
+    const long long t0 = clock64();
+    for (int i = 0; i < (1 << 16) && clock64() - t0 < 200000; ++i) __nanosleep(100);
   }
   __device__ __forceinline__ void done_a() {
     ++na;
@@ -83,12 +100,12 @@ struct ClusterComm {
   }
   // The end of a phase whose sends are on their way: every thread waits for the expected bytes.
   __device__ void finish_a() {
-    if (threadIdx.x == 0) mbar_expect(bar_a(), pend_a);
+    if (threadIdx.x == 0 && !broken) mbar_expect(bar_a(), pend_a);
     wait(bar_a(), (na >> 1) & 1);
     done_a();
   }
   __device__ void finish_n() {
-    if (threadIdx.x == 0) mbar_expect(bar_n(), pend_n);
+    if (threadIdx.x == 0 && !broken) mbar_expect(bar_n(), pend_n);
     wait(bar_n(), (nn >> 1) & 1);
     ++nn;
     pend_n = 0;
@@ -112,24 +129,26 @@ struct ClusterComm {
     }
     __syncthreads();
     if (warp == 0) {
+      // the same in the whole warp: every earlier wait of the CTA lies before the block barrier
+      broken = dead();
       union { uint4 u[kWords]; T t[16 * kWords / sizeof(T)]; } pk;
 #pragma unroll
       for (int w = 0; w < kWords; ++w) pk.u[w] = make_uint4(0, 0, 0, 0);
 #pragma unroll
       for (int i = 0; i < NV; ++i) pk.t[i] = half_warp_sum(lane < nwarps ? rb.warp[lane][i] : T{});
-      if (lane < cs) {
+      if (lane < cs && !broken) {
         const unsigned b = mapa_u32(smem_u32(bar_a()), (unsigned)lane);
 #pragma unroll
         for (int w = 0; w < kWords; ++w)
           st_async16(mapa_u32(smem_u32(&rs.slot[na & 1][w][rank()]), (unsigned)lane), pk.u[w], b);
       }
-      if (lane == 0) mbar_expect(bar_a(), pend_a + 16u * kWords * (unsigned)cs);
+      if (lane == 0 && !broken) mbar_expect(bar_a(), pend_a + 16u * kWords * (unsigned)cs);
       wait(bar_a(), (na >> 1) & 1);
 #pragma unroll
       for (int w = 0; w < kWords; ++w) pk.u[w] = rs.slot[na & 1][w][lane < cs ? lane : 0];
       T t[NV + NX];
 #pragma unroll
-      for (int i = 0; i < NV; ++i) t[i] = half_warp_sum(lane < cs ? pk.t[i] : T{});
+      for (int i = 0; i < NV; ++i) t[i] = half_warp_sum(broken ? not_a_number<T>() : lane < cs ? pk.t[i] : T{});
 #pragma unroll
       for (int i = NV; i < NV + NX; ++i) t[i] = T{};
       post(t);
@@ -140,6 +159,7 @@ struct ClusterComm {
     }
     done_a();
     __syncthreads();
+    broken = dead();
 #pragma unroll
     for (int i = 0; i < NV + NX; ++i) v[i] = rb.bcast[i];
   }
@@ -148,6 +168,7 @@ struct ClusterComm {
   // and above (their rows dst_lo / dst_hi), counting on `bar` there.
   __device__ __forceinline__ void send_rows(const void* first, const void* last, const void* dst_lo, const void* dst_hi,
                                             int words16, int rank_, int cs, unsigned long long* bar) {
+    if (broken) return;
     if (rank_ > 0) {
       const unsigned d = mapa_u32(smem_u32(dst_lo), (unsigned)(rank_ - 1)), b = mapa_u32(smem_u32(bar), (unsigned)(rank_ - 1));
       const uint4* s = reinterpret_cast<const uint4*>(first);
@@ -189,6 +210,7 @@ struct ClusterComm {
   __device__ void begin_edges() {}
   template <class T>
   __device__ void put_edge(T* edge, int lr, int col, const T (&v)[4], const Slab& sb) {
+    if (broken) return;
     unsigned long long* bar = bar_n();
     union { uint4 u[sizeof(T) / 4]; T t[4]; } pk;
 #pragma unroll
@@ -215,6 +237,7 @@ struct ClusterComm {
   // the 16 lanes `sub` = 0..15 of a half-warp share the destinations.  Part of the next all-to-all
   // phase; expect_tl adds the bytes that all ranks together send to each.
   __device__ void publish_tl(float* slot, int dst, const float4& chunk, int sub, int cs) {
+    if (broken) return;
     const uint4 u = make_uint4(__float_as_uint(chunk.x), __float_as_uint(chunk.y), __float_as_uint(chunk.z),
                                __float_as_uint(chunk.w));
     for (int q = sub; q < cs; q += 16)
@@ -266,6 +289,7 @@ struct GridComm {
   int pending_bytes = 0;         // bytes of one row
   int hset = 0;                  // slot set of the latest push
   unsigned epoch = 0;            // barriers this CTA has passed in the launch
+  bool broken = false;           // thread 0: a wait of the group ran out; its reductions return NaN
 
   __device__ GridComm(const StepParams& P_, RedSmem& rs_)
       : P(P_), rs(rs_), G(P_.cs), gid((int)blockIdx.x / P_.cs), base(((int)blockIdx.x / P_.cs) * P_.cs) {}
@@ -295,20 +319,29 @@ struct GridComm {
   // every load after the next block barrier; a fence on top of each would cost a round trip.
   __device__ __forceinline__ void arrive_and_wait() {
     unsigned* count = P.g_bar + 4 * gid;
-    unsigned* broken = count + 2;
+    unsigned* flag = count + 2;
     ++epoch;
     const unsigned target = epoch * (unsigned)G;
     red_release_add_gpu(count, 1u);
+    if (broken) return;
     const long long limit = P.wait_limit > 0 ? P.wait_limit : (long long)kGridSpinLimit;
     long long spins = 0;
     while ((int)(ld_acquire_gpu(count) - target) < 0) {
-      if ((++spins & 255) == 0 && ld_acquire_gpu(broken) != 0u) break;
+      if ((++spins & 255) == 0 && ld_acquire_gpu(flag) != 0u) {
+        broken = true;
+        break;
+      }
       if (spins >= limit) {
-        record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
-        atomicExch(broken, 1u);
+        give_up();
         break;
       }
     }
+  }
+  // One thread: a wait ran out.  Every later wait of the group returns at once.
+  __device__ void give_up() {
+    record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
+    atomicExch(P.g_bar + 4 * gid + 2, 1u);
+    broken = true;
   }
   __device__ void sync() { barrier(); }
   // every phase of a group is its barrier, a release and an acquire at gpu scope: nothing left to order
@@ -342,7 +375,7 @@ struct GridComm {
       T t[NV + NX];
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        T a = T{};
+        T a = broken ? not_a_number<T>() : T{};
         for (int r = lane; r < G; r += 32) a = a + ldcg(slots + (base + r) * kPer + i);
         t[i] = warp_sum(a);
       }

@@ -61,6 +61,17 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar) {
 __device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
+// whether the phase is complete, without waiting; mbar_try may wait a little
+__device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned parity) {
+  unsigned done;
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+               "selp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done)
+               : "r"(smem_u32(bar)), "r"(parity)
+               : "memory");
+  return done != 0;
+}
 __device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigned parity) {
   unsigned done;
   asm volatile("{\n\t.reg .pred p;\n\t"
@@ -71,6 +82,26 @@ __device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigned parit
                : "memory");
   return done != 0;
 }
+
+// A bounded wait: false where it ran out, after kMbarPolls polls or after `limit` of them if positive
+// (then without the waiting form of the poll, so that a limit of one poll runs out at once).
+constexpr int kMbarPolls = 1 << 20;
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long long limit) {
+  if (limit > 0) {
+    for (long long i = 1; i < limit; ++i)
+      if (mbar_test(bar, parity)) return true;
+    return false;
+  }
+  for (int i = 0; i < kMbarPolls; ++i)
+    if (mbar_try(bar, parity)) return true;
+  return false;
+}
+
+// A not-a-number: what the reductions of a launch return once a wait of theirs has run out
+template <class T> __device__ __forceinline__ T not_a_number();
+template <> __device__ __forceinline__ float not_a_number<float>() { return __int_as_float(0x7fffffff); }
+template <> __device__ __forceinline__ double not_a_number<double>() { return __hiloint2double(0x7fffffff, -1); }
+template <> __device__ __forceinline__ ff not_a_number<ff>() { return make_ff(__int_as_float(0x7fffffff)); }
 
 // Shared scratch for reductions (static shared memory of the stepper kernel).
 template <class T>
@@ -84,6 +115,7 @@ struct RedSmem {
   RedBank<ff> p;
   uint4 slot[2][2][kMaxCluster]; // [phase][16-byte word][source rank]: that rank's partials
   unsigned long long bar[4];     // the cluster's mbarriers (comm.cuh): two for all-to-all, two for neighbour phases
+  volatile int dead;             // a wait of this CTA ran out (ClusterComm)
 };
 template <class T> __device__ __forceinline__ RedBank<T>& bank(RedSmem& rs);
 template <> __device__ __forceinline__ RedBank<float>& bank<float>(RedSmem& rs) { return rs.f; }

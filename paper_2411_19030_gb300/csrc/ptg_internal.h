@@ -167,7 +167,8 @@ struct StepParams {
   int wide_tasks;            // tasks of a grid-wide launch (group g runs g, g + groups, ...)
   double* g_red;             // [2][kMaxGrid][4] reduction partials
   unsigned* g_bar;           // [4 per group] barrier: arrival count, unused, broken flag (zeroed per launch)
-  long long wait_limit;      // polls of a grid barrier before it reports PTG_ETIMEOUT (<= 0: kGridSpinLimit)
+  long long wait_limit;      // polls of a wait (grid barrier, cluster phase, row ring) before it reports
+                             // PTG_ETIMEOUT (<= 0: kGridSpinLimit, kMbarPolls)
   void* g_halo;              // [2 sets][kMaxGrid][2] rows of g_halo_row_bytes: first / last owned row
   int g_halo_row_bytes;      // W * 8 (a row of doubles; float rows use the first half)
   float* g_tl;               // [kMaxGrid][ncp] restricted partials of the two-level preconditioner

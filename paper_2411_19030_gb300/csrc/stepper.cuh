@@ -1794,6 +1794,7 @@ __global__ void __launch_bounds__(THREADS, 1) stepper_kernel(const __grid_consta
   run_task<Real, NG, KIND>(st, (int)(blockIdx.x / (unsigned)P.cs));
   // no CTA leaves while another may still read or write its shared memory
   cluster_sync_all();
+  comm.drain();
 }
 
 // Systems spread over groups of CTAs of a cooperative launch: the grid holds gridDim.x / P.cs
@@ -1825,27 +1826,37 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) stepper_batch_kernel(const
                                                                        int* __restrict__ queue) {
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   __shared__ RedSmem rs;
-  __shared__ int s_task;
+  __shared__ int s_task, s_dead;               // s_dead (of rank 0): a CTA of the cluster gave up
   ClusterComm comm(rs);
   const unsigned rank = comm.cl.block_rank();
+  if (threadIdx.x == 0) s_dead = 0;
   cluster_sync_all();                          // all CTAs running before any DSMEM store
   for (;;) {
     // rank 0 claims the next task and writes it into every CTA of the cluster; the barrier
-    // publishes it (and orders it after the previous task's last shared-memory access)
+    // publishes it (and orders it after the previous task's last shared-memory access).  Once a wait has
+    // run out the cluster's exchanges are of no use any more: it claims on (~t), so that the designs
+    // whose tasks it takes learn of it, and runs none of them.
     if (rank == 0 && threadIdx.x == 0) {
-      const int t = atomicAdd(queue, 1);
-      for (unsigned r = 0; r < comm.cl.num_blocks(); ++r) *comm.cl.map_shared_rank(&s_task, r) = t;
+      const int t = atomicAdd(queue, 1), claim = s_dead ? ~t : t;
+      for (unsigned r = 0; r < comm.cl.num_blocks(); ++r) *comm.cl.map_shared_rank(&s_task, r) = claim;
     }
     cluster_sync_all();
-    const int t = s_task;                      // identical in every CTA: the loop is uniform
+    const int claim = s_task, t = claim < 0 ? ~claim : claim;   // identical in every CTA: the loop is uniform
     if (t >= ntasks) break;
     const int2 tk = tasks[t];
-    comm.bind(table[tk.x]);
-    Stepper<Real, NG, ClusterComm, kCoarseStep<KIND>> st(table[tk.x], comm, dyn_smem);
-    cluster_sync_all();
-    run_task<Real, NG, KIND>(st, tk.y);
+    if (claim < 0) {
+      if (rank == 0 && threadIdx.x == 0) record_error(table[tk.x].stats, PTG_ETIMEOUT, table[tk.x].stats_kind, -1);
+    } else {
+      comm.bind(table[tk.x]);
+      Stepper<Real, NG, ClusterComm, kCoarseStep<KIND>> st(table[tk.x], comm, dyn_smem);
+      cluster_sync_all();
+      run_task<Real, NG, KIND>(st, tk.y);
+      __syncthreads();
+      if (threadIdx.x == 0 && comm.dead()) *comm.cl.map_shared_rank(&s_dead, 0u) = 1;
+    }
     cluster_sync_all();
   }
+  comm.drain();
 }
 
 }  // namespace ptg

@@ -87,9 +87,10 @@ struct Streamer {
   float* ring_sm;
   unsigned long long* ring_bar;
   unsigned& ring_phase;
+  bool& ring_dead;               // a wait for rows ran out (the same in every thread)
 
-  __device__ Streamer(const StepParams& P_, GridComm& comm_, float* sm, unsigned long long* bar, unsigned& phase)
-      : P(P_), comm(comm_), ring_sm(sm), ring_bar(bar), ring_phase(phase) {
+  __device__ Streamer(const StepParams& P_, GridComm& comm_, float* sm, unsigned long long* bar, unsigned& phase, bool& dead)
+      : P(P_), comm(comm_), ring_sm(sm), ring_bar(bar), ring_phase(phase), ring_dead(dead) {
     rank = comm.rank();
     slab_rows(P.ny + 1, P.cs, rank, r0, R);
     nn = P.nx + 1;
@@ -208,11 +209,13 @@ struct Streamer {
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
   }
-  __device__ __forceinline__ void ring_wait(int slot) {
-    bool in = false;
-    for (int i = 0; i < (1 << 20) && !in; ++i) in = mbar_try(ring_bar + slot, (ring_phase >> slot) & 1u);
-    if (!in) record_error(P.stats, PTG_ETIMEOUT, P.stats_kind, -1);
+  // Waits for a chunk; false where the wait ran out (P.wait_limit).
+  __device__ __forceinline__ bool ring_wait(int slot) {
+    unsigned long long* bar = ring_bar + slot;
+    const unsigned parity = (ring_phase >> slot) & 1u;
+    if (!mbar_test(bar, parity) && !mbar_wait(bar, parity, P.wait_limit)) return false;
     ring_phase ^= 1u << slot;
+    return true;
   }
   // The rows below, at and above a group's row in the ring: the vector (v) and the weights (w, array
   // a of C, E, N, NE, NW, omega/diag, or of omega/diag, k, m)
@@ -229,9 +232,13 @@ struct Streamer {
   // level's weights in shared memory (every lane calls it; one without a group has ok = false and
   // the last group's operands), then after(y_done) runs behind a block barrier, rows below y_done
   // visited.  The rows ya-1 .. yb+1 (all inside the padded layout) come in chunks of CR rows, one
-  // mbarrier and two bulk copies each; a chunk's slot is filled again once its rows are done.
+  // mbarrier and two bulk copies each; a chunk's slot is filled again once its rows are done.  Where a
+  // wait of any thread runs out, the CTA learns of it at the trip's block barrier: thread 0 waits for the
+  // copies in flight, the group gives up (its reductions return NaN, which ends the solve), and this CTA
+  // starts no march any more.
   template <int NW, class Body, class After>
   __device__ __forceinline__ void march(int l, const float* vec, int ya, int yb, Body body, After after) {
+    if (ring_dead) return;
     const int Wl = P.mg[l].W, G4l = Wl / kGroup, first = ya - 1, nr = yb - ya + 3, n = (yb - ya + 1) * G4l;
     const int Smax = pipe_rows(G4l, NW), CR = nr <= Smax ? nr : chunk_rows(Smax, trip_rows(G4l));
     const int NS = Smax / CR, S = NS * CR, nchunks = (nr + CR - 1) / CR;
@@ -255,7 +262,11 @@ struct Streamer {
     for (int t0 = 0; t0 < n; t0 += kStreamThreads) {
       const int t = t0 + (int)threadIdx.x, tc = min(t, n - 1);
       const int need = ((min(n, t0 + kStreamThreads) - 1) / G4l + 2) / CR;   // last chunk of the trip
-      for (; ready <= need; ++ready) ring_wait(ready % NS);
+      bool out = false;
+      for (; ready <= need; ++ready) {
+        out = !ring_wait(ready % NS);
+        if (out) break;
+      }
       const int ry = tc / G4l, g = tc - ry * G4l;
       RowRef<NW> rr;
       rr.vec = svec;
@@ -265,7 +276,14 @@ struct Streamer {
       rr.sm = rr.so + 1 == S ? 0 : rr.so + 1;
       rr.su = rr.sm + 1 == S ? 0 : rr.sm + 1;
       body(rr, ya + ry, g, t < n);
-      __syncthreads();
+      if (__syncthreads_or(out)) {
+        ring_dead = true;
+        if (threadIdx.x == 0) {
+          for (; ready < issued; ++ready) mbar_wait(ring_bar + ready % NS, (ring_phase >> (ready % NS)) & 1u, 0);
+          comm.give_up();
+        }
+        break;
+      }
       const int done = min(n, t0 + kStreamThreads) / G4l;   // whole rows visited: chunks below are free
       issue(min(nchunks, done / CR + NS));
       after(ya + done);
@@ -1486,8 +1504,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
   }
   __syncthreads();
   unsigned ring_phase = 0;
+  bool ring_dead = false;
   GridComm comm(P, rs);
-  Streamer<Real, KIND> st(P, comm, stream_smem, ring_bar, ring_phase);
+  Streamer<Real, KIND> st(P, comm, stream_smem, ring_bar, ring_phase, ring_dead);
   const int ngroups = (int)gridDim.x / P.cs;
   for (int task = comm.gid; task < P.wide_tasks; task += ngroups) {
     if constexpr (KIND == KIND_FINE_PRI) st.fine_primal(task);
