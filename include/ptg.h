@@ -101,7 +101,9 @@ typedef struct {
 
 typedef struct {
     int precision;     /* PTG_FP64, PTG_FP32_REFINE or PTG_FP32_REFINE_ALL */
-    double rtol;       /* stop when ||b - A x||_2 <= rtol ||b||_2 (FP64 residual) */
+    double rtol;       /* a solve stops when ||b - A x||_2 <= rtol ||b||_2, evaluated in FP64.  Below the
+                          rounding of x and of A x to FP64 (2^-51 ||diag(A) x||_2) no state does: FP32
+                          and streamed solves then stop there, FP64 solves on chip report PTG_ENOCONV */
     double inner_rtol; /* relative residual reduction of each FP32 CG (FP32 solves only) */
     int cg_iters_max;  /* iteration limit of one CG */
     int refine_max;    /* limit of refinement sweeps of one solve */

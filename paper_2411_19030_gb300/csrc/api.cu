@@ -41,7 +41,7 @@ struct ptg_op {
   // 1/C ([6][PN]), the FP64 1/C ([PN]), and the workspace of st_groups concurrent slices
   float* w32 = nullptr;         // [3][PEe] FP32 element weights (D, S, T) of C/dt + K
   float* w32_inv = nullptr;     // [PN] FP32 1/C
-  double* st_w64 = nullptr;     // [st_groups][3][PN] (x, x, b), padded node layout
+  double* st_w64 = nullptr;     // [st_groups][4][PN] (x, x, b, residual), padded node layout
   void* st_wr = nullptr;        // [st_groups][5][PN] (r, z, p, q, d) of the FP64 CG kinds
   void* st_wr32 = nullptr;      // the same for the FP32 CG kinds: the two layouts never share
                                 // memory, whose padding rows must stay zero for both
@@ -639,7 +639,7 @@ int run(ptg_op* op, StepParams& P, int ntasks, cudaStream_t stream, int stats_ki
       if (P.kind == KIND_CORRECT_PRI || P.kind == KIND_CORRECT_ADJ) {
         // the sweep's own group of the workspace, partials and barrier
         const size_t g = (size_t)op->st_groups;
-        P.st_w64 = op->st_w64 + g * 3 * (size_t)P.st_pv;
+        P.st_w64 = op->st_w64 + g * 4 * (size_t)P.st_pv;
         P.st_wr = static_cast<char*>(P.st_wr) + g * 5 * (size_t)P.st_pv * rbytes;
         P.mg_ws = op->mg_ws + g * (size_t)op->mg_ws_stride;
         P.g_red = op->sw_red;
@@ -1020,11 +1020,11 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
     const bool f32 = (fine_st && pf != PTG_FP64) || (op->mg_L > 0 && pc != PTG_FP64);
     A(&op->w32, 3 * PEs * sizeof(float));
     A(&op->w32_inv, PNs * sizeof(float));
-    A(&op->st_w64, ng * 3 * PNs * sizeof(double));
+    A(&op->st_w64, ng * 4 * PNs * sizeof(double));
     if (f64) A(&op->st_wr, ng * 5 * PNs * sizeof(double));
     if (f32) A(&op->st_wr32, ng * 5 * PNs * sizeof(float));
     // the padded vectors are zero outside the unknowns; only unknowns are ever written
-    if (e == cudaSuccess) e = cudaMemset(op->st_w64, 0, ng * 3 * PNs * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemset(op->st_w64, 0, ng * 4 * PNs * sizeof(double));
     if (e == cudaSuccess && f64) e = cudaMemset(op->st_wr, 0, ng * 5 * PNs * sizeof(double));
     if (e == cudaSuccess && f32) e = cudaMemset(op->st_wr32, 0, ng * 5 * PNs * sizeof(float));
     if (op->mg_L > 0 || op->mg_Lf > 0) {

@@ -83,7 +83,8 @@ __device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigned parit
   return done != 0;
 }
 
-// A bounded wait: false where it ran out, after kMbarPolls polls or after `limit` of them if positive
+// A bounded wait: false where it ran out, after kMbarPolls polls (of 7 800 cycles when nothing arrives: four
+// seconds) or after `limit` of them if positive
 // (then without the waiting form of the poll, so that a limit of one poll runs out at once).
 constexpr int kMbarPolls = 1 << 20;
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long long limit) {
@@ -198,6 +199,11 @@ __device__ __forceinline__ void slab_rows(int rows_total, int cs, int rank, int&
   r0 = rank * base + (rank < rem ? rank : rem);
   R = base + (rank < rem ? 1 : 0);
 }
+
+// The residual that rounding leaves: x rounded to FP64 and A x evaluated in FP64 each contribute up to
+// 2^-53 || |A| |x| ||, and |A| |x| is about 2 diag(A) |x| (the couplings of a Q1 element's node add up to about
+// its diagonal), so || b - A x ||^2 of about 2^-102 sum (diag(A) x)^2 cannot be lowered.
+constexpr double kRounding2 = 0x1p-102;
 
 // x^e for an integer exponent e >= 1 by squaring, without the multiplications by one (exact
 // operation order is fixed so every CTA and every run computes the same value).

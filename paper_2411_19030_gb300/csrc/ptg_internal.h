@@ -151,7 +151,7 @@ struct StepParams {
   int l3_W1;                 // padded row width of the 2h buffers
   int l3_r1max;              // most 2h rows owned by a CTA of the launch
   const double* A1;          // [9][(ny1 + 1) (nx1 + 1)] 2h stencil, k = (dJ + 1) * 3 + (dI + 1)
-  // streamed propagators (stream.cuh): per group of P.cs CTAs, three FP64 vectors (x, x, b) and the
+  // streamed propagators (stream.cuh): per group of P.cs CTAs, four FP64 vectors (x, x, b, residual) and the
   // CG vectors (r, z, p, q, d) of one float array each, two in the FP64 kinds (float pairs), st_pv
   // entries an array in the padded node layout with its slack; the FP32 element weights (D, S, T)
   // of C/dt + K, w32_stride floats apart in the padded element layout; 1/C of C/dt + K (0 off the

@@ -40,7 +40,7 @@ struct Stepper {
   Slab sb;
   // shared memory (each pointer at the first non-slack entry)
   double* x64;      // FP64 state, rows -1..R
-  double* b64;      // FP64 right-hand side, rows 0..R-1 (in an FP32 kind's solve: the residual)
+  double* b64;      // FP64 right-hand side, rows 0..R-1
   float* zbuf;      // CG stencil operand, rows -1..R
   float* dinv;      // Jacobi inverse diagonal, rows 0..R-1 (0 on Dirichlet and pad nodes)
   float* wk = nullptr;  // FP32 element weights, element rows r0-1..r0+R-1 (FP32 CG, V-cycle): the conductivity
@@ -1305,41 +1305,20 @@ struct Stepper {
   }
 
   // After an FP32 CG (d with its halo rows in zbuf): x64's halo rows follow their owners' update bit
-  // for bit, and the residual in b64 follows x64 += unscale d by
-  //   r -= unscale A d,
-  // A d summed in float pairs: d is a small correction of x64, so the 48 bits of its product are
-  // finer than the rounding of an FP64 b - A x64, and a refinement costs 3 FP64 instructions per
-  // node here instead of 11.  Returns the local sum of r^2.
-  __device__ double update_residual(double unscale, double (&r64)[NG][4]) {
+  // for bit, without an exchange.
+  __device__ void update_halos(double unscale) {
     for (int i = threadIdx.x; i < 2 * sb.W; i += blockDim.x) {
       const int l = halo_offset(i);
       x64[l] = fma(widen(zbuf[l]), unscale, x64[l]);
     }
-    const double us = -unscale / ffw.scale;   // powers of two
-    double rr = 0.0;
-#pragma unroll
-    for (int k = 0; k < NG; ++k) {
-      const int l0 = loc0[k];
-#pragma unroll
-      for (int j = 0; j < kGroup; ++j) r64[k][j] = 0.0;
-      if (l0 < 0) continue;
-      ff y[4];
-      stencil_ff(zbuf, l0, ffw, l0 + gshift, sb.W, y);
-#pragma unroll
-      for (int j = 0; j < kGroup; ++j) {
-        if (!unknown(k, j)) continue;
-        const double t = fma(widen(y[j].l), us, fma(widen(y[j].h), us, b64[l0 + j]));
-        if (ax64) ax64[l0 + j] -= t - b64[l0 + j];
-        b64[l0 + j] = t;
-        r64[k][j] = t;
-        rr = fma(t, t, rr);
-      }
-    }
-    return rr;
+    __syncthreads();
   }
 
   // Solve (C/dt + K) x = b64 with x64 (owned + halos) as initial guess; on return x64 holds
   // the solution with valid halos in every CTA.  `step` is the fine index for error reports.
+  // What decides is b - A x in FP64, evaluated after every CG: a residual that follows x by
+  // recurrence misses the rounding of x and that of A d, and would accept solves that do not meet rtol.
+  // An FP32 kind ends a solve that rounding keeps above rtol too (kRounding2); an FP64 kind reports it.
   // `reuse_ax`: x64 is the previous solution of the same operator, so the A x64 saved by that
   // solve's final residual check gives the first residual without another stencil.
   __device__ void solve(int step, bool reuse_ax = false) {
@@ -1351,17 +1330,15 @@ struct Stepper {
       const int l0 = loc0[k];
       if (l0 < 0) continue;
 #pragma unroll
-      for (int j = 0; j < kGroup; ++j) {
-        bb_rr[0] = fma(b64[l0 + j], b64[l0 + j], bb_rr[0]);
-        if constexpr (kMixed) b64[l0 + j] = r64[k][j];   // the residual from here on (update_residual)
-      }
+      for (int j = 0; j < kGroup; ++j) bb_rr[0] = fma(b64[l0 + j], b64[l0 + j], bb_rr[0]);
     }
     allreduce<double, 2>(bb_rr);
     const double bb = bb_rr[0];
     double rr = bb_rr[1];
     const double tol2 = P.rtol * P.rtol * bb;
     int sweeps = 0, its = 0;
-    while (rr > tol2 && sweeps < P.refmax) {
+    bool rounded = false;
+    while (rr > tol2 && !rounded && sweeps < P.refmax) {
       // scale the residual by 2^-k to a squared norm in [1, 4), so that the CG works on O(1) values
       const int k2 = (((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1;
       const double rr0 = rr * exp2_int(-k2) * exp2_int(-k2);
@@ -1378,19 +1355,26 @@ struct Stepper {
         }
       }
       // (the pairs carry a residual to about 1e-15 of its start)
-      const float target2 = fmaxf((float)(fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr) * rr0), 1e-30f);
+      const double inner2 = P.inner_rtol * P.inner_rtol, final2 = 0.25 * tol2 / rr;
+      const float target2 = fmaxf((float)(fmax(inner2, final2) * rr0), 1e-30f);
       // A d = r in the scale of the float pairs gives d / scale
       const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
       its += cg_correct(r, (float)rr0, target2, unscale);
       ++sweeps;
-      double v[1];
-      if constexpr (kMixed) {
-        v[0] = update_residual(unscale, r64);
-      } else {
+      if constexpr (kMixed)
+        update_halos(unscale);
+      else
         exchange_x64();
-        v[0] = residual(r64);
-      }
+      double v[1] = {residual(r64)};
       allreduce<double, 1>(v);
+      if constexpr (kMixed) {
+        // a CG that aimed at the tolerance, or gained little: whether rounding is what is left
+        if (v[0] > tol2 && (inner2 <= final2 || v[0] > 0.01 * rr)) {
+          double u[1] = {diag_x2()};
+          allreduce<double, 1>(u);
+          rounded = v[0] <= kRounding2 * u[0];
+        }
+      }
       rr = v[0];
     }
     ax_valid = true;
@@ -1404,10 +1388,26 @@ struct Stepper {
       atomicAdd(&P.stats->kind_refinements[P.stats_kind], (unsigned long long)sweeps);
       if (!(rr == rr) || !(bb == bb) || isinf(rr)) {
         record_error(P.stats, PTG_ENONFINITE, P.stats_kind, step);
-      } else if (rr > tol2) {
+      } else if (rr > tol2 && !rounded) {
         record_error(P.stats, PTG_ENOCONV, P.stats_kind, step);
       }
     }
+  }
+
+  // the local sum of (diag(A) x)^2 (kRounding2)
+  __device__ double diag_x2() const {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < NG; ++k) {
+      const int l0 = loc0[k];
+      if (l0 < 0) continue;
+#pragma unroll
+      for (int j = 0; j < kGroup; ++j) {
+        const double t = unknown(k, j) ? A.C[l0 + gshift + j] * x64[l0 + j] : 0.0;
+        s = fma(t, t, s);
+      }
+    }
+    return s;
   }
 
   // sum over owned free nodes of x64^p, reduced over the cluster (FP64)

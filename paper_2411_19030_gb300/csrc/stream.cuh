@@ -7,7 +7,7 @@
 // shared memory and registers of about 50 SMs and only 3 of 128 slices run at once.  Here every
 // slice is a group of G CTAs of one launch (G = 1 or 2 at 512 x 512, one or two per SM), and
 // its vectors stream from HBM: x (FP64, two buffers: the state a step starts from and the one
-// it solves for), the right-hand side b (FP64), and the CG vectors r, p, q, d (precision Real).
+// it solves for), the right-hand side b and the residual (FP64), and the CG vectors r, p, q, d.
 // All Ntau slices then advance together and the solves are bound by HBM bandwidth.
 //
 // Each step is the same as the stepper's (stepper.cuh): b = (C/dt) x_{j-1} + source, the start
@@ -74,7 +74,7 @@ struct Streamer {
   int G4 = 0;                    // groups of 4 nodes per padded row (W / 4)
   // group workspace, padded node layout (node (iy, ix) at (iy + 1) W + ix + 1, the layout of the
   // per-node weights), zero off the unknowns
-  double *xa = nullptr, *xb = nullptr, *b = nullptr;
+  double *xa = nullptr, *xb = nullptr, *b = nullptr, *res = nullptr;
   float *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *d = nullptr;   // high parts; low parts
   size_t lo = 0;                                                                // `lo` floats after (FP64 kinds)
   double step_dt = 0.0, inv_dt = 0.0;
@@ -97,10 +97,11 @@ struct Streamer {
     G4 = P.W / kGroup;
     const int grp = (int)blockIdx.x / P.cs;
     const size_t pv = (size_t)P.st_pv;                 // entries of one padded vector incl. slack
-    double* w64 = P.st_w64 + (size_t)grp * 3 * pv + kSlack;
+    double* w64 = P.st_w64 + (size_t)grp * 4 * pv + kSlack;
     xa = w64;
     xb = w64 + pv;
     b = w64 + 2 * pv;
+    res = w64 + 3 * pv;
     constexpr int kParts = kMixed ? 1 : 2;
     float* wr = reinterpret_cast<float*>(P.st_wr) + (size_t)grp * 5 * kParts * pv + kSlack;
     lo = pv;
@@ -809,7 +810,7 @@ struct Streamer {
     return rz;
   }
 
-  // b <- b - A x (FP64, 0 off the unknowns); the local (b, b) of the old b and (r, r)
+  // res = b - A x (FP64, 0 off the unknowns); the local (b, b) and (r, r)
   __device__ __forceinline__ void residual(const double* __restrict__ x, double& bb, double& rr) const {
     bb = 0.0;
     rr = 0.0;
@@ -825,40 +826,63 @@ struct Streamer {
         bv[j] = di[j] != 0.f ? bv[j] - y[j] : 0.0;
         rr = fma(bv[j], bv[j], rr);
       }
-      st4d(b, loc, bv);
+      st4d(res, loc, bv);
     });
   }
-  // After a CG: x += unscale d, and b <- b - unscale A d with A d summed in float pairs (see
-  // Stepper::update_residual: d is a small correction of x, so the 48 bits of its product are finer
-  // than the rounding of an FP64 b - A x); returns the local (r, r)
+  // the local sum of (diag(A) x)^2 (kRounding2); x is 0 off the unknowns
+  __device__ __forceinline__ double diag_x2(const double* __restrict__ x) const {
+    double s = 0.0;
+    for_groups([&](int loc, int, int) {
+      double xv[4], cv[4];
+      load4(x + loc, xv);
+      load4(A64.C + loc, cv);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double t = cv[j] * xv[j];
+        s = fma(t, t, s);
+      }
+    });
+    return s;
+  }
+  // After a CG: x += unscale d
+  __device__ __forceinline__ void update(double* __restrict__ x, double unscale) const {
+    for_groups([&](int loc, int, int) {
+      V dv[4];
+      double xv[4];
+      ldv(d, loc, dv);
+      load4(x + loc, xv);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if constexpr (!kMixed) xv[j] = fma(widen(dv[j].l), unscale, xv[j]);
+        xv[j] = fma(widen(f32(dv[j])), unscale, xv[j]);
+      }
+      st4d(x, loc, xv);
+    });
+  }
+  // The same in an FP32 kind, with the residual following: res <- res - unscale A d, A d summed in
+  // float pairs.  Cheaper than a new residual (3 FP64 instructions per node instead of 11), but
+  // without the rounding of x and with the pairs' 48 bits: good enough for the next CG to work on, never to
+  // end a solve.  Returns the local (r, r).
   __device__ __forceinline__ double update_residual(double* __restrict__ x, double unscale) const {
     const double us = -unscale / ffw.scale;
     double rr = 0.0;
     for_groups([&](int loc, int, int) {
       ff y[4];
       stencil_ff(d, loc, ffw, loc, P.W, y);
-      if constexpr (!kMixed) {
-        ff yl[4];
-        stencil_ff(d + lo, loc, ffw, loc, P.W, yl);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) y[j] = y[j] + yl[j];
-      }
-      V dv[4];
-      double xv[4], bv[4];
-      float di[4];
-      ldv(d, loc, dv);
+      float dv[4], di[4];
+      double xv[4], rv[4];
+      ld4f(d, loc, dv);
       load4(x + loc, xv);
-      load4(b + loc, bv);
+      load4(res + loc, rv);
       dinv4(loc, di);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if constexpr (!kMixed) xv[j] = fma(widen(dv[j].l), unscale, xv[j]);
-        xv[j] = fma(widen(f32(dv[j])), unscale, xv[j]);
-        bv[j] = di[j] != 0.f ? fma(widen(y[j].l), us, fma(widen(y[j].h), us, bv[j])) : 0.0;
-        rr = fma(bv[j], bv[j], rr);
+        xv[j] = fma(widen(dv[j]), unscale, xv[j]);
+        rv[j] = di[j] != 0.f ? fma(widen(y[j].l), us, fma(widen(y[j].h), us, rv[j])) : 0.0;
+        rr = fma(rv[j], rv[j], rr);
       }
       st4d(x, loc, xv);
-      st4d(b, loc, bv);
+      st4d(res, loc, rv);
     });
     return rr;
   }
@@ -933,7 +957,10 @@ struct Streamer {
     return acc;
   }
 
-  // Solve (C/dt + K) x = b from the start in x (every row of x readable); b becomes the residual.
+  // Solve (C/dt + K) x = b from the start in x (every row of x readable).  What decides is b - A x in FP64.
+  // After a CG that was to reach the tolerance it is evaluated; after one that was to reach inner_rtol
+  // alone the residual may follow x (update_residual), and it is evaluated before it ends the solve.  A
+  // solve that rounding keeps above rtol ends too (kRounding2).
   __device__ __forceinline__ void solve(double* __restrict__ x, int step) {
     double v2[2];
     residual(x, v2[0], v2[1]);
@@ -943,11 +970,13 @@ struct Streamer {
     const double tol2 = P.rtol * P.rtol * bb;
     const bool mg = P.mg_levels > 0;
     int sweeps = 0, its = 0;
-    while (rr > tol2 && sweeps < P.refmax) {
+    bool rounded = false;
+    while (rr > tol2 && !rounded && sweeps < P.refmax) {
       // r / 2^k of squared norm in [1, 4)
       const int k2 = (((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1;
       const double rr0 = rr * exp2_int(-k2) * exp2_int(-k2);
-      const float target2 = fmaxf((float)(fmax(P.inner_rtol * P.inner_rtol, 0.25 * tol2 / rr) * rr0), 1e-30f);
+      const double inner2 = P.inner_rtol * P.inner_rtol, final2 = 0.25 * tol2 / rr;
+      const float target2 = fmaxf((float)(fmax(inner2, final2) * rr0), 1e-30f);
       V rz = V{}, beta = V{};
       int it = -1;                     // -1: the start, whose z and (r, z) open the iteration
       bool done = !((float)rr0 > target2);
@@ -959,7 +988,7 @@ struct Streamer {
           for_groups([&](int loc, int, int) {
             double bv[4];
             V rv[4];
-            load4(b + loc, bv);
+            load4(res + loc, bv);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const ff s = split_scaled(bv[j], -k2);
@@ -1023,9 +1052,34 @@ struct Streamer {
       ++sweeps;
       if (none) break;                             // no iteration: there is no d
       const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
-      double w1[1] = {update_residual(x, unscale)};
-      allreduce<double, 1>(w1);
-      rr = w1[0];
+      bool follow = kMixed && inner2 > final2;
+      double w1[1];
+      if constexpr (kMixed) {
+        if (follow) {
+          w1[0] = update_residual(x, unscale);
+          allreduce<double, 1>(w1);
+          rr = w1[0];
+          follow = rr > tol2;
+        } else {
+          update(x, unscale);
+          comm.sync();
+        }
+      } else {
+        update(x, unscale);
+        comm.sync();
+      }
+      if (!follow) {
+        const double before = rr;
+        residual(x, v2[0], w1[0]);
+        allreduce<double, 1>(w1);
+        rr = w1[0];
+        // a CG that aimed at the tolerance, or gained little: whether rounding is what is left
+        if (rr > tol2 && (inner2 <= final2 || rr > 0.01 * before)) {
+          double u[1] = {diag_x2(x)};
+          allreduce<double, 1>(u);
+          rounded = rr <= kRounding2 * u[0];
+        }
+      }
     }
     if (threadIdx.x == 0 && rank == 0) {
       atomicAdd(&P.stats->solves, 1ull);
@@ -1037,7 +1091,7 @@ struct Streamer {
       atomicAdd(&P.stats->kind_refinements[P.stats_kind], (unsigned long long)sweeps);
       if (!(rr == rr) || !(bb == bb) || isinf(rr)) {
         record_error(P.stats, PTG_ENONFINITE, P.stats_kind, step);
-      } else if (rr > tol2) {
+      } else if (rr > tol2 && !rounded) {
         record_error(P.stats, PTG_ENOCONV, P.stats_kind, step);
       }
     }
