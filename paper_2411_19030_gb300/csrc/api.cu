@@ -1221,15 +1221,15 @@ int ptg_fe_assemble_operator(ptg_op* op, const double* rho_d, cudaStream_t strea
   PTG_CUDA(launch_assemble(op->g.nx, op->g.ny, op->g.h, op->mat, op->tm.dt, op->dtau, rho_d, op->q_elem,
                            op->dirichlet, out, op->stats, stream));
   if (op->w32)
-    PTG_CUDA(launch_stream_weights((int)PEe, (int)PN, op->wE, op->nodew, op->dirichlet, op->g.nx, op->g.ny, op->W,
+    PTG_CUDA(launch_stream_weights((int)PEe, (int)PN, op->wE, op->nodew, op->ff_scale[0], op->dirichlet, op->g.nx, op->g.ny, op->W,
                                    op->w32, op->w32_inv, stream));
   if (op->mg_L > 0) {
     NodeWeights Ac{out.node[5], out.node[6], out.node[7], out.node[8], out.node[9]};
-    PTG_CUDA(launch_mg_setup(Ac, out.wEc, (int)PEe, op->dirichlet, op->mg_lv, op->mg_L, op->mg_w, op->mg_elem, stream));
+    PTG_CUDA(launch_mg_setup(Ac, out.wEc, (int)PEe, op->ff_scale[1], op->dirichlet, op->mg_lv, op->mg_L, op->mg_w, op->mg_elem, stream));
   }
   if (op->mg_Lf > 0) {
     NodeWeights Af{out.node[0], out.node[1], out.node[2], out.node[3], out.node[4]};
-    PTG_CUDA(launch_mg_setup(Af, out.wEf, (int)PEe, op->dirichlet, op->mg_lv, op->mg_Lf, op->mg_wf, op->mg_elemf, stream));
+    PTG_CUDA(launch_mg_setup(Af, out.wEf, (int)PEe, op->ff_scale[0], op->dirichlet, op->mg_lv, op->mg_Lf, op->mg_wf, op->mg_elemf, stream));
   }
   if (op->tl_m) {
     NodeWeights Ac;
@@ -1238,10 +1238,10 @@ int ptg_fe_assemble_operator(ptg_op* op, const double* rho_d, cudaStream_t strea
     Ac.N = out.node[7];
     Ac.NE = out.node[8];
     Ac.NW = out.node[9];
-    PTG_CUDA(launch_coarse_setup(op->g.nx, op->g.ny, op->W, op->tl_m, Ac, op->dirichlet, op->tl_Ac, op->tl_band,
+    PTG_CUDA(launch_coarse_setup(op->g.nx, op->g.ny, op->W, op->tl_m, Ac, op->ff_scale[1], op->dirichlet, op->tl_Ac, op->tl_band,
                                  op->tl_X, op->tl_Ainv, stream));
     if (op->tl3_m > 0)
-      PTG_CUDA(launch_threelevel_setup(op->g.nx, op->g.ny, op->W, Ac, op->dirichlet, op->tl3_m, op->tl3_A1,
+      PTG_CUDA(launch_threelevel_setup(op->g.nx, op->g.ny, op->W, Ac, op->ff_scale[1], op->dirichlet, op->tl3_m, op->tl3_A1,
                                        op->tl3_Ac, op->tl3_band, op->tl3_X, op->tl3_Ainv, stream));
   }
   if (op->mesh) {                // the 2h-mesh op on the averaged design

@@ -273,22 +273,22 @@ cudaError_t launch_adjoint_combine(long long n_l, long long n_g, const double* T
 // ptg_internal.h).  Node entry i of the padded layout (slack included) is row i / W - 1 after the
 // kSlack leading entries.
 __global__ void stream_weights_kernel(int PE, int PN, const double* __restrict__ wE, const double* __restrict__ C,
-                                      const uint8_t* __restrict__ dirichlet, int nx, int ny, int W,
+                                      double scale, const uint8_t* __restrict__ dirichlet, int nx, int ny, int W,
                                       float* __restrict__ w32, float* __restrict__ w32_inv) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < 3 * PE) w32[i] = (float)wE[i];
+  if (i < 3 * PE) w32[i] = (float)(scale * wE[i]);
   if (i < PN) {
     const int k = i - kSlack;
     const int iy = k >= 0 ? k / W - 1 : -2, ix = k >= 0 ? k % W - 1 : -2;
     const bool unknown = iy >= 0 && iy <= ny && ix >= 0 && ix <= nx && dirichlet[iy * (nx + 1) + ix] == 0;
-    w32_inv[i] = unknown ? (float)(1.0 / C[i]) : 0.f;
+    w32_inv[i] = unknown ? (float)(1.0 / (scale * C[i])) : 0.f;
   }
 }
 
-cudaError_t launch_stream_weights(int PE, int PN, const double* wE, const double* C_node, const uint8_t* dirichlet,
-                                  int nx, int ny, int W, float* w32, float* w32_inv, cudaStream_t stream) {
+cudaError_t launch_stream_weights(int PE, int PN, const double* wE, const double* C_node, double scale,
+                                  const uint8_t* dirichlet, int nx, int ny, int W, float* w32, float* w32_inv, cudaStream_t stream) {
   const int n = 3 * PE > PN ? 3 * PE : PN;
-  stream_weights_kernel<<<(n + 255) / 256, 256, 0, stream>>>(PE, PN, wE, C_node, dirichlet, nx, ny, W, w32, w32_inv);
+  stream_weights_kernel<<<(n + 255) / 256, 256, 0, stream>>>(PE, PN, wE, C_node, scale, dirichlet, nx, ny, W, w32, w32_inv);
   return cudaGetLastError();
 }
 

@@ -10,7 +10,8 @@
 // nay = (ny + 1) / m aggregates per direction (at least 1), the last ones absorbing the
 // remainder.  Ac = P^T A P restricted to the free nodes.  This file builds Ac in FP64,
 // factors its band (half-bandwidth nax + 1) as L D L^T in FP32 and forms the dense inverse in
-// FP32 (symmetrised, rows padded to a multiple of 4), which the stepper reads row-wise.
+// FP32 (symmetrised, rows padded to a multiple of 4), which the stepper reads row-wise.  A is taken times
+// the power of two that the CG works with (FFWeights::scale).
 #include <cstdint>
 #include "ptg_internal.h"
 
@@ -18,9 +19,9 @@ namespace ptg {
 
 // One CTA per aggregate a = (ay, ax); the threads stride over its nodes.  For a free node i
 // the 9-point row of A is split by the aggregate of each free neighbour j (one of the 3 x 3
-// aggregates around a): Ac[a][b] = sum over i in a, j in b of A_ij.  Fixed-order block sums.
+// aggregates around a): Ac[a][b] = scale times the sum over i in a, j in b of A_ij.  Fixed-order block sums.
 __global__ void galerkin_kernel(int nx, int ny, int W, int m, int nax, int nay, NodeWeights A,
-                                const uint8_t* __restrict__ dirichlet, double* __restrict__ Ac) {
+                                double scale, const uint8_t* __restrict__ dirichlet, double* __restrict__ Ac) {
   const int a = blockIdx.x;
   const int ax = a % nax, ay = a / nax;
   const int nc = nax * nay;
@@ -70,7 +71,7 @@ __global__ void galerkin_kernel(int nx, int ny, int W, int m, int nax, int nay, 
     double s = 0.0;
     for (int w = 0; w < nw; ++w) s += part[k][w];
     const int bx = ax + k % 3 - 1, by = ay + k / 3 - 1;
-    if (bx >= 0 && bx < nax && by >= 0 && by < nay) Ac[(size_t)a * nc + by * nax + bx] = s;
+    if (bx >= 0 && bx < nax && by >= 0 && by < nay) Ac[(size_t)a * nc + by * nax + bx] = scale * s;
   }
 }
 
@@ -190,11 +191,11 @@ __global__ void pack_inverse_kernel(int nax, int nay, const float* __restrict__ 
 // (2I + di, 2J + dj), |di|, |dj| <= 1, takes the weight w(di) w(dj) of 2h node (I, J), with
 // w(0) = 1 and w(+-1) = 1/2; rows of P1 at Dirichlet fine nodes are zero.  A1 = P1^T A P1 is a
 // 9-point operator; one thread per (2h node a, neighbour b) sums P1(i, a) A(i, j) P1(j, b) over
-// the free fine nodes i in the support of a and their free fine neighbours j (fixed order).
+// the free fine nodes i in the support of a and their free fine neighbours j (fixed order), times scale.
 // A 2h node whose support holds no free fine node gets the identity row.
 __device__ __forceinline__ double p1_weight(int d) { return d == 0 ? 1.0 : 0.5; }
 
-__global__ void galerkin_l1_kernel(int nx, int ny, int W, NodeWeights A, const uint8_t* __restrict__ dirichlet,
+__global__ void galerkin_l1_kernel(int nx, int ny, int W, NodeWeights A, double scale, const uint8_t* __restrict__ dirichlet,
                                    int nx1, int ny1, double* __restrict__ A1) {
   const int n1 = (nx1 + 1) * (ny1 + 1);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -229,6 +230,7 @@ __global__ void galerkin_l1_kernel(int nx, int ny, int W, NodeWeights A, const u
       }
     }
   }
+  sum *= scale;
   if (k == 4 && !(sum > 0.0)) sum = 1.0;   // no free fine node in the support
   A1[(size_t)k * n1 + a] = sum;
 }
@@ -279,13 +281,13 @@ __global__ void galerkin_l2_kernel(int nx1, int ny1, int m, int nax, int nay, co
   }
 }
 
-cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A, const uint8_t* dirichlet, int m,
+cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A, double scale, const uint8_t* dirichlet, int m,
                                     double* A1, double* Ac, float* band, float* X, float* Ainv, cudaStream_t stream) {
   const int nx1 = nx / 2, ny1 = ny / 2, n1 = (nx1 + 1) * (ny1 + 1);
   const int nax = coarse_aggregates(nx1, m), nay = coarse_aggregates(ny1, m);   // (n1 + 1) / m 2h nodes
   const int nc = nax * nay, ncp = coarse_row_stride(nax) * nay;
   const int b = nax + 1;
-  galerkin_l1_kernel<<<(9 * n1 + 255) / 256, 256, 0, stream>>>(nx, ny, W, A, dirichlet, nx1, ny1, A1);
+  galerkin_l1_kernel<<<(9 * n1 + 255) / 256, 256, 0, stream>>>(nx, ny, W, A, scale, dirichlet, nx1, ny1, A1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(Ac, 0, sizeof(double) * nc * nc, stream)) != cudaSuccess) return e;
@@ -303,14 +305,14 @@ cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A,
   return cudaGetLastError();
 }
 
-cudaError_t launch_coarse_setup(int nx, int ny, int W, int m, const NodeWeights& A, const uint8_t* dirichlet,
+cudaError_t launch_coarse_setup(int nx, int ny, int W, int m, const NodeWeights& A, double scale, const uint8_t* dirichlet,
                                 double* Ac, float* band, float* X, float* Ainv, cudaStream_t stream) {
   const int nax = coarse_aggregates(nx, m), nay = coarse_aggregates(ny, m);
   const int nc = nax * nay, ncp = coarse_row_stride(nax) * nay;
   const int b = nax + 1;
   cudaError_t e = cudaMemsetAsync(Ac, 0, sizeof(double) * nc * nc, stream);
   if (e != cudaSuccess) return e;
-  galerkin_kernel<<<nc, 256, 0, stream>>>(nx, ny, W, m, nax, nay, A, dirichlet, Ac);
+  galerkin_kernel<<<nc, 256, 0, stream>>>(nx, ny, W, m, nax, nay, A, scale, dirichlet, Ac);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t ldlt_smem = sizeof(float) * nc * (b + 1);
   const size_t inv_smem = sizeof(float) * ((nc + kBandMax) * (kBandMax + 1) + (nc + 2 * kBandMax) * 32);

@@ -36,14 +36,14 @@ __device__ __forceinline__ double coupling(const float* __restrict__ w, int W, i
 
 __device__ __forceinline__ double hat(int a) { return a == 0 ? 1.0 : 0.5; }   // |a| <= 1
 
-// Level 0: FP32 copy of the FP64 node weights; omega/diag on the unknowns.  One thread per
+// Level 0: FP32 copy of the FP64 node weights times scale; omega/diag on the unknowns.  One thread per
 // padded entry (rows -1 .. ny + 1); entries outside the grid are zero.
 // Beside them the element form (omega/diag of the nodes of row y, then k = k_e/6 and m = c_e h^2/(36
 // step) of the elements above it) interleaved row by row, from the element weights wE (D = 4 (k + m)
 // and S = 2 m - k, PE apart, rows ey = -1 .. ny).
 __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ dirichlet, int nx, int ny, int W,
                                  float* __restrict__ w, float omega, const double* __restrict__ wE, int PE,
-                                 float* __restrict__ elem) {
+                                 double scale, float* __restrict__ elem) {
   const int n = (ny + 3) * W;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int iy = t / W - 1, ix = t % W - 1;
@@ -51,12 +51,12 @@ __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ diri
     const int loc = t;
     float c = 0.f, e = 0.f, no = 0.f, ne = 0.f, nw = 0.f, wd = 0.f;
     if (in) {
-      c = (float)A.C[loc];
-      e = (float)A.E[loc];
-      no = (float)A.N[loc];
-      ne = (float)A.NE[loc];
-      nw = (float)A.NW[loc];
-      if (!dirichlet[iy * (nx + 1) + ix] && A.C[loc] > 0.0) wd = (float)(omega / A.C[loc]);
+      c = (float)(scale * A.C[loc]);
+      e = (float)(scale * A.E[loc]);
+      no = (float)(scale * A.N[loc]);
+      ne = (float)(scale * A.NE[loc]);
+      nw = (float)(scale * A.NW[loc]);
+      if (!dirichlet[iy * (nx + 1) + ix] && A.C[loc] > 0.0) wd = (float)(omega / (scale * A.C[loc]));
     }
     const int o = 6 * (t / W) * W + t % W;
     w[o] = c;
@@ -67,7 +67,7 @@ __global__ void mg_level0_kernel(NodeWeights A, const uint8_t* __restrict__ diri
     w[o + 5 * W] = wd;
     // the node rows are -1 .. ny + 1, the element rows -1 .. ny
     const bool row = t < (ny + 2) * W;
-    const double Dw = row ? wE[t] : 0.0, Sw = row ? wE[PE + t] : 0.0;
+    const double Dw = row ? scale * wE[t] : 0.0, Sw = row ? scale * wE[PE + t] : 0.0;
     const int oe = 3 * (t / W) * W + t % W;
     elem[oe] = wd;
     elem[oe + W] = (float)(fma(-2.0, Sw, Dw) * (1.0 / 6.0));
@@ -153,13 +153,13 @@ long long mg_layout(int nx, int ny, MgLevel* lv, int L, long long* ws_floats) {
   return woff;
 }
 
-cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, const uint8_t* dirichlet, const MgLevel* lv, int L,
-                            float* w, float* elem, cudaStream_t stream) {
+cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, double scale, const uint8_t* dirichlet,
+                            const MgLevel* lv, int L, float* w, float* elem, cudaStream_t stream) {
   const MgLevel& l0 = lv[0];
   const int threads = 256;
   auto blocks = [&](long long n) { return (int)std::min<long long>((n + threads - 1) / threads, 4096); };
   mg_level0_kernel<<<blocks((long long)(l0.ny + 3) * l0.W), threads, 0, stream>>>(
-      A, dirichlet, l0.nx, l0.ny, l0.W, w + l0.woff + kSlack, kMgOmega, wE, PE, elem + kSlack);
+      A, dirichlet, l0.nx, l0.ny, l0.W, w + l0.woff + kSlack, kMgOmega, wE, PE, scale, elem + kSlack);
   for (int l = 0; l + 1 < L; ++l) {
     const MgLevel& f = lv[l];
     const MgLevel& c = lv[l + 1];

@@ -55,7 +55,9 @@ struct NodeWeights {
 
 // The same weights as float pairs for the CG of the FP64 kinds (ff.cuh): ten arrays in the padded
 // node layout, stride floats apart, the high parts of (C, E, N, NE, NW) and then their low parts,
-// times a power of two (scale) that makes the largest of order one.
+// times a power of two (scale) that makes the largest of order one.  Every CG, FP32 and float pairs,
+// and every preconditioner works with the operator times scale: its floats then do not depend on the
+// units of the materials.
 struct FFWeights {
   const float* w;            // the first non-slack entry of the first array
   int stride;
@@ -324,12 +326,12 @@ cudaError_t launch_stepper(const StepParams& P, const Plan& plan, int precision,
 cudaError_t launch_stepper_batch(int precision, int kind, const Plan& plan, const StepParams* table, const int2* tasks,
                                  int ntasks, int* queue, int nclusters, cudaStream_t stream);
 cudaError_t query_batch_occupancy(int precision, int kind, int cs, int ng, int nthreads, size_t smem, int* nclusters);
-cudaError_t launch_coarse_setup(int nx, int ny, int W, int m, const NodeWeights& A, const uint8_t* dirichlet,
+cudaError_t launch_coarse_setup(int nx, int ny, int W, int m, const NodeWeights& A, double scale, const uint8_t* dirichlet,
                                 double* Ac, float* band, float* X, float* Ainv, cudaStream_t stream);
 // Three-level set-up from the coarse-step operator's node weights: the 2h Galerkin stencil A1
 // ([9][(ny/2 + 1)(nx/2 + 1)]), then the aggregates of m x m 2h nodes: A2 = P2^T A1 P2 (dense FP64
 // in Ac), its band LDL^T and dense inverse in FP32, packed as for the fine aggregates.
-cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A, const uint8_t* dirichlet, int m,
+cudaError_t launch_threelevel_setup(int nx, int ny, int W, const NodeWeights& A, double scale, const uint8_t* dirichlet, int m,
                                     double* A1, double* Ac, float* band, float* X, float* Ainv, cudaStream_t stream);
 // Raise a kernel's dynamic shared-memory limit (and allow non-portable cluster sizes) once per
 // device; later calls with no larger footprint make no attribute call.
@@ -372,19 +374,19 @@ cudaError_t launch_sensitivities(int nx, int ny, int Nt, double h, double dt, in
                                  const double* dc, const double* lam, int j0, int j1, const double* T, int hist_j0,
                                  double* partial, int nchunks, double* grad, cudaStream_t stream);
 
-// For the streamed fine propagators: FP32 copies of the 3 x PE FP64 element weights (D, S, T) of
-// C/dt + K (slack included), and 1/C in FP32 (0 off the unknowns) on the PN entries of
+// For the streamed fine propagators, of C/dt + K times scale: FP32 copies of the 3 x PE FP64 element
+// weights (D, S, T; slack included), and 1/C in FP32 (0 off the unknowns) on the PN entries of
 // the padded node layout (slack included; C the node weight array with its slack).
-cudaError_t launch_stream_weights(int PE, int PN, const double* wE, const double* C_node, const uint8_t* dirichlet,
-                                  int nx, int ny, int W, float* w32, float* w32_inv, cudaStream_t stream);
+cudaError_t launch_stream_weights(int PE, int PN, const double* wE, const double* C_node, double scale,
+                                  const uint8_t* dirichlet, int nx, int ny, int W, float* w32, float* w32_inv, cudaStream_t stream);
 cudaError_t launch_stream(const StepParams& P, int precision, int ngroups, cudaStream_t stream);
 // Multigrid hierarchy: the number of levels of an nx x ny grid (1: no coarsening), the layout of
 // L levels (returns the floats of the weight buffer; *ws_floats the floats of one group's
 // workspace), and the set-up of every level's weights from the FP64 node weights A and element
-// weights wE (buffers zeroed beforehand: the slack and the rows outside the grid stay zero).
+// weights wE times scale (buffers zeroed beforehand: the slack and the rows outside the grid stay zero).
 int mg_level_count(int nx, int ny);
 long long mg_layout(int nx, int ny, MgLevel* lv, int L, long long* ws_floats);
-cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, const uint8_t* dirichlet, const MgLevel* lv, int L,
+cudaError_t launch_mg_setup(NodeWeights A, const double* wE, int PE, double scale, const uint8_t* dirichlet, const MgLevel* lv, int L,
                             float* w, float* elem, cudaStream_t stream);
 // G_l = H_l + c S_l ([n_l]) and G_g = H_g + c S_g ([n_g]), c the adjoint source scale of Theta
 cudaError_t launch_adjoint_combine(long long n_l, long long n_g, const double* Theta, double p, int Ne, int modified,

@@ -292,8 +292,9 @@ struct Stepper {
   }
 
   // Select the operator C/dt + K (fine) or C/dtau + K (coarse): per-node FP64 weights for the
-  // residual (and the FP64 CG), FP32 element weights in shared memory for the FP32 CG, and
-  // the Jacobi inverse diagonal (zero on Dirichlet and pad nodes).
+  // residual, and, of the operator times ffw.scale, float pairs (FP64 kinds' CG), FP32 element weights
+  // in shared memory (FP32 CG, V-cycle) and the Jacobi inverse diagonal (zero on Dirichlet and pad
+  // nodes).  The 2h level and the aggregates' inverse are built from the operator times scale too.
   __device__ void set_operator() {
     constexpr bool coarse = COARSE;
     A = coarse ? P.A_coarse : P.A_fine;
@@ -321,8 +322,8 @@ struct Stepper {
       const double* src = wE + sb.r0 * W;               // padded element row r0 = element row r0 - 1
       for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const double Dw = src[i], Sw = src[PE + i];   // 4 (k + m) and 2 m - k
-        wk[i] = (float)(fma(-2.0, Sw, Dw) * (1.0 / 6.0));
-        wm[i] = (float)(fma(4.0, Sw, Dw) * (1.0 / 12.0));
+        wk[i] = (float)(ffw.scale * (fma(-2.0, Sw, Dw) * (1.0 / 6.0)));
+        wm[i] = (float)(ffw.scale * (fma(4.0, Sw, Dw) * (1.0 / 12.0)));
       }
     }
     fmask = 0;
@@ -335,10 +336,7 @@ struct Stepper {
         const int g = gnode(l0, j);
         float v = 0.f;
         if (g >= 0 && P.dirichlet[g] == 0) {
-          // the float pairs are scaled: the CG of the FP64 kinds without a two-level form takes 1/C
-          // in their scale
-          const double c = A.C[l0 + gshift + j];
-          v = 1.f / (float)(kMixed || tl ? c : c * ffw.scale);
+          v = 1.f / (float)(ffw.scale * A.C[l0 + gshift + j]);
           fmask |= 1u << (kGroup * k + j);
         }
         dinv[l0 + j] = v;
@@ -361,7 +359,7 @@ struct Stepper {
         const int lr = i / W - 1, ix = i - (lr + 1) * W - 1, row = sb.r0 + lr;
         float v = 0.f;
         if (row >= 0 && row <= P.ny && ix >= 0 && ix <= P.nx && P.dirichlet[row * (P.nx + 1) + ix] == 0)
-          v = (float)((double)P.tl_omega / A.C[i + gshift]);
+          v = (float)((double)P.tl_omega / (ffw.scale * A.C[i + gshift]));
         vsd[i] = v;
       }
     }
@@ -1357,8 +1355,8 @@ struct Stepper {
       // (the pairs carry a residual to about 1e-15 of its start)
       const double inner2 = P.inner_rtol * P.inner_rtol, final2 = 0.25 * tol2 / rr;
       const float target2 = fmaxf((float)(fmax(inner2, final2) * rr0), 1e-30f);
-      // A d = r in the scale of the float pairs gives d / scale
-      const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
+      // (scale A) d = r gives d / scale
+      const double unscale = exp2_int(k2) * ffw.scale;
       its += cg_correct(r, (float)rr0, target2, unscale);
       ++sweeps;
       if constexpr (kMixed)

@@ -1051,7 +1051,7 @@ struct Streamer {
       its += it;
       ++sweeps;
       if (none) break;                             // no iteration: there is no d
-      const double unscale = exp2_int(k2) * (kMixed ? 1.0 : ffw.scale);
+      const double unscale = exp2_int(k2) * ffw.scale;
       bool follow = kMixed && inner2 > final2;
       double w1[1];
       if constexpr (kMixed) {
