@@ -262,8 +262,18 @@ size_t wide_twolevel_bytes(const void* ctx, int G) {
   return twolevel_bytes(c->op, c->precision, c->kind, G, c->tl_mode, false);
 }
 
+// From this ratio of K to C / step (diagonals, of the materials' extremes) the CG on chip forms (p, q) with
+// dot products of its own (Stepper::cg_correct says why and what they cost).  Iterations without over
+// with them, FP64 kinds, 16 x 16 to 64 x 64 nodes, uniform, near-binary and block designs: Jacobi 1.00 at
+// ratios up to 800, up to 1.2 at 1.5e3 to 6e3, 1.5 at 2e4, 1.7 at 6e5; a two-level form, which takes the
+// slow modes out, 1.00 to 1.04 up to 2e4, up to 1.4 at 6e5.
+constexpr double kDotsRatio = 2e3, kDotsRatioTwoLevel = 1e5;
+
 void twolevel_params(const ptg_op* op, int precision, StepParams& P, int tl_mode) {
   P.tl_naj = twolevel_rows(op, precision, P.kind, P.cs, tl_mode);
+  const double step = coarse_kind(P.kind) ? op->dtau : op->tm.dt;
+  P.cg_dots = 6.0 * std::max(op->mat.k0, op->mat.kmin) * step >
+              (P.tl_naj > 0 ? kDotsRatioTwoLevel : kDotsRatio) * std::min(op->mat.c0, op->mat.cmin) * op->g.h * op->g.h;
   P.tl_vc = P.tl_naj > 0 && uses_vcycle(op, tl_mode);
   P.tl_omega = kVcycleOmega;
   P.tl_nu = op->tl_nu;
@@ -1032,7 +1042,7 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
       const long long wf = mg_layout(grid->nx, grid->ny, op->mg_lv, std::max(op->mg_L, op->mg_Lf), &wsf);
       op->mg_ws_stride = wsf;
       A(&op->mg_ws, ng * (size_t)wsf * sizeof(float));
-      A(&op->sw_red, 2 * kMaxGrid * 4 * sizeof(double));
+      A(&op->sw_red, 2 * kMaxGrid * 2 * kRedWords * sizeof(double));
       A(&op->sw_bar, 4 * sizeof(unsigned));
       // rows and columns outside each level's grid and the slack stay zero
       if (e == cudaSuccess) e = cudaMemset(op->mg_ws, 0, ng * (size_t)wsf * sizeof(float));
@@ -1048,7 +1058,7 @@ int ptg_op_create(const ptg_grid* grid, const ptg_material* mat, const ptg_time*
     }
   }
   A(&op->scratch, 2 * sizeof(double));
-  A(&op->g_red, 2 * kMaxGrid * 4 * sizeof(double));
+  A(&op->g_red, 2 * kMaxGrid * 2 * kRedWords * sizeof(double));
   A(&op->g_bar, 4 * kMaxGrid * sizeof(unsigned));
   A(&op->g_halo, (size_t)2 * kMaxGrid * 2 * op->W * sizeof(double));
   A(&op->stats, sizeof(DevStats));

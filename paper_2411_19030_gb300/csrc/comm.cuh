@@ -117,9 +117,9 @@ struct ClusterComm {
   // same order: the same bits everywhere.
   template <class T, int NV, int NX, class Post>
   __device__ void allreduce(T (&v)[NV + NX], int cs, Post post) {
-    constexpr int kWords = NV * (int)sizeof(T) > 16 ? 2 : 1;
-    static_assert(NV <= 4 && NV * sizeof(T) <= 32, "two 16-byte words per rank");
-    RedBank<T>& rb = bank<T>(rs);
+    constexpr int kWords = (NV * (int)sizeof(T) + 15) / 16;
+    static_assert(NV <= kMaxReduce && NV + NX <= 8 && kWords <= kRedWords, "16-byte words per rank");
+    const RedBank<T> rb(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
@@ -349,7 +349,7 @@ struct GridComm {
 
   template <class T, int NV, int NX, class Post>
   __device__ __forceinline__ void allreduce(T (&v)[NV + NX], int /*cs*/, Post post) {
-    RedBank<T>& rb = bank<T>(rs);
+    const RedBank<T> rb(rs);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
@@ -358,10 +358,11 @@ struct GridComm {
       for (int i = 0; i < NV; ++i) rb.warp[warp][i] = v[i];
     }
     __syncthreads();
-    // 32 bytes per block whatever T: the groups of a launch are not in step, and one may reduce floats
+    // the same bytes per block whatever T: the groups of a launch are not in step, and one may reduce floats
     // while another reduces doubles
-    constexpr int kPer = 32 / (int)sizeof(T);
-    T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 4);
+    constexpr int kPer = 16 * kRedWords / (int)sizeof(T);
+    static_assert(NV <= kPer && NV <= kMaxReduce && NV + NX <= 8, "a block's part of g_red");
+    T* slots = reinterpret_cast<T*>(P.g_red + (size_t)phase * kMaxGrid * 2 * kRedWords);
     // warp 0 alone: the CTA's sums into its slots, the barrier, lane-strided sums over the ranks and
     // the warp's sum, then `post`; broadcast
     if (warp == 0) {

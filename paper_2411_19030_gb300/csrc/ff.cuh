@@ -92,6 +92,10 @@ __device__ __forceinline__ ff vmul(const ff& a, const ff& b) {
 }
 __device__ __forceinline__ float vdiv(float a, float b) { return a / b; }
 __device__ __forceinline__ ff vdiv(const ff& a, const ff& b) { return ff_div(a, b); }
+// a float as one of the CG's scalars
+template <class V> __device__ __forceinline__ V vfloat(float a);
+template <> __device__ __forceinline__ float vfloat<float>(float a) { return a; }
+template <> __device__ __forceinline__ ff vfloat<ff>(float a) { return make_ff(a); }
 __device__ __forceinline__ float vneg(float a) { return -a; }
 __device__ __forceinline__ ff vneg(const ff& a) { return make_ff(-a.h, -a.l); }
 

@@ -105,23 +105,24 @@ template <> __device__ __forceinline__ double not_a_number<double>() { return __
 template <> __device__ __forceinline__ ff not_a_number<ff>() { return make_ff(__int_as_float(0x7fffffff)); }
 
 // Shared scratch for reductions (static shared memory of the stepper kernel).
-template <class T>
-struct RedBank {
-  T warp[kMaxWarps][4];       // per-warp partials of this CTA
-  T bcast[8];                 // finalised values
-};
+constexpr int kMaxReduce = 5;      // values of one all-reduce (of floats; 4 of the 8-byte types)
 struct RedSmem {
-  RedBank<float> f;
-  RedBank<double> d;
-  RedBank<ff> p;
-  uint4 slot[2][2][kMaxCluster]; // [phase][16-byte word][source rank]: that rank's partials
+  // per-warp partials of this CTA and finalised values, of whatever type is being reduced: partials are
+  // read between the two block barriers of a reduction and written outside them, final values the other way
+  // round, so reductions of different types share the memory
+  double warp[kMaxWarps * kMaxReduce];
+  double bcast[8];
+  uint4 slot[2][kRedWords][kMaxCluster]; // [phase][16-byte word][source rank]: that rank's partials
   unsigned long long bar[4];     // the cluster's mbarriers (comm.cuh): two for all-to-all, two for neighbour phases
   volatile int dead;             // a wait of this CTA ran out (ClusterComm)
 };
-template <class T> __device__ __forceinline__ RedBank<T>& bank(RedSmem& rs);
-template <> __device__ __forceinline__ RedBank<float>& bank<float>(RedSmem& rs) { return rs.f; }
-template <> __device__ __forceinline__ RedBank<double>& bank<double>(RedSmem& rs) { return rs.d; }
-template <> __device__ __forceinline__ RedBank<ff>& bank<ff>(RedSmem& rs) { return rs.p; }
+template <class T>
+struct RedBank {
+  T (*warp)[kMaxReduce];
+  T* bcast;
+  __device__ __forceinline__ explicit RedBank(RedSmem& rs)
+      : warp(reinterpret_cast<T (*)[kMaxReduce]>(rs.warp)), bcast(reinterpret_cast<T*>(rs.bcast)) {}
+};
 
 struct NoPost {
   template <class T>

@@ -78,6 +78,9 @@ struct MgLevel {
 };
 
 // Everything one stepper launch needs (passed by value in parameter space).
+// What a CTA contributes to an all-reduce (comm.cuh), in 16-byte words: 4 doubles or float pairs, 5 floats.
+constexpr int kRedWords = 2;
+
 struct StepParams {
   // problem
   int nx, ny, Nn, Ne, Nt, Ntau, M;
@@ -95,6 +98,7 @@ struct StepParams {
   // solver
   double rtol, inner_rtol;
   int itmax, refmax;
+  int cg_dots;               // kinds on chip: (p, q) with dot products of its own (Stepper::cg_correct)
   // op data (device, FP64, padded layouts; pointers at the first non-slack entry)
   const double* wE_fine;     // [3][(ny+2) W] element (D, S, T) weights of C/dt + K
   const double* wE_coarse;   // [3][(ny+2) W] element (D, S, T) weights of C/dtau + K
@@ -167,7 +171,7 @@ struct StepParams {
   // one system over a whole cooperative grid (GridComm): global scratch of the op
   int wide;                  // 1: launched as stepper_wide_kernel, groups of cs CTAs
   int wide_tasks;            // tasks of a grid-wide launch (group g runs g, g + groups, ...)
-  double* g_red;             // [2][kMaxGrid][4] reduction partials
+  double* g_red;             // [2][kMaxGrid][2 kRedWords] reduction partials
   unsigned* g_bar;           // [4 per group] barrier: arrival count, unused, broken flag (zeroed per launch)
   long long wait_limit;      // polls of a wait (grid barrier, cluster phase, row ring) before it reports
                              // PTG_ETIMEOUT (<= 0: kGridSpinLimit, kMbarPolls)

@@ -1203,9 +1203,18 @@ struct Stepper {
   // of two to a squared 2-norm rr0 in [1, 4); on return x64 += unscale * d.  Stops when
   // ||r||^2 <= target2 (scaled units) or at the iteration limit; returns the iteration count.
   // Vectors, scalars and dot products are V; z is float.
-  // One reduction per iteration (Chronopoulos and Gear's arrangement): A z instead of A p, with
-  // q = A p and (p, q) by recurrence, so the iteration waits for the neighbours' rows of z and for
-  // one all-reduce instead of two.
+  // One reduction per iteration (after Chronopoulos and Gear): A z instead of A p, with q = A p by
+  // recurrence, so the iteration waits for the neighbours' rows of z and for one all-reduce instead of
+  // two.  (p, q) of the new direction p = z + beta p_old comes from that reduction as well,
+  //   (p, q) = (z, w) + beta (2 (z, q_old) + beta (p, q)_old),
+  // or, where K does not outweigh C/dt by much (P.cg_dots == 0), as (z, w) - beta^2 (p, q)_old.  That takes z
+  // for conjugate to p_old, which it is to 2^-24 only, being the FP32 result of a preconditioner, and where
+  // (p, q) is far below (z, w) the error decides: with K over C/dt of 1e5 and more it took 1.2 to 4 times
+  // the iterations of a CG with a dot product of its own for (p, q) (16 x 16 nodes, FP64 kinds), or
+  // 16 000 instead of 400 without an end (FP32 kinds).  With (z, q_old) it takes as many.  In FP32
+  // (p, q)_old carried from iteration to iteration loses its own bits there too, so it is a dot product
+  // of the same reduction.  One more dot product costs 3 to 4% of a pass (128 x 128 FP64 43.0 -> 44.4 ms,
+  // 96 x 96 gradient 99.9 -> 104.8), the two of FP32 5% (100 x 100 28.0 -> 29.6): hence the rule.
   // The float pairs of the FP64 kinds: on a slab of 9 x 132 nodes (128 x 128 over 16 CTAs) an
   // iteration's stencil, updates and dot products took 10 100 cycles on the FP64 pipe (17 FP64
   // instructions per node) and take about 180 FP32 instructions per node in pairs.
@@ -1229,12 +1238,12 @@ struct Stepper {
         put_edges(vrh, r);
         comm.finish_edges();
       }
-      // z = M^-1 r and w = A z; (r, z), (z, w) and (r, r) in one reduction; then
-      //   beta = (r, z) / (r, z)_old,  (p, q) = (z, w) - beta^2 (p, q)_old,  alpha = (r, z) / (p, q)
-      V v[6] = {V{}, V{}, V{}, V{}, V{}, V{}};
-      v[0] = precondition(r);
+      // z = M^-1 r and w = A z; (r, z), (z, w), (r, r) and what (p, q) needs in one reduction; then beta,
+      // (p, q) and alpha = (r, z) / (p, q).  (r, r), for the stop alone, needs no more than a float.
+      const V rz_part = precondition(r);
       exchange(zbuf);
-      V w[NG][4];
+      V w[NG][4], zw = V{}, zq = V{}, pq = V{};
+      float rr = 0.f;
 #pragma unroll
       for (int k = 0; k < NG; ++k) {
         const int l0 = loc0[k];
@@ -1244,24 +1253,60 @@ struct Stepper {
 #pragma unroll
         for (int j = 0; j < kGroup; ++j) {
           if (!unknown(k, j)) w[k][j] = V{};
-          v[1] = vdot(v[1], w[k][j], zbuf[l0 + j]);
-          v[2] = vdot(v[2], r[k][j], r[k][j]);
+          zw = vdot(zw, w[k][j], zbuf[l0 + j]);
+          rr = fmaf(f32(r[k][j]), f32(r[k][j]), rr);
+        }
+      }
+      if (P.cg_dots) {
+#pragma unroll
+        for (int k = 0; k < NG; ++k) {
+          const int l0 = loc0[k];
+          if (l0 < 0) continue;
+#pragma unroll
+          for (int j = 0; j < kGroup; ++j) {
+            zq = vdot(zq, q[k][j], zbuf[l0 + j]);
+            if constexpr (kMixed) pq = vdot(pq, p[k][j], q[k][j]);
+          }
         }
       }
       const bool start = it == 0;
-      allreduce<V, 3, 3>(v, [start, rz_old, pq_old](V* t) {
-        if (start) {
-          t[5] = t[1];
-        } else {
-          t[4] = vdiv(t[0], rz_old);
-          t[5] = vfma(vneg(vmul(t[4], t[4])), pq_old, t[1]);
+      // alpha, beta and (p, q) into o, from (r, z), (z, w) and what (p, q) has beside (z, w)
+      auto lengths = [start](const V& rz_, const V& zw_, const V& b, const V& more, V* o) {
+        o[1] = start ? V{} : b;
+        o[2] = zw_;
+        if (!start) o[2] = vfma(b, more, zw_);
+        if (!(f32(o[2]) > 0.f)) {        // nothing left of (p, q) but rounding: start again from z
+          o[1] = V{};
+          o[2] = zw_;
         }
-        t[3] = vdiv(t[0], t[5]);
-      });
-      if (!((start ? rr0 : f32(v[2])) > target2)) break;
-      const V alpha = v[3], nalpha = vneg(alpha), beta = v[4];
-      rz_old = v[0];
-      pq_old = v[5];
+        o[0] = vdiv(rz_, o[2]);
+      };
+      V o[3];
+      if (P.cg_dots) {
+        constexpr int NV = kMixed ? 5 : 4;
+        V v[NV + 3] = {rz_part, zw, vfloat<V>(rr), zq};
+        if constexpr (kMixed) v[4] = pq;
+        allreduce<V, NV, 3>(v, [&lengths, rz_old, pq_old](V* t) {
+          const V b = vdiv(t[0], rz_old), pq_ = kMixed ? t[NV - 1] : pq_old;
+          lengths(t[0], t[1], b, vfma(b, pq_, t[3] + t[3]), t + NV);
+        });
+        rr = f32(v[2]);
+        rz_old = v[0];
+        for (int i = 0; i < 3; ++i) o[i] = v[NV + i];
+      } else {
+        V v[6] = {rz_part, zw, vfloat<V>(rr)};
+        allreduce<V, 3, 3>(v, [&lengths, rz_old, pq_old](V* t) {
+          const V b = vdiv(t[0], rz_old);
+          lengths(t[0], t[1], b, vneg(vmul(b, pq_old)), t + 3);
+        });
+        rr = f32(v[2]);
+        rz_old = v[0];
+        for (int i = 0; i < 3; ++i) o[i] = v[3 + i];
+      }
+      const V alpha = o[0], beta = o[1];
+      pq_old = o[2];
+      if (!((start ? rr0 : rr) > target2)) break;
+      const V nalpha = vneg(alpha);
       // p = z + beta p, q = w + beta q, d += alpha p, r -= alpha q
 #pragma unroll
       for (int k = 0; k < NG; ++k) {
