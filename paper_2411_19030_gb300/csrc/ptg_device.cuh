@@ -441,9 +441,10 @@ __device__ __forceinline__ void stencil_km32(const float* __restrict__ z, const 
                                              const float* __restrict__ wm, int loc0, int W, int lane, float (&y)[4],
                                              bool no_lo = false, bool no_hi = false) {
   float zl[6], zm[6], zh[6], kl[5], ml[5], ku[5], mu[5];
-  warp_window(z, loc0 - W, lane, zl);
+  // (a row that is left out is not read either: a neighbour may be writing it)
+  warp_window(z, no_lo ? loc0 : loc0 - W, lane, zl);
   warp_window(z, loc0, lane, zm);
-  warp_window(z, loc0 + W, lane, zh);
+  warp_window(z, no_hi ? loc0 : loc0 + W, lane, zh);
   warp_ewindow(wk, loc0 - W, lane, kl);
   warp_ewindow(wm, loc0 - W, lane, ml);
   warp_ewindow(wk, loc0, lane, ku);

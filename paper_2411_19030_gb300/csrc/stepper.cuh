@@ -1152,7 +1152,7 @@ struct Stepper {
       for (int j = 0; j < kGroup; ++j) z[k][j] = 0.f;
       const int lr = l0 / sb.W - 1;
       float t[4];
-      apply32(zbuf, k, t, lr == 0, lr == sb.R - 1);
+      apply32(zbuf, k, t, lr <= 0, lr < 0 || lr == sb.R - 1);   // (lr = -1: no group, computes on the first row)
       if (l0 < 0) continue;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) z[k][j] = fmaf(om * dinv[l0 + j], f32(r[k][j]) - t[j], e[k][j]);
