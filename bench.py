@@ -520,14 +520,14 @@ def run_gpu(args):
 # beside them.  Any other workload, precision or source hash reports traffic as null.
 NCU_TRAFFIC = {
     "captured": "2026-12-05",
-    "sources_sha16": "3568ff7231bf5f38",
+    "sources_sha16": "373a8ad1d74de613",
     "workload": WORKLOAD,
     "precision": "fp32_refine",
     # the adjoint coarse propagator runs as its two Theta-free parts (two launches per pass)
-    "bytes": {"fine_primal": 10.605824e6 + 129.631488e6, "coarse_primal": 7.128576e6 + 0.269056e6,
-              "correct_primal": 11.402496e6 + 0.0, "fine_adjoint": 151.732992e6 + 8.669440e6,
-              "coarse_adjoint": (15.538944e6 + 0.282112e6) + (6.909952e6 + 0.419584e6),
-              "correct_adjoint": 23.983104e6 + 256.0},
+    "bytes": {"fine_primal": 10.139392e6 + 132.496640e6, "coarse_primal": 7.083776e6 + 0.314368e6,
+              "correct_primal": 11.618560e6 + 768.0, "fine_adjoint": 150.571008e6 + 7.012864e6,
+              "coarse_adjoint": (15.418624e6 + 0.649984e6) + (6.985728e6 + 0.487424e6),
+              "correct_adjoint": 23.916800e6 + 0.0},
 }
 STEPPER_SOURCES = ("stepper.cuh", "comm.cuh", "ff.cuh", "ptg_device.cuh", "stepper_inst.cu", "stepper_launch.cuh",
                    "plan.cu")

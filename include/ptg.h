@@ -58,9 +58,11 @@ extern "C" {
                                 outside the op's allocations; the launch was skipped */
 
 /* precision of the fine-propagator CG (Sec. 2.2 solves; precision pattern of the port) */
-#define PTG_FP64            0  /* CG and every accumulation in FP64 */
+#define PTG_FP64            0  /* states, right-hand sides, residuals b - A x and every accumulation of
+                                  results in FP64; the CG that lowers a residual works in pairs of
+                                  floats (48 bits), its preconditioner in FP32 */
 #define PTG_FP32_REFINE     1  /* fine-step solves: CG in FP32 on the FP64 residual, refined in FP64;
-                                  coarse-step solves (G and the correction sweeps): FP64 CG */
+                                  coarse-step solves (G and the correction sweeps): as PTG_FP64 */
 #define PTG_FP32_REFINE_ALL 2  /* every solve as the fine-step solves of PTG_FP32_REFINE */
 
 /* slice scheduling of ptg_fine_propagate_slices / ptg_adjoint_sweep */
@@ -186,8 +188,8 @@ typedef struct {
                           roughly 300 x 300 and more), on chip elsewhere.  Other values:
                           PTG_EINVAL. */
     int coarse_stream; /* coarse-step solves (G_pri, G_adj and the correction sweeps, a3 and a4) with
-                          the Krylov vectors in global memory: FP64 CG (FP32 under
-                          PTG_FP32_REFINE_ALL) preconditioned by one V(1,1)-cycle of geometric
+                          the Krylov vectors in global memory: the CG of PTG_FP64
+                          (FP32 under PTG_FP32_REFINE_ALL) preconditioned by one V(1,1)-cycle of geometric
                           multigrid in FP32: level l+1 the nodes (2I, 2J) of level l down to a
                           grid of at most 8 elements across (while nx and ny stay even), Galerkin
                           operators P^T A P of bilinear interpolation P, damped-Jacobi smoothing

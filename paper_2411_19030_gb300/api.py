@@ -56,8 +56,9 @@ def twolevel_code(v) -> int:
 
 @dataclass
 class SolveConfig:
-    precision: str = "fp64"          # "fp64"; "fp32_refine": fine-step CG in FP32 with FP64 refinement,
-    #                                  coarse-step solves in FP64; "fp32_refine_all": every CG in FP32
+    precision: str = "fp64"          # "fp64": FP64 residuals, states and sums, CG in pairs of floats;
+    #                                  "fp32_refine": fine-step CG in FP32 with FP64 refinement,
+    #                                  coarse-step solves as "fp64"; "fp32_refine_all": every CG in FP32
     rtol: float = 1e-13
     inner_rtol: float = 1e-4
     cg_iters_max: int = 2000

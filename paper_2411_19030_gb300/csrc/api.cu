@@ -222,26 +222,33 @@ size_t twolevel_bytes(const ptg_op* op, int precision, int kind, int cs, int tl_
 // omega lambda_max stays below 1.8 < 2 for every step size.
 constexpr float kVcycleOmega = 0.8f;
 // Default preconditioner of FP32 CG solves without a two-level form (ptg_solve.local_steps = 0):
-// Jacobi on cluster launches, the two slab-local steps on cooperative-grid launches (run()).  The two slab-local steps cut the fine-step CG iterations (128 x 128 pass: 34 -> 27
-// primal, 31 -> 24.5 adjoint) but cost more than they save there (fine kernels 7.6 + 8.5 ->
-// 8.6 + 9.4 ms); on high-contrast 512 x 512 designs they pay (one-shot design iteration 13.2 ->
-// 11.5 s).
+// Jacobi on cluster launches, the two slab-local steps on cooperative-grid launches (run()).  The
+// two steps cut the fine-step CG iterations but cost more than they save on clusters (128 x 128:
+// 18.9 -> 15.3 iterations, 5.4 -> 6.3 ms per fine propagator; 256 x 256: 24.8 -> 20.0, 51.0 -> 60.7 ms).
+// On cooperative-grid launches they paid on high-contrast 512 x 512 designs with the solver before (one-shot
+// design iteration 13.2 -> 11.5 s), which now stream; at 320 x 320, rho in 0.2 .. 0.8, they do not
+// (66.3 -> 53.5 iterations, 54.6 -> 64.8 ms).
 constexpr int kLocalSteps = 1;
 // Default smoothing steps of the V-cycle (ptg_solve.smooth_steps = 0): four slab-local Jacobi
-// steps before and after the coarse correction.  Measured on the 128 x 128 one-shot pass
-// (FP64 coarse-step CG): 1 global step 66.1 ms; 2, 3, 4, 6 local steps 59.2, 56.5, 55.9,
-// 56.8 ms, the CG iterations per correction solve falling from 34 to 26, 23, 21, 19.
+// steps before and after the coarse correction.  Measured on the 128 x 128 one-shot pass: 1 global
+// step 34.8 ms; 2, 3, 4, 6 local steps 31.8, 31.4, 31.8, 33.4 ms, the CG iterations per correction
+// solve falling from 25 to 19, 16.8, 15.7, 14.6.
 constexpr int kVcycleSmoothSteps = 4;
-// Default smoothing steps of the three-level cycle on both its smoothed levels: a numpy model of
-// the 128 x 128 coarse-step operator (slab-local Jacobi on 16 slabs, aggregates of 4 x 4 2h nodes)
-// needs 13 PCG iterations with 3 or 4 steps, 14 with 2 on one level, 15 with 2 on both.
+// Default smoothing steps of the three-level cycle on both its smoothed levels.  Measured on the
+// 128 x 128 one-shot pass: 1, 2, 3, 4, 6 steps 27.7, 26.9, 27.3, 28.0, 29.8 ms at 12.2, 10.0, 9.3, 8.8, 8.4
+// CG iterations per correction solve.
 constexpr int kThreeLevelSmoothSteps = 3;
 
-// Node count from which a single FP64 system runs grid-wide (see choose_plan).
+// Node count from which a single FP64 system runs grid-wide (see choose_plan).  Chained FP64 passes of
+// two steps per row, on a cluster against grid-wide: 128 x 128 82 / 155 ms, 160 x 160 135 / 215,
+// 200 x 200 215 / 300, 240 x 240 394 / 369, 280 x 280 609 / 392.  The line was drawn with FP64 CG vectors;
+// with float pairs the two meet at about 55 000 nodes.
 constexpr int kWideMinNodes = 40000;
 // Node count from which the coarse-step solves stream by default (multigrid-preconditioned FP64 CG
-// with the vectors in HBM): 192 x 192 (37 249 nodes) and up.  On chip, a 192 x 192 one-shot pass
-// took longer than a 256 x 256 one with the same slices (214 against 187 ms at 64 slices).
+// with the vectors in HBM): 192 x 192 (37 249 nodes) and up.  One-shot passes of 32 steps per slice, on
+// chip against streamed: 128 x 128 27 / 49 ms, 160 x 160 47 / 73, 176 x 176 74 / 92, 192 x 192 103 / 114,
+// 224 x 224 191 / 159, 256 x 256 261 / 203.  The line was drawn with FP64 CG vectors; with float pairs the
+// two meet at about 42 000 nodes for rho in 0.2 .. 0.8.
 constexpr int kCoarseStreamMinNodes = 30000;
 // Streamed coarse-step solves (stream.cuh, mg.cu): node rows per CTA of a correction sweep's
 // group, the damped-Jacobi steps on the multigrid's coarsest level, and the levels with at most
@@ -414,8 +421,9 @@ int choose_plan(ptg_op* op, int precision, int kind, int ntasks, Plan* out) {
       op->sv.fine_stream != 1) {
     // fine_stream 0: streamed where no cluster holds a slice (the grouped launches of large
     // grids run only a few slices at a time: at 512 x 512, 3 of 128); measured there the one-shot
-    // design iteration takes 4.4-4.8 s streamed against 7.6-9.0 s on chip.  Where clusters fit
-    // (256 x 256) both take the same time and the on-chip path stays.
+    // design iteration took 4.4-4.8 s streamed against 7.6-9.0 s on chip.  Where clusters fit the
+    // on-chip path is faster (fine propagator at 128 x 128 5.4 against 19.5 ms, 192 x 192 19.7 / 41.8,
+    // 256 x 256 51 / 94, 300 x 300 78 / 116).
     bool want = op->sv.fine_stream == 2;
     if (!want && op->sv.fine_stream == 0) {
       Plan c;
@@ -443,15 +451,15 @@ int choose_plan(ptg_op* op, int precision, int kind, int ntasks, Plan* out) {
       return PTG_OK;
     }
   }
-  // One FP64 system: a cluster runs its CG on 16 SMs, bound by their FP64 pipes; a grid-wide
-  // launch spreads the FP64 work over every SM, but each of its reductions costs a few
-  // microseconds of global-memory round trips against about one for a cluster.  Measured on
-  // GB300 the cluster wins at 128 x 128; the grid wins once the per-iteration FP64 work of 16
-  // SMs dominates (kWideMinNodes).  Grids whose slabs do not fit 16 CTAs (512 x 512) run in
-  // groups of CTAs of one cooperative launch.  grid_wide: 0 never, 1 by these rules, 2 always.
-  // The strongest two-level form whose plan fits (and, for FP32 CG, adds no wave over
-  // Jacobi's: FP64 CG on GB300 is bound by the FP64 pipe, so the cut in iterations outweighs
-  // extra waves; FP32 CG is bound by latency).
+  // One FP64 system: a cluster runs its float-pair CG on 16 SMs; a grid-wide launch spreads the work
+  // over every SM, but each of its reductions costs a few microseconds of global-memory round trips
+  // against less than one for a cluster.  The cluster wins on small grids, the grid once the work per
+  // iteration of 16 SMs dominates (kWideMinNodes).  Grids whose slabs do not fit 16 CTAs
+  // (512 x 512) run in groups of CTAs of one cooperative launch.  grid_wide: 0 never, 1 by these
+  // rules, 2 always.
+  // The strongest two-level form whose plan fits (and, for FP32 CG, adds no wave over Jacobi's: a
+  // float-pair iteration costs more than an FP32 one, so the cut in iterations, three to ten times at
+  // 128 x 128, outweighs extra waves sooner; chosen with FP64 CG vectors and not measured again).
   // A plan may leave out the saved A x of the last residual (one more FP64 stencil per step) when
   // that lets a two-level form, or any plan at all, fit.
   Plan jac, two;
@@ -1804,9 +1812,9 @@ constexpr int kBatchSweepCtas = 16;
 constexpr int kBatchSideStreams = 24;
 // Designs of this many nodes or more take their own path in a batch even with on-chip solves:
 // the persistent launch's geometry is sized by its largest design, and their own cluster
-// launches run beside it.  Measured on the 48-design workload: 1.98 s per batched pass with
-// 15000 (128 x 128 and larger on their own path), 2.12 s with 30000, 2.60 s with only the
-// streamed designs on it; 9000 gained nothing over 15000.
+// launches run beside it.  Measured on the 48-design workload: 1.23 s per batched pass with
+// 15000 (128 x 128 and larger on their own path) and with 9000, 1.32 s with 30000 and with only the
+// streamed designs on it.
 constexpr int kBatchOwnMinNodes = 15000;
 
 // Phase ph of design d through its op's own launches (the per-op entry points on the batch's

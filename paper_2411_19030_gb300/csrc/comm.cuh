@@ -10,9 +10,9 @@
 //                systems run side by side (one cluster each).
 //   GridComm     groups of G CTAs of one cooperative launch (up to kMaxGrid CTAs in all, one
 //                per SM), each group running one system at a time: global memory and a
-//                counting barrier per group.  Used for a single system whose solves are bound
-//                by the FP64 pipe (1/58 of the FP32 rate on this chip), spread over every SM
-//                instead of one cluster, and for grids whose slabs do not fit 16 CTAs.
+//                counting barrier per group.  Used for a single large FP64 system, spread over
+//                every SM instead of one cluster (kWideMinNodes in api.cu has the times), and for
+//                grids whose slabs do not fit 16 CTAs.
 //
 // Both produce bitwise identical reductions in every CTA (fixed summation orders).
 #pragma once

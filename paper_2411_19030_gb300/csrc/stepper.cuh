@@ -585,9 +585,9 @@ struct Stepper {
   // the accuracy); P is piecewise constant on aggregates of m x m nodes aligned to the 4-node groups, so the
   // restriction P^T v is a sum of group sums and the prolongation adds one value per group.
   // Every CTA sends its partial sums for the aggregates its slab touches to every CTA of the
-  // cluster (16-byte stores of 4 aggregates); the next cluster barrier (the one of the
-  // following all-reduce) makes them visible.  coarse_gather then adds, chunk by chunk, the
-  // partials of the covering ranks in rank order and multiplies by the CTA's rows of Ac^-1.
+  // cluster (16-byte stores of 4 aggregates); comm.finish_tl() waits for all of them.
+  // coarse_gather then adds, chunk by chunk, the partials of the covering ranks in rank order
+  // and multiplies by the CTA's rows of Ac^-1.
   template <class T>
   __device__ void coarse_restrict_push(const T (&v)[NG][4]) {
     const int G = sb.G, m4 = P.cm / 4, nax = P.nax, naxp = coarse_row_stride(nax), ncp = naxp * P.nay;
@@ -720,8 +720,8 @@ struct Stepper {
   // so that I - M^-1 A = (I - S A)(I - P Ac^-1 P^T A)(I - S A) (symmetric).  The halo rows of r
   // (vrh) are the owners' rows, and every CTA computes ec for the
   // aggregate rows its halo rows touch from the same restricted vector, so y and u on a halo
-  // row equal the owner's values: M^-1 is one operator across the CTAs.  One cluster barrier
-  // (the restricted partials).  z goes to zbuf on the owned rows; returns the local (r, z).
+  // row equal the owner's values: M^-1 is one operator across the CTAs.  One all-to-all
+  // phase (the restricted partials).  z goes to zbuf on the owned rows; returns the local (r, z).
   __device__ V vcycle(const V (&r)[NG][4]) {
     const int W = sb.W, G = sb.G;
     float rf[NG][4];   // r in FP32, converted once (FP64 conversions run on the FP64 pipe)
@@ -816,9 +816,9 @@ struct Stepper {
   // Two-grid cycle with the slab-local smoother S_s of smooth_local before and after the coarse
   // correction: e1 = S_s r;  ec = Ac^-1 P^T (r - A e1);  u = e1 + P ec;  z = u + S_s (r - A u),
   // so that I - M^-1 A = (I - S_s A)(I - P Ac^-1 P^T A)(I - S_s A).  e1's edge rows are
-  // exchanged (a cluster barrier) before the residual; u on the halo rows is then the owner's
-  // value (e1 from the owner, ec computed from the same restricted vector).  Two cluster
-  // barriers.  z goes to zbuf on the owned rows; returns the local (r, z).
+  // exchanged before the residual; u on the halo rows is then the owner's value (e1 from the
+  // owner, ec computed from the same restricted vector).  One neighbour exchange and one
+  // all-to-all phase.  z goes to zbuf on the owned rows; returns the local (r, z).
   __device__ V vcycle_local(const V (&r)[NG][4]) {
     const int W = sb.W, G = sb.G;
     float rf[NG][4], e[NG][4], w[NG][4];
@@ -1038,7 +1038,8 @@ struct Stepper {
   // A2 = P2^T A1 P2.  Each level's correction is the exact adjoint of its restriction and every
   // smoother is symmetric, so M^-1 is symmetric.  Values on halo rows equal the owners' (e0 and
   // e1 exchanged, ec from the same restricted vector in every CTA, z1 exchanged), so M^-1 is one
-  // operator across the CTAs.  Five cluster barriers.  z goes to zbuf; returns the local (r, z).
+  // operator across the CTAs.  Four neighbour exchanges and one all-to-all
+  // phase.  z goes to zbuf; returns the local (r, z).
   __device__ V vcycle3(const V (&r)[NG][4]) {
     const int W = sb.W;
     float e[NG][4], w[NG][4];
@@ -1126,9 +1127,6 @@ struct Stepper {
   // not read, so the neighbours may already be writing their new edge rows into them.  No
   // communication; two block barriers.  z goes to zbuf; returns the local (r, z).
   __device__ V precond_local2(const V (&r)[NG][4]) {
-    if constexpr (!kMixed) {
-      return V{};       // not used: FP64 CG has no FP32 element weights
-    } else {
     const float om = P.tl_omega;
     float e[NG][4];
 #pragma unroll
@@ -1170,7 +1168,6 @@ struct Stepper {
       }
     }
     return rz;
-    }
   }
 
   // z = M^-1 r to zbuf (owned rows); returns the local (r, z)

@@ -1043,7 +1043,7 @@ struct Streamer {
         const V rz_c = rz;
         allreduce<V, 2, 1>(v, [rz_c, start](V* t) { if (!start) t[2] = vdiv(t[0], rz_c); });
         ++it;
-        if (!start && !(f32(v[1]) > target2)) done = true;   // NaN keeps iterating until the limit
+        if (!start && !(f32(v[1]) > target2)) done = true;   // a NaN ends it too
         beta = v[2];
         rz = v[0];
         if (done || it >= P.itmax) break;
